@@ -492,8 +492,9 @@ template <int S, int MODE>
 struct RowCfg {
     static constexpr int BK = Pipe<S, MODE>::BK;
     static constexpr int A_TILE = NP * BK * 2;                 // 4 or 8 KB
-    // fixed-matrix rows of a stage: 2 x 48 at N = 96 (EPI_SLICEH), else up to 128
-    static constexpr int BROWS = MODE == EPI_SLICEH ? 96 : NP;
+    // fixed-matrix rows of a stage: up to 128 in the two-pass modes (2 x 48 in EPI_SLICEH), 64 in
+    // the one-pass modes, whose tiles are at most 32 complex columns wide
+    static constexpr int BROWS = MODE == EPI_SLICEH ? 96 : Pipe<S, MODE>::two ? NP : 64;
     static constexpr int B_TILE = BROWS * BK * 2;
     static constexpr int STAGE_BYTES = S * (A_TILE + B_TILE);
     // level-3 hold: [4 column groups][8 float4 slots][128 rows]
@@ -2120,6 +2121,11 @@ static void launch_rows(Plan& p, const char* name, const DataOp& A, const FixedO
         a.num_tiles = a.num_tiles / a.ncol_tiles * (rad / wide);
         a.ncol_tiles = rad / wide;
         a.bnc = wide;
+    }
+    if (!Pipe<S, MODE>::two && a.bnc > 32) {   // one-pass stages hold 32 columns (see RowCfg)
+        a.num_tiles = a.num_tiles / a.ncol_tiles * (a.bnc * a.ncol_tiles / 32);
+        a.ncol_tiles = a.bnc * a.ncol_tiles / 32;
+        a.bnc = 32;
     }
     a.kch = (kprime + bk - 1) / bk;            // K' past kprime holds zeros on both sides
     a.lgR = (a.R > 0 && (a.R & (a.R - 1)) == 0) ? __builtin_ctzll((unsigned long long)a.R) : -1;
