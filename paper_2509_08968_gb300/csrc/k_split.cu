@@ -226,16 +226,26 @@ __device__ __forceinline__ long long df_round_i64(dfl x)
     return ((long long)t << 24) + __float2int_rn(rem + x.lo);
 }
 
-// Per-row values of the quotient epilogues.
-struct RowInfo {
-    double2 sigma;        // sum of the row's p eigenvalues minus lambda_i (lambda_{p_N} alone
-                          // when the per-column sums carry the rest)
-    double mult_base;     // N! / prod(run lengths)!
+// One row of the divide's operand (a slot): a sorted tuple (p_2 <= .. <= p_N). The table holds the
+// slots of one upper index (it does not depend on the index) and is refreshed with the modes.
+struct SlotRow {
+    double2 sigma;        // lambda_{p_2} + .. + lambda_{p_N}
     tfl sr, si;           // sigma as exact triple-floats
-    dfl f_row, f_first;   // mult_base / N! (and with the first run one longer) as double-floats
-    int run1;
-    float fmb;            // mult_base / N! in FP32 (exponent estimates)
+    dfl f_row, f_first;   // 1 / prod(run lengths)! of the tuple (f_first: the first run one longer)
+    float fmb;            // f_row in FP32 (exponent estimates)
+    int den, run1;        // prod(run lengths)!, length of the first run
+    int firstp;           // p_2, or -1 for a padding slot
+    int rbase;            // reduction row of (p_1, .., p_{N-1}) = rbase + p_1
+    int kpos;             // p_N, the K position in that row
+    int seg;              // segment within the 128-row tile; bit 8: the segment's first row
+    int pad;
 };
+// What the quotient reads per element, copied to shared memory (one per tile row).
+struct RowInfo {
+    tfl sr, si;
+    dfl f_row, f_first;
+};
+constexpr int SEGS = 8;   // segments a 128-row divide tile may hold
 
 // 1 / d for a small positive integer d as a double-float (relative error ~2^-46), without FP64.
 __device__ __forceinline__ dfl rcp_small(int d)
@@ -389,12 +399,7 @@ __global__ void k_prep_at(const double* __restrict__ A, int64_t P, int n,
 // column <= first p when `colmask`) and the padding (digits >= n) decide which tiles run (a tile
 // runs when any sub-block does) and which elements count.
 // ---------------------------------------------------------------------------------------
-enum { EPI_F64T = 0, EPI_SLICE = 1, EPI_DIVIDE = 2, EPI_SLAB = 3, EPI_REDUCE = 4, EPI_SLICEH = 5 };
-// EPI_SLICEH: the mode products' re-slicing epilogue on 48-column tiles (N = 96, three column
-// tiles per 128-wide radix) with the level-3 hold and two passes over K. An MMA at N = 96 costs
-// ~56 cycles against ~55 at N = 64 and 64 at N = 128 (back-to-back MMAs, M = 128, K = 16), and
-// the hold lets the level-3 pass of the next tile (15 of the 21 slice pairs) run beside the epilogue.
-__host__ __device__ constexpr bool is_slice(int mode) { return mode == EPI_SLICE || mode == EPI_SLICEH; }
+enum { EPI_F64T = 0, EPI_SLICE = 1, EPI_DIVIDE = 2, EPI_SLAB = 3, EPI_REDUCE = 4 };
 
 // Tensor maps of one operand: every slice plane in one box (`all`), and the planes of levels
 // 0..2 only (`low`, the second pass of a tile with the level-3 hold).
@@ -418,26 +423,34 @@ struct RowArgs {
     int digits;          // 1: r carries N-1 index digits (0 for the packed-tuple rows of P1)
     int rp;              // leading p digits in r
     int colmask;         // new column must be <= the first p
-    int kfrom;           // EPI_REDUCE: skip the K' chunks below the tile's last shared p
+    int kfrom;           // EPI_REDUCE: skip the K' chunks below the tile's smallest p_{N-1}
     int aswap;           // EPI_SLICE: only tiles with non-decreasing shared a's run, and each
                          // output row is also written for the swapped pair of shared a's
                          // (orders <= 4 have at most two shared a's)
-    int64_t R;           // rows per outer index (output layout [outer][q][r])
+    int64_t R;           // rows per outer index
+    int RB;              // > 0: every outer index starts a tile and has RB of them (the last one may
+                         // read rows of the next index, which are masked); 0: tiles of 128 rows run
+                         // over all rows
     int lgR;             // log2(R) when R is a power of two (digit rows), else -1
     int lgncol;          // log2(ncol_tiles), or -1 when ncol_tiles is not a power of two
-    // compact reduction rows (order >= 3, row radix 128): the reduction's operand rows are the
-    // sorted tuples (i, p_1 <= .. <= p_{N-1}) in lexicographic rank, RT rows per upper index (Q of
-    // them valid, then padding to whole tiles). EPI_DIVIDE writes them, EPI_REDUCE reads them.
-    int cmp;
-    int64_t Q, RT;
-    const int64_t* cnt;      // tuple-rank table: cnt[r*(n+1) + v] = non-decreasing r-tuples in [v, n)
-    const uint32_t* tuples;  // the sorted (N-1)-tuples in rank order, 8 bits per index
-    const float4* wpre;      // prod_{m <= N-2} W[p_m][k] per sorted (N-2)-tuple (rank) and k,
+    // EPI_SLICE, last mode product: output rows are the divide's slots, RS per upper index
+    int last;
+    int64_t RS;
+    const int* segbase;      // first slot of the segment (p_2, .., p_{N-1}), by its colex rank
+    // EPI_DIVIDE, EPI_SLAB: the slots; EPI_DIVIDE writes reduction rows, RT per upper index
+    const SlotRow* srow;
+    const uint32_t* stup;    // the slots' tuples, 8 bits per index (all ones: padding)
+    const int* tpmax;        // largest p_2 of each tile's slots
+    int64_t RT;
+    // EPI_REDUCE: rows are the sorted tuples (p_1 <= .. <= p_{N-1}) in colexicographic rank
+    const uint32_t* tuples;  // 8 bits per index
+    const float4* wpre;      // prod_{m <= N-2} W[p_m][k] per sorted (N-2)-tuple (colex rank) and k,
                              // as double-float complex
     const int* tiles;        // the tiles that run (nullptr: every tile, skipped ones tested)
     const unsigned* ntiles_run;   // their count
     int npc;             // extent of the new index in the output layout
     int lg;              // log2 of the row radix (digits, and the next operand's K extent)
+    int lgout;           // EPI_DIVIDE: log2 of the K extent of a reduction row
     int n;               // states (range of the a digits and of the reduction's columns k)
     int nm;              // modes in use (range of i and of the p digits; n unless a subset is set)
     int ncv;             // valid columns of this launch (modes, or states for the reduction)
@@ -449,9 +462,7 @@ struct RowArgs {
     int64_t ld_f64;
     // EPI_DIVIDE / EPI_SLAB / EPI_REDUCE
     const double2* lam;
-    const double2* V;        // psi_{p k} at p*n + k
-    const float4* psi_df;    // the same as double-float
-    const float* lam_t;      // lambda_p as exact triple-floats [n][Re a, b, c, Im a, b, c]
+    const float4* psi_df;    // the reduction weights W[p][k] (psi_{p k}) as double-float, at p*n + k
     int i0;
     double invfact, eps;
     int divide;
@@ -478,10 +489,10 @@ __device__ __forceinline__ unsigned long long global_ns()
 // fast as TMA refills shared memory, and a second pass would re-read planes 0..2.
 template <int S, int MODE>
 struct Pipe {
-    static constexpr bool two = Lev<S>::N == 4 && (MODE == EPI_DIVIDE || MODE == EPI_REDUCE || MODE == EPI_SLICEH);
+    static constexpr bool two = Lev<S>::N == 4 && (MODE == EPI_DIVIDE || MODE == EPI_REDUCE);
     // K' elements per stage: 16 (32-byte rows) where the 64 KB hold leaves three 48 KB stages,
-    // 32 (64-byte rows) otherwise (the 48-column tiles: two 84 KB stages beside a 48 KB hold)
-    static constexpr int BK = (two && MODE != EPI_SLICEH) ? 16 : 32;
+    // 32 (64-byte rows) otherwise
+    static constexpr int BK = two ? 16 : 32;
     static constexpr int KS = BK / KSTEP;        // MMA K steps per stage
     // K steps per stage of the second pass, which reads planes 0..2 only: as many as the
     // stage's S plane slots hold, so the ring keeps as many bytes in flight as in the first pass
@@ -492,40 +503,56 @@ template <int S, int MODE>
 struct RowCfg {
     static constexpr int BK = Pipe<S, MODE>::BK;
     static constexpr int A_TILE = NP * BK * 2;                 // 4 or 8 KB
-    // fixed-matrix rows of a stage: up to 128 in the two-pass modes (2 x 48 in EPI_SLICEH), 64 in
-    // the one-pass modes, whose tiles are at most 32 complex columns wide
-    static constexpr int BROWS = MODE == EPI_SLICEH ? 96 : Pipe<S, MODE>::two ? NP : 64;
+    // fixed-matrix rows of a stage: up to 128 in the two-pass modes, 64 in the one-pass modes, whose
+    // tiles are at most 32 complex columns wide (three 72 KB stages at six slices instead of two of
+    // 96 KB: the mode products wait for staging, not for the tensor core; n = 120, orders 3 + 4:
+    // 659 -> 614 ms a call)
+    static constexpr int BROWS = Pipe<S, MODE>::two ? NP : 64;
     static constexpr int B_TILE = BROWS * BK * 2;
     static constexpr int STAGE_BYTES = S * (A_TILE + B_TILE);
-    // level-3 hold: [4 column groups][8 float4 slots][128 rows]
     // level-3 hold: [4 column groups][HSLOT float4 slots][128 rows]; a thread holds the Re and Im
-    // level-3 values of its column units (up to 4 at 64 columns, 3 at 48)
-    static constexpr int HSLOT = MODE == EPI_SLICEH ? 6 : 8;
+    // level-3 values of its column units (up to 4 at 64 columns)
+    static constexpr int HSLOT = 8;
     static constexpr int HOLD_BYTES = Pipe<S, MODE>::two ? 4 * HSLOT * NP * 16 : 0;
-    // barriers, column tables, reduction partials and row tables (< 17 KB), and 1 KB of
-    // alignment slack
-    // (the re-slicing epilogue uses only the barriers and the column tables)
-    static constexpr int TABLES = is_slice(MODE) ? 3 * 1024 : 19 * 1024;
+    // barriers, column tables, reduction partials and row tables, and 1 KB of alignment slack
+    // (the other epilogues use only the barriers, the column tables and the output rows)
+    static constexpr int TABLES = MODE == EPI_DIVIDE || MODE == EPI_REDUCE ? 14 * 1024 : 4 * 1024;
     static_assert(2 * 8 * 8 + 5 * 8 + 8 <= 256, "barriers fit the first 256 bytes of the tables");
     static constexpr int SMEM_MAX = 227 * 1024;
     static constexpr int STAGES_FIT = (SMEM_MAX - TABLES - HOLD_BYTES) / STAGE_BYTES;
     static constexpr int STAGES = STAGES_FIT < 8 ? STAGES_FIT : 8;
     static constexpr int SMEM = STAGES * STAGE_BYTES + HOLD_BYTES + TABLES;
-    static_assert(STAGES >= 3 || ((!Pipe<S, MODE>::two || MODE == EPI_SLICEH) && STAGES >= 2), "pipeline stages");
+    static_assert(STAGES >= 3, "pipeline stages");
     static_assert(SMEM <= SMEM_MAX, "shared memory");
 };
 
-// Compact reduction input: the reduction launch (kfrom) with compact rows.
-#define MODE_IS_COMPACT_INPUT(a) ((a).cmp && (a).kfrom)
-// Column tile and first local row of a tile index (tiles are ordered row block major).
-__device__ __forceinline__ void tile_pos(const RowArgs& a, int64_t tile, int& ct, int64_t& row0)
+// Position of a tile (tiles are ordered row block major).
+struct TilePos {
+    int ct;         // column tile
+    int outer;      // upper index of the launch (RB > 0)
+    int rr0;        // first row within the upper index (RB > 0)
+    int64_t row0;   // first row of the operand
+};
+__device__ __forceinline__ TilePos tile_pos(const RowArgs& a, int64_t tile)
 {
-    if (a.lgncol >= 0) { ct = (int)(tile & (a.ncol_tiles - 1)); row0 = (tile >> a.lgncol) * NP; }
-    else { const int64_t rb = tile / a.ncol_tiles; ct = (int)(tile - rb * a.ncol_tiles); row0 = rb * NP; }
+    const unsigned t = (unsigned)tile;   // (launch_rows bounds the tile count to 2^31)
+    const unsigned rb = a.lgncol >= 0 ? t >> a.lgncol : t / (unsigned)a.ncol_tiles;
+    TilePos p;
+    p.ct = (int)(t - rb * (unsigned)a.ncol_tiles);
+    if (a.RB > 0) {
+        p.outer = (int)(rb / (unsigned)a.RB);
+        p.rr0 = (int)(rb - (unsigned)p.outer * (unsigned)a.RB) * NP;
+        p.row0 = (int64_t)p.outer * a.R + p.rr0;
+    } else {
+        p.outer = 0;
+        p.rr0 = 0;
+        p.row0 = (int64_t)rb * NP;
+    }
+    return p;
 }
 
-// Row index within / across the outer index (shifts for the power-of-two digit layouts: 64-bit
-// divisions by a runtime divisor cost ~70 instructions, and every role decodes every tile).
+// Row index within / across the outer index (RB = 0; shifts for the power-of-two digit layouts:
+// 64-bit divisions by a runtime divisor cost ~70 instructions, and every role decodes every tile).
 __device__ __forceinline__ int64_t row_in_outer(const RowArgs& a, int64_t o)
 {
     return a.lgR >= 0 ? (o & ((1ll << a.lgR) - 1)) : o % a.R;
@@ -557,34 +584,23 @@ __device__ __forceinline__ bool block_skipped(const RowArgs& a, int lg, int64_t 
 }
 
 // lg: the row radix (a compile-time 7 in the kernels without sub-blocks)
-__device__ __forceinline__ bool tile_skipped(const RowArgs& a, int lg, int64_t row0_local, int ct)
+__device__ __forceinline__ bool tile_skipped(const RowArgs& a, int lg, const TilePos& p)
 {
-    if (ct * a.bnc >= a.ncv) return true;                  // every column is padding
-    if (MODE_IS_COMPACT_INPUT(a)) return row_in_outer(a, row0_local) >= a.Q;   // padding rows
+    if (p.ct * a.bnc >= a.ncv) return true;                // every column is padding
+    if (a.tpmax) return p.ct * a.bnc > a.tpmax[p.rr0 / NP];   // slots: columns p_1 <= p_2
     if (!a.digits) return false;
     for (int sb = 0; sb < (NP >> lg); ++sb)
-        if (!block_skipped(a, lg, row0_local + ((int64_t)sb << lg), ct)) return false;
+        if (!block_skipped(a, lg, p.row0 + ((int64_t)sb << lg), p.ct)) return false;
     return true;
 }
 
-// First K' chunk a tile needs. In the reduction (kfrom = 1) the rows are (i, p_1..p_{N-1}) and
-// K = p_N; only non-decreasing tuples are formed, so every valid row of a tile has
-// p_N >= p_{N-1} >= p_{N-2} (its last shared digit) and the chunks below p_{N-2} are zero.
-__device__ __forceinline__ int first_chunk(const RowArgs& a, int lg, int64_t row0_local, int bk)
+// First K' chunk a tile needs. In the reduction (kfrom = 1) the rows are (p_1, .., p_{N-1}) in
+// colexicographic order and K = p_N >= p_{N-1}, which never decreases along the rows: the chunks
+// below the first row's p_{N-1} are not read.
+__device__ __forceinline__ int first_chunk(const RowArgs& a, const TilePos& p, int bk)
 {
-    if (!a.kfrom || a.N < 3) return 0;
-    if (MODE_IS_COMPACT_INPUT(a)) {
-        // rank order: p_1 never decreases along the rows, and every K = p_N >= p_1
-        const int r = (int)row_in_outer(a, row0_local);
-        return (int)(a.tuples[r] & 255u) / (bk / 2);
-    }
-    int d[8];
-    row_digits(row_in_outer(a, row0_local), a.N - 1, lg, d);   // sub-block 0: smallest p_{N-2}
-    int kmin = 0;
-#pragma unroll
-    for (int m = 0; m < 8; ++m)
-        if (m == a.N - 3) kmin = d[m];
-    return kmin / (bk / 2);   // bk / 2 complex K entries per stage of bk K'
+    if (!a.kfrom) return 0;
+    return (int)((a.tuples[p.rr0] >> (8 * (a.N - 2))) & 255u) / (bk / 2);
 }
 
 // Wait with the same limits and no early exit (draining copies after an error).
@@ -692,8 +708,7 @@ static __global__ void k_tile_list(RowArgs a, int lg, int* __restrict__ list, un
     const int64_t tile = (int64_t)blockIdx.x * 256 + threadIdx.x;
     bool run = false;
     if (tile < a.num_tiles) {
-        int ct; int64_t row0; tile_pos(a, tile, ct, row0);
-        run = !tile_skipped(a, lg, row0, ct);
+        run = !tile_skipped(a, lg, tile_pos(a, tile));
     }
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const unsigned bal = __ballot_sync(0xffffffffu, run);
@@ -709,8 +724,9 @@ static __global__ void k_tile_list(RowArgs a, int lg, int* __restrict__ list, un
 }
 
 static_assert(sizeof(tfl) == 12 && 6144 + 128 * sizeof(tfl) <= 7680, "table layout");
-static_assert(7680 + 128 * sizeof(RowInfo) + 1024 <= 19 * 1024, "tables and alignment slack");
-static_assert(1280 + 64 * 4 + 1024 <= 3 * 1024, "re-slicing tables (barriers, colE, colEb) and alignment slack");
+static_assert(7680 + 128 * sizeof(RowInfo) + 1024 <= 14 * 1024, "tables and alignment slack");
+static_assert(1536 + 4 * 64 * 4 + 1024 <= 4 * 1024, "re-slicing tables and alignment slack");
+static_assert(1536 + SEGS * 64 * 4 <= 5632, "the divide's segment exponents lie in the partials' place");
 
 template <int S, int MODE, bool SUBB>
 __global__ void __launch_bounds__(ROW_THREADS, 1)
@@ -733,9 +749,12 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
     uint64_t* t3empty = tempty + 2;            // epilogue -> MMA: level 3 copied to the hold
     uint32_t* tmem_slot = (uint32_t*)(t3empty + 1);
     int* stop = (int*)(tmem_slot + 1);
-    int* colE = (int*)(tables + 256);          // [4 sub-blocks][64] column exponent keys
+    // column exponent keys: [4 sub-blocks][64], or the divide's [SEGS][64] in the partials' place
+    int* colE = (int*)(tables + (MODE == EPI_DIVIDE ? 1536 : 256));
     int* colEb = (int*)(tables + 1280);        // 64 fixed-matrix column exponents
+    int* srowq = (int*)(tables + 1536);        // EPI_SLICE, last: [4 sub-blocks][64] output slots
     float4* red = (float4*)(tables + 1536);    // [4 lane quarters][64 columns] reduction partials
+    int* qpin = (int*)(tables + 5632);         // EPI_REDUCE: p_{N-1} of each lane quarter's rows, or -1
     float2* lamf = (float2*)(tables + 5632);   // 64 lambda_q in FP32 (exponent estimates)
     tfl* lamt = (tfl*)(tables + 6144);         // 64 x (Re, Im) lambda_q as exact triple-floats
     RowInfo* rowinfo = (RowInfo*)(tables + 7680);   // [128]
@@ -787,10 +806,11 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
             bool alive = true;
             for (int64_t k = blockIdx.x; k < nloop && alive; k += gridDim.x) {
                 const int64_t tile = args.tiles ? (int64_t)args.tiles[k] : k;
-                int ct; int64_t row0; tile_pos(args, tile, ct, row0);
-                if (!args.tiles && tile_skipped(args, lg, row0, ct)) continue;
-                const int bc = ct * bnc;
-                const int k0 = first_chunk(args, lg, row0, BKm);
+                const TilePos tp = tile_pos(args, tile);
+                if (!args.tiles && tile_skipped(args, lg, tp)) continue;
+                const int64_t row0 = tp.row0;
+                const int bc = tp.ct * bnc;
+                const int k0 = first_chunk(args, tp, BKm);
                 for (int pass = TWO ? 1 : 0; pass <= (TWO ? 2 : 0) && alive; ++pass) {
                     const int np = pass_planes<S>(pass);
                     const int kstride = pass == 2 ? Pipe<S, MODE>::P2 : 1;
@@ -838,9 +858,9 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
             bool alive = true;
             for (int64_t k = blockIdx.x; k < nloop && alive; k += gridDim.x) {
                 const int64_t tile = args.tiles ? (int64_t)args.tiles[k] : k;
-                int ct; int64_t row0; tile_pos(args, tile, ct, row0);
-                if (!args.tiles && tile_skipped(args, lg, row0, ct)) continue;
-                const int k0 = first_chunk(args, lg, row0, BKm);
+                const TilePos tp = tile_pos(args, tile);
+                if (!args.tiles && tile_skipped(args, lg, tp)) continue;
+                const int k0 = first_chunk(args, tp, BKm);
                 const int set = nset == 2 ? (int)(t & 1) : 0;
                 const uint32_t use = nset == 2 ? t >> 1 : t;     // earlier tiles on this set
                 const uint32_t tm = tmem + (uint32_t)set * (TMEM_COLS / 2);
@@ -923,31 +943,30 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
         uint32_t t = 0;
         for (int64_t k = blockIdx.x; k < nloop; k += gridDim.x) {
             const int64_t tile = args.tiles ? (int64_t)args.tiles[k] : k;
-            int ct; int64_t row0; tile_pos(args, tile, ct, row0);
-            if (!args.tiles && tile_skipped(args, lg, row0, ct)) continue;
+            const TilePos tp = tile_pos(args, tile);
+            if (!args.tiles && tile_skipped(args, lg, tp)) continue;
             unsigned long long* trc = args.trace ? args.trace + tile * 6 : nullptr;
-            const int qbase = ct * bnc;
-            const int64_t o = row0 + rl;                      // local row of the launch
-            const int ea = args.ea[o >> args.ea_shift];
-            const int64_t outer = outer_of(args, o);
-            const int64_t rr = row_in_outer(args, o);
-            const int64_t rblk = rr >> lg;                    // the next operand's row within [outer][q]
-            const int64_t rperq = args.R >> lg;
-            const int64_t row_base = outer * args.npc * rperq + rblk;   // + qc rperq: next row
-            const int kpos = rl & ((1 << lg) - 1);            // ... and the K position in it
+            const int qbase = tp.ct * bnc;
+            const int64_t o = tp.row0 + rl;                   // row of the operand
+            const int64_t outer = args.RB > 0 ? (int64_t)tp.outer : outer_of(args, o);
+            const int64_t rr = args.RB > 0 ? (int64_t)(tp.rr0 + rl) : row_in_outer(args, o);
+            const bool row_in = args.RB == 0 || rr < args.R;  // (a last block reads past its index)
+            const int ea = row_in ? args.ea[o >> args.ea_shift] : 0;
             const int sb = rl >> lg;                          // sub-block of the tile (warp-uniform)
             // columns of this tile that any row uses: below the modes in use and, with the
-            // sorted-tuple mask, at most the largest leading p of the tile's sub-blocks. Columns
+            // sorted-tuple mask, at most the largest leading p of the tile's rows. Columns
             // past them are neither read nor written (the rows they would fill are never used),
             // so the column groups split only the used ones, in units of 4.
             int vcols = min(bnc, args.ncv - qbase);
-            if (args.colmask && args.digits && args.rp >= 1 && N - 1 >= 2) {
+            if (MODE == EPI_DIVIDE) {
+                vcols = min(vcols, args.tpmax[tp.rr0 / NP] - qbase + 1);
+            } else if (MODE == EPI_SLICE && args.colmask && N - 1 >= 2) {
                 // the leading p is a shared digit (for N - 1 = 1 it is the innermost one and
                 // takes every value within a sub-block)
                 int pmax = 0;
                 for (int b = 0; b < (NP >> lg); ++b) {
                     int d0[8];
-                    row_digits(row_in_outer(args, row0 + ((int64_t)b << lg)), N - 1, lg, d0);
+                    row_digits(row_in_outer(args, tp.row0 + ((int64_t)b << lg)), N - 1, lg, d0);
                     pmax = max(pmax, d0[0]);
                 }
                 vcols = min(vcols, pmax - qbase + 1);
@@ -956,12 +975,42 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
             const int cbeg = 4 * ((grp * units) / NGRP);
             const int cols = 4 * (((grp + 1) * units) / NGRP) - cbeg;
 
-            // row digits: the first rp are p's (must be in order and < n), then a's (< n)
+            // Row digits (mode products): the first rp are p's (must be in order and < n), then
+            // a's (< n). The divide's and the slab's rows are slots: their tuple (p_2, .., p_N).
             int dg[8];
-            row_digits(rr, N - 1, lg, dg);
-            bool row_ok = true;
-            int firstp = NP;
-            if (args.digits) {
+            bool row_ok = row_in;
+            int firstp = NP;                                  // the new index is <= firstp
+            int warpp = NP;                                   // largest firstp of the warp's rows
+            int rbase = 0, kpos = 0, seg = 0, run1 = 1;
+            bool segfirst = false;
+            float fmb = 1.0f;
+            if (MODE == EPI_DIVIDE) {
+                const SlotRow& sr = args.srow[rr];            // (the table covers whole tiles)
+                firstp = sr.firstp;
+                row_ok = firstp >= 0;
+                rbase = sr.rbase;
+                kpos = sr.kpos;
+                seg = sr.seg & 255;
+                segfirst = (sr.seg & 256) != 0;
+                run1 = sr.run1;
+                fmb = sr.fmb;
+                warpp = __reduce_max_sync(0xffffffffu, firstp);
+                if (grp == 2) {
+                    RowInfo ri;
+                    ri.sr = sr.sr;
+                    ri.si = sr.si;
+                    ri.f_row = sr.f_row;
+                    ri.f_first = sr.f_first;
+                    rowinfo[rl] = ri;
+                }
+            } else if (MODE == EPI_SLAB) {
+                const uint32_t tup = N >= 2 ? args.stup[rr] : 0u;
+#pragma unroll
+                for (int m = 0; m < 8; ++m) dg[m] = m < N - 1 ? (int)((tup >> (8 * (m & 3))) & 255u) : 0;
+                row_ok = N >= 2 ? tup != 0xFFFFFFFFu : outer < args.nouter;
+                if (N >= 2) firstp = row_ok ? dg[0] : -1;
+            } else if (MODE == EPI_SLICE) {
+                row_digits(rr, N - 1, lg, dg);
 #pragma unroll
                 for (int m = 0; m < 7; ++m) {
                     if (m < N - 1) {
@@ -970,179 +1019,97 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                     }
                 }
                 if (args.rp >= 1) firstp = dg[0];
-                // rows past the batch: sub-blocks, and order 1 (one row per upper index)
-                if (SUBB || args.R == 1) row_ok &= outer < args.nouter;
+                if (SUBB) row_ok &= outer < args.nouter;      // rows past the batch
+                kpos = rl & ((1 << lg) - 1);                  // K position in the next operand's row
             }
 
             // rows of the swapped pair of shared a's (digits rp, rp + 1 when both are shared):
             // offset of that row in the output's row index (shared digits, base 2^lg). A row
             // whose shared a's decrease is not formed: its output rows are the mirrored writes of
             // the non-decreasing one (its operand row was never written), so it writes nothing.
-            int64_t swap_off = 0;
+            int64_t swap_off = 0, row_base = 0;
             bool no_write = false;
-            if (is_slice(MODE) && args.aswap) {
-                const int j = args.rp, nd = N - 1;
-                if (j + 1 <= nd - 2) {
-                    if (dg[j] < dg[j + 1]) {
-                        const int64_t wj = ipow_rad(nd - 2 - j, lg), wj1 = ipow_rad(nd - 3 - j, lg);
-                        swap_off = (int64_t)(dg[j + 1] - dg[j]) * wj + (int64_t)(dg[j] - dg[j + 1]) * wj1;
+            const int64_t rperq = args.R >> lg;
+            if (MODE == EPI_SLICE) {
+                row_base = outer * args.npc * rperq + (rr >> lg);   // + qc rperq: next row
+                if (args.aswap) {
+                    const int j = args.rp, nd = N - 1;
+                    if (j + 1 <= nd - 2) {
+                        if (dg[j] < dg[j + 1]) {
+                            const int64_t wj = ipow_rad(nd - 2 - j, lg), wj1 = ipow_rad(nd - 3 - j, lg);
+                            swap_off = (int64_t)(dg[j + 1] - dg[j]) * wj + (int64_t)(dg[j] - dg[j + 1]) * wj1;
+                        }
+                        no_write = SUBB && dg[j] > dg[j + 1];   // (whole tiles are skipped at radix 128)
                     }
-                    no_write = SUBB && dg[j] > dg[j + 1];   // (whole tiles are skipped at radix 128)
                 }
+                if (SUBB && outer >= args.nouter) no_write = true;   // padding rows past the batch
             }
-            if (SUBB && outer >= args.nouter) no_write = true;   // padding rows past the batch
-            // per-tile tables: column exponents, the fixed matrix's column exponents, lambda_q
-            // (FP32 and as exact triple-floats); per row (one thread of each row): sigma of the
-            // row p's minus lambda_i, the multiplicity base and the first run length
-            // Divide tiles without sub-blocks share every row digit but the innermost (p_N), so
-            // D = sigma_row + lambda_q = (shared p's lambdas - lambda_i + lambda_q) + lambda_{p_N}:
-            // the bracket once per column in FP64, lambda_{p_N} per row from a triple-float
-            // table, the multiplicities from integer run lengths (FP64 runs at a small fraction
-            // of the FP32 rate, and the per-row sums and divisions made this set-up longer than
-            // the tile's epilogue).
+            // Per-tile tables. Column exponents; the divide's columns: lambda_q - lambda_i (FP32
+            // and as exact triple-floats), so that D = sigma_row + (lambda_q - lambda_i) needs no
+            // FP64 per row (FP64 runs at a small fraction of the FP32 rate); the last mode
+            // product's output slots.
             if (trc && et == 0) trc[5] = global_ns();         // set-up starts
-            // The three set-up jobs run on three warp groups at once: the column tables (warps of
-            // group 0), the column sums and eigenvalues (group 1), the row table (group 2).
-            const bool fastdiv = MODE == EPI_DIVIDE && !SUBB && !args.fp64_quotient;
-            if (et < 64) {
-#pragma unroll
-                for (int b = 0; b < 4; ++b) colE[64 * b + et] = 0;
-                colEb[et] = args.eb[qbase + et];
-            }
+            if (MODE == EPI_DIVIDE) colE[et] = 0;
+            else if (et < 256) colE[et] = 0;
+            if (et < 64) colEb[et] = args.eb[qbase + et];
             if (MODE == EPI_DIVIDE && et >= 128 && et < 192) {
-                {
-                    const int c = et - 128;
-                    const int q = qbase + c;
-                    double2 lq = q < args.ncv ? args.lam[q] : make_double2(0.0, 0.0);
-                    if (fastdiv) {
-                        lq = csub(lq, args.lam[args.i0 + (int)outer]);
-#pragma unroll
-                        for (int m = 0; m < 6; ++m)
-                            if (m < N - 2) lq = cadd(lq, args.lam[dg[m]]);
-                    }
-                    lamf[c] = make_float2((float)lq.x, (float)lq.y);
-                    lamt[2 * c] = to_tfl(lq.x);
-                    lamt[2 * c + 1] = to_tfl(lq.y);
-                    if (args.cmp) {
-                        // compact reduction row of (p_1 = q, the tile's shared p's)
-                        int tup[8];
-                        tup[0] = q;
-                        bool srt = q < args.ncv && q <= dg[0];
-#pragma unroll
-                        for (int m = 0; m < 6; ++m)
-                            if (m < N - 2) tup[m + 1] = dg[m];
-                        ((int*)red)[c] = srt ? (int)tuple_rank(tup, N - 1, args.cnt, n) : -1;
-                    }
-                }
+                const int c = et - 128;
+                const int q = qbase + c;
+                const double2 lq = q < args.ncv ? csub(args.lam[q], args.lam[args.i0 + (int)outer])
+                                                : make_double2(0.0, 0.0);
+                lamf[c] = make_float2((float)lq.x, (float)lq.y);
+                lamt[2 * c] = to_tfl(lq.x);
+                lamt[2 * c + 1] = to_tfl(lq.y);
             }
-            if (MODE == EPI_REDUCE && args.cmp && grp == 2) {
-                // compact rows: the row's tuple, its last index p_{N-1} and the rank of its prefix
-                const int64_t r = rr;
-                int v = -1;
-                if (r < args.Q) {
-                    const uint32_t tp = args.tuples[r];
-                    int tup[8];
-                    bool okr = true;
-#pragma unroll
-                    for (int m = 0; m < 7; ++m) {
-                        tup[m] = (int)((tp >> (8 * (m & 3))) & 255u);
-                        if (m < N - 1) okr &= tup[m] < args.nm;
+            if (MODE == EPI_SLICE && args.last && et >= 256) {
+                // output slot of (p_2 = q, the sub-block's shared p's); order 2: slot q
+                const int b = (et - 256) >> 6, c = et & 63, q = qbase + c;
+                int slot = q;
+                if (N >= 3) {
+                    slot = 0;
+                    int d0[8];
+                    const int64_t rb0 = tp.row0 + ((int64_t)b << lg);
+                    if (b < (NP >> lg)) row_digits(row_in_outer(args, rb0), N - 1, lg, d0);
+                    if (b < (NP >> lg) && q <= d0[0] && d0[0] < args.nm) {
+                        if (N == 3) slot = args.segbase[q] + d0[0] - q;
+                        else if (d0[1] >= d0[0] && d0[1] < args.nm)
+                            slot = args.segbase[d0[0] * (d0[0] + 1) / 2 + q] + d0[1] - d0[0];
                     }
-                    int pin = 0;
-#pragma unroll
-                    for (int m = 0; m < 7; ++m)
-                        if (m == N - 2) pin = tup[m];
-                    const int pre = N >= 3 ? (int)tuple_rank(tup, N - 2, args.cnt, n) : 0;
-                    v = okr ? (pin | (pre << 8)) : -1;
                 }
-                ((int*)rowinfo)[rl] = v;
+                srowq[64 * b + c] = slot;
             }
-            if (fastdiv && grp == 2) {
-                int den = 1, run = 1, r1 = 1;
-                bool first_run = true;
-                int pN = 0;
+            // sigma of the row's p's minus lambda_i in FP64 (slabs, and the FP64 quotient)
+            double2 sigma = make_double2(0.0, 0.0);
+            if (MODE == EPI_SLAB && row_ok) {
 #pragma unroll
-                for (int m = 1; m < 8; ++m) {
-                    if (m == N - 1) pN = dg[m - 1];
-                    if (m > N - 1) break;
-                    if (m < N - 1 && dg[m] == dg[m - 1]) {
-                        ++run;
-                    } else {
-                        if (first_run) r1 = run;
-                        first_run = false;
-                        for (int u = 2; u <= run; ++u) den *= u;
-                        run = 1;
-                    }
-                }
-                RowInfo ri;
-                ri.mult_base = 0.0;   // not read on this path
-                ri.run1 = r1;
-                ri.fmb = 1.0f / (float)den;
-                ri.f_row = rcp_small(den);
-                ri.f_first = rcp_small(den * (r1 + 1));
+                for (int m = 0; m < 7; ++m)
+                    if (m < N - 1) sigma = cadd(sigma, args.lam[dg[m]]);
+                sigma = csub(sigma, args.lam[args.i0 + (int)outer]);
+            }
+            if (MODE == EPI_DIVIDE && args.fp64_quotient && row_ok)
+                sigma = csub(args.srow[rr].sigma, args.lam[args.i0 + (int)outer]);
+            // EPI_REDUCE: the row's last index p_{N-1} and the rank of its prefix
+            int pin = 0, pre = -1;
+            bool uni = false;
+            if (MODE == EPI_REDUCE) {
                 if (row_ok) {
-                    const float* lt = args.lam_t + 6 * pN;
-                    ri.sr = {lt[0], lt[1], lt[2]};
-                    ri.si = {lt[3], lt[4], lt[5]};
-                    ri.sigma = args.lam[pN];
-                } else {
-                    ri.sr = {0.f, 0.f, 0.f};
-                    ri.si = {0.f, 0.f, 0.f};
-                    ri.sigma = make_double2(0.0, 0.0);
+                    const uint32_t tup = args.tuples[rr];
+                    const int p0 = (int)(tup & 255u), p1 = (int)((tup >> 8) & 255u);
+                    pin = (int)((tup >> (8 * (N - 2))) & 255u);
+                    if (N == 3) pre = p0;
+                    if (N >= 4) pre = p1 * (p1 + 1) / 2 + p0;
                 }
-                rowinfo[rl] = ri;
-            } else if ((MODE == EPI_DIVIDE || MODE == EPI_SLAB) && grp == 2) {
-                double2 sg = make_double2(0, 0);
-                const int np_row = args.rp;
-                if (row_ok) {
-#pragma unroll
-                    for (int m = 0; m < 7; ++m)
-                        if (m < np_row) sg = cadd(sg, args.lam[dg[m]]);
-                    sg = csub(sg, args.lam[args.i0 + (int)outer]);
-                }
-                double denom = 1.0;
-                int run = 1, r1 = 1;
-                bool first_run = true;
-#pragma unroll
-                for (int m = 1; m < 8; ++m) {
-                    if (m > np_row) break;
-                    if (m < np_row && dg[m] == dg[m - 1]) {
-                        ++run;
-                    } else {
-                        if (first_run) r1 = run;
-                        first_run = false;
-                        for (int u = 2; u <= run; ++u) denom *= u;
-                        run = 1;
-                    }
-                }
-                double nf = 1.0;
-                for (int u = 2; u <= N; ++u) nf *= u;
-                RowInfo ri;
-                ri.sigma = sg;
-                ri.mult_base = nf / denom;
-                ri.run1 = r1;
-                ri.sr = to_tfl(sg.x);
-                ri.si = to_tfl(sg.y);
-                const double f = args.invfact * ri.mult_base;
-                ri.f_row = to_dfl(f);
-                ri.f_first = to_dfl(f / (r1 + 1));
-                ri.fmb = (float)f;
-                rowinfo[rl] = ri;
+                // rows in colex order mostly share p_{N-1}: its weight is then applied once to the
+                // quarter's sum instead of to every element
+                const int hi = __reduce_max_sync(0xffffffffu, row_ok ? pin : -1);
+                const int lo = __reduce_min_sync(0xffffffffu, row_ok ? pin : NP);
+                uni = N >= 3 && hi >= 0 && hi == lo;
+                if (grp == 0 && lane == 0) qpin[q4] = uni ? hi : -1;
             }
             // another role's error is picked up every 8 tiles (the waits see it at once)
             if (et == 0 && (t & 7) == 0) *stop = *(volatile int*)args.err;
             epi_sync();
             if (*stop) break;                                // uniform over the epilogue warps
-            double2 sigma = make_double2(0, 0);
-            double mult_base = 1.0;
-            int run1 = 1;
-            float fmb = 1.0f;
-            if (MODE == EPI_DIVIDE || MODE == EPI_SLAB) {
-                sigma = rowinfo[rl].sigma;
-                mult_base = rowinfo[rl].mult_base;
-                run1 = rowinfo[rl].run1;
-                fmb = rowinfo[rl].fmb;
-            }
             if (trc && et == 0) {
                 trc[0] = global_ns();
                 trc[4] = blockIdx.x + 1;
@@ -1153,8 +1120,8 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
             const uint32_t trow = trow0 + (uint32_t)set * (TMEM_COLS / 2);
             const bool ok = __all_sync(0xffffffffu, tc::mbar_wait(&tfull[set], use & 1, args.err, kErrTimeout));
             tc::fence_after_sync();
-            // this thread's level-3 slots of the hold: Re columns of unit u at slot u, Im at 4 + u
-            // (Re columns of unit u at slot u, Im at HSLOT / 2 + u)
+            // this thread's level-3 slots of the hold: Re columns of unit u at slot u, Im at
+            // HSLOT / 2 + u
             constexpr int HS2 = C::HSLOT / 2;
             float4* held = hold + ((size_t)grp * C::HSLOT * NP + rl);
             if (TWO && ok) {
@@ -1179,9 +1146,9 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
             // V * 2^(ea+eb-VEXP) / N! (times the multiplicity for the reduction), divided by the
             // clamped denominator
             auto quotient = [&](long long Vr, long long Vi, int eb, int qc) -> double2 {
-                const double mult = (qc == firstp) ? mult_base / (run1 + 1) : mult_base;
-                const double sc = pow2d(ea + eb - VEXP) * args.invfact *
-                                  (MODE == EPI_DIVIDE ? mult : 1.0);
+                double f = args.invfact;                      // 1 / N!, or 1 / prod(run lengths)!
+                if (MODE == EPI_DIVIDE) f = 1.0 / (double)(args.srow[rr].den * (qc == firstp ? run1 + 1 : 1));
+                const double sc = pow2d(ea + eb - VEXP) * f;
                 double2 h = make_double2((double)Vr * sc, (double)Vi * sc);
                 if (args.divide) {
                     // h / D = h conj(D) / |D|^2, D clamped per Alg. 2 step 9
@@ -1197,15 +1164,22 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                 return h;
             };
 
-            if (is_slice(MODE) || MODE == EPI_DIVIDE) {
-                // pass 1: column exponents (max over the tile's valid rows). For the quotients an
-                // FP32 upper bound of |h| = |V| 2^(ea+eb-VEXP) f / |D| with a lower bound of the
-                // clamped |D| (FP32 error of sigma + lambda_q bounded by 4 ulp of its terms).
-                const float2 sf = make_float2((float)sigma.x, (float)sigma.y);
-
+            if (MODE == EPI_SLICE || MODE == EPI_DIVIDE) {
+                // pass 1: column exponents (max over the tile's valid rows, per next operand row).
+                // For the quotients an FP32 upper bound of |h| = |V| 2^(ea+eb-VEXP) f / |D| with a
+                // lower bound of the clamped |D| (FP32 error of the sum bounded by 4 ulp of its
+                // terms).
+                float2 sf = make_float2(0.f, 0.f);
+                int seg0 = 0, seg1 = 0;                       // segments of this warp's rows
+                if (MODE == EPI_DIVIDE) {
+                    sf = make_float2(rowinfo[rl].sr.a, rowinfo[rl].si.a);
+                    seg0 = __reduce_min_sync(0xffffffffu, row_ok ? seg : SEGS);
+                    seg1 = __reduce_max_sync(0xffffffffu, row_ok ? seg : -1);
+                }
                 if (ok) {
                     constexpr float deep = deep_level_bound(S);
                     for (int c4 = cbeg; c4 < cbeg + cols; c4 += 4) {
+                        if (MODE == EPI_DIVIDE && qbase + c4 > warpp) break;   // no row of the warp
                         uint32_t rv[2][4], iv[2][4];   // levels 0 and 1 only
                         tc::tmem_ld4(trow + c4, rv[0]);
                         tc::tmem_ld4(trow + c4 + lstride, rv[1]);
@@ -1221,30 +1195,36 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                             // L3) 2^30)
                             const float br = level_bound01(rv[0][c], rv[1][c], deep);
                             const float bi = level_bound01(iv[0][c], iv[1][c], deep);
-                            const bool valid = row_ok && !no_write && qc < args.ncv &&
-                                               (!args.colmask || qc <= firstp);
                             unsigned key = 0;
-                            if (is_slice(MODE)) {
+                            if (MODE == EPI_SLICE) {
+                                const bool valid = row_ok && !no_write && qc < args.ncv &&
+                                                   (!args.colmask || qc <= firstp);
                                 // bitlen(V) <= exponent(bound) + 30
                                 const float bm = fmaxf(br, bi);
                                 if (valid && bm > 0.f)
                                     key = (unsigned)(f32_exponent(bm) + 30 + ea + eb - VEXP + 8192);
-                            } else if (valid && (br > 0.f || bi > 0.f)) {
-                                float lb = 1.0f;
-                                if (args.divide) {
-                                    const float2 lq = lamf[cl];
-                                    const float dx = sf.x + lq.x, dy = sf.y + lq.y;
-                                    const float del = 2.4e-7f * (fabsf(sf.x) + fabsf(sf.y) +
-                                                                fabsf(lq.x) + fabsf(lq.y));
-                                    lb = fmaxf(sqrtf(fmaf(dx, dx, dy * dy)) - del, (float)args.eps);
+                                const unsigned wmax = __reduce_max_sync(0xffffffffu, key);
+                                if (lane == 0 && wmax) atomicMax(&colE[64 * sb + cl], (int)wmax);
+                            } else {
+                                if (qc < args.ncv && qc <= firstp && (br > 0.f || bi > 0.f)) {
+                                    float lb = 1.0f;
+                                    if (args.divide) {
+                                        const float2 lq = lamf[cl];
+                                        const float dx = sf.x + lq.x, dy = sf.y + lq.y;
+                                        const float del = 2.4e-7f * (fabsf(sf.x) + fabsf(sf.y) +
+                                                                    fabsf(lq.x) + fabsf(lq.y));
+                                        lb = fmaxf(sqrtf(fmaf(dx, dx, dy * dy)) - del, (float)args.eps);
+                                    }
+                                    const float fm = qc == firstp ? fmb / (float)(run1 + 1) : fmb;
+                                    const float hm = sqrtf(fmaf(br, br, bi * bi)) * fm / lb *
+                                                     (1.0f + 0.0009765625f);
+                                    key = (unsigned)(f32_exponent(hm) + 30 + ea + eb - VEXP + 8192);
                                 }
-                                const float fm = qc == firstp ? fmb / (float)(run1 + 1) : fmb;
-                                const float hm = sqrtf(fmaf(br, br, bi * bi)) * fm / lb *
-                                                 (1.0f + 0.0009765625f);
-                                key = (unsigned)(f32_exponent(hm) + 30 + ea + eb - VEXP + 8192);
+                                for (int g = seg0; g <= seg1; ++g) {
+                                    const unsigned wmax = __reduce_max_sync(0xffffffffu, seg == g ? key : 0u);
+                                    if (lane == 0 && wmax) atomicMax(&colE[64 * g + cl], (int)wmax);
+                                }
                             }
-                            const unsigned wmax = __reduce_max_sync(0xffffffffu, key);
-                            if (lane == 0 && wmax) atomicMax(&colE[64 * sb + cl], (int)wmax);
                         }
                     }
                 }
@@ -1253,21 +1233,10 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
             }
 
             if (MODE == EPI_REDUCE && ok) {
-                // G[c'][k] psi_{p_{N-1} k} in double-float, summed over the warp's 32 rows by a
-                // transposing butterfly: the first two exchanges halve the columns each lane
-                // carries (4 -> 2 -> 1), the last three finish one column per lane group
-                int pin = 0;   // innermost row digit p_{N-1} (static indices)
-#pragma unroll
-                for (int m = 0; m < 7; ++m)
-                    if (m == N - 2) pin = dg[m];
-                int pre = -1;  // compact rows: the prefix weight's rank, applied per element
-                bool rok = row_ok;
-                if (args.cmp) {
-                    const int v = ((const int*)rowinfo)[rl];
-                    rok = v >= 0;
-                    pin = v & 255;
-                    pre = N >= 3 ? (v >> 8) : -1;
-                }
+                // G[c'][k] times the weights of the row's p's in double-float, summed over the
+                // warp's 32 rows by a transposing butterfly: the first two exchanges halve the
+                // columns each lane carries (4 -> 2 -> 1), the last three finish one column per
+                // lane group
                 const bool b4 = (lane & 16) != 0, b3 = (lane & 8) != 0;
                 for (int c4 = cbeg; c4 < cbeg + cols; c4 += 4) {
                     uint32_t rv[4][4], iv[4][4];
@@ -1284,14 +1253,16 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                         pi[c] = {0.f, 0.f};
                         const dfl vr = level_sum_df(rv[0][c], rv[1][c], rv[2][c], rv[3][c]);
                         const dfl vi = level_sum_df(iv[0][c], iv[1][c], iv[2][c], iv[3][c]);
-                        if (rok && qc < args.ncv && (vr.hi != 0.f || vi.hi != 0.f)) {
+                        if (row_ok && qc < args.ncv && (vr.hi != 0.f || vi.hi != 0.f)) {
                             const int sc = ea + colEb[cl] - VEXP + 30;
                             const dfl gr = {ldexpf(vr.hi, sc), ldexpf(vr.lo, sc)};
                             const dfl gi = {ldexpf(vi.hi, sc), ldexpf(vi.lo, sc)};
-                            const float4 w = args.psi_df[(int64_t)pin * n + qc];
+                            // prod_{m <= N-2} W[p_m][k], and W[p_{N-1}][k] unless it is left to the sum
+                            const float4 w = pre >= 0 ? args.wpre[(int64_t)pre * n + qc]
+                                                      : args.psi_df[(int64_t)pin * n + qc];
                             dfl wr = {w.x, w.y}, wi = {w.z, w.w};
-                            if (pre >= 0) {   // times prod_{m <= N-2} W[p_m][k] of the row
-                                const float4 x = args.wpre[(int64_t)pre * n + qc];
+                            if (pre >= 0 && !uni) {
+                                const float4 x = args.psi_df[(int64_t)pin * n + qc];
                                 const dfl xr = {x.x, x.y}, xi = {x.z, x.w};
                                 const dfl tr = df_add(df_mul(wr, xr), df_neg(df_mul(wi, xi)));
                                 wi = df_add(df_mul(wr, xi), df_mul(wi, xr));
@@ -1343,6 +1314,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
             if (MODE != EPI_REDUCE && ok) {
                 // pass 2 (or the only pass): outputs
                 for (int c4 = cbeg; c4 < cbeg + cols; c4 += 4) {
+                    if (MODE == EPI_DIVIDE && qbase + c4 > warpp) break;
                     uint32_t rv[4][4], iv[4][4];
                     const int u = (c4 - cbeg) / 4;
                     load_levels<S, TWO>(trow + c4, lstride, rv, held + (size_t)u * NP);
@@ -1353,12 +1325,12 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                         const int cl = c4 + c;
                         const int qc = qbase + cl;
                         const int eb = colEb[cl];
-                        const long long Vr = combine(rv[0][c], rv[1][c], rv[2][c], rv[3][c]);
-                        const long long Vi = combine(iv[0][c], iv[1][c], iv[2][c], iv[3][c]);
                         if (qc >= args.npc) continue;
                         if (MODE == EPI_F64T) {
                             if (qc < args.ncv) {
                                 const double sc = pow2d(ea + eb - VEXP);
+                                const long long Vr = combine(rv[0][c], rv[1][c], rv[2][c], rv[3][c]);
+                                const long long Vi = combine(iv[0][c], iv[1][c], iv[2][c], iv[3][c]);
                                 args.out_f64[(int64_t)qc * args.ld_f64 + o] =
                                     make_double2((double)Vr * sc, (double)Vi * sc);
                             }
@@ -1367,11 +1339,13 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                         const bool valid = row_ok && qc < args.ncv && (!args.colmask || qc <= firstp);
                         if (MODE == EPI_SLAB) {
                             // store h^i_{pre, q} when the multiset (q, row p's) minus pre is {extra}
+                            const long long Vr = combine(rv[0][c], rv[1][c], rv[2][c], rv[3][c]);
+                            const long long Vi = combine(iv[0][c], iv[1][c], iv[2][c], iv[3][c]);
                             if (!valid || !(Vr | Vi)) continue;
                             const double2 h = quotient(Vr, Vi, eb, qc);
                             int tt[8];
                             tt[0] = qc;
-                            for (int m = 0; m < args.rp; ++m) tt[m + 1] = dg[m];
+                            for (int m = 0; m < N - 1; ++m) tt[m + 1] = dg[m];
                             int used[8] = {0, 0, 0, 0, 0, 0, 0, 0};
                             int matched = 0, extra = -1, nextra = 0;
                             for (int a = 0; a < N; ++a) {
@@ -1385,24 +1359,50 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                                 args.out_f64[(int64_t)(args.i0 + outer) * n + extra] = h;
                             continue;
                         }
-                        if (args.colmask && qc > firstp && is_slice(MODE)) continue;   // unused rows
-                        if (no_write) continue;
-                        int64_t rowp = row_base + (int64_t)qc * rperq;
-                        if (MODE == EPI_DIVIDE && args.cmp) {   // compact reduction row, if sorted
-                            const int rk = ((const int*)red)[cl];
-                            if (rk < 0) continue;
-                            rowp = outer * args.RT + rk;
-                        }
-                        const int key = colE[64 * sb + cl];
-                        const int E = key ? key - 8192 : EXP_NONE;
                         uint32_t w[S];
-                        if (key == 0 || !valid) {
+                        if (MODE == EPI_SLICE) {
+                            if ((args.colmask && qc > firstp) || no_write) continue;   // unused rows
+                            // the last mode product writes the divide's slots (rows of unused
+                            // shared p's have none)
+                            if (args.last && N >= 3 && (firstp >= args.nm || (N >= 4 && (dg[1] < firstp || dg[1] >= args.nm))))
+                                continue;
+                            const int64_t rowp = args.last ? outer * args.RS + srowq[64 * sb + cl]
+                                                           : row_base + (int64_t)qc * rperq;
+                            const int key = colE[64 * sb + cl];
+                            const int E = key ? key - 8192 : EXP_NONE;
+                            if (key == 0 || !valid) {
+#pragma unroll
+                                for (int s = 0; s < S; ++s) w[s] = 0u;
+                            } else {
+                                const long long Vr = combine(rv[0][c], rv[1][c], rv[2][c], rv[3][c]);
+                                const long long Vi = combine(iv[0][c], iv[1][c], iv[2][c], iv[3][c]);
+                                const int sh = ea + eb - VEXP - E + 7 + 8 * (S - 1);
+                                digit_pairs<S>(shift_round(Vr, sh), shift_round(Vi, sh), w);
+                            }
+                            // next operand row rowp: 2^lg complex K entries (BF16 pairs), K = kpos
+                            uint32_t* dst = reinterpret_cast<uint32_t*>(args.out_planes) + (rowp << lg) + kpos;
+#pragma unroll
+                            for (int s = 0; s < S; ++s) dst[s * (args.out_plane_stride / 2)] = w[s];
+                            if (kpos == 0) args.out_exp[rowp] = E;
+                            if (swap_off != 0) {   // the same row, shared a's swapped
+                                uint32_t* d2 = dst + (swap_off << lg);
+#pragma unroll
+                                for (int s = 0; s < S; ++s) d2[s * (args.out_plane_stride / 2)] = w[s];
+                                if (kpos == 0) args.out_exp[rowp + swap_off] = E;
+                            }
+                            continue;
+                        }
+                        // EPI_DIVIDE: reduction row (p_1 = q, .., p_{N-1}), K = p_N
+                        if (!valid) continue;
+                        const int64_t rowp = outer * args.RT + rbase + qc;
+                        const int key = colE[64 * seg + cl];
+                        const int E = key ? key - 8192 : EXP_NONE;
+                        if (key == 0) {
 #pragma unroll
                             for (int s = 0; s < S; ++s) w[s] = 0u;
-                        } else if (is_slice(MODE)) {
-                            const int sh = ea + eb - VEXP - E + 7 + 8 * (S - 1);
-                            digit_pairs<S>(shift_round(Vr, sh), shift_round(Vi, sh), w);
                         } else if (args.fp64_quotient) {
+                            const long long Vr = combine(rv[0][c], rv[1][c], rv[2][c], rv[3][c]);
+                            const long long Vi = combine(iv[0][c], iv[1][c], iv[2][c], iv[3][c]);
                             const double2 h = quotient(Vr, Vi, eb, qc);
                             const double sc = pow2d(7 + 8 * (S - 1) - E);
                             digit_pairs<S>(__double2ll_rn(h.x * sc), __double2ll_rn(h.y * sc), w);
@@ -1434,49 +1434,42 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                             digit_pairs<S>(df_round_i64(dfl{ldexpf(qr.hi, k), ldexpf(qr.lo, k)}),
                                            df_round_i64(dfl{ldexpf(qi.hi, k), ldexpf(qi.lo, k)}), w);
                         }
-                        // next operand row rowp: 2^lg complex K entries (BF16 pairs), K = kpos
-                        uint32_t* dst = reinterpret_cast<uint32_t*>(args.out_planes) + (rowp << lg) + kpos;
+                        uint32_t* dst = reinterpret_cast<uint32_t*>(args.out_planes) + (rowp << args.lgout) + kpos;
 #pragma unroll
                         for (int s = 0; s < S; ++s) dst[s * (args.out_plane_stride / 2)] = w[s];
-                        if (kpos == 0) args.out_exp[rowp] = E;
-                        if (is_slice(MODE) && swap_off != 0) {   // the same row, shared a's swapped
-                            uint32_t* d2 = dst + (swap_off << lg);
-#pragma unroll
-                            for (int s = 0; s < S; ++s) d2[s * (args.out_plane_stride / 2)] = w[s];
-                            if (kpos == 0) args.out_exp[rowp + swap_off] = E;
-                        }
+                        // the row's first entry holds p_N = p_{N-1} (order 2: p_2 = p_1 = q)
+                        if (N >= 3 ? segfirst : kpos == qc) args.out_exp[rowp] = E;
                     }
                 }
             }
             if (MODE == EPI_REDUCE) {
-                // the four lane quarters' partials of every column, the prefix weight
-                // prod_{m<=N-2} psi_{p_m k}, and -sum into Psi_N[i][k]
+                // the four lane quarters' partials of every column, their common weight
+                // W[p_{N-1}][k] where it was left out, and -sum into Psi_N[i][k]
                 epi_sync();
                 const int cl = et;
                 const int qc = qbase + cl;
                 if (ok && cl < bnc && qc < args.ncv) {
-                    // each sub-block shares (i, p_1..p_{N-2}); its lane quarters' partials
-                    const int nsb = NP >> lg, qps = 4 / nsb;
-                    for (int b = 0; b < nsb; ++b) {
-                        dfl ar = {0.f, 0.f}, ai = {0.f, 0.f};
-                        for (int pp = 0; pp < qps; ++pp) {
-                            const float4 g = red[(b * qps + pp) * 64 + cl];
-                            ar = df_add(ar, dfl{g.x, g.y});
-                            ai = df_add(ai, dfl{g.z, g.w});
+                    dfl ar = {0.f, 0.f}, ai = {0.f, 0.f};
+                    double2 v = make_double2(0.0, 0.0);
+                    for (int pp = 0; pp < 4; ++pp) {
+                        const float4 g = red[pp * 64 + cl];
+                        ar = df_add(ar, dfl{g.x, g.y});
+                        ai = df_add(ai, dfl{g.z, g.w});
+                        const int wp = qpin[pp];
+                        if (pp < 3 && qpin[pp + 1] == wp) continue;   // same weight: one product
+                        double2 s = make_double2(df_to_d(ar), df_to_d(ai));
+                        if (wp >= 0) {
+                            const float4 x = args.psi_df[(int64_t)wp * n + qc];
+                            s = cmul(s, make_double2((double)x.x + (double)x.y, (double)x.z + (double)x.w));
                         }
-                        if (ar.hi == 0.f && ai.hi == 0.f) continue;
-                        // recover (i, p_1..p_{N-2}) from the sub-block's first row
-                        const int64_t rb = row0 + ((int64_t)b << lg);
-                        int d0[8];
-                        row_digits(row_in_outer(args, rb), N - 1, lg, d0);
-                        double2 wgt = make_double2(1.0, 0.0);   // compact rows: applied already
-#pragma unroll
-                        for (int m = 0; m < 6; ++m)
-                            if (m < N - 2 && !args.cmp) wgt = cmul(wgt, args.V[(int64_t)d0[m] * n + qc]);
-                        const int i = args.i0 + (int)outer_of(args, rb);
-                        const double2 v = cmul(make_double2(df_to_d(ar), df_to_d(ai)), wgt);
-                        atomicAdd(&args.out_f64[(int64_t)i * n + qc].x, -v.x);
-                        atomicAdd(&args.out_f64[(int64_t)i * n + qc].y, -v.y);
+                        v = cadd(v, s);
+                        ar = {0.f, 0.f};
+                        ai = {0.f, 0.f};
+                    }
+                    if (v.x != 0.0 || v.y != 0.0) {
+                        const int64_t at = (int64_t)(args.i0 + tp.outer) * n + qc;
+                        atomicAdd(&args.out_f64[at].x, -v.x);
+                        atomicAdd(&args.out_f64[at].y, -v.y);
                     }
                 }
             }
@@ -1660,6 +1653,79 @@ __global__ void k_expand_sorted(const uint4* __restrict__ rec, int64_t P, int n,
     }
 }
 
+// Slot rows (SlotRow) of the tuples tup[0, count): eigenvalue sums, run lengths and the place in
+// the reduction's operand.
+static __global__ void k_slot_rows(int N, int64_t count, const uint32_t* __restrict__ tup,
+                                   const int* __restrict__ segs, const double2* __restrict__ lam,
+                                   SlotRow* __restrict__ out)
+{
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= count) return;
+    SlotRow r{};
+    r.firstp = -1;
+    r.den = 1;
+    r.run1 = 1;
+    const uint32_t t = tup[idx];
+    if (t != 0xFFFFFFFFu) {
+        int d[3];
+        double2 sg = make_double2(0.0, 0.0);
+        const int np = N - 1;
+        for (int m = 0; m < 3; ++m) {
+            d[m] = (int)((t >> (8 * m)) & 255u);
+            if (m < np) sg = cadd(sg, lam[d[m]]);
+        }
+        int den = 1, run = 1, r1 = 1;
+        bool first_run = true;
+        for (int m = 1; m <= np; ++m) {
+            if (m < np && d[m] == d[m - 1]) { ++run; continue; }
+            if (first_run) r1 = run;
+            first_run = false;
+            for (int u = 2; u <= run; ++u) den *= u;
+            run = 1;
+        }
+        r.sigma = sg;
+        r.sr = to_tfl(sg.x);
+        r.si = to_tfl(sg.y);
+        r.den = den;
+        r.run1 = r1;
+        r.fmb = 1.0f / (float)den;
+        r.f_row = rcp_small(den);
+        r.f_first = rcp_small(den * (r1 + 1));
+        r.firstp = d[0];
+        r.kpos = d[np - 1];
+        if (N == 3) r.rbase = d[0] * (d[0] + 1) / 2;
+        if (N == 4) r.rbase = d[1] * (d[1] + 1) * (d[1] + 2) / 6 + d[0] * (d[0] + 1) / 2;
+        r.seg = segs[idx];
+    }
+    out[idx] = r;
+}
+
+// Zeros in the reduction rows' K entries that its tiles read but the divide does not write: from
+// the chunk of the tile's smallest p_{N-1} up to the row's own p_{N-1}, and from nm to the end of
+// the last chunk. kc: complex K entries a chunk. One thread per (upper index, row, 8th entry).
+template <int S>
+__global__ void k_zero_heads(int N, int nm, int kc, int lg, int Q, int64_t RT, int nouter,
+                             const uint32_t* __restrict__ tuples, uint32_t* __restrict__ planes,
+                             int64_t plane_stride_u32)
+{
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int e = (int)(idx & 7);
+    const int64_t row = idx >> 3;
+    if (row >= (int64_t)Q * nouter) return;
+    const int outer = (int)(row / Q), r = (int)(row - (int64_t)outer * Q);
+    const int sh = 8 * (N - 2);
+    const int p = (int)((tuples[r] >> sh) & 255u);
+    const int p0 = (int)((tuples[r & ~(NP - 1)] >> sh) & 255u);
+    uint32_t* dst = planes + (((int64_t)outer * RT + r) << lg);
+    for (int k = p0 / kc * kc + e; k < p; k += 8)
+#pragma unroll
+        for (int s = 0; s < S; ++s) dst[s * plane_stride_u32 + k] = 0u;
+    const int end = min(1 << lg, (nm + kc - 1) / kc * kc);
+    for (int k = nm + e; k < end; k += 8)
+#pragma unroll
+        for (int s = 0; s < S; ++s) dst[s * plane_stride_u32 + k] = 0u;
+}
+
 // Prefix weights of the compact reduction: out[t][k] = prod_{m < M} W[p_m][k] for the t-th sorted
 // M-tuple (p_0..p_{M-1}) (8 bits per index in tup[t]), FP64 products stored as double-float
 // complex (Re hi, Re lo, Im hi, Im lo).
@@ -1691,7 +1757,6 @@ struct SplitOperand {
     __nv_bfloat16* psir = nullptr;  int* psir_e = nullptr;   // Psi, real K (j), columns i
     __nv_bfloat16* red = nullptr;   int* red_e = nullptr;    // Psi^T rows k, complex K (p)
     float4* psi_df = nullptr;
-    float* lam_t = nullptr;         // lambda_p as exact triple-floats [n][Re a, b, c, Im a, b, c]
     int* tile_list = nullptr;       // running tiles of the current launch (k_tile_list)
     unsigned* tile_count = nullptr;
     int64_t tile_cap = 0;
@@ -1702,6 +1767,18 @@ struct SplitOperand {
     uint32_t* prefixes[kMaxOrder + 1] = {};   // non-decreasing (a_1..a_{N-1}), 8 bits per index
     int64_t nprefix[kMaxOrder + 1] = {};
     const double* at_src[kMaxOrder + 1] = {};
+    // per order, for the modes in use: the divide's slots (128 a tile) and the tables around them
+    int slot_nm[kMaxOrder + 1] = {};          // modes the tables were built for (0: none)
+    int slot_tiles[kMaxOrder + 1] = {};
+    SlotRow* srow[kMaxOrder + 1] = {};
+    uint32_t* stup[kMaxOrder + 1] = {};
+    int* sseg[kMaxOrder + 1] = {};
+    int* stpmax[kMaxOrder + 1] = {};
+    int* segbase[kMaxOrder + 1] = {};
+    // sorted M-tuples over the modes in use in colexicographic order, 8 bits per index
+    uint32_t* ptup[4] = {};
+    int64_t nptup[4] = {};
+    int ptup_nm[4] = {};
     int* err = nullptr;
     // reduction weights other than Psi (mode-interaction NPFs): planes of W^T, exponents, W in
     // double-float
@@ -1859,12 +1936,16 @@ void split_release(Plan& p)
     cudaFree(so->psir); cudaFree(so->psir_e);
     cudaFree(so->red); cudaFree(so->red_e);
     cudaFree(so->psi_df);
-    cudaFree(so->lam_t);
     cudaFree(so->tile_list);
     cudaFree(so->tile_count);
     for (int N = 0; N <= kMaxOrder; ++N) { cudaFree(so->at[N]); cudaFree(so->at_e[N]); }
     cudaFree(so->wred); cudaFree(so->wred_e); cudaFree(so->w_df);
-    for (int N = 0; N <= kMaxOrder; ++N) cudaFree(so->prefixes[N]);
+    for (int N = 0; N <= kMaxOrder; ++N) {
+        cudaFree(so->prefixes[N]);
+        cudaFree(so->srow[N]); cudaFree(so->stup[N]); cudaFree(so->sseg[N]);
+        cudaFree(so->stpmax[N]); cudaFree(so->segbase[N]);
+    }
+    for (int M = 0; M < 4; ++M) cudaFree(so->ptup[M]);
     cudaFree(so->err);
     delete so;
     p.split = nullptr;
@@ -1887,12 +1968,8 @@ static void set_smem_attrs()
     smem_attr<S, EPI_SLICE, false>();
     smem_attr<S, EPI_SLICE, true>();
     smem_attr<S, EPI_DIVIDE, false>();
-    smem_attr<S, EPI_DIVIDE, true>();
     smem_attr<S, EPI_SLAB, false>();
-    smem_attr<S, EPI_SLAB, true>();
     smem_attr<S, EPI_REDUCE, false>();
-    smem_attr<S, EPI_REDUCE, true>();
-    if constexpr (S == 4 || S == 6) smem_attr<S, EPI_SLICEH, false>();
     done = true;
 }
 
@@ -1934,21 +2011,6 @@ static void fill_fixed(Plan& p, SplitOperand* so)
         pdf[t] = make_float4(rh, (float)(V[t].x - rh), ih, (float)(V[t].y - ih));
     }
     put(so->psi_df, pdf);
-    // eigenvalues as exact triple-floats (24 + 24 + 5 significant bits of a double)
-    std::vector<double2> lam(n);
-    NPF_CUDA(cudaMemcpy(lam.data(), p.d_lam, n * sizeof(double2), cudaMemcpyDeviceToHost));
-    std::vector<float> lt((size_t)6 * n);
-    auto split3 = [](double x, float* o) {
-        o[0] = (float)x;
-        const double r = x - (double)o[0];
-        o[1] = (float)r;
-        o[2] = (float)(r - (double)o[1]);
-    };
-    for (int q = 0; q < n; ++q) {
-        split3(lam[q].x, &lt[6 * q]);
-        split3(lam[q].y, &lt[6 * q + 3]);
-    }
-    put(so->lam_t, lt);
 }
 
 static SplitOperand& prepare(Plan& p)
@@ -1986,12 +2048,101 @@ static void prepare_weights(Plan& p, SplitOperand& so, const double2* dW)
     put(so.w_df, wdf);
 }
 
+// Slot rows of the order's tuples from the plan's eigenvalues.
+static void fill_slots(Plan& p, SplitOperand& so, int N)
+{
+    const int64_t count = (int64_t)so.slot_tiles[N] * NP;
+    LaunchScope ls(&p.prof, "split_slot_rows", p.stream);
+    k_slot_rows<<<(unsigned)((count + 127) / 128), 128, 0, p.stream>>>(N, count, so.stup[N], so.sseg[N],
+                                                                      p.d_lam, so.srow[N]);
+    NPF_CUDA(cudaGetLastError());
+}
+
 #ifndef NPF_SPLIT_LOW
 void split_refresh_modes(Plan& p)
 {
-    if (p.split) fill_fixed(p, p.split);   // same n and S: the buffers (and graphs) stay valid
+    if (!p.split) return;
+    fill_fixed(p, p.split);   // same n and S: the buffers (and graphs) stay valid
+    bool any = false;
+    for (int N = 2; N <= 4; ++N)
+        if (p.split->slot_nm[N] == p.nm) { fill_slots(p, *p.split, N); any = true; }
+    if (any) NPF_CUDA(cudaStreamSynchronize(p.stream));   // (a batch's graph runs on other streams)
 }
 #endif
+
+// Sorted M-tuples (1 <= M <= 3) over the modes in use, colexicographic.
+static void ensure_ptuples(Plan& p, SplitOperand& so, int M)
+{
+    if (so.ptup_nm[M] == p.nm) return;
+    cudaFree(so.ptup[M]);
+    so.ptup[M] = nullptr;
+    so.ptup_nm[M] = 0;
+    std::vector<uint32_t> t;
+    for (int r = 0; r < (M >= 3 ? p.nm : 1); ++r)
+        for (int q = 0; q < (M >= 3 ? r + 1 : M == 2 ? p.nm : 1); ++q)
+            for (int x = 0; x < (M >= 2 ? q + 1 : p.nm); ++x)
+                t.push_back((uint32_t)x | (M >= 2 ? (uint32_t)q << 8 : 0u) | (M >= 3 ? (uint32_t)r << 16 : 0u));
+    so.ptup[M] = upload(t);
+    so.nptup[M] = (int64_t)t.size();
+    so.ptup_nm[M] = p.nm;
+}
+
+// The slots of order N: the sorted tuples (p_2 <= .. <= p_N) in 128-row tiles. A segment (the
+// tuples that share p_2 .. p_{N-1}) fills one row of the reduction's operand per p_1, whose
+// exponent it shares, so it never straddles two tiles. A tile runs the columns p_1 <= its largest
+// p_2, so it takes segments of nearby p_2 only (within 8), the longest first.
+static void ensure_slots(Plan& p, SplitOperand& so, int N)
+{
+    if (so.slot_nm[N] == p.nm) return;
+    cudaFree(so.srow[N]); cudaFree(so.stup[N]); cudaFree(so.sseg[N]); cudaFree(so.stpmax[N]);
+    cudaFree(so.segbase[N]);
+    so.srow[N] = nullptr; so.stup[N] = nullptr; so.sseg[N] = nullptr; so.stpmax[N] = nullptr;
+    so.segbase[N] = nullptr;
+    so.slot_nm[N] = 0;
+    const int nm = p.nm;
+    struct Seg { int p2, p3, len; };         // p3: the last shared p (p_{N-1})
+    std::vector<Seg> segs;
+    if (N == 2) segs.push_back({nm - 1, 0, nm});
+    for (int p2 = 0; N >= 3 && p2 < nm; ++p2)
+        for (int p3 = p2; p3 < (N == 3 ? p2 + 1 : nm); ++p3) segs.push_back({p2, p3, nm - p3});
+    struct Bin { int p2, used; std::vector<int> seg; };
+    std::vector<Bin> bins;
+    size_t open = 0;                         // bins before it are full or of far smaller p_2
+    for (int g = 0; g < (int)segs.size(); ++g) {
+        while (open < bins.size() && (bins[open].p2 + 8 < segs[g].p2 || bins[open].used == NP)) ++open;
+        size_t b = open;
+        while (b < bins.size() && (bins[b].p2 + 8 < segs[g].p2 || bins[b].used + segs[g].len > NP ||
+                                   (int)bins[b].seg.size() >= SEGS)) ++b;
+        if (b == bins.size()) bins.push_back({segs[g].p2, 0, {}});
+        bins[b].seg.push_back(g);
+        bins[b].used += segs[g].len;
+    }
+    std::vector<uint32_t> tup(bins.size() * NP, 0xFFFFFFFFu);
+    std::vector<int> seg(bins.size() * NP, 0), tpmax(bins.size(), 0);
+    std::vector<int> base(N == 4 ? nm * (nm + 1) / 2 : N == 3 ? nm : 1, 0);
+    for (size_t b = 0; b < bins.size(); ++b) {
+        int pos = (int)b * NP;
+        for (int k = 0; k < (int)bins[b].seg.size(); ++k) {
+            const Seg& x = segs[bins[b].seg[k]];
+            tpmax[b] = std::max(tpmax[b], x.p2);
+            base[N == 4 ? x.p3 * (x.p3 + 1) / 2 + x.p2 : N == 3 ? x.p2 : 0] = pos;
+            for (int r = 0; r < x.len; ++r, ++pos) {
+                const uint32_t pn = (uint32_t)(N == 2 ? r : x.p3 + r);
+                tup[pos] = N == 2 ? pn : N == 3 ? (uint32_t)x.p2 | pn << 8
+                                                : (uint32_t)x.p2 | (uint32_t)x.p3 << 8 | pn << 16;
+                seg[pos] = k | (r == 0 ? 256 : 0);
+            }
+        }
+    }
+    so.slot_tiles[N] = (int)bins.size();
+    so.stup[N] = upload(tup);
+    so.sseg[N] = upload(seg);
+    so.stpmax[N] = upload(tpmax);
+    so.segbase[N] = upload(base);
+    NPF_CUDA(cudaMalloc(&so.srow[N], tup.size() * sizeof(SlotRow)));
+    so.slot_nm[N] = nm;
+    fill_slots(p, so, N);
+}
 
 // A^T digit planes of the packed tensor (part of the tensor upload; redone when the tensor or the
 // slice count changes).
@@ -2110,12 +2261,11 @@ static void launch_rows(Plan& p, const char* name, const DataOp& A, const FixedO
                         RowArgs a)
 {
     constexpr int bk = RowCfg<S, MODE>::BK;
-    if (Pipe<S, MODE>::two && MODE != EPI_SLICEH && a.bnc < 64) {
+    if (Pipe<S, MODE>::two && a.bnc < 64) {
         // the divide's and the reduction's two-pass tiles keep one TMEM accumulator set and the
         // level-3 hold, so a narrower tile only adds MMA issues (an M = 128 MMA costs ~55 cycles
         // at N <= 64, 64 at N = 128): they run 64 complex columns wide (or the whole radix)
-        // whatever the tuned width. (The 48-column mode-product tiles have stages and a hold
-        // sized for 48 columns and keep their width.)
+        // whatever the tuned width
         const int rad = a.bnc * a.ncol_tiles;
         const int wide = rad < 64 ? rad : 64;
         a.num_tiles = a.num_tiles / a.ncol_tiles * (rad / wide);
@@ -2133,28 +2283,29 @@ static void launch_rows(Plan& p, const char* name, const DataOp& A, const FixedO
     a.klast = (kprime + KSTEP - 1) / KSTEP - (bk / KSTEP) * (a.kch - 1);
     const TMaps tA = plane_maps<S>(A, bk);
     const TMaps tB = fixed_maps<S>(B, a.bnc, bk);
-    // the running tiles, listed on the device (stream order puts the list before the launch)
-    SplitOperand& so = *p.split;
-    if (!so.tile_list || so.tile_cap < a.num_tiles) {
-        if (p.capturing) fail(NPF_ERR_CUDA, "tile list would grow during graph capture");
-        cudaFree(so.tile_list);
-        cudaFree(so.tile_count);
-        so.tile_list = nullptr;
-        so.tile_count = nullptr;
-        NPF_CUDA(cudaMalloc(&so.tile_list, (size_t)a.num_tiles * sizeof(int)));
-        NPF_CUDA(cudaMalloc(&so.tile_count, sizeof(unsigned)));
-        so.tile_cap = a.num_tiles;
-    }
     if (a.num_tiles >= (int64_t)1 << 31) fail(NPF_ERR_UNSUPPORTED, "too many tiles in one launch");
-    NPF_CUDA(cudaMemsetAsync(so.tile_count, 0, sizeof(unsigned), p.stream));
-    {
+    if (MODE == EPI_SLICE || MODE == EPI_DIVIDE) {
+        // the running tiles, listed on the device (stream order puts the list before the launch);
+        // the other modes run every tile
+        SplitOperand& so = *p.split;
+        if (!so.tile_list || so.tile_cap < a.num_tiles) {
+            if (p.capturing) fail(NPF_ERR_CUDA, "tile list would grow during graph capture");
+            cudaFree(so.tile_list);
+            cudaFree(so.tile_count);
+            so.tile_list = nullptr;
+            so.tile_count = nullptr;
+            NPF_CUDA(cudaMalloc(&so.tile_list, (size_t)a.num_tiles * sizeof(int)));
+            NPF_CUDA(cudaMalloc(&so.tile_count, sizeof(unsigned)));
+            so.tile_cap = a.num_tiles;
+        }
+        NPF_CUDA(cudaMemsetAsync(so.tile_count, 0, sizeof(unsigned), p.stream));
         LaunchScope ls(&p.prof, "split_tile_list", p.stream);
         k_tile_list<<<(unsigned)((a.num_tiles + 255) / 256), 256, 0, p.stream>>>(a, a.lg, so.tile_list,
                                                                                 so.tile_count);
         NPF_CUDA(cudaGetLastError());
+        a.tiles = so.tile_list;
+        a.ntiles_run = so.tile_count;
     }
-    a.tiles = so.tile_list;
-    a.ntiles_run = so.tile_count;
     static const bool tracing = getenv("NPF_TRACE_TILES") != nullptr;
     unsigned long long* dtrace = nullptr;
     if (tracing) {
@@ -2170,7 +2321,7 @@ static void launch_rows(Plan& p, const char* name, const DataOp& A, const FixedO
         int64_t grid = std::min<int64_t>(a.num_tiles, sm_count());
         if (grid > 1 && a.ncol_tiles > 1 && grid % 2 == 0) grid -= 1;
         const unsigned g = (unsigned)std::max<int64_t>(grid, 1);
-        if constexpr (MODE != EPI_F64T && MODE != EPI_SLICEH) {   // (48-column tiles: radix 128 only)
+        if constexpr (MODE == EPI_SLICE) {
             if (a.lg < 7) k_rows<S, MODE, true><<<g, ROW_THREADS, RowCfg<S, MODE>::SMEM, p.stream>>>(tA, tB, a);
             else k_rows<S, MODE, false><<<g, ROW_THREADS, RowCfg<S, MODE>::SMEM, p.stream>>>(tA, tB, a);
         } else {
@@ -2221,10 +2372,9 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     set_smem_attrs<S>();
     prepare_tensor<S>(p, so, N);
     ensure_tuples(p, so, N);
-    // compact reduction rows (order >= 3, row radix 128): sorted (N-1)-tuples per upper index
-    const int lg_run = p.n <= 32 ? 5 : p.n <= 64 ? 6 : 7;
-    const bool cmp = lg_run == 7 && N >= 3 && prefix == nullptr;
-    if (cmp) ensure_tuples(p, so, N - 1);
+    if (N >= 2) ensure_slots(p, so, N);
+    if (N >= 2 && !prefix) ensure_ptuples(p, so, N - 1);
+    if (N == 4 && !prefix) ensure_ptuples(p, so, 2);
     int* const err = p.err_override ? p.err_override : so.err;   // a batch zeroes and checks its own
     if (!p.err_override) NPF_CUDA(cudaMemsetAsync(err, 0, sizeof(int), p.stream));
     const int n = p.n;
@@ -2237,13 +2387,9 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     const int lg = n <= 32 ? 5 : n <= 64 ? 6 : 7;
     const int rad = 1 << lg;
     const int64_t npN1 = ipow64(rad, N - 1);
-    // complex columns per tile. A width of 48 means 48-column mode-product tiles with the level-3 hold (the 4- and 6-slice
-    // forms at radix 128; three column tiles per radix) and 32 for every other launch and radix.
-    // The slab path runs untuned: 32 when the plan autotunes.
-    const int want = p.tile_n > 0 ? p.tile_n : 32;
-    bool wide48 = false;
-    if constexpr (S == 4 || S == 6) wide48 = want == 48 && lg == 7;
-    const int bnc = std::min(want == 48 ? 32 : want, rad);
+    // complex columns per tile (the slab path runs untuned: 32 when the plan autotunes); the mode
+    // products run at most 32 columns, the divide and the reduction 64 (launch_rows)
+    const int bnc = std::min(p.tile_n > 0 ? (p.tile_n == 48 ? 32 : p.tile_n) : 32, rad);
     const bool slab = prefix != nullptr;
 
     // ---- memory plan (Algorithm 1's rule on the upper-index space)
@@ -2257,11 +2403,10 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     const int64_t t_rows = ((int64_t)ib * npN1 + NP - 1) / NP * NP;
     const size_t tbytes = (size_t)t_rows * 2 * rad * 2 * S;
     const size_t ebytes = (size_t)t_rows * 4;
-    // compact reduction: RT rows per upper index, and the prefix weights of its rows
-    const int64_t Qc = so.nprefix[N];
-    const int64_t RTc = (Qc + NP - 1) / NP * NP;
-    const int64_t Q2 = cmp ? so.nprefix[N - 1] : 0;
-    const size_t wbytes = cmp && N >= 4 ? (size_t)Q2 * n * sizeof(float4) : 0;
+    // reduction rows per upper index (sorted (N-1)-tuples) and, at order 4, the weights of the pairs
+    const int64_t Qc = N >= 2 ? so.nptup[N - 1] : 0;
+    const int64_t Q2 = N == 4 && !slab ? so.nptup[2] : 0;
+    const size_t wbytes = (size_t)Q2 * n * sizeof(float4);
     Arena& ar = p.scratch();
     ar.reserve(s_bytes + rec_bytes + 2 * (tbytes + ebytes) + wbytes + 8 * 256 + 1024);
     uint8_t* base = (uint8_t*)ar.base;
@@ -2272,18 +2417,13 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     __nv_bfloat16* T[2] = {(__nv_bfloat16*)take(tbytes), (__nv_bfloat16*)take(tbytes)};
     int* E[2] = {(int*)take(ebytes), (int*)take(ebytes)};
     // order 3: the prefix weight is W itself (the double-float copy); order 4: pairs' products
-    const float4* wpre = nullptr;
-    if (cmp) {
-        if (N >= 4) {
-            float4* wp = (float4*)take(wbytes);
-            LaunchScope ls(&p.prof, "split_prefix_weights", p.stream);
-            k_prefix_weights<<<1024, 256, 0, p.stream>>>(N - 2, n, Q2, so.prefixes[N - 1],
-                                                         W ? W : p.d_V, wp);
-            NPF_CUDA(cudaGetLastError());
-            wpre = wp;
-        } else {
-            wpre = W ? so.w_df : so.psi_df;
-        }
+    const float4* wpre = W ? so.w_df : so.psi_df;
+    if (N == 4 && !slab) {
+        float4* wp = (float4*)take(wbytes);
+        LaunchScope ls(&p.prof, "split_prefix_weights", p.stream);
+        k_prefix_weights<<<1024, 256, 0, p.stream>>>(N - 2, n, Q2, so.ptup[2], W ? W : p.d_V, wp);
+        NPF_CUDA(cudaGetLastError());
+        wpre = wp;
     }
 
     // a slab entry whose accumulator is exactly zero is not stored, so the slab starts at zero
@@ -2302,9 +2442,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     base0.nm = nm;
     base0.ncv = nm;
     base0.N = N;
-    base0.V = W ? W : p.d_V;              // reduction weights (the prefix factors)
     base0.psi_df = W ? so.w_df : so.psi_df;
-    base0.lam_t = so.lam_t;
     base0.lam = p.d_lam;
     base0.invfact = 1.0 / factorial(N);
     base0.eps = p.eps;
@@ -2378,46 +2516,55 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
             a.out_plane_stride = t_rows * 2 * rad;
             a.out_exp = E[cb ^ 1];
             if (c < N) {
-                bool done48 = false;
-                if constexpr (S == 4 || S == 6) {
-                    if (wide48) {
-                        a.bnc = 48; a.ncol_tiles = 3; a.num_tiles = rows / NP * 3;
-                        launch_rows<S, EPI_SLICEH>(p, "split_mode_product", *tT[cb], tPhi, 2 * n, a);
-                        done48 = true;
-                    }
-                }
-                if (!done48) launch_rows<S, EPI_SLICE>(p, "split_mode_product", *tT[cb], tPhi, 2 * n, a);
-            } else if (slab) {
-                a.out_f64 = d_out;
-                launch_rows<S, EPI_SLAB>(p, "split_mode_divide", *tT[cb], tPhi, 2 * n, a);
+                a.last = c == N - 1;
+                a.RS = N == 2 ? rad : (int64_t)so.slot_tiles[N] * NP;
+                a.segbase = so.segbase[N];
+                launch_rows<S, EPI_SLICE>(p, "split_mode_product", *tT[cb], tPhi, 2 * n, a);
             } else {
-                a.cmp = cmp;
-                a.Q = Qc;
-                a.RT = RTc;
-                a.cnt = p.d_cnt;
-                launch_rows<S, EPI_DIVIDE>(p, "split_mode_divide", *tT[cb], tPhi, 2 * n, a);
+                if (N >= 2) {   // rows are slots
+                    a.digits = 0;
+                    a.ea_shift = 0;
+                    a.R = N == 2 ? rad : (int64_t)so.slot_tiles[N] * NP;
+                    a.RB = so.slot_tiles[N];
+                    a.srow = so.srow[N];
+                    a.stup = so.stup[N];
+                    a.num_tiles = (int64_t)cur * a.RB * a.ncol_tiles;
+                    a.lg = 7;
+                    a.lgout = lg;
+                }
+                if (slab) {
+                    a.out_f64 = d_out;
+                    launch_rows<S, EPI_SLAB>(p, "split_mode_divide", *tT[cb], tPhi, 2 * n, a);
+                } else {
+                    a.tpmax = so.stpmax[N];
+                    a.RT = Qc;
+                    launch_rows<S, EPI_DIVIDE>(p, "split_mode_divide", *tT[cb], tPhi, 2 * n, a);
+                }
             }
             cb ^= 1;
         }
         if (slab) continue;
-        // ---- reduction: rows c' = (i, p_1..p_{N-1}), K = p_N, columns k (Psi^T)
+        {
+            LaunchScope ls(&p.prof, "split_zero_heads", p.stream);
+            const int64_t tot = Qc * cur * 8;
+            k_zero_heads<S><<<(unsigned)((tot + 255) / 256), 256, 0, p.stream>>>(
+                N, nm, RowCfg<S, EPI_REDUCE>::BK / 2, lg, (int)Qc, Qc, cur, so.ptup[N - 1],
+                (uint32_t*)T[cb], t_rows * rad);
+            NPF_CUDA(cudaGetLastError());
+        }
+        // ---- reduction: rows c' = (i, p_1 <= .. <= p_{N-1}), K = p_N, columns k (Psi^T)
         RowArgs a = base0;
         a.a_rows = (int)t_rows;
         a.ncv = n;                         // columns: states k
-        a.kfrom = 1;                       // K = p_N >= the tile's last shared p
+        a.kfrom = 1;                       // K = p_N >= the tile's smallest p_{N-1}
         a.ea = E[cb];
         a.ea_shift = 0;
         a.eb = W ? so.wred_e : so.red_e;
-        a.num_tiles = (cmp ? (int64_t)cur * RTc : rows) / NP * a.ncol_tiles;
-        a.digits = 1;
-        a.rp = N - 1;
-        a.colmask = 0;
-        a.R = cmp ? RTc : npN1;
-        a.cmp = cmp;
-        a.Q = Qc;
-        a.RT = RTc;
-        a.cnt = p.d_cnt;
-        a.tuples = so.prefixes[N];
+        a.R = Qc;
+        a.RB = (int)((Qc + NP - 1) / NP);
+        a.num_tiles = (int64_t)cur * a.RB * a.ncol_tiles;
+        a.lg = 7;
+        a.tuples = so.ptup[N - 1];
         a.wpre = wpre;
         a.npc = rad;
         a.i0 = i0;
