@@ -18,22 +18,22 @@
 // [Re W_0p, -Im W_0p, Re W_1p, -Im W_1p, ..] and Im-row p = [Im W_0p, Re W_0p, ..], so one real
 // GEMM yields Re and Im of X.W; a real operand row has K' = 128 plain entries.
 //
-// Dataflow of one order N (Algorithm 2), indices padded to the row radix 2^lg (32, 64 or 128,
-// at least n; see split_run):
+// Dataflow of one order N (Algorithm 2). h and every intermediate are symmetric in their a's and in
+// their p's, so only sorted tuples are formed, stored in colexicographic rank:
 //   P1     : S[i][Q] = sum_j psi_{ij} A^j_Q on the packed (sorted) lower tuples Q (real rows Q,
 //            K = j), then per-i digit records of S (the upper index first: step 4 moved ahead,
 //            which the contraction order allows).
-//   batches of `ib` upper indices i (the output index space of Algorithm 1's sizing rule):
-//   expand : rows (i, a_1..a_{N-1}), K = a_N, digits of S^i_{sort(a)}
-//   c = 1..N-1 : contract the innermost a with Phi, new index p in front of the other p's:
-//            [i][p_{N-c+1}][p_{N-c+2}..p_N][a_1..a_{N-c}]
-//   c = N  : last a with Phi, 1/N!, resonance denominator (clamped), multiplicity -> h
-//            [i][p_1][p_2..p_N]
-//   reduce : G^T[k][c'] = sum_{p_N} psi_{p_N k} h[c'][p_N], c' = (i, p_1..p_{N-1}), folded with
-//            psi_{p_{N-1} k} and prod_{m<=N-2} psi_{p_m k} into Psi_N[i][k].
-// h is symmetric in its lower indices, so only non-decreasing tuples p_1 <= .. <= p_N are formed
-// (tiles whose shared p's are unsorted are skipped; elements out of order are masked) and each
-// is weighted by its multiplicity N! / prod(run lengths)! in the reduction.
+//   expand : rows (i, sorted (a_1..a_{N-1})), K = a_N, digits of S^i_{sort(a)}
+//   c = 1..N-2 : contract an a with Phi; V (the exact 64-bit accumulators) per
+//            (i, sorted p's, sorted a's), regathered into the digit rows
+//            (i, sorted p's, sorted a's less one), K = the remaining a, with exact row exponents
+//   c = N-1: rows (i, sorted (p_3..p_N), a_1), K = a_2; the output is re-sliced in the epilogue
+//            into rows (i, sorted (p_2..p_N)), K = a_1 (a 128-row tile holds every a_1 of a row)
+//   c = N  : last a with Phi, 1/N!, resonance denominator (clamped), multiplicity -> h in rows
+//            (i, sorted (p_1..p_{N-1})), K = p_N
+//   reduce : G^T[k][c'] = sum_{p_N} psi_{p_N k} h[c'][p_N], folded with psi_{p_{N-1} k} and
+//            prod_{m<=N-2} psi_{p_m k} into Psi_N[i][k]; each tuple carries its multiplicity
+//            N! / prod(run lengths)!.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
@@ -77,6 +77,12 @@ __device__ __forceinline__ long long shift_round(long long V, int sh)
     const int r = -sh;
     if (r >= 63) return 0;
     return (V + (1ll << (r - 1))) >> r;
+}
+
+// The same for shifts to the left by up to 47 (a row whose exponent is its exact bit length).
+__device__ __forceinline__ long long shift_full(long long V, int sh)
+{
+    return sh >= 0 ? (sh < 48 ? V << sh : 0) : shift_round(V, sh);
 }
 
 // 2^e for |e| < 1000 (double) / |e| < 127 (float)
@@ -323,23 +329,11 @@ __device__ __forceinline__ void load_levels(uint32_t taddr, int stride, uint32_t
     }
 }
 
-// Row digits use the radix 2^lg (32, 64 or 128 >= n): a 128-row tile holds 128 >> lg sub-blocks
-// of 2^lg rows, each one next-stage operand row (its innermost digit is the next K index).
-__host__ __device__ constexpr int64_t ipow_rad(int e, int lg) { return e <= 0 ? 1 : (int64_t)1 << (lg * e); }
-
-// digits of r (N-1 digits base 2^lg, most significant first) into d[0..N-2]
-__device__ __forceinline__ void row_digits(int64_t r, int nd, int lg, int (&d)[8])
+// Colexicographic ranks of sorted pairs and triples.
+__host__ __device__ __forceinline__ int rank2(int a, int b) { return b * (b + 1) / 2 + a; }   // a <= b
+__host__ __device__ __forceinline__ int rank3(int a, int b, int c)                            // a <= b <= c
 {
-    const int64_t mask = ((int64_t)1 << lg) - 1;
-#pragma unroll
-    for (int m = 7; m >= 0; --m) {   // unrolled with static indices: d stays in registers
-        if (m < nd) {
-            d[m] = (int)(r & mask);
-            r >>= lg;
-        } else {
-            d[m] = 0;
-        }
-    }
+    return c * (c + 1) * (c + 2) / 6 + b * (b + 1) / 2 + a;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -392,14 +386,16 @@ __global__ void k_prep_at(const double* __restrict__ A, int64_t P, int n,
 // Row-data GEMM: data rows on the M side (128 per tile), the fixed complex matrix on the N side
 // (bnc complex columns per tile -> 2*bnc real columns: Re block then Im block).
 //
-// A launch works on rows o = outer * R + r where r holds N-1 base-2^lg digits (most significant
-// first; 2^lg = 32, 64 or 128 >= n): `rp` leading lower output indices p followed by lower input
-// indices a. The innermost digit varies within a sub-block of 2^lg rows, the others are shared by
-// it; a 128-row tile holds 128 >> lg sub-blocks. The non-decreasing rule (only p's in order, new
-// column <= first p when `colmask`) and the padding (digits >= n) decide which tiles run (a tile
-// runs when any sub-block does) and which elements count.
+// Index layouts. A_N and every intermediate are symmetric in the lower indices not yet contracted
+// and in the p's already formed, so the operands hold sorted tuples only, in colexicographic rank:
+//   mode product c < N - 1 : rows (i, (p's) sorted (c-1)-tuple, (a's) sorted (N-c)-tuple)
+//   mode product c = N - 1 : rows (i, sorted (N-2)-tuple (p_3..p_N), a_1), 2^lg rows a tuple; a
+//                            128-row tile holds 128 >> lg of them (sub-blocks)
+//   divide (c = N)         : rows (i, slot), a slot per sorted tuple (p_2..p_N)
+//   reduction              : rows (i, sorted (p_1..p_{N-1})), K = p_N
+// Each forms only new indices p <= the row's first p.
 // ---------------------------------------------------------------------------------------
-enum { EPI_F64T = 0, EPI_SLICE = 1, EPI_DIVIDE = 2, EPI_SLAB = 3, EPI_REDUCE = 4 };
+enum { EPI_F64T = 0, EPI_SLICE = 1, EPI_DIVIDE = 2, EPI_SLAB = 3, EPI_REDUCE = 4, EPI_V = 5 };
 
 // Tensor maps of one operand: every slice plane in one box (`all`), and the planes of levels
 // 0..2 only (`low`, the second pass of a tile with the level-3 hold).
@@ -408,33 +404,31 @@ struct TMaps {
 };
 
 struct RowArgs {
-    int a_rows;          // rows per plane in the A tensor map
     int kch;             // pipeline stages of K' (16 or 32 wide; K' past the operands' length is
                          // zero on both sides)
     int klast;           // 16-wide steps in the last stage (1 or 2 for 32-wide stages): the rest
                          // is padding
-    const int* ea;       // row exponents, indexed by (local row) >> ea_shift
-    int ea_shift;
+    const int* ea;       // row exponents, by operand row or (ea_outer) by outer index
+    int ea_outer;
     const int* eb;       // column exponents of the fixed matrix (256 entries)
     int bnc;             // complex columns per tile (16, 32, 48 or 64)
     int ncol_tiles;
     int64_t num_tiles;
     int N;               // order
-    int digits;          // 1: r carries N-1 index digits (0 for the packed-tuple rows of P1)
-    int rp;              // leading p digits in r
-    int colmask;         // new column must be <= the first p
+    int colmask;         // new index <= the row's first p
     int kfrom;           // EPI_REDUCE: skip the K' chunks below the tile's smallest p_{N-1}
-    int aswap;           // EPI_SLICE: only tiles with non-decreasing shared a's run, and each
-                         // output row is also written for the swapped pair of shared a's
-                         // (orders <= 4 have at most two shared a's)
     int64_t R;           // rows per outer index
     int RB;              // > 0: every outer index starts a tile and has RB of them (the last one may
                          // read rows of the next index, which are masked); 0: tiles of 128 rows run
                          // over all rows
-    int lgR;             // log2(R) when R is a power of two (digit rows), else -1
     int lgncol;          // log2(ncol_tiles), or -1 when ncol_tiles is not a power of two
-    // EPI_SLICE, last mode product: output rows are the divide's slots, RS per upper index
-    int last;
+    // EPI_V: V (two 64-bit integers) at out_v[(new tuple) * R + row]; colmask: outer = (i, p), and
+    // the new tuple (i, rank2(q, p)), else (i, q)
+    longlong2* out_v;
+    // EPI_SLICE: rows (tuple t of nt sorted (p_3..p_N), a_1); output rows are the divide's slots, RS
+    // per upper index
+    int nt;
+    const uint32_t* ttup;    // order 4: the pairs (p_3, p_4), 8 bits per index
     int64_t RS;
     const int* segbase;      // first slot of the segment (p_2, .., p_{N-1}), by its colex rank
     // EPI_DIVIDE, EPI_SLAB: the slots; EPI_DIVIDE writes reduction rows, RT per upper index
@@ -448,13 +442,13 @@ struct RowArgs {
                              // as double-float complex
     const int* tiles;        // the tiles that run (nullptr: every tile, skipped ones tested)
     const unsigned* ntiles_run;   // their count
-    int npc;             // extent of the new index in the output layout
-    int lg;              // log2 of the row radix (digits, and the next operand's K extent)
+    int kout;            // K entries written per row of the next operand (whole chunks of it)
+    int lg;              // EPI_SLICE: log2 of the row radix (and of the next operand's K extent)
     int lgout;           // EPI_DIVIDE: log2 of the K extent of a reduction row
     int n;               // states (range of the a digits and of the reduction's columns k)
     int nm;              // modes in use (range of i and of the p digits; n unless a subset is set)
     int ncv;             // valid columns of this launch (modes, or states for the reduction)
-    int nouter;          // upper indices of this launch: rows of later ones pad the last tile
+    int nouter;          // upper indices of this launch (order-1 slabs: one row each)
     __nv_bfloat16* out_planes;
     int64_t out_plane_stride;
     int* out_exp;
@@ -551,36 +545,15 @@ __device__ __forceinline__ TilePos tile_pos(const RowArgs& a, int64_t tile)
     return p;
 }
 
-// Row index within / across the outer index (RB = 0; shifts for the power-of-two digit layouts:
-// 64-bit divisions by a runtime divisor cost ~70 instructions, and every role decodes every tile).
-__device__ __forceinline__ int64_t row_in_outer(const RowArgs& a, int64_t o)
+// Largest first p of a tile's rows (mode products with colmask).
+__device__ __forceinline__ int tile_pmax(const RowArgs& a, int lg, const TilePos& p)
 {
-    return a.lgR >= 0 ? (o & ((1ll << a.lgR) - 1)) : o % a.R;
-}
-__device__ __forceinline__ int64_t outer_of(const RowArgs& a, int64_t o)
-{
-    return a.lgR >= 0 ? (o >> a.lgR) : o / a.R;
-}
-
-// A sub-block (rows row0_local .. + 2^lg - 1, which share every digit but the innermost) whose
-// rows are all padding, or that the sorted-tuple rules exclude.
-__device__ __forceinline__ bool block_skipped(const RowArgs& a, int lg, int64_t row0_local, int ct)
-{
-    int d[8];
-    row_digits(row_in_outer(a, row0_local), a.N - 1, lg, d);
-    const int nd = a.N - 1;
-#pragma unroll
-    for (int m = 0; m < 7; ++m) {
-        if (m + 1 >= nd) break;                            // shared digits: 0 .. nd-2
-        if (d[m] >= (m < a.rp ? a.nm : a.n)) return true;  // padding index: rows are zero
-        if (m >= 1 && m < a.rp && d[m - 1] > d[m]) return true;
-        // shared a's: the output is symmetric in them, so only non-decreasing ones are formed
-        // and the epilogue writes each row to every ordering (aswap)
-        if (a.aswap && m > a.rp && d[m - 1] > d[m]) return true;
-    }
-    const bool first_shared = a.rp >= 1 && nd >= 2;
-    if (a.colmask && first_shared && ct * a.bnc > d[0]) return true;
-    return false;
+    if (a.out_v) return p.outer % a.nm;
+    const int t1 = min(((p.rr0 + NP - 1) >> lg), a.nt - 1);
+    if (a.N == 3) return t1;
+    int m = 0;
+    for (int t = p.rr0 >> lg; t <= t1; ++t) m = max(m, (int)(a.ttup[t] & 255u));
+    return m;
 }
 
 // lg: the row radix (a compile-time 7 in the kernels without sub-blocks)
@@ -588,10 +561,7 @@ __device__ __forceinline__ bool tile_skipped(const RowArgs& a, int lg, const Til
 {
     if (p.ct * a.bnc >= a.ncv) return true;                // every column is padding
     if (a.tpmax) return p.ct * a.bnc > a.tpmax[p.rr0 / NP];   // slots: columns p_1 <= p_2
-    if (!a.digits) return false;
-    for (int sb = 0; sb < (NP >> lg); ++sb)
-        if (!block_skipped(a, lg, p.row0 + ((int64_t)sb << lg), p.ct)) return false;
-    return true;
+    return a.colmask && p.ct * a.bnc > tile_pmax(a, lg, p);
 }
 
 // First K' chunk a tile needs. In the reduction (kfrom = 1) the rows are (p_1, .., p_{N-1}) in
@@ -948,10 +918,11 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
             unsigned long long* trc = args.trace ? args.trace + tile * 6 : nullptr;
             const int qbase = tp.ct * bnc;
             const int64_t o = tp.row0 + rl;                   // row of the operand
-            const int64_t outer = args.RB > 0 ? (int64_t)tp.outer : outer_of(args, o);
-            const int64_t rr = args.RB > 0 ? (int64_t)(tp.rr0 + rl) : row_in_outer(args, o);
+            // (RB = 0: packed tuples, and order-1 slabs, whose rows are the outer indices)
+            const int64_t outer = args.RB > 0 ? (int64_t)tp.outer : o;
+            const int rr = tp.rr0 + rl;
             const bool row_in = args.RB == 0 || rr < args.R;  // (a last block reads past its index)
-            const int ea = row_in ? args.ea[o >> args.ea_shift] : 0;
+            const int ea = row_in ? args.ea[args.ea_outer ? outer : o] : 0;
             const int sb = rl >> lg;                          // sub-block of the tile (warp-uniform)
             // columns of this tile that any row uses: below the modes in use and, with the
             // sorted-tuple mask, at most the largest leading p of the tile's rows. Columns
@@ -960,23 +931,14 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
             int vcols = min(bnc, args.ncv - qbase);
             if (MODE == EPI_DIVIDE) {
                 vcols = min(vcols, args.tpmax[tp.rr0 / NP] - qbase + 1);
-            } else if (MODE == EPI_SLICE && args.colmask && N - 1 >= 2) {
-                // the leading p is a shared digit (for N - 1 = 1 it is the innermost one and
-                // takes every value within a sub-block)
-                int pmax = 0;
-                for (int b = 0; b < (NP >> lg); ++b) {
-                    int d0[8];
-                    row_digits(row_in_outer(args, tp.row0 + ((int64_t)b << lg)), N - 1, lg, d0);
-                    pmax = max(pmax, d0[0]);
-                }
-                vcols = min(vcols, pmax - qbase + 1);
+            } else if ((MODE == EPI_SLICE || MODE == EPI_V) && args.colmask) {
+                vcols = min(vcols, tile_pmax(args, lg, tp) - qbase + 1);
             }
             const int units = (max(vcols, 0) + 3) / 4;
             const int cbeg = 4 * ((grp * units) / NGRP);
             const int cols = 4 * (((grp + 1) * units) / NGRP) - cbeg;
 
-            // Row digits (mode products): the first rp are p's (must be in order and < n), then
-            // a's (< n). The divide's and the slab's rows are slots: their tuple (p_2, .., p_N).
+            // The divide's and the slab's rows are slots: their tuple (p_2, .., p_N).
             int dg[8];
             bool row_ok = row_in;
             int firstp = NP;                                  // the new index is <= firstp
@@ -1010,40 +972,19 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                 row_ok = N >= 2 ? tup != 0xFFFFFFFFu : outer < args.nouter;
                 if (N >= 2) firstp = row_ok ? dg[0] : -1;
             } else if (MODE == EPI_SLICE) {
-                row_digits(rr, N - 1, lg, dg);
-#pragma unroll
-                for (int m = 0; m < 7; ++m) {
-                    if (m < N - 1) {
-                        row_ok &= dg[m] < (m < args.rp ? args.nm : n);
-                        if (m >= 1 && m < args.rp) row_ok &= dg[m - 1] <= dg[m];
-                    }
-                }
-                if (args.rp >= 1) firstp = dg[0];
-                if (SUBB) row_ok &= outer < args.nouter;      // rows past the batch
+                // row (p_3..p_N, a_1)
+                const int tt = rr >> lg;
+                row_ok = tt < args.nt;
+                if (N == 3) firstp = tt;
+                if (N >= 4) firstp = row_ok ? (int)(args.ttup[tt] & 255u) : 0;
                 kpos = rl & ((1 << lg) - 1);                  // K position in the next operand's row
+            } else if (MODE == EPI_V && args.colmask) {
+                firstp = (int)(tp.outer % args.nm);
             }
-
-            // rows of the swapped pair of shared a's (digits rp, rp + 1 when both are shared):
-            // offset of that row in the output's row index (shared digits, base 2^lg). A row
-            // whose shared a's decrease is not formed: its output rows are the mirrored writes of
-            // the non-decreasing one (its operand row was never written), so it writes nothing.
-            int64_t swap_off = 0, row_base = 0;
-            bool no_write = false;
-            const int64_t rperq = args.R >> lg;
-            if (MODE == EPI_SLICE) {
-                row_base = outer * args.npc * rperq + (rr >> lg);   // + qc rperq: next row
-                if (args.aswap) {
-                    const int j = args.rp, nd = N - 1;
-                    if (j + 1 <= nd - 2) {
-                        if (dg[j] < dg[j + 1]) {
-                            const int64_t wj = ipow_rad(nd - 2 - j, lg), wj1 = ipow_rad(nd - 3 - j, lg);
-                            swap_off = (int64_t)(dg[j + 1] - dg[j]) * wj + (int64_t)(dg[j] - dg[j + 1]) * wj1;
-                        }
-                        no_write = SUBB && dg[j] > dg[j + 1];   // (whole tiles are skipped at radix 128)
-                    }
-                }
-                if (SUBB && outer >= args.nouter) no_write = true;   // padding rows past the batch
-            }
+            int64_t vbase = 0;                                // EPI_V: V of the new index 0
+            if (MODE == EPI_V)
+                vbase = (args.colmask ? (int64_t)(tp.outer / args.nm) * rank2(0, args.nm) + rank2(0, firstp)
+                                      : (int64_t)tp.outer * args.nm) * args.R + rr;
             // Per-tile tables. Column exponents; the divide's columns: lambda_q - lambda_i (FP32
             // and as exact triple-floats), so that D = sigma_row + (lambda_q - lambda_i) needs no
             // FP64 per row (FP64 runs at a small fraction of the FP32 rate); the last mode
@@ -1061,19 +1002,18 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                 lamt[2 * c] = to_tfl(lq.x);
                 lamt[2 * c + 1] = to_tfl(lq.y);
             }
-            if (MODE == EPI_SLICE && args.last && et >= 256) {
+            if (MODE == EPI_SLICE && et >= 256) {
                 // output slot of (p_2 = q, the sub-block's shared p's); order 2: slot q
                 const int b = (et - 256) >> 6, c = et & 63, q = qbase + c;
+                const int tt = (tp.rr0 >> lg) + b;
                 int slot = q;
                 if (N >= 3) {
                     slot = 0;
-                    int d0[8];
-                    const int64_t rb0 = tp.row0 + ((int64_t)b << lg);
-                    if (b < (NP >> lg)) row_digits(row_in_outer(args, rb0), N - 1, lg, d0);
-                    if (b < (NP >> lg) && q <= d0[0] && d0[0] < args.nm) {
-                        if (N == 3) slot = args.segbase[q] + d0[0] - q;
-                        else if (d0[1] >= d0[0] && d0[1] < args.nm)
-                            slot = args.segbase[d0[0] * (d0[0] + 1) / 2 + q] + d0[1] - d0[0];
+                    if (tt < args.nt) {
+                        const uint32_t pp = N == 3 ? (uint32_t)tt : args.ttup[tt];
+                        const int p3 = (int)(pp & 255u), p4 = (int)((pp >> 8) & 255u);
+                        if (q <= p3) slot = N == 3 ? args.segbase[q] + p3 - q
+                                                   : args.segbase[rank2(q, p3)] + p4 - p3;
                     }
                 }
                 srowq[64 * b + c] = slot;
@@ -1197,8 +1137,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                             const float bi = level_bound01(iv[0][c], iv[1][c], deep);
                             unsigned key = 0;
                             if (MODE == EPI_SLICE) {
-                                const bool valid = row_ok && !no_write && qc < args.ncv &&
-                                                   (!args.colmask || qc <= firstp);
+                                const bool valid = row_ok && kpos < n && qc < args.ncv && qc <= firstp;
                                 // bitlen(V) <= exponent(bound) + 30
                                 const float bm = fmaxf(br, bi);
                                 if (valid && bm > 0.f)
@@ -1325,7 +1264,15 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                         const int cl = c4 + c;
                         const int qc = qbase + cl;
                         const int eb = colEb[cl];
-                        if (qc >= args.npc) continue;
+                        if (MODE == EPI_V) {
+                            if (row_in && qc < args.ncv && qc <= firstp) {
+                                longlong2 v;
+                                v.x = combine(rv[0][c], rv[1][c], rv[2][c], rv[3][c]);
+                                v.y = combine(iv[0][c], iv[1][c], iv[2][c], iv[3][c]);
+                                args.out_v[vbase + (int64_t)qc * args.R] = v;
+                            }
+                            continue;
+                        }
                         if (MODE == EPI_F64T) {
                             if (qc < args.ncv) {
                                 const double sc = pow2d(ea + eb - VEXP);
@@ -1336,7 +1283,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                             }
                             continue;
                         }
-                        const bool valid = row_ok && qc < args.ncv && (!args.colmask || qc <= firstp);
+                        const bool valid = row_ok && qc < args.ncv && qc <= firstp;
                         if (MODE == EPI_SLAB) {
                             // store h^i_{pre, q} when the multiset (q, row p's) minus pre is {extra}
                             const long long Vr = combine(rv[0][c], rv[1][c], rv[2][c], rv[3][c]);
@@ -1361,16 +1308,11 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                         }
                         uint32_t w[S];
                         if (MODE == EPI_SLICE) {
-                            if ((args.colmask && qc > firstp) || no_write) continue;   // unused rows
-                            // the last mode product writes the divide's slots (rows of unused
-                            // shared p's have none)
-                            if (args.last && N >= 3 && (firstp >= args.nm || (N >= 4 && (dg[1] < firstp || dg[1] >= args.nm))))
-                                continue;
-                            const int64_t rowp = args.last ? outer * args.RS + srowq[64 * sb + cl]
-                                                           : row_base + (int64_t)qc * rperq;
+                            if (!valid || kpos >= args.kout) continue;   // unused rows and entries
+                            const int64_t rowp = outer * args.RS + srowq[64 * sb + cl];
                             const int key = colE[64 * sb + cl];
                             const int E = key ? key - 8192 : EXP_NONE;
-                            if (key == 0 || !valid) {
+                            if (key == 0 || kpos >= n) {
 #pragma unroll
                                 for (int s = 0; s < S; ++s) w[s] = 0u;
                             } else {
@@ -1384,12 +1326,6 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
 #pragma unroll
                             for (int s = 0; s < S; ++s) dst[s * (args.out_plane_stride / 2)] = w[s];
                             if (kpos == 0) args.out_exp[rowp] = E;
-                            if (swap_off != 0) {   // the same row, shared a's swapped
-                                uint32_t* d2 = dst + (swap_off << lg);
-#pragma unroll
-                                for (int s = 0; s < S; ++s) d2[s * (args.out_plane_stride / 2)] = w[s];
-                                if (kpos == 0) args.out_exp[rowp + swap_off] = E;
-                            }
                             continue;
                         }
                         // EPI_DIVIDE: reduction row (p_1 = q, .., p_{N-1}), K = p_N
@@ -1548,18 +1484,15 @@ __global__ void k_s_records(const double2* __restrict__ Sd, int64_t ld, int64_t 
     }
 }
 
-// Dense expansion by sorted row prefix: one warp per (upper index i, non-decreasing prefix
-// (a_1..a_{N-1}) over [0, n)). Lane t covers a_N = lane + 32 t. The 128 K' digit records
-// S^i_{sort(prefix, a_N)} are gathered once and written to every distinct ordering of the
-// prefix (the dense rows that share them), so a record is read once per prefix rather than once
-// per ordering. Layout: row (i - i0, a_1..a_{N-1}) (digits base 2^lg >= n), K' pair a_N (2^lg
-// pairs a row); rows with an index >= n are not written (they only feed their own, discarded,
-// outputs) and K' entries past n are zeros (they meet the fixed matrix's zero rows, where stale
-// bit patterns could be NaN).
+// Expansion: one warp per (upper index i, sorted (N-1)-tuple of a's, colexicographic rank). Lane t
+// covers a_N = lane + 32 t: the digit records S^i_{sort(tuple, a_N)} are gathered (rec holds the
+// packed, lexicographic order) into the first mode product's operand row. Layout: row
+// (i - i0) R + rank, 2^lg complex K entries a row of which kout are written (entries past n are
+// zeros: they meet the fixed matrix's zero rows, where stale bit patterns could be NaN).
 template <int S>
 __global__ void k_expand_sorted(const uint4* __restrict__ rec, int64_t P, int n, int N, int i0,
-                                int ib, int lg, const int64_t* __restrict__ cnt,
-                                const uint32_t* __restrict__ prefixes, int64_t npre,
+                                int ib, int lg, int kout, const int64_t* __restrict__ cnt,
+                                const uint32_t* __restrict__ tuples, int64_t ntup, int64_t R,
                                 uint32_t* __restrict__ planes, int64_t plane_stride_u32)
 {
     // the rank table (rows 0..N of C(n - v + r - 1, r), <= 5 x 129 entries) in shared memory:
@@ -1572,11 +1505,10 @@ __global__ void k_expand_sorted(const uint4* __restrict__ rec, int64_t P, int n,
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int nd = N - 1;
-    const int64_t rows_per_i = ipow_rad(nd, lg);
-    const int kw = 1 << lg;   // K' pairs a row
-    for (int64_t item = warp; item < npre * ib; item += nwarps) {
-        const int il = (int)(item / npre);
-        const uint32_t pk = prefixes[item % npre];
+    for (int64_t item = warp; item < ntup * ib; item += nwarps) {
+        const int il = (int)(item / ntup);
+        const int64_t r0row = item - il * ntup;
+        const uint32_t pk = tuples[r0row];
         int pre[3];
 #pragma unroll
         for (int m = 0; m < 3; ++m) pre[m] = (int)((pk >> (8 * m)) & 255u);
@@ -1618,38 +1550,97 @@ __global__ void k_expand_sorted(const uint4* __restrict__ rec, int64_t P, int n,
                 r1[t] = rec[((int64_t)(i0 + il) * P + qv[t]) * 2 + 1];
             }
         }
-        uint32_t w[4][S];
+        uint32_t* dst = planes + (((int64_t)il * R + r0row) << lg) + lane;
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
             const uint32_t rr[8] = {r0[t].x, r0[t].y, r0[t].z, r0[t].w, r1[t].x, r1[t].y, r1[t].z, r1[t].w};
+            if (lane + 32 * t < kout)
 #pragma unroll
-            for (int s = 0; s < S; ++s) w[t][s] = rr[s];
+                for (int s = 0; s < S; ++s) dst[s * plane_stride_u32 + 32 * t] = rr[s];
         }
-        // every distinct ordering of the prefix whose shared indices (all but the last) are
-        // non-decreasing, which is what the first contraction runs: for x <= y <= z these are
-        // (x, y, z), (x, z, y) when y < z and (y, z, x) when x < y; (x, y) and (y, x) when x < y
-        auto write_row = [&](int o0, int o1, int o2) {
-            int64_t row = o0;
-            if (nd >= 2) row = (row << lg) + o1;
-            if (nd >= 3) row = (row << lg) + o2;
-            uint32_t* dst = planes + (((int64_t)il * rows_per_i + row) << lg) + lane;
-#pragma unroll
-            for (int t = 0; t < 4; ++t)
-                if (32 * t < kw)
-#pragma unroll
-                    for (int s = 0; s < S; ++s) dst[s * plane_stride_u32 + 32 * t] = w[t][s];
-        };
-        const int x = pre[0], y = pre[1], z = pre[2];
-        if (nd <= 1) {   // (order 1: one empty prefix, row 0)
-            write_row(x, 0, 0);
-        } else if (nd == 2) {
-            write_row(x, y, 0);
-            if (x != y) write_row(y, x, 0);
-        } else {
-            write_row(x, y, z);
-            if (y != z) write_row(x, z, y);
-            if (x != y) write_row(y, z, x);
+    }
+}
+
+// Operand rows of the next mode product from a mode product's V (EPI_V): one warp per row
+// (outer, sorted M-tuple of a's), outer = (i, sorted tuple of p's). Lane t covers a = lane + 32 t:
+// it gathers V[outer][rank(sort(tuple, a))], and the row gets its exact exponent (the largest
+// bit length) and its digits. V is in units of 2^(ea + eb - VEXP) with eb of the newest p.
+//   ea: by upper index (M + 1 = N - 1: the first product's operand has one exponent per index) or
+//       (ea_row) by the source product's operand row, (i, p, rank) with p the tuple's other index
+// Neighbouring rows gather neighbouring entries (colexicographic rank), so the warps of a block
+// share sectors. Bound: HBM writes (4 S bytes an entry against 16 read per source entry): 0.69 ms
+// per upper index and product at n = 120, order 4 (3.2 GB: 4.7 TB/s). It pays because the products
+// before it run on sorted a's only: 614 ms of mode products became 245 + 166 here.
+template <int S, int M>
+__global__ void __launch_bounds__(256)
+    k_regather(const longlong2* __restrict__ V, int64_t Rsrc, int n, int nm, int nt, const uint32_t* __restrict__ ttup,
+               const int* __restrict__ ea, int ea_row, const int* __restrict__ eb, int lg, int kout,
+               int nrows, int64_t Rdst, int64_t nouter, const uint32_t* __restrict__ tuples,
+               uint32_t* __restrict__ planes, int64_t plane_stride_u32, int* __restrict__ out_exp)
+{
+    const int lane = threadIdx.x & 31;
+    const int chunks = (nrows + 7) / 8;                      // 8 rows (one a warp) a step
+    const int64_t steps = nouter * chunks;
+    for (int64_t st = blockIdx.x; st < steps; st += gridDim.x) {
+        const int64_t outer = st / chunks;
+        const int row = (int)(st - outer * chunks) * 8 + (int)(threadIdx.x >> 5);
+        if (row >= nrows) continue;
+        const int64_t i = outer / nt;
+        const int t = (int)(outer - i * nt);
+        const uint32_t tp = ea_row ? ttup[t] : (uint32_t)t;  // the newest p in the low byte
+        const int q = (int)(tp & 255u);
+        const int e0 = eb[q] - VEXP + (ea_row ? 0 : ea[i]);
+        const int* earow = ea_row ? ea + (i * nm + (int)((tp >> 8) & 255u)) * Rsrc : nullptr;
+        int x = row, y = 0;
+        if (M == 2) {
+            const uint32_t pk = tuples[row];
+            x = (int)(pk & 255u);
+            y = (int)((pk >> 8) & 255u);
         }
+        const longlong2* src = V + outer * Rsrc;
+        longlong2 v[4];
+        int ex[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int a = lane + 32 * k;
+            v[k] = make_longlong2(0ll, 0ll);
+            ex[k] = 0;
+            if (a < n) {
+                const int rk = M == 1 ? (a <= x ? rank2(a, x) : rank2(x, a))
+                                      : (a <= x ? rank3(a, x, y) : a <= y ? rank3(x, a, y) : rank3(x, y, a));
+                v[k] = src[rk];
+                if (ea_row) ex[k] = earow[rk];
+            }
+        }
+        int key = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const unsigned long long m = (unsigned long long)(v[k].x < 0 ? ~v[k].x : v[k].x) |
+                                         (unsigned long long)(v[k].y < 0 ? ~v[k].y : v[k].y);
+            // bit length of max(|x|, |y|) (one less for a negative power of two, which the top
+            // digit's range [-128, 128] holds)
+            if (v[k].x | v[k].y) key = max(key, 64 - __clzll((long long)m) + ex[k] + e0 + 8192);
+        }
+        key = (int)__reduce_max_sync(0xffffffffu, (unsigned)key);
+        const int E = key ? key - 8192 : EXP_NONE;
+        const int sh = e0 - E + 7 + 8 * (S - 1);
+        const int64_t rowp = outer * Rdst + row;
+        uint32_t* dst = planes + (rowp << lg) + lane;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (lane + 32 * k < kout) {
+                uint32_t w[S];
+                if (key) {
+                    digit_pairs<S>(shift_full(v[k].x, sh + ex[k]), shift_full(v[k].y, sh + ex[k]), w);
+                } else {
+#pragma unroll
+                    for (int s = 0; s < S; ++s) w[s] = 0u;
+                }
+#pragma unroll
+                for (int s = 0; s < S; ++s) dst[s * plane_stride_u32 + 32 * k] = w[s];
+            }
+        }
+        if (lane == 0) out_exp[rowp] = E;
     }
 }
 
@@ -1764,8 +1755,9 @@ struct SplitOperand {
     __nv_bfloat16* at[kMaxOrder + 1] = {};
     int* at_e[kMaxOrder + 1] = {};
     int64_t at_rows[kMaxOrder + 1] = {};
-    uint32_t* prefixes[kMaxOrder + 1] = {};   // non-decreasing (a_1..a_{N-1}), 8 bits per index
-    int64_t nprefix[kMaxOrder + 1] = {};
+    // sorted M-tuples of states in colexicographic order, 8 bits per index (M = 0: one empty tuple)
+    uint32_t* atup[4] = {};
+    int64_t natup[4] = {};
     const double* at_src[kMaxOrder + 1] = {};
     // per order, for the modes in use: the divide's slots (128 a tile) and the tables around them
     int slot_nm[kMaxOrder + 1] = {};          // modes the tables were built for (0: none)
@@ -1941,11 +1933,10 @@ void split_release(Plan& p)
     for (int N = 0; N <= kMaxOrder; ++N) { cudaFree(so->at[N]); cudaFree(so->at_e[N]); }
     cudaFree(so->wred); cudaFree(so->wred_e); cudaFree(so->w_df);
     for (int N = 0; N <= kMaxOrder; ++N) {
-        cudaFree(so->prefixes[N]);
         cudaFree(so->srow[N]); cudaFree(so->stup[N]); cudaFree(so->sseg[N]);
         cudaFree(so->stpmax[N]); cudaFree(so->segbase[N]);
     }
-    for (int M = 0; M < 4; ++M) cudaFree(so->ptup[M]);
+    for (int M = 0; M < 4; ++M) { cudaFree(so->ptup[M]); cudaFree(so->atup[M]); }
     cudaFree(so->err);
     delete so;
     p.split = nullptr;
@@ -1970,6 +1961,7 @@ static void set_smem_attrs()
     smem_attr<S, EPI_DIVIDE, false>();
     smem_attr<S, EPI_SLAB, false>();
     smem_attr<S, EPI_REDUCE, false>();
+    smem_attr<S, EPI_V, false>();
     done = true;
 }
 
@@ -2070,21 +2062,36 @@ void split_refresh_modes(Plan& p)
 }
 #endif
 
-// Sorted M-tuples (1 <= M <= 3) over the modes in use, colexicographic.
-static void ensure_ptuples(Plan& p, SplitOperand& so, int M)
+// Sorted M-tuples (M <= 3) over [0, count) in colexicographic order, 8 bits per index.
+static std::vector<uint32_t> colex_tuples(int M, int count)
+{
+    std::vector<uint32_t> t;
+    if (M == 0) t.push_back(0u);
+    for (int r = 0; r < (M >= 3 ? count : M >= 1 ? 1 : 0); ++r)
+        for (int q = 0; q < (M >= 3 ? r + 1 : M == 2 ? count : 1); ++q)
+            for (int x = 0; x < (M >= 2 ? q + 1 : count); ++x)
+                t.push_back((uint32_t)x | (M >= 2 ? (uint32_t)q << 8 : 0u) | (M >= 3 ? (uint32_t)r << 16 : 0u));
+    return t;
+}
+
+static void ensure_ptuples(Plan& p, SplitOperand& so, int M)   // over the modes in use
 {
     if (so.ptup_nm[M] == p.nm) return;
     cudaFree(so.ptup[M]);
     so.ptup[M] = nullptr;
     so.ptup_nm[M] = 0;
-    std::vector<uint32_t> t;
-    for (int r = 0; r < (M >= 3 ? p.nm : 1); ++r)
-        for (int q = 0; q < (M >= 3 ? r + 1 : M == 2 ? p.nm : 1); ++q)
-            for (int x = 0; x < (M >= 2 ? q + 1 : p.nm); ++x)
-                t.push_back((uint32_t)x | (M >= 2 ? (uint32_t)q << 8 : 0u) | (M >= 3 ? (uint32_t)r << 16 : 0u));
+    const std::vector<uint32_t> t = colex_tuples(M, p.nm);
     so.ptup[M] = upload(t);
     so.nptup[M] = (int64_t)t.size();
     so.ptup_nm[M] = p.nm;
+}
+
+static void ensure_atuples(Plan& p, SplitOperand& so, int M)   // over the states
+{
+    if (so.atup[M]) return;
+    const std::vector<uint32_t> t = colex_tuples(M, p.n);
+    so.atup[M] = upload(t);
+    so.natup[M] = (int64_t)t.size();
 }
 
 // The slots of order N: the sorted tuples (p_2 <= .. <= p_N) in 128-row tiles. A segment (the
@@ -2278,15 +2285,14 @@ static void launch_rows(Plan& p, const char* name, const DataOp& A, const FixedO
         a.bnc = 32;
     }
     a.kch = (kprime + bk - 1) / bk;            // K' past kprime holds zeros on both sides
-    a.lgR = (a.R > 0 && (a.R & (a.R - 1)) == 0) ? __builtin_ctzll((unsigned long long)a.R) : -1;
     a.lgncol = (a.ncol_tiles & (a.ncol_tiles - 1)) == 0 ? __builtin_ctz((unsigned)a.ncol_tiles) : -1;
     a.klast = (kprime + KSTEP - 1) / KSTEP - (bk / KSTEP) * (a.kch - 1);
     const TMaps tA = plane_maps<S>(A, bk);
     const TMaps tB = fixed_maps<S>(B, a.bnc, bk);
     if (a.num_tiles >= (int64_t)1 << 31) fail(NPF_ERR_UNSUPPORTED, "too many tiles in one launch");
-    if (MODE == EPI_SLICE || MODE == EPI_DIVIDE) {
+    if (a.colmask) {
         // the running tiles, listed on the device (stream order puts the list before the launch);
-        // the other modes run every tile
+        // without a column mask every tile runs
         SplitOperand& so = *p.split;
         if (!so.tile_list || so.tile_cap < a.num_tiles) {
             if (p.capturing) fail(NPF_ERR_CUDA, "tile list would grow during graph capture");
@@ -2340,30 +2346,9 @@ static void launch_rows(Plan& p, const char* name, const DataOp& A, const FixedO
 
 static double factorial(int N) { double f = 1; for (int t = 2; t <= N; ++t) f *= t; return f; }
 
-// so.prefixes[M]: the non-decreasing (M-1)-tuples over [0, n) in lexicographic order, 8 bits per
-// index (M - 1 = 0: one empty tuple).
-static void ensure_tuples(Plan& p, SplitOperand& so, int M)
-{
-    if (so.prefixes[M]) return;
-    std::vector<uint32_t> pre;
-    std::vector<int> t(std::max(M - 1, 0), 0);
-    while (true) {
-        uint32_t pk = 0;
-        for (int m = 0; m < M - 1; ++m) pk |= (uint32_t)t[m] << (8 * m);
-        pre.push_back(pk);
-        int m = M - 2;
-        while (m >= 0 && t[m] == p.n - 1) --m;
-        if (m < 0) break;
-        ++t[m];
-        for (int r = m + 1; r < M - 1; ++r) t[r] = t[m];
-    }
-    so.prefixes[M] = upload(pre);
-    so.nprefix[M] = (int64_t)pre.size();
-}
-
-// Device memory of one order: S (FP64, n x P), records (n x P x 32 B), and per i of a batch two
-// operand buffers of R^(N-1) rows x 2R K' x S planes (BF16) plus exponents, R = 2^lg the row
-// radix.
+// Device memory of one order: S (FP64, n x P), records (n x P x 32 B), and per upper index of a
+// batch two buffers that the stages alternate (A: the operands of the mode products and of the
+// reduction, B: V and the divide's slots) plus the row exponents.
 template <int S>
 static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const double2* W)
 {
@@ -2371,51 +2356,64 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     if (W) prepare_weights(p, so, W);
     set_smem_attrs<S>();
     prepare_tensor<S>(p, so, N);
-    ensure_tuples(p, so, N);
+    const bool slab = prefix != nullptr;
+    for (int M = N >= 4 ? 2 : std::max(N - 1, 0); M <= N - 1; ++M) ensure_atuples(p, so, M);
     if (N >= 2) ensure_slots(p, so, N);
-    if (N >= 2 && !prefix) ensure_ptuples(p, so, N - 1);
-    if (N == 4 && !prefix) ensure_ptuples(p, so, 2);
+    if (N >= 2 && !slab) ensure_ptuples(p, so, N - 1);
+    if (N == 4) ensure_ptuples(p, so, 2);
     int* const err = p.err_override ? p.err_override : so.err;   // a batch zeroes and checks its own
     if (!p.err_override) NPF_CUDA(cudaMemsetAsync(err, 0, sizeof(int), p.stream));
     const int n = p.n;
     const int nm = p.nm;                 // modes in use (a critical-mode subset comes first)
     const int64_t P = p.packed_count[N];
     const int64_t Prows = so.at_rows[N];
-    // row radix 2^lg >= n: 32 or 64 for small systems (a 128-row tile then holds 4 or 2 operand
-    // rows instead of one padded to 128), else 128. For order 2 a tile can span several upper
-    // indices, and the rows of a batch are padded to whole tiles (rows past it write nothing).
+    // K extent of an operand row: the radix 2^lg >= n
     const int lg = n <= 32 ? 5 : n <= 64 ? 6 : 7;
     const int rad = 1 << lg;
-    const int64_t npN1 = ipow64(rad, N - 1);
     // complex columns per tile (the slab path runs untuned: 32 when the plan autotunes); the mode
     // products run at most 32 columns, the divide and the reduction 64 (launch_rows)
     const int bnc = std::min(p.tile_n > 0 ? (p.tile_n == 48 ? 32 : p.tile_n) : 32, rad);
-    const bool slab = prefix != nullptr;
 
-    // ---- memory plan (Algorithm 1's rule on the upper-index space)
+    // ---- rows per upper index of every stage
+    const int64_t npairs = (int64_t)nm * (nm + 1) / 2;
+    auto arows = [&](int M) { return M <= 0 ? (int64_t)1 : packed_count(n, M); };   // sorted M-tuples of a's
+    const int64_t nt = N <= 2 ? 1 : N == 3 ? nm : npairs;         // sorted (N-2)-tuples of p's
+    const int64_t R0 = N == 1 ? 1 : N == 2 ? rad : arows(N - 1);  // first product
+    const int64_t R1 = N == 4 ? nm * arows(2) : 0;                // second product (order 4)
+    const int64_t R2 = N >= 3 ? nt * rad : 0;                     // last mode product
+    const int64_t RS = N == 2 ? rad : N >= 3 ? (int64_t)so.slot_tiles[N] * NP : 0;   // divide
+    const int64_t Qc = N >= 2 ? packed_count(nm, N - 1) : 0;      // reduction
+    const int64_t v_per = N == 4 ? std::max(nm * arows(3), npairs * arows(2)) : N == 3 ? nm * arows(2) : 0;
+
+    // ---- memory plan (Algorithm 1's rule on the upper-index space). A call is accepted when the
+    // dense rows of one upper index (rad^(N-1) rows in two buffers) fit: the sorted rows take less.
+    const size_t row_bytes = (size_t)rad * 4 * S;
     const size_t s_bytes = (size_t)n * Prows * sizeof(double2);
     const size_t rec_bytes = (size_t)n * P * 32;
-    const size_t per_i = 2 * ((size_t)npN1 * 2 * rad * 2 * S + (size_t)npN1 * 4) + 4096;
+    const size_t dense_i = 2 * ((size_t)ipow64(rad, N - 1) * (row_bytes + 4)) + 4096;
+    const size_t a_per = (size_t)std::max(std::max(R0, R1), std::max(R2, Qc)) * row_bytes;
+    const size_t b_per = std::max((size_t)v_per * sizeof(longlong2), (size_t)RS * row_bytes);
+    const size_t e_per = (size_t)(R1 + R2 + RS + Qc) * sizeof(int);
+    const size_t per_i = std::min(dense_i, a_per + b_per + e_per);
     const size_t budget = effective_budget(p);
-    if (s_bytes + rec_bytes + per_i > budget)
+    if (s_bytes + rec_bytes + dense_i > budget)
         fail(NPF_ERR_OOM, "memory budget too small for one upper-index batch");
     const int ib = (int)std::min<size_t>((size_t)nm, (budget - s_bytes - rec_bytes) / per_i);
-    const int64_t t_rows = ((int64_t)ib * npN1 + NP - 1) / NP * NP;
-    const size_t tbytes = (size_t)t_rows * 2 * rad * 2 * S;
-    const size_t ebytes = (size_t)t_rows * 4;
-    // reduction rows per upper index (sorted (N-1)-tuples) and, at order 4, the weights of the pairs
-    const int64_t Qc = N >= 2 ? so.nptup[N - 1] : 0;
-    const int64_t Q2 = N == 4 && !slab ? so.nptup[2] : 0;
+    const int64_t Q2 = N == 4 && !slab ? npairs : 0;              // order 4: weights of the pairs
     const size_t wbytes = (size_t)Q2 * n * sizeof(float4);
     Arena& ar = p.scratch();
-    ar.reserve(s_bytes + rec_bytes + 2 * (tbytes + ebytes) + wbytes + 8 * 256 + 1024);
+    ar.reserve(s_bytes + rec_bytes + (size_t)ib * (a_per + b_per + e_per) + wbytes + 10 * 256 + 1024);
     uint8_t* base = (uint8_t*)ar.base;
     auto take = [&](size_t bytes) { uint8_t* r = base; base += (bytes + 255) & ~(size_t)255; return r; };
     double2* Sd = (double2*)take(s_bytes);
     uint4* rec = (uint4*)take(rec_bytes);
     int* sE = (int*)take(256 * sizeof(int));
-    __nv_bfloat16* T[2] = {(__nv_bfloat16*)take(tbytes), (__nv_bfloat16*)take(tbytes)};
-    int* E[2] = {(int*)take(ebytes), (int*)take(ebytes)};
+    uint8_t* bufA = take((size_t)ib * a_per);
+    uint8_t* bufB = take((size_t)ib * b_per);
+    int* E1 = (int*)take((size_t)ib * R1 * sizeof(int));
+    int* E2 = (int*)take((size_t)ib * R2 * sizeof(int));
+    int* ES = (int*)take((size_t)ib * RS * sizeof(int));
+    int* ER = (int*)take((size_t)ib * Qc * sizeof(int));
     // order 3: the prefix weight is W itself (the double-float copy); order 4: pairs' products
     const float4* wpre = W ? so.w_df : so.psi_df;
     if (N == 4 && !slab) {
@@ -2433,9 +2431,6 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     const FixedOp tPsiR{so.psir, NP};
     const FixedOp tRed{W ? so.wred : so.red, KP};
     const DataOp tAT{so.at[N], NP, Prows};
-    const DataOp tT0{T[0], 2 * rad, t_rows};
-    const DataOp tT1{T[1], 2 * rad, t_rows};
-    const DataOp* tT[2] = {&tT0, &tT1};
 
     RowArgs base0{};
     base0.n = n;
@@ -2453,22 +2448,19 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     base0.err = err;
     base0.bnc = bnc;
     base0.ncol_tiles = rad / bnc;
-    base0.lg = lg;
+    base0.lg = 7;
+    base0.segbase = N >= 2 ? so.segbase[N] : nullptr;
+    base0.ttup = N == 4 ? so.ptup[2] : nullptr;
     if (slab)
         for (int m = 0; m < N - 1; ++m) base0.pre[m] = prefix[m];
 
     // ---- P1: S[i][Q] = sum_j psi_ij A^j_Q (rows Q, real K = j)
     {
         RowArgs a = base0;
-        a.a_rows = (int)Prows;
         a.ea = so.at_e[N];
-        a.ea_shift = 0;
         a.eb = so.psir_e;
         a.num_tiles = Prows / NP * a.ncol_tiles;
-        a.digits = 0;
-        a.lg = 7;                    // plain rows (packed tuples), no digits
         a.R = Prows;
-        a.npc = n;
         a.out_f64 = Sd;
         a.ld_f64 = Prows;
         launch_rows<S, EPI_F64T>(p, "split_upper_contraction", tAT, tPsiR, n, a);   // K = j < n
@@ -2484,93 +2476,124 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
         NPF_CUDA(cudaGetLastError());
     }
 
+    // K entries a launch reads: whole chunks of its pipeline
+    auto chunked = [&](int bk) { return std::min(rad, (n + bk / 2 - 1) / (bk / 2) * (bk / 2)); };
+    const int kmode = chunked(RowCfg<S, EPI_SLICE>::BK), kdiv = chunked(RowCfg<S, EPI_DIVIDE>::BK);
+    const int kslab = chunked(RowCfg<S, EPI_SLAB>::BK);
+
     const int rlo = std::max(0, p.row_lo);                       // upper-index rows to form
     const int rhi = p.row_hi < 0 ? nm : std::min(p.row_hi, nm);
     for (int i0 = rlo; i0 < rhi; i0 += ib) {
         const int cur = std::min(ib, rhi - i0);
-        const int64_t rows = ((int64_t)cur * npN1 + NP - 1) / NP * NP;   // whole tiles
+        auto operand = [&](const uint8_t* buf, int64_t R) { return DataOp{buf, 2 * rad, cur * R}; };
+        auto plane = [&](int64_t R) { return cur * R * rad; };   // plane stride in complex entries
         {
             LaunchScope ls(&p.prof, "split_expand", p.stream);
-            k_expand_sorted<S><<<8192, 256, 0, p.stream>>>(rec, P, n, N, i0, cur, lg, p.d_cnt,
-                                                           so.prefixes[N], so.nprefix[N],
-                                                           (uint32_t*)T[0], t_rows * rad);
+            k_expand_sorted<S><<<8192, 256, 0, p.stream>>>(rec, P, n, N, i0, cur, lg, kmode, p.d_cnt,
+                                                           so.atup[N - 1], so.natup[N - 1], R0,
+                                                           (uint32_t*)bufA, plane(R0));
             NPF_CUDA(cudaGetLastError());
         }
-        int cb = 0;
-        for (int c = 1; c <= N; ++c) {
+        // ---- the first N - 2 mode products: V per sorted tuple, regathered into the next operand
+        for (int c = 1; c <= N - 2; ++c) {
+            const int64_t Ra = arows(N - c), outers = c == 1 ? cur : (int64_t)cur * nm;
             RowArgs a = base0;
-            a.a_rows = (int)t_rows;
-            a.ea = c == 1 ? sE + i0 : E[cb];
-            a.ea_shift = c == 1 ? lg * (N - 1) : 0;   // c = 1: one exponent per upper index
+            a.ea = c == 1 ? sE + i0 : E1;
+            a.ea_outer = c == 1;
             a.eb = so.phi_e;
-            a.num_tiles = rows / NP * a.ncol_tiles;
-            a.digits = 1;
-            a.rp = c - 1;              // p_{N-c+2}..p_N lead the row, then a_1..a_{N-c}
-            a.colmask = c >= 2;        // new index p_{N-c+1} <= p_{N-c+2}
-            a.aswap = c < N;           // mode products: shared a's non-decreasing, rows mirrored
-            a.R = npN1;
-            a.npc = rad;
+            a.colmask = c >= 2;                                  // new index p_3 <= p_4
+            a.R = Ra;
+            a.RB = (int)((Ra + NP - 1) / NP);
+            a.num_tiles = outers * a.RB * a.ncol_tiles;
+            a.out_v = (longlong2*)bufB;
+            launch_rows<S, EPI_V>(p, "split_mode_product", operand(bufA, outers / cur * Ra), tPhi, 2 * n, a);
+            const bool pairs = N - c - 1 == 2;                   // rows of the next operand: pairs of a's, or a_1
+            const int64_t outs = c == 1 ? (int64_t)cur * nm : cur * npairs;
+            const int nrows = pairs ? (int)so.natup[2] : n;
+            const int64_t Rdst = pairs ? nrows : rad;
+            LaunchScope ls(&p.prof, "split_regather", p.stream);
+            const unsigned grid = (unsigned)std::min<int64_t>(outs * ((nrows + 7) / 8), 1 << 16);
+            auto kern = pairs ? k_regather<S, 2> : k_regather<S, 1>;
+            kern<<<grid, 256, 0, p.stream>>>((const longlong2*)bufB, Ra, n, nm, (int)(outs / cur), base0.ttup,
+                                             c == 1 ? sE + i0 : E1, c == 2, so.phi_e, lg, kmode, nrows, Rdst,
+                                             outs, so.atup[2], (uint32_t*)bufA, outs * Rdst * rad,
+                                             pairs ? E1 : E2);
+            NPF_CUDA(cudaGetLastError());
+        }
+        // ---- the last mode product (its output rows are the divide's slots)
+        if (N >= 2) {
+            RowArgs a = base0;
+            a.lg = lg;
+            a.ea = N == 2 ? sE + i0 : E2;
+            a.ea_outer = N == 2;
+            a.eb = so.phi_e;
+            a.colmask = N >= 3;                                  // p_2 <= p_3
+            a.nt = (int)nt;
+            a.R = nt * rad;
+            a.RB = (int)((a.R + NP - 1) / NP);
+            a.num_tiles = (int64_t)cur * a.RB * a.ncol_tiles;
+            a.RS = RS;
+            a.kout = slab ? kslab : kdiv;
+            a.out_planes = (__nv_bfloat16*)bufB;
+            a.out_plane_stride = 2 * plane(RS);
+            a.out_exp = ES;
+            launch_rows<S, EPI_SLICE>(p, "split_mode_product", operand(bufA, a.R), tPhi, 2 * n, a);
+        }
+        // ---- the last contraction: divide, or the slab's entries
+        {
+            RowArgs a = base0;
+            a.eb = so.phi_e;
             a.i0 = i0;
             a.nouter = cur;
-            a.out_planes = T[cb ^ 1];
-            a.out_plane_stride = t_rows * 2 * rad;
-            a.out_exp = E[cb ^ 1];
-            if (c < N) {
-                a.last = c == N - 1;
-                a.RS = N == 2 ? rad : (int64_t)so.slot_tiles[N] * NP;
-                a.segbase = so.segbase[N];
-                launch_rows<S, EPI_SLICE>(p, "split_mode_product", *tT[cb], tPhi, 2 * n, a);
-            } else {
-                if (N >= 2) {   // rows are slots
-                    a.digits = 0;
-                    a.ea_shift = 0;
-                    a.R = N == 2 ? rad : (int64_t)so.slot_tiles[N] * NP;
-                    a.RB = so.slot_tiles[N];
-                    a.srow = so.srow[N];
-                    a.stup = so.stup[N];
-                    a.num_tiles = (int64_t)cur * a.RB * a.ncol_tiles;
-                    a.lg = 7;
-                    a.lgout = lg;
-                }
-                if (slab) {
-                    a.out_f64 = d_out;
-                    launch_rows<S, EPI_SLAB>(p, "split_mode_divide", *tT[cb], tPhi, 2 * n, a);
-                } else {
-                    a.tpmax = so.stpmax[N];
-                    a.RT = Qc;
-                    launch_rows<S, EPI_DIVIDE>(p, "split_mode_divide", *tT[cb], tPhi, 2 * n, a);
-                }
+            if (N >= 2) {
+                a.ea = ES;
+                a.R = RS;
+                a.RB = so.slot_tiles[N];
+                a.num_tiles = (int64_t)cur * a.RB * a.ncol_tiles;
+                a.srow = so.srow[N];
+                a.stup = so.stup[N];
+            } else {                                             // order 1: a row per upper index
+                a.ea = sE + i0;
+                a.R = 1;
+                a.num_tiles = (int64_t)((cur + NP - 1) / NP) * a.ncol_tiles;
             }
-            cb ^= 1;
+            const DataOp op = N >= 2 ? operand(bufB, RS) : operand(bufA, 1);
+            if (slab) {
+                a.out_f64 = d_out;
+                launch_rows<S, EPI_SLAB>(p, "split_mode_divide", op, tPhi, 2 * n, a);
+                continue;
+            }
+            a.colmask = 1;
+            a.tpmax = so.stpmax[N];
+            a.RT = Qc;
+            a.lgout = lg;
+            a.out_planes = (__nv_bfloat16*)bufA;
+            a.out_plane_stride = 2 * plane(Qc);
+            a.out_exp = ER;
+            launch_rows<S, EPI_DIVIDE>(p, "split_mode_divide", op, tPhi, 2 * n, a);
         }
-        if (slab) continue;
         {
             LaunchScope ls(&p.prof, "split_zero_heads", p.stream);
             const int64_t tot = Qc * cur * 8;
             k_zero_heads<S><<<(unsigned)((tot + 255) / 256), 256, 0, p.stream>>>(
                 N, nm, RowCfg<S, EPI_REDUCE>::BK / 2, lg, (int)Qc, Qc, cur, so.ptup[N - 1],
-                (uint32_t*)T[cb], t_rows * rad);
+                (uint32_t*)bufA, plane(Qc));
             NPF_CUDA(cudaGetLastError());
         }
-        // ---- reduction: rows c' = (i, p_1 <= .. <= p_{N-1}), K = p_N, columns k (Psi^T)
+        // ---- reduction: rows (i, p_1 <= .. <= p_{N-1}), K = p_N, columns k (Psi^T)
         RowArgs a = base0;
-        a.a_rows = (int)t_rows;
         a.ncv = n;                         // columns: states k
         a.kfrom = 1;                       // K = p_N >= the tile's smallest p_{N-1}
-        a.ea = E[cb];
-        a.ea_shift = 0;
+        a.ea = ER;
         a.eb = W ? so.wred_e : so.red_e;
         a.R = Qc;
         a.RB = (int)((Qc + NP - 1) / NP);
         a.num_tiles = (int64_t)cur * a.RB * a.ncol_tiles;
-        a.lg = 7;
         a.tuples = so.ptup[N - 1];
         a.wpre = wpre;
-        a.npc = rad;
         a.i0 = i0;
-        a.nouter = cur;
         a.out_f64 = d_out;
-        launch_rows<S, EPI_REDUCE>(p, "split_reduce", *tT[cb], tRed, 2 * nm, a);   // K = p_N < nm
+        launch_rows<S, EPI_REDUCE>(p, "split_reduce", operand(bufA, Qc), tRed, 2 * nm, a);   // K = p_N < nm
     }
     if (p.err_override) return;   // the batch reads the shared flag after its graph has run
     int herr = 0;

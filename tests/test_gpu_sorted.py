@@ -1,0 +1,86 @@
+"""Sorted-tuple operands of the tensor-core path: the first mode products' regathered rows, the
+divide's slots (segments packed into 128-row tiles) and the reduction's colexicographic rows, at
+the sizes where their tables have remainders: odd n, one mode, segments of length 1, tiles of
+several short segments, n just past a row radix, a mode subset of odd size, batches of a few upper
+indices, the FP32 form and a slab. Tolerances are the library's bars for the forms (1e-10, 1e-5)."""
+from math import comb
+
+import numpy as np
+import pytest
+
+import npf_synth as S
+import oracle
+from tests._util import rel_fro
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def npf():
+    from paper_2509_08968_gb300 import build
+    build.build()
+    import paper_2509_08968_gb300 as m
+    return m
+
+
+def _odd_system(n, N, seed):
+    """Conjugate pairs and, for odd n, one real mode; eigenvectors from a real similarity."""
+    rng = np.random.default_rng(seed)
+    lam, W = np.empty(n, np.complex128), np.zeros((n, n), np.complex128)
+    for b in range(n // 2):
+        s, w = rng.uniform(-2.0, -0.05), rng.uniform(0.5, 15.0)
+        lam[2 * b:2 * b + 2] = s + 1j * w, s - 1j * w
+        W[2 * b, 2 * b:2 * b + 2] = 1.0
+        W[2 * b + 1, 2 * b:2 * b + 2] = 1j, -1j
+    if n % 2:
+        lam[-1], W[-1, -1] = rng.uniform(-2.0, -0.05), 1.0
+    U = (np.eye(n) + 0.3 / np.sqrt(n) * rng.standard_normal((n, n))) @ W
+    return lam, U, np.linalg.inv(U), S.random_packed_tensor(n, N, seed + N)
+
+
+@pytest.mark.parametrize("n,N,precision", [
+    (1, 3, "split_bf16"), (3, 2, "split_bf16"), (3, 4, "split_bf16"), (9, 3, "split_bf16"),
+    (11, 4, "split_bf16"), (33, 3, "split_bf16"), (35, 3, "fp32"), (17, 4, "fp32"), (19, 4, "split_bf16"),
+    (65, 3, "split_bf16"), (67, 2, "split_bf16"), (71, 3, "fp32")])
+def test_term_odd_sizes(npf, n, N, precision):
+    lam, U, V, A = _odd_system(n, N, 40 * n + N)
+    ref = oracle.psiN(A, n, N, U, V, lam, p1_block=8)
+    with npf.Plan(lam, U, V, N, precision=precision) as p:
+        p.set_tensor(N, A)
+        assert rel_fro(p.term(N), ref) < (1e-10 if precision == "split_bf16" else 1e-5)
+
+
+@pytest.mark.parametrize("n,N,m", [(9, 3, 1), (21, 3, 5), (13, 4, 7), (67, 3, 33)])
+def test_subset_odd_sizes(npf, n, N, m):
+    lam, U, V, A = _odd_system(n, N, 50 * n + N)
+    modes = np.random.default_rng(n).permutation(n)[:m]
+    ref = oracle.psiN_subset(A, n, N, U, V, lam, modes)
+    with npf.Plan(lam, U, V, N) as p:
+        p.set_tensor(N, A)
+        full = p.term(N)                       # the tables of every mode, then of the subset
+        p.set_mode_subset(modes)
+        assert rel_fro(p.term(N), ref) < 1e-10
+        p.set_mode_subset(None)
+        assert rel_fro(p.term(N), full) < 1e-12
+
+
+@pytest.mark.parametrize("n,N", [(9, 3), (11, 4), (35, 3)])
+def test_few_upper_indices_and_new_modes(npf, n, N):
+    """Batches of a few upper indices, and modal data replaced in a plan whose tables exist."""
+    lam, U, V, A = _odd_system(n, N, 60 * n + N)
+    lam2, U2, V2, _ = _odd_system(n, N, 61 * n + N)
+    rad = 32 if n <= 32 else 64
+    dense = 2 * (rad ** (N - 1) * (rad * 4 * 6 + 4)) + 4096
+    fixed = n * (-(-comb(n + N - 1, N) // 128) * 128) * 16 + n * comb(n + N - 1, N) * 32
+    with npf.Plan(lam2, U2, V2, N) as p:
+        p.set_tensor(N, A)
+        p.term(N)
+        p.set_option(npf.OPT_MEM_BUDGET, fixed + dense)
+        p.set_modes(lam, U, V)
+        assert rel_fro(p.term(N), oracle.psiN(A, n, N, U, V, lam, p1_block=8)) < 1e-10
+        pre = [n - 1] * (N - 1)
+        assert rel_fro(p.modal_slab(N, pre), oracle.h_slab(A, n, N, U, V, lam, pre)) < 1e-10
+        p.set_option(npf.OPT_MEM_BUDGET, fixed + dense - 1)   # below one dense upper index: refused
+        with pytest.raises(npf.NpfError) as e:
+            p.term(N)
+        assert e.value.status == npf.NPF_ERR_OOM
