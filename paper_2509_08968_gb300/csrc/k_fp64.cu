@@ -192,7 +192,7 @@ static DivideArgs divide_args(const Plan& p, int N)
 }
 
 // Psi_N for one order, native FP64.
-void fp64_term(Plan& p, int N, double2* d_out, const double2* W)
+void fp64_term(Plan& p, int N, double2* d_out, const double2* W, bool accumulate)
 {
     if (p.nm != p.n)
         fail(NPF_ERR_UNSUPPORTED, "a critical-mode subset needs the tensor-core forms");
@@ -200,18 +200,27 @@ void fp64_term(Plan& p, int N, double2* d_out, const double2* W)
     const int n = p.n;
     const int64_t nN = ipow64(n, N);
     const int64_t P = p.packed_count[N];
+    // (a chain's scratch is far below any default budget: its size is not looked up)
+    if (!p.mem_budget && chain_fits(p, N, (size_t)1 << 30)) {
+        chain_term(p, N, d_out, W, accumulate);
+        return;
+    }
     const size_t budget = effective_budget(p);
     // Two ping-pong buffers of nb * n^N and one of nb * n^(N-1) complex doubles.
     const size_t per_nb = (2 * (size_t)nN + (size_t)nN / n) * sizeof(double2);
     int nb = (int)std::min<size_t>((size_t)n, budget / per_nb);
     if (nb < 1) fail(NPF_ERR_OOM, "memory budget too small for one output-index batch");
+    if (chain_fits(p, N, budget)) {
+        chain_term(p, N, d_out, W, accumulate);
+        return;
+    }
     Arena& ar = p.scratch();
     ar.reserve(per_nb * nb);
     double2* bufA = (double2*)ar.base;
     double2* bufB = bufA + (size_t)nb * nN;
     double2* bufC = bufB + (size_t)nb * nN;
 
-    launch_zero(p, d_out, (int64_t)n * n);
+    if (!accumulate) launch_zero(p, d_out, (int64_t)n * n);
     DivideArgs none = divide_args(p, N);
     for (int b0 = 0; b0 < n; b0 += nb) {
         const int cur = std::min(nb, n - b0);

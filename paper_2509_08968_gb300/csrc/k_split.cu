@@ -1919,7 +1919,22 @@ static T* upload(const std::vector<T>& v)
     return d;
 }
 
+// Bytes of the dense rows of one upper index (rad^(N-1) rows in two buffers).
+static size_t dense_bytes(int n, int N, int S)
+{
+    const int rad = n <= 32 ? 32 : n <= 64 ? 64 : 128;
+    return 2 * ((size_t)ipow64(rad, N - 1) * ((size_t)rad * 4 * S + 4)) + 4096;
+}
+
 #ifndef NPF_SPLIT_LOW
+// A term is accepted when S, its records and the dense rows of one upper index fit the budget (the
+// sorted rows it forms take less).
+size_t split_min_bytes(const Plan& p, int N)
+{
+    const int64_t P = p.packed_count[N], rows = (P + NP - 1) / NP * NP;
+    return (size_t)p.n * rows * sizeof(double2) + (size_t)p.n * P * 32 + dense_bytes(p.n, N, default_slices(p));
+}
+
 void split_release(Plan& p)
 {
     SplitOperand* so = p.split;
@@ -2350,7 +2365,7 @@ static double factorial(int N) { double f = 1; for (int t = 2; t <= N; ++t) f *=
 // batch two buffers that the stages alternate (A: the operands of the mode products and of the
 // reduction, B: V and the divide's slots) plus the row exponents.
 template <int S>
-static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const double2* W)
+static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const double2* W, bool accumulate)
 {
     SplitOperand& so = prepare(p);
     if (W) prepare_weights(p, so, W);
@@ -2385,18 +2400,16 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     const int64_t Qc = N >= 2 ? packed_count(nm, N - 1) : 0;      // reduction
     const int64_t v_per = N == 4 ? std::max(nm * arows(3), npairs * arows(2)) : N == 3 ? nm * arows(2) : 0;
 
-    // ---- memory plan (Algorithm 1's rule on the upper-index space). A call is accepted when the
-    // dense rows of one upper index (rad^(N-1) rows in two buffers) fit: the sorted rows take less.
+    // ---- memory plan (Algorithm 1's rule on the upper-index space)
     const size_t row_bytes = (size_t)rad * 4 * S;
     const size_t s_bytes = (size_t)n * Prows * sizeof(double2);
     const size_t rec_bytes = (size_t)n * P * 32;
-    const size_t dense_i = 2 * ((size_t)ipow64(rad, N - 1) * (row_bytes + 4)) + 4096;
     const size_t a_per = (size_t)std::max(std::max(R0, R1), std::max(R2, Qc)) * row_bytes;
     const size_t b_per = std::max((size_t)v_per * sizeof(longlong2), (size_t)RS * row_bytes);
     const size_t e_per = (size_t)(R1 + R2 + RS + Qc) * sizeof(int);
-    const size_t per_i = std::min(dense_i, a_per + b_per + e_per);
+    const size_t per_i = std::min(dense_bytes(n, N, S), a_per + b_per + e_per);
     const size_t budget = effective_budget(p);
-    if (s_bytes + rec_bytes + dense_i > budget)
+    if (split_min_bytes(p, N) > budget)
         fail(NPF_ERR_OOM, "memory budget too small for one upper-index batch");
     const int ib = (int)std::min<size_t>((size_t)nm, (budget - s_bytes - rec_bytes) / per_i);
     const int64_t Q2 = N == 4 && !slab ? npairs : 0;              // order 4: weights of the pairs
@@ -2425,7 +2438,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     }
 
     // a slab entry whose accumulator is exactly zero is not stored, so the slab starts at zero
-    launch_zero(p, d_out, (int64_t)n * n);
+    if (!accumulate) launch_zero(p, d_out, (int64_t)n * n);
 
     const FixedOp tPhi{so.phi, KP};
     const FixedOp tPsiR{so.psir, NP};
@@ -2604,32 +2617,38 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
 
 // The 2..5-slice runs live in a second translation unit (k_split_low.cu, these sources compiled
 // with NPF_SPLIT_LOW), so that the kernel instantiations of the two halves build in parallel.
-void split_run_low(Plan& p, int S, int N, double2* d_out, const int* prefix, const double2* W);
+void split_run_low(Plan& p, int S, int N, double2* d_out, const int* prefix, const double2* W, bool accumulate);
 
 #ifdef NPF_SPLIT_LOW
-void split_run_low(Plan& p, int S, int N, double2* d_out, const int* prefix, const double2* W)
+void split_run_low(Plan& p, int S, int N, double2* d_out, const int* prefix, const double2* W, bool accumulate)
 {
     switch (S) {
-    case 2: split_run<2>(p, N, d_out, prefix, W); break;
-    case 3: split_run<3>(p, N, d_out, prefix, W); break;
-    case 4: split_run<4>(p, N, d_out, prefix, W); break;
-    case 5: split_run<5>(p, N, d_out, prefix, W); break;
+    case 2: split_run<2>(p, N, d_out, prefix, W, accumulate); break;
+    case 3: split_run<3>(p, N, d_out, prefix, W, accumulate); break;
+    case 4: split_run<4>(p, N, d_out, prefix, W, accumulate); break;
+    case 5: split_run<5>(p, N, d_out, prefix, W, accumulate); break;
     default: fail(NPF_ERR_UNSUPPORTED, "slices must be in [2, 6] on the tensor-core path");
     }
 }
 #else
-static void split_any(Plan& p, int N, double2* d_out, const int* prefix, const double2* W)
+static void split_any(Plan& p, int N, double2* d_out, const int* prefix, const double2* W, bool accumulate)
 {
     if (N < 1 || (N == 1 && !prefix)) fail(NPF_ERR_ARG, "order must be >= 2 (order 1: modal slabs only)");
     if (N > 4) fail(NPF_ERR_UNSUPPORTED, "the tensor-core path supports orders <= 4 (use NPF_PREC_FP64)");
     const int S = default_slices(p);
-    if (S == 6) split_run<6>(p, N, d_out, prefix, W);
-    else if (S >= 2 && S <= 5) split_run_low(p, S, N, d_out, prefix, W);
+    if (S == 6) split_run<6>(p, N, d_out, prefix, W, accumulate);
+    else if (S >= 2 && S <= 5) split_run_low(p, S, N, d_out, prefix, W, accumulate);
     else fail(NPF_ERR_UNSUPPORTED, "slices must be in [2, 6] on the tensor-core path");
 }
 
-void split_term(Plan& p, int N, double2* d_out, const double2* W) { split_any(p, N, d_out, nullptr, W); }
-void split_slab(Plan& p, int N, const int* prefix, double2* d_out) { split_any(p, N, d_out, prefix, nullptr); }
+void split_term(Plan& p, int N, double2* d_out, const double2* W, bool accumulate)
+{
+    split_any(p, N, d_out, nullptr, W, accumulate);
+}
+void split_slab(Plan& p, int N, const int* prefix, double2* d_out)
+{
+    split_any(p, N, d_out, prefix, nullptr, false);
+}
 #endif
 
 }  // namespace npf

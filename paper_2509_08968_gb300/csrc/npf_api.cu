@@ -235,19 +235,39 @@ int tuned_tile(Plan& p, int N)
 }
 
 // -sum_p h^i_p prod_m W[p_m][k] into out (W = nullptr: the left eigenvectors, i.e. Psi_N).
-void compute_term(Plan& p, int N, double2* out, const double2* W = nullptr)
+// Small systems: the tensor-core forms run the FP64 chain too (k_chain.cu), two launches an order
+// instead of eight to ten. Time of one call, orders 2 / 3 / 4, chain against tensor-core path:
+// n = 40 / 20 / 12: 122 / 118 / 131 us against 161 / 157 / 177; n = 48 / 24 / 14: 183 / 193 / 266
+// against 168 / 168 / 211 (its work grows as n^4 / n^5 / n^6 on the FP64 pipe). Options that choose
+// how the tensor-core path works keep it, and a budget too small for it is refused as before.
+bool small_system(const Plan& p, int N)
+{
+    constexpr int limit[5] = {0, 0, 44, 22, 12};
+    if (N < 2 || N > 4 || p.n > limit[N] || p.slices || p.tile_n != 32 || p.fp64_quotient || p.debug_stall)
+        return false;
+    if (p.mem_budget && npf::split_min_bytes(p, N) > p.mem_budget)
+        npf::fail(NPF_ERR_OOM, "memory budget too small for one upper-index batch");
+    return npf::chain_fits(p, N, p.mem_budget ? p.mem_budget : (size_t)-1);
+}
+
+// accumulate: added to out.
+void compute_term(Plan& p, int N, double2* out, const double2* W = nullptr, bool accumulate = false)
 {
     if (p.precision == NPF_PREC_FP64) {
-        npf::fp64_term(p, N, out, W);
+        npf::fp64_term(p, N, out, W, accumulate);
+        return;
+    }
+    if (small_system(p, N)) {
+        npf::chain_term(p, N, out, W, accumulate);
         return;
     }
     if (p.tile_n != 0) {
-        npf::split_term(p, N, out, W);
+        npf::split_term(p, N, out, W, accumulate);
         return;
     }
     p.tile_n = tuned_tile(p, N);
     try {
-        npf::split_term(p, N, out, W);
+        npf::split_term(p, N, out, W, accumulate);
     } catch (...) {
         p.tile_n = 0;
         throw;
@@ -258,14 +278,13 @@ void compute_term(Plan& p, int N, double2* out, const double2* W = nullptr)
 // Psi_m for every order 2..order that has a tensor, summed into d_sum; NPF into d_npf.
 void compute_npf(Plan& p, int order)
 {
-    const int64_t nn = (int64_t)p.n * p.n;
-    npf::launch_zero(p, p.d_sum, nn);
+    bool any = false;
     for (int m = 2; m <= order; ++m) {
         if (!p.d_tensor[m]) continue;
-        compute_term(p, m, p.d_psiN[m]);
-        npf::launch_add(p, p.d_sum, p.d_psiN[m], nn);
+        compute_term(p, m, p.d_sum, nullptr, any);   // the first term replaces d_sum
+        any = true;
     }
-    npf::launch_finish(p, order >= 2 ? p.d_sum : nullptr, p.d_npf);
+    npf::launch_finish(p, any ? p.d_sum : nullptr, p.d_npf);
     if (p.permuted()) {   // modes back to the caller's order
         npf::launch_unpermute(p, p.d_npf, p.d_tmp, true);
         NPF_CUDA(cudaMemcpyAsync(p.d_npf, p.d_tmp, (size_t)p.n * p.n * sizeof(double2),

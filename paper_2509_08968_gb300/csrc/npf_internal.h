@@ -136,14 +136,22 @@ size_t effective_budget(const Plan& p);
 // Native FP64 path (k_fp64.cu).
 // ----------------------------------------------------------------------------------------
 // Psi_N [n][n] = -sum_p h^i_p prod_m W[p_m][k]; W = nullptr: the left eigenvectors (W = V).
-void fp64_term(Plan& p, int N, double2* d_out, const double2* W = nullptr);
+// accumulate: added to d_out instead of replacing it.
+void fp64_term(Plan& p, int N, double2* d_out, const double2* W = nullptr, bool accumulate = false);
 void fp64_slab(Plan& p, int N, const int* prefix, double2* d_out /* h [n][n] */);
+
+// ----------------------------------------------------------------------------------------
+// Native FP64 term with the chain in shared memory (k_chain.cu): orders 2 to 4 that fit.
+// ----------------------------------------------------------------------------------------
+bool chain_fits(const Plan& p, int N, size_t budget);
+void chain_term(Plan& p, int N, double2* d_out, const double2* W, bool accumulate);
 
 // ----------------------------------------------------------------------------------------
 // Split BF16 tensor-core path (k_split.cu).
 // ----------------------------------------------------------------------------------------
-void split_term(Plan& p, int N, double2* d_out, const double2* W = nullptr);
+void split_term(Plan& p, int N, double2* d_out, const double2* W = nullptr, bool accumulate = false);
 void split_slab(Plan& p, int N, const int* prefix, double2* d_out);
+size_t split_min_bytes(const Plan& p, int N);   // smallest budget a term is accepted with
 void split_release(Plan& p);
 void split_prepare_tensor(Plan& p, int N);   // digit planes of a newly uploaded tensor
 const void* split_tensor_planes(const Plan& p, int N);   // device address of those planes

@@ -35,7 +35,7 @@ def _odd_system(n, N, seed):
     if n % 2:
         lam[-1], W[-1, -1] = rng.uniform(-2.0, -0.05), 1.0
     U = (np.eye(n) + 0.3 / np.sqrt(n) * rng.standard_normal((n, n))) @ W
-    return lam, U, np.linalg.inv(U), S.random_packed_tensor(n, N, seed + N)
+    return lam, U, np.linalg.inv(U), S.random_packed_tensor_dense_fill(n, N, seed + N)
 
 
 @pytest.mark.parametrize("n,N,precision", [
