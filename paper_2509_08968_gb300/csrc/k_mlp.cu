@@ -21,32 +21,45 @@
 namespace npf {
 namespace mlp {
 
-constexpr int TM = 64, TN = 64, TK = 32, PAD = 8;
+constexpr int TM = 64, TN = 64, TK = 32, STAGES = 4;
 constexpr int kMaxRows = 65536;
+constexpr int kMaxLayers = 8;
+// a stage of one operand: 64 rows of 32 + 8 K-contiguous elements, or 32 K rows of 64 + 8
+// (both strides keep the eight rows of an ldmatrix on different banks)
+constexpr int LDN = TK + 8, LDT = TM + 8;
+constexpr int STAGE = TM * LDN > TK * LDT ? TM * LDN : TK * LDT;
 
-enum { EPI_F32 = 0, EPI_RELU_BF16 = 1, EPI_MASK_BF16 = 2 };
+enum { EPI_F32 = 0, EPI_RELU_BF16 = 1, EPI_MASK_BF16 = 2, EPI_LOSS = 3, EPI_ADAM = 4 };
 
 // C[e] = op(A[e]) op(B[e]) over M x N with inner dimension K.
-//   A element (m, k): a_t == 0 -> A[m * lda + k], a_t == 1 -> A[k * lda + m]
-//   B element (k, n): b_t == 0 -> B[n * ldb + k], b_t == 1 -> B[k * ldb + n]
+//   A element (m, k): AT == 0 -> A[m * lda + k], AT == 1 -> A[k * lda + m]
+//   B element (k, n): BT == 0 -> B[n * ldb + k], BT == 1 -> B[k * ldb + n]
+// Leading dimensions are multiples of 8 and rows start on 16 bytes; elements between K (or M, N)
+// and the leading dimension are zero or feed outputs that are not stored.
 struct Gemm {
     int M, N, K;
     const __nv_bfloat16* A;
     int64_t lda, sA;
-    int a_t;
     const __nv_bfloat16* B;
     int64_t ldb, sB;
-    int b_t;
     void* C;
     int64_t ldc, sC;
     const __nv_bfloat16* mask;   // EPI_MASK_BF16: keep C(m, n) where mask(m, n) > 0
     int64_t ldm, sM;
+    const float* T;              // EPI_LOSS: targets [M][N]; C holds the output error in BF16
+    int64_t sT;
+    double* loss;                // EPI_LOSS: per member, += sum (Y - T)^2 / (M N)
 };
 
-__device__ __forceinline__ uint32_t ld_pair(const __nv_bfloat16* p)
-{
-    return *reinterpret_cast<const uint32_t*>(p);
-}
+// EPI_ADAM: the weight gradients of every layer in one launch, each tile updating its weights.
+struct AdamStep {
+    int layers;
+    int tile0[kMaxLayers + 1];   // first tile of a layer
+    Gemm g[kMaxLayers];          // C: offset of the layer's block in the parameter arrays, in floats
+    float *W, *M1, *M2;
+    __nv_bfloat16* Wb;
+    float lr, b1, b2, eps, c1, c2;
+};
 
 // D (16x8, FP32) += A (16x16, BF16, row-major fragment) * B (16x8, BF16, column fragment).
 __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4],
@@ -59,97 +72,185 @@ __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4],
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-// 64 x 64 output tile per CTA, four warps of 32 x 32, K in steps of 32 staged in shared memory
-// (rows K-contiguous whatever the source layout; out-of-range elements read as zero).
-template <int EPI>
-__global__ void __launch_bounds__(128) k_gemm(Gemm g)
+template <bool TRANS>
+__device__ __forceinline__ void ldmatrix4(uint32_t (&r)[4], const __nv_bfloat16* p)
 {
-    __shared__ __align__(16) __nv_bfloat16 sA[TM][TK + PAD];
-    __shared__ __align__(16) __nv_bfloat16 sB[TN][TK + PAD];
-    const int e = blockIdx.z;
+    const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+    if (TRANS)
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
+    else
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
+}
+
+// 16 bytes global -> shared, zeros when `ok` is false (the source is not read then).
+__device__ __forceinline__ void copy16(__nv_bfloat16* dst, const __nv_bfloat16* src, bool ok)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                 ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(ok ? 16 : 0) : "memory");
+}
+
+// One operand's stage: rows r0.. (TRANS: K rows k0.., columns r0..) of a matrix with R rows (K-contiguous
+// layout) or columns, K extent K.
+template <bool TRANS>
+__device__ __forceinline__ void load_stage(__nv_bfloat16* s, const __nv_bfloat16* src, int64_t ld, int r0,
+                                           int R, int k0, int K)
+{
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const int idx = (int)threadIdx.x + 128 * j;
+        if (TRANS) {
+            const int k = idx / (TM / 8), c = idx % (TM / 8) * 8;
+            const bool ok = k0 + k < K && r0 + c + 8 <= ld;
+            copy16(s + k * LDT + c, ok ? src + (int64_t)(k0 + k) * ld + r0 + c : src, ok);
+        } else {
+            const int r = idx / (TK / 8), c = idx % (TK / 8) * 8;
+            const bool ok = r0 + r < R && k0 + c + 8 <= ld;
+            copy16(s + r * LDN + c, ok ? src + (int64_t)(r0 + r) * ld + k0 + c : src, ok);
+        }
+    }
+}
+
+// 64 x 64 output tile per CTA, four warps of 32 x 32, K in steps of 32 through a ring of four
+// shared-memory stages filled by 16-byte asynchronous copies; fragments by ldmatrix (transposed
+// where the source is M- or N-contiguous). The products are small (256 x 272 x 256 a layer and
+// member), so the time is the latency of the K loop: with scalar loads and one stage a step of the
+// 4-256-256-256-64 ensemble of five took 203 us at 256 rows.
+template <bool AT, bool BT>
+__device__ __forceinline__ void gemm_tile(const Gemm& g, int e, int m0, int n0, __nv_bfloat16* sA,
+                                          __nv_bfloat16* sB, float (&acc)[2][4][4])
+{
     const __nv_bfloat16* A = g.A + e * g.sA;
     const __nv_bfloat16* B = g.B + e * g.sB;
-    const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
-    const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
-    const int wm = warp / 2, wn = warp % 2;
-    const int gq = lane / 4, tq = lane % 4;
-    float acc[2][4][4];
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int wm = warp / 2 * 32, wn = warp % 2 * 32;
 #pragma unroll
     for (int mi = 0; mi < 2; ++mi)
 #pragma unroll
         for (int ni = 0; ni < 4; ++ni)
 #pragma unroll
             for (int c = 0; c < 4; ++c) acc[mi][ni][c] = 0.f;
-    const __nv_bfloat16 zero = __float2bfloat16(0.f);
-
-    for (int k0 = 0; k0 < g.K; k0 += TK) {
-        for (int j = 0; j < TM * TK / 128; ++j) {
-            const int idx = tid + 128 * j;
-            const int m = g.a_t ? idx % TM : idx / TK;
-            const int k = g.a_t ? idx / TM : idx % TK;
-            const int gm = m0 + m, gk = k0 + k;
-            __nv_bfloat16 v = zero;
-            if (gm < g.M && gk < g.K)
-                v = g.a_t ? A[(int64_t)gk * g.lda + gm] : A[(int64_t)gm * g.lda + gk];
-            sA[m][k] = v;
+    const int steps = (g.K + TK - 1) / TK;
+    auto fetch = [&](int st) {
+        if (st < steps) {
+            load_stage<AT>(sA + (st % STAGES) * STAGE, A, g.lda, m0, g.M, st * TK, g.K);
+            load_stage<BT>(sB + (st % STAGES) * STAGE, B, g.ldb, n0, g.N, st * TK, g.K);
         }
-        for (int j = 0; j < TN * TK / 128; ++j) {
-            const int idx = tid + 128 * j;
-            const int n = g.b_t ? idx % TN : idx / TK;
-            const int k = g.b_t ? idx / TN : idx % TK;
-            const int gn = n0 + n, gk = k0 + k;
-            __nv_bfloat16 v = zero;
-            if (gn < g.N && gk < g.K)
-                v = g.b_t ? B[(int64_t)gk * g.ldb + gn] : B[(int64_t)gn * g.ldb + gk];
-            sB[n][k] = v;
-        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+#pragma unroll
+    for (int st = 0; st < STAGES - 1; ++st) fetch(st);
+    const int l8 = lane % 8, lq = lane / 8;   // row within an 8 x 8 matrix, matrix of the four
+    for (int st = 0; st < steps; ++st) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
         __syncthreads();
+        fetch(st + STAGES - 1);
+        const __nv_bfloat16* a = sA + (st % STAGES) * STAGE;
+        const __nv_bfloat16* b = sB + (st % STAGES) * STAGE;
 #pragma unroll
         for (int ks = 0; ks < TK; ks += 16) {
             uint32_t af[2][4], bf[4][2];
-            const int c = ks + tq * 2;
 #pragma unroll
             for (int mi = 0; mi < 2; ++mi) {
-                const int r = wm * 32 + mi * 16 + gq;
-                af[mi][0] = ld_pair(&sA[r][c]);
-                af[mi][1] = ld_pair(&sA[r + 8][c]);
-                af[mi][2] = ld_pair(&sA[r][c + 8]);
-                af[mi][3] = ld_pair(&sA[r + 8][c + 8]);
+                // matrices (m, k): (0, 0), (8, 0), (0, 8), (8, 8)
+                const int m = wm + mi * 16 + (lq & 1) * 8, k = ks + (lq >> 1) * 8;
+                if (AT) ldmatrix4<true>(af[mi], a + (k + l8) * LDT + m);
+                else ldmatrix4<false>(af[mi], a + (m + l8) * LDN + k);
             }
 #pragma unroll
-            for (int ni = 0; ni < 4; ++ni) {
-                const int nn = wn * 32 + ni * 8 + gq;
-                bf[ni][0] = ld_pair(&sB[nn][c]);
-                bf[ni][1] = ld_pair(&sB[nn][c + 8]);
+            for (int nj = 0; nj < 2; ++nj) {
+                // matrices (n, k): (0, 0), (0, 8), (8, 0), (8, 8)
+                const int n = wn + nj * 16 + (lq >> 1) * 8, k = ks + (lq & 1) * 8;
+                uint32_t r[4];
+                if (BT) ldmatrix4<true>(r, b + (k + l8) * LDT + n);
+                else ldmatrix4<false>(r, b + (n + l8) * LDN + k);
+                bf[2 * nj][0] = r[0]; bf[2 * nj][1] = r[1];
+                bf[2 * nj + 1][0] = r[2]; bf[2 * nj + 1][1] = r[3];
             }
 #pragma unroll
             for (int mi = 0; mi < 2; ++mi)
 #pragma unroll
                 for (int ni = 0; ni < 4; ++ni) mma16816(acc[mi][ni], af[mi], bf[ni]);
         }
-        __syncthreads();
     }
+}
 
+// f(m, n, value) for the thread's elements of the tile that lie in the matrix.
+template <class F>
+__device__ __forceinline__ void for_outputs(const Gemm& g, int m0, int n0, const float (&acc)[2][4][4], F&& f)
+{
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
 #pragma unroll
     for (int mi = 0; mi < 2; ++mi)
 #pragma unroll
         for (int ni = 0; ni < 4; ++ni)
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const int m = m0 + wm * 32 + mi * 16 + gq + (q >= 2 ? 8 : 0);
-                const int n = n0 + wn * 32 + ni * 8 + tq * 2 + (q & 1);
-                if (m >= g.M || n >= g.N) continue;
-                const float v = acc[mi][ni][q];
-                const int64_t o = e * g.sC + (int64_t)m * g.ldc + n;
-                if (EPI == EPI_F32) {
-                    static_cast<float*>(g.C)[o] = v;
-                } else if (EPI == EPI_RELU_BF16) {
-                    static_cast<__nv_bfloat16*>(g.C)[o] = __float2bfloat16_rn(fmaxf(v, 0.f));
-                } else {
-                    const float mk = __bfloat162float(g.mask[e * g.sM + (int64_t)m * g.ldm + n]);
-                    static_cast<__nv_bfloat16*>(g.C)[o] = __float2bfloat16_rn(mk > 0.f ? v : 0.f);
-                }
+                const int m = m0 + warp / 2 * 32 + mi * 16 + lane / 4 + (q >= 2 ? 8 : 0);
+                const int n = n0 + warp % 2 * 32 + ni * 8 + lane % 4 * 2 + (q & 1);
+                if (m < g.M && n < g.N) f(m, n, acc[mi][ni][q]);
             }
+}
+
+template <int EPI, bool AT, bool BT>
+__global__ void __launch_bounds__(128) k_gemm(const __grid_constant__ Gemm g)
+{
+    __shared__ __align__(16) __nv_bfloat16 sA[STAGES * STAGE], sB[STAGES * STAGE];
+    const int e = blockIdx.z, m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
+    float acc[2][4][4];
+    gemm_tile<AT, BT>(g, e, m0, n0, sA, sB, acc);
+    double part = 0.0;
+    const float scale2 = EPI == EPI_LOSS ? (float)(2.0 * (1.0 / ((double)g.M * g.N))) : 0.f;
+    for_outputs(g, m0, n0, acc, [&](int m, int n, float v) {
+        const int64_t o = e * g.sC + (int64_t)m * g.ldc + n;
+        if (EPI == EPI_F32) {
+            static_cast<float*>(g.C)[o] = v;
+        } else if (EPI == EPI_RELU_BF16) {
+            static_cast<__nv_bfloat16*>(g.C)[o] = __float2bfloat16_rn(fmaxf(v, 0.f));
+        } else if (EPI == EPI_MASK_BF16) {
+            const float mk = __bfloat162float(g.mask[e * g.sM + (int64_t)m * g.ldm + n]);
+            static_cast<__nv_bfloat16*>(g.C)[o] = __float2bfloat16_rn(mk > 0.f ? v : 0.f);
+        } else {   // mean squared error: the output's error 2 (Y - T) / (M N), and the loss
+            const float d = v - g.T[e * g.sT + (int64_t)m * g.N + n];
+            static_cast<__nv_bfloat16*>(g.C)[o] = __float2bfloat16_rn(scale2 * d);
+            part += (double)d * d;
+        }
+    });
+    if (EPI == EPI_LOSS) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+        __shared__ double red[4];
+        if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = part;
+        __syncthreads();
+        if (threadIdx.x == 0)
+            atomicAdd(&g.loss[e], (red[0] + red[1] + red[2] + red[3]) * (1.0 / ((double)g.M * g.N)));
+    }
+}
+
+// Weight gradients G_l = dZ_l^T H_l of every layer and the Adam step of their weights: no gradient
+// array, and one launch instead of one a layer and one over all parameters. The back-propagation has
+// read the weights before.
+__global__ void __launch_bounds__(128) k_grad_adam(const __grid_constant__ AdamStep s)
+{
+    __shared__ __align__(16) __nv_bfloat16 sA[STAGES * STAGE], sB[STAGES * STAGE];
+    int l = 0;
+    while (l + 1 < s.layers && (int)blockIdx.x >= s.tile0[l + 1]) ++l;
+    const Gemm& g = s.g[l];
+    const int t = (int)blockIdx.x - s.tile0[l], nt = (g.N + TN - 1) / TN;
+    const int e = blockIdx.z, m0 = t / nt * TM, n0 = t % nt * TN;
+    float acc[2][4][4];
+    gemm_tile<true, true>(g, e, m0, n0, sA, sB, acc);
+    for_outputs(g, m0, n0, acc, [&](int m, int n, float gr) {
+        const int64_t o = e * g.sC + reinterpret_cast<int64_t>(g.C) + (int64_t)m * g.ldc + n;
+        const float m1 = s.b1 * s.M1[o] + (1.f - s.b1) * gr;
+        const float m2 = s.b2 * s.M2[o] + (1.f - s.b2) * gr * gr;
+        s.M1[o] = m1;
+        s.M2[o] = m2;
+        const float w = s.W[o] - s.lr * (m1 / s.c1) / (sqrtf(m2 / s.c2) + s.eps);
+        s.W[o] = w;
+        s.Wb[o] = __float2bfloat16_rn(w);
+    });
 }
 
 // Augmented BF16 inputs Xa[e][b][ip] = (X[r][0..w0-1], 1, 0, ..) with r = idx[e][b] (or b), and
@@ -190,51 +291,6 @@ __global__ void k_const_cols(int E, int64_t cap, int w, int ip, __nv_bfloat16* _
         const int c = (int)(t % pad);
         const int64_t row = t / pad;
         h[row * ip + w + c] = __float2bfloat16_rn(c == 0 ? 1.f : 0.f);
-    }
-}
-
-// Mean squared error: dY = 2 (Y - T) / (Bn wo) in BF16 and loss[e] += sum (Y - T)^2 / (Bn wo).
-__global__ void k_loss(int Bn, int wo, int64_t cap, const float* __restrict__ Y,
-                       const float* __restrict__ Tb, __nv_bfloat16* __restrict__ dY,
-                       double* __restrict__ loss)
-{
-    const int e = blockIdx.y;
-    const int64_t tot = (int64_t)Bn * wo;
-    const double scale = 1.0 / (double)tot;
-    double part = 0.0;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < tot;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t o = (int64_t)e * cap * wo + t;
-        const float d = Y[o] - Tb[o];
-        dY[o] = __float2bfloat16_rn((float)(2.0 * scale) * d);
-        part += (double)d * d;
-    }
-    __shared__ double red[256];
-    red[threadIdx.x] = part;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) atomicAdd(&loss[e], red[0] * scale);
-}
-
-// Adam step over every parameter of every member; BF16 copy of the updated weights.
-__global__ void k_adam(int64_t total, float* __restrict__ W, float* __restrict__ M1,
-                       float* __restrict__ M2, const float* __restrict__ G,
-                       __nv_bfloat16* __restrict__ Wb, float lr, float b1, float b2, float eps,
-                       float c1, float c2)
-{
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const float g = G[t];
-        const float m = b1 * M1[t] + (1.f - b1) * g;
-        const float v = b2 * M2[t] + (1.f - b2) * g * g;
-        M1[t] = m;
-        M2[t] = v;
-        const float w = W[t] - lr * (m / c1) / (sqrtf(v / c2) + eps);
-        W[t] = w;
-        Wb[t] = __float2bfloat16_rn(w);
     }
 }
 
@@ -312,7 +368,8 @@ struct npf_mlp {
     // activations, capacity `cap` rows per member
     int64_t cap = 0;
     std::vector<__nv_bfloat16*> H;    // H[l]: [E][cap][ip_l], l < L
-    std::vector<__nv_bfloat16*> dZ;   // dZ[l]: [E][cap][w_{l+1}]
+    std::vector<__nv_bfloat16*> dZ;   // dZ[l]: [E][cap][zp_l], zero past w_{l+1}
+    std::vector<int> zp;      // leading dimensions of dZ: w_{l+1} rounded up to 8
     float* Y = nullptr;               // [E][cap][w_L]
     float* Tb = nullptr;              // [E][cap][w_L]
     double* d_loss = nullptr;         // [E]
@@ -377,7 +434,11 @@ void reserve_rows(npf_mlp& m, int64_t rows)
     release_acts(m);
     const int64_t cap = std::max<int64_t>(rows, 256);
     for (int l = 0; l < m.L; ++l) m.H.push_back(dalloc<__nv_bfloat16>(m.E * cap * m.ip[l]));
-    for (int l = 0; l < m.L; ++l) m.dZ.push_back(dalloc<__nv_bfloat16>(m.E * cap * m.w[l + 1]));
+    for (int l = 0; l < m.L; ++l) {
+        m.dZ.push_back(dalloc<__nv_bfloat16>(m.E * cap * m.zp[l]));
+        if (m.zp[l] != m.w[l + 1])
+            NPF_CUDA(cudaMemsetAsync(m.dZ[l], 0, (size_t)m.E * cap * m.zp[l] * sizeof(__nv_bfloat16), m.s));
+    }
     m.Y = dalloc<float>(m.E * cap * m.w[m.L]);
     m.Tb = dalloc<float>(m.E * cap * m.w[m.L]);
     m.cap = cap;
@@ -400,12 +461,12 @@ void stage(float*& dst, int64_t& capf, const float* src, int64_t count, cudaStre
     NPF_CUDA(cudaMemcpyAsync(dst, src, (size_t)count * sizeof(float), cudaMemcpyDefault, s));
 }
 
-template <int EPI>
+template <int EPI, bool AT, bool BT>
 void gemm(npf_mlp& m, const char* name, const Gemm& g)
 {
     npf::LaunchScope ls(nullptr, name, m.s);
     dim3 grid((unsigned)((g.N + TN - 1) / TN), (unsigned)((g.M + TM - 1) / TM), (unsigned)m.E);
-    k_gemm<EPI><<<grid, 128, 0, m.s>>>(g);
+    k_gemm<EPI, AT, BT><<<grid, 128, 0, m.s>>>(g);
     NPF_CUDA(cudaGetLastError());
 }
 
@@ -419,54 +480,58 @@ void gather(npf_mlp& m, int rows, const float* dX, const float* dT, const int* i
     NPF_CUDA(cudaGetLastError());
 }
 
-void forward(npf_mlp& m, int rows)
+// loss: the last layer's epilogue forms the output's error and the loss instead of storing Y
+void forward(npf_mlp& m, int rows, bool loss)
 {
     for (int l = 0; l < m.L; ++l) {
         Gemm g{};
         g.M = rows;
         g.N = m.w[l + 1];
         g.K = m.ip[l];
-        g.A = m.H[l]; g.lda = m.ip[l]; g.sA = m.cap * m.ip[l]; g.a_t = 0;
-        g.B = m.Wb + m.off[l]; g.ldb = m.ip[l]; g.sB = m.P; g.b_t = 0;
+        g.A = m.H[l]; g.lda = m.ip[l]; g.sA = m.cap * m.ip[l];
+        g.B = m.Wb + m.off[l]; g.ldb = m.ip[l]; g.sB = m.P;
         if (l + 1 < m.L) {
             g.C = m.H[l + 1]; g.ldc = m.ip[l + 1]; g.sC = m.cap * m.ip[l + 1];
-            gemm<EPI_RELU_BF16>(m, "mlp_forward_relu", g);
-        } else {
+            gemm<EPI_RELU_BF16, false, false>(m, "mlp_forward_relu", g);
+        } else if (!loss) {
             g.C = m.Y; g.ldc = m.w[m.L]; g.sC = m.cap * m.w[m.L];
-            gemm<EPI_F32>(m, "mlp_forward_out", g);
+            gemm<EPI_F32, false, false>(m, "mlp_forward_out", g);
+        } else {
+            g.C = m.dZ[l]; g.ldc = m.zp[l]; g.sC = m.cap * m.zp[l];
+            g.T = m.Tb; g.sT = m.cap * m.w[m.L];
+            g.loss = m.d_loss;
+            gemm<EPI_LOSS, false, false>(m, "mlp_forward_loss", g);
         }
     }
 }
 
-void loss_and_backward(npf_mlp& m, int rows)
+// Errors of the hidden layers: dZ_{l-1} = (dZ_l W_l)[:, :w_l] o (h_l > 0)
+void backward(npf_mlp& m, int rows)
 {
-    const int wo = m.w[m.L];
-    {
-        npf::LaunchScope ls(nullptr, "mlp_loss", m.s);
-        dim3 grid(grid_for((int64_t)rows * wo, 256 * 8), (unsigned)m.E);
-        k_loss<<<grid, 256, 0, m.s>>>(rows, wo, m.cap, m.Y, m.Tb, m.dZ[m.L - 1], m.d_loss);
-        NPF_CUDA(cudaGetLastError());
-    }
-    for (int l = m.L - 1; l >= 0; --l) {
-        Gemm g{};   // weight gradient: G_l = dZ_l^T H_l  ([w_{l+1}] x [ip_l], K = rows)
-        g.M = m.w[l + 1];
-        g.N = m.ip[l];
-        g.K = rows;
-        g.A = m.dZ[l]; g.lda = m.w[l + 1]; g.sA = m.cap * m.w[l + 1]; g.a_t = 1;
-        g.B = m.H[l]; g.ldb = m.ip[l]; g.sB = m.cap * m.ip[l]; g.b_t = 1;
-        g.C = m.G + m.off[l]; g.ldc = m.ip[l]; g.sC = m.P;
-        gemm<EPI_F32>(m, "mlp_weight_grad", g);
-        if (l == 0) break;
-        Gemm d{};   // error of the layer below: dZ_{l-1} = (dZ_l W_l)[:, :w_l] o (h_l > 0)
+    for (int l = m.L - 1; l >= 1; --l) {
+        Gemm d{};
         d.M = rows;
         d.N = m.w[l];
         d.K = m.w[l + 1];
-        d.A = m.dZ[l]; d.lda = m.w[l + 1]; d.sA = m.cap * m.w[l + 1]; d.a_t = 0;
-        d.B = m.Wb + m.off[l]; d.ldb = m.ip[l]; d.sB = m.P; d.b_t = 1;
-        d.C = m.dZ[l - 1]; d.ldc = m.w[l]; d.sC = m.cap * m.w[l];
+        d.A = m.dZ[l]; d.lda = m.zp[l]; d.sA = m.cap * m.zp[l];
+        d.B = m.Wb + m.off[l]; d.ldb = m.ip[l]; d.sB = m.P;
+        d.C = m.dZ[l - 1]; d.ldc = m.zp[l - 1]; d.sC = m.cap * m.zp[l - 1];
         d.mask = m.H[l]; d.ldm = m.ip[l]; d.sM = m.cap * m.ip[l];
-        gemm<EPI_MASK_BF16>(m, "mlp_backprop", d);
+        gemm<EPI_MASK_BF16, false, true>(m, "mlp_backprop", d);
     }
+}
+
+// Weight gradient of a layer: G_l = dZ_l^T H_l ([w_{l+1}] x [ip_l], K = rows)
+Gemm weight_grad(const npf_mlp& m, int rows, int l)
+{
+    Gemm g{};
+    g.M = m.w[l + 1];
+    g.N = m.ip[l];
+    g.K = rows;
+    g.A = m.dZ[l]; g.lda = m.zp[l]; g.sA = m.cap * m.zp[l];
+    g.B = m.H[l]; g.ldb = m.ip[l]; g.sB = m.cap * m.ip[l];
+    g.ldc = m.ip[l]; g.sC = m.P;
+    return g;
 }
 
 void sync(npf_mlp& m) { NPF_CUDA(cudaStreamSynchronize(m.s)); }
@@ -523,6 +588,7 @@ npf_mlp* npf_mlp_create(int ensemble, int layers, const int* widths, const float
             m->ip.push_back((m->w[l] + 1 + 15) / 16 * 16);
             m->off.push_back(m->P);
             m->offp.push_back(m->Ppub);
+            m->zp.push_back((m->w[l + 1] + 7) / 8 * 8);
             m->P += (int64_t)m->w[l + 1] * m->ip[l];
             m->Ppub += (int64_t)m->w[l + 1] * (m->w[l] + 1);
         }
@@ -574,7 +640,7 @@ int npf_mlp_forward(npf_mlp* m, int rows, const float* X, float* Y)
         reserve_rows(*m, rows);
         stage(m->d_X, m->xcap, X, (int64_t)rows * m->w[0], m->s);
         gather(*m, rows, m->d_X, nullptr, nullptr, 0);
-        forward(*m, rows);
+        forward(*m, rows, false);
         const int wo = m->w[m->L];
         NPF_CUDA(cudaMemcpy2DAsync(Y, (size_t)rows * wo * sizeof(float), m->Y,
                                    (size_t)m->cap * wo * sizeof(float),
@@ -595,8 +661,13 @@ int npf_mlp_loss_grad(npf_mlp* m, int rows, const float* X, const float* T, floa
         stage(m->d_T, m->tcap, T, (int64_t)rows * m->w[m->L], m->s);
         NPF_CUDA(cudaMemsetAsync(m->d_loss, 0, m->E * sizeof(double), m->s));
         gather(*m, rows, m->d_X, m->d_T, nullptr, 0);
-        forward(*m, rows);
-        loss_and_backward(*m, rows);
+        forward(*m, rows, true);
+        backward(*m, rows);
+        for (int l = 0; l < m->L; ++l) {
+            Gemm g = weight_grad(*m, rows, l);
+            g.C = m->G + m->off[l];
+            gemm<EPI_F32, true, true>(*m, "mlp_weight_grad", g);
+        }
         std::vector<float> in((size_t)m->E * m->P), pub((size_t)m->E * m->Ppub);
         std::vector<double> l(m->E);
         NPF_CUDA(cudaMemcpyAsync(in.data(), m->G, in.size() * sizeof(float), cudaMemcpyDeviceToHost, m->s));
@@ -628,8 +699,15 @@ int npf_mlp_train(npf_mlp* m, int rows, const float* X, const float* T, int epoc
         std::vector<uint64_t> st(m->E);
         for (int e = 0; e < m->E; ++e) st[e] = seed + 7919ull * (uint64_t)e;
         std::vector<int> perm((size_t)m->E * rows);
-        const int64_t tot = (int64_t)m->E * m->P;
-        const float b1 = 0.9f, b2 = 0.999f;
+        AdamStep ad{};
+        ad.layers = m->L;
+        ad.W = m->W; ad.M1 = m->M1; ad.M2 = m->M2; ad.Wb = m->Wb;
+        ad.lr = (float)lr; ad.b1 = 0.9f; ad.b2 = 0.999f; ad.eps = 1e-8f;
+        for (int l = 0; l < m->L; ++l) {
+            ad.g[l] = weight_grad(*m, batch, l);
+            ad.g[l].C = reinterpret_cast<void*>(m->off[l]);
+            ad.tile0[l + 1] = ad.tile0[l] + (ad.g[l].M + TM - 1) / TM * ((ad.g[l].N + TN - 1) / TN);
+        }
         for (int ep = 0; ep < epochs; ++ep) {
             for (int e = 0; e < m->E; ++e) {   // Fisher-Yates with splitmix64
                 int* p = perm.data() + (size_t)e * rows;
@@ -645,14 +723,13 @@ int npf_mlp_train(npf_mlp* m, int rows, const float* X, const float* T, int epoc
             NPF_CUDA(cudaMemsetAsync(m->d_loss, 0, m->E * sizeof(double), m->s));
             for (int k = 0; k < steps; ++k) {
                 gather(*m, batch, m->d_X, m->d_T, m->d_idx + (int64_t)k * batch, rows);
-                forward(*m, batch);
-                loss_and_backward(*m, batch);
+                forward(*m, batch, true);
+                backward(*m, batch);
                 ++m->step;
-                const float c1 = (float)(1.0 - std::pow((double)b1, (double)m->step));
-                const float c2 = (float)(1.0 - std::pow((double)b2, (double)m->step));
-                npf::LaunchScope ls(nullptr, "mlp_adam", m->s);
-                k_adam<<<grid_for(tot), 256, 0, m->s>>>(tot, m->W, m->M1, m->M2, m->G, m->Wb,
-                                                        (float)lr, b1, b2, 1e-8f, c1, c2);
+                ad.c1 = (float)(1.0 - std::pow((double)ad.b1, (double)m->step));
+                ad.c2 = (float)(1.0 - std::pow((double)ad.b2, (double)m->step));
+                npf::LaunchScope ls(nullptr, "mlp_grad_adam", m->s);
+                k_grad_adam<<<dim3((unsigned)ad.tile0[m->L], 1, (unsigned)m->E), 128, 0, m->s>>>(ad);
                 NPF_CUDA(cudaGetLastError());
             }
             if (epoch_loss) {
@@ -694,7 +771,7 @@ int npf_mlp_predict(npf_mlp* m, int rows, const float* X, const float* mu, const
             m->mcap = rows;
         }
         gather(*m, rows, m->d_X, nullptr, nullptr, 0);
-        forward(*m, rows);
+        forward(*m, rows, false);
         {
             npf::LaunchScope ls(nullptr, "mlp_ensemble_gate", m->s);
             k_ens_stats<<<rows, 128, 0, m->s>>>(m->E, wo, m->cap, m->Y, m->d_mu, m->d_sig,
