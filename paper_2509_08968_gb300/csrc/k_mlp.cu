@@ -58,7 +58,7 @@ struct AdamStep {
     Gemm g[kMaxLayers];          // C: offset of the layer's block in the parameter arrays, in floats
     float *W, *M1, *M2;
     __nv_bfloat16* Wb;
-    float lr, b1, b2, eps, c1, c2;
+    float lr, b1, b2, eps, ic1, ic2;   // ic: 1 / (1 - b^step)
 };
 
 // D (16x8, FP32) += A (16x16, BF16, row-major fragment) * B (16x8, BF16, column fragment).
@@ -176,23 +176,33 @@ __device__ __forceinline__ void gemm_tile(const Gemm& g, int e, int m0, int n0, 
     }
 }
 
-// f(m, n, value) for the thread's elements of the tile that lie in the matrix.
+// Row and first column of the thread's accumulators acc[mi][ni][2 h], acc[mi][ni][2 h + 1].
+__device__ __forceinline__ int out_row(int m0, int mi, int h)
+{
+    return m0 + (int)threadIdx.x / 64 * 32 + mi * 16 + (int)threadIdx.x % 32 / 4 + 8 * h;
+}
+__device__ __forceinline__ int out_col(int n0, int ni)
+{
+    return n0 + (int)threadIdx.x / 32 % 2 * 32 + ni * 8 + (int)threadIdx.x % 4 * 2;
+}
+
+// f(m, n, value, j) for the thread's elements of the tile that lie in the matrix (j: 0..31).
 template <class F>
 __device__ __forceinline__ void for_outputs(const Gemm& g, int m0, int n0, const float (&acc)[2][4][4], F&& f)
 {
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
 #pragma unroll
     for (int mi = 0; mi < 2; ++mi)
 #pragma unroll
         for (int ni = 0; ni < 4; ++ni)
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const int m = m0 + warp / 2 * 32 + mi * 16 + lane / 4 + (q >= 2 ? 8 : 0);
-                const int n = n0 + warp % 2 * 32 + ni * 8 + lane % 4 * 2 + (q & 1);
-                if (m < g.M && n < g.N) f(m, n, acc[mi][ni][q]);
+                const int m = out_row(m0, mi, q / 2), n = out_col(n0, ni) + q % 2;
+                if (m < g.M && n < g.N) f(m, n, acc[mi][ni][q], (mi * 4 + ni) * 4 + q);
             }
 }
 
+// The epilogues read what they need (mask, targets, Adam's state) into registers before they store
+// anything, so that the loads are in flight together instead of one after each store.
 template <int EPI, bool AT, bool BT>
 __global__ void __launch_bounds__(128) k_gemm(const __grid_constant__ Gemm g)
 {
@@ -200,19 +210,54 @@ __global__ void __launch_bounds__(128) k_gemm(const __grid_constant__ Gemm g)
     const int e = blockIdx.z, m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
     float acc[2][4][4];
     gemm_tile<AT, BT>(g, e, m0, n0, sA, sB, acc);
+    if (EPI == EPI_RELU_BF16 || EPI == EPI_MASK_BF16) {
+        // hidden widths are multiples of 16: a thread's column pairs are whole
+        uint32_t mk[2][4][2];
+#pragma unroll
+        for (int mi = 0; mi < 2; ++mi)
+#pragma unroll
+            for (int ni = 0; ni < 4; ++ni)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int m = out_row(m0, mi, h), n = out_col(n0, ni);
+                    mk[mi][ni][h] = 0u;
+                    if (EPI == EPI_MASK_BF16 && m < g.M && n < g.N)
+                        mk[mi][ni][h] = *reinterpret_cast<const uint32_t*>(g.mask + e * g.sM + (int64_t)m * g.ldm + n);
+                }
+#pragma unroll
+        for (int mi = 0; mi < 2; ++mi)
+#pragma unroll
+            for (int ni = 0; ni < 4; ++ni)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int m = out_row(m0, mi, h), n = out_col(n0, ni);
+                    if (m >= g.M || n >= g.N) continue;
+                    float x = acc[mi][ni][2 * h], y = acc[mi][ni][2 * h + 1];
+                    if (EPI == EPI_RELU_BF16) {
+                        x = fmaxf(x, 0.f);
+                        y = fmaxf(y, 0.f);
+                    } else {   // the activations' BF16 bits: positive where the unit was active
+                        x = __uint_as_float(mk[mi][ni][h] << 16) > 0.f ? x : 0.f;
+                        y = __uint_as_float(mk[mi][ni][h] & 0xFFFF0000u) > 0.f ? y : 0.f;
+                    }
+                    *reinterpret_cast<__nv_bfloat162*>(static_cast<__nv_bfloat16*>(g.C) + e * g.sC +
+                                                       (int64_t)m * g.ldc + n) = __floats2bfloat162_rn(x, y);
+                }
+        return;
+    }
+    float aux[32];
+    if (EPI == EPI_LOSS)
+        for_outputs(g, m0, n0, acc, [&](int m, int n, float, int j) {
+            aux[j] = g.T[e * g.sT + (int64_t)m * g.N + n];
+        });
     double part = 0.0;
     const float scale2 = EPI == EPI_LOSS ? (float)(2.0 * (1.0 / ((double)g.M * g.N))) : 0.f;
-    for_outputs(g, m0, n0, acc, [&](int m, int n, float v) {
+    for_outputs(g, m0, n0, acc, [&](int m, int n, float v, int j) {
         const int64_t o = e * g.sC + (int64_t)m * g.ldc + n;
         if (EPI == EPI_F32) {
             static_cast<float*>(g.C)[o] = v;
-        } else if (EPI == EPI_RELU_BF16) {
-            static_cast<__nv_bfloat16*>(g.C)[o] = __float2bfloat16_rn(fmaxf(v, 0.f));
-        } else if (EPI == EPI_MASK_BF16) {
-            const float mk = __bfloat162float(g.mask[e * g.sM + (int64_t)m * g.ldm + n]);
-            static_cast<__nv_bfloat16*>(g.C)[o] = __float2bfloat16_rn(mk > 0.f ? v : 0.f);
         } else {   // mean squared error: the output's error 2 (Y - T) / (M N), and the loss
-            const float d = v - g.T[e * g.sT + (int64_t)m * g.N + n];
+            const float d = v - aux[j];
             static_cast<__nv_bfloat16*>(g.C)[o] = __float2bfloat16_rn(scale2 * d);
             part += (double)d * d;
         }
@@ -241,16 +286,80 @@ __global__ void __launch_bounds__(128) k_grad_adam(const __grid_constant__ AdamS
     const int e = blockIdx.z, m0 = t / nt * TM, n0 = t % nt * TN;
     float acc[2][4][4];
     gemm_tile<true, true>(g, e, m0, n0, sA, sB, acc);
-    for_outputs(g, m0, n0, acc, [&](int m, int n, float gr) {
-        const int64_t o = e * g.sC + reinterpret_cast<int64_t>(g.C) + (int64_t)m * g.ldc + n;
-        const float m1 = s.b1 * s.M1[o] + (1.f - s.b1) * gr;
-        const float m2 = s.b2 * s.M2[o] + (1.f - s.b2) * gr * gr;
-        s.M1[o] = m1;
-        s.M2[o] = m2;
-        const float w = s.W[o] - s.lr * (m1 / s.c1) / (sqrtf(m2 / s.c2) + s.eps);
-        s.W[o] = w;
-        s.Wb[o] = __float2bfloat16_rn(w);
-    });
+    // the gradient tile through shared memory, so that the state moves in coalesced 16-byte accesses
+    constexpr int LDG = TN + 4;
+    float* tile = reinterpret_cast<float*>(sA);
+    static_assert(TM * LDG * sizeof(float) <= sizeof(sA), "the gradient tile fits one operand's stages");
+    __syncthreads();
+#pragma unroll
+    for (int mi = 0; mi < 2; ++mi)
+#pragma unroll
+        for (int ni = 0; ni < 4; ++ni)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                *reinterpret_cast<float2*>(tile + out_row(0, mi, h) * LDG + out_col(0, ni)) =
+                    make_float2(acc[mi][ni][2 * h], acc[mi][ni][2 * h + 1]);
+    __syncthreads();
+    const int64_t base = e * g.sC + reinterpret_cast<int64_t>(g.C);
+    const int c = (int)threadIdx.x % 16 * 4, r0 = (int)threadIdx.x / 16;
+    float4 w[8], m1[8], m2[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const int m = m0 + r0 + 8 * j;
+        if (m >= g.M || n0 + c >= g.N) continue;   // (N = ip is a multiple of 16)
+        const int64_t o = base + (int64_t)m * g.ldc + n0 + c;
+        w[j] = *reinterpret_cast<const float4*>(s.W + o);
+        m1[j] = *reinterpret_cast<const float4*>(s.M1 + o);
+        m2[j] = *reinterpret_cast<const float4*>(s.M2 + o);
+    }
+    // Reciprocals of the bias corrections from the host, and no operand that is zero in a division or
+    // square root (units that never fire have zero moments, and zeros take the slow branch of both:
+    // 150 instructions an element, 26 us a launch). sqrt(1e-36) = 1e-18 does not change eps = 1e-8.
+    auto adam = [&](float gr, float& x, float& a, float& v) {
+        a = s.b1 * a + (1.f - s.b1) * gr;
+        v = s.b2 * v + (1.f - s.b2) * gr * gr;
+        x = x - s.lr * (a * s.ic1) * __frcp_rn(sqrtf(fmaxf(v * s.ic2, 1e-36f)) + s.eps);
+    };
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const int m = m0 + r0 + 8 * j;
+        if (m >= g.M || n0 + c >= g.N) continue;
+        const int64_t o = base + (int64_t)m * g.ldc + n0 + c;
+        const float4 gr = *reinterpret_cast<const float4*>(tile + (r0 + 8 * j) * LDG + c);
+        adam(gr.x, w[j].x, m1[j].x, m2[j].x);
+        adam(gr.y, w[j].y, m1[j].y, m2[j].y);
+        adam(gr.z, w[j].z, m1[j].z, m2[j].z);
+        adam(gr.w, w[j].w, m1[j].w, m2[j].w);
+        *reinterpret_cast<float4*>(s.W + o) = w[j];
+        *reinterpret_cast<float4*>(s.M1 + o) = m1[j];
+        *reinterpret_cast<float4*>(s.M2 + o) = m2[j];
+        __nv_bfloat162 b[2] = {__floats2bfloat162_rn(w[j].x, w[j].y), __floats2bfloat162_rn(w[j].z, w[j].w)};
+        *reinterpret_cast<uint2*>(s.Wb + o) = *reinterpret_cast<uint2*>(b);
+    }
+}
+
+// Weights between the public layout [w_{l+1}][w_l + 1] and the internal one [w_{l+1}][ip_l] (padding
+// columns keep their zeros), member by member; to_pub: internal -> public.
+struct Layout {
+    int layers;
+    int w[kMaxLayers + 1], ip[kMaxLayers];
+    int64_t off[kMaxLayers + 1], offp[kMaxLayers + 1];   // one past the end: P, Ppub
+};
+__global__ void k_relayout(const __grid_constant__ Layout a, int E, const float* __restrict__ src,
+                           float* __restrict__ dst, int to_pub)
+{
+    const int64_t Ppub = a.offp[a.layers], P = a.off[a.layers];
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < E * Ppub;
+         t += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t e = t / Ppub;
+        const int r = (int)(t - e * Ppub);
+        int l = 0;
+        while (l + 1 < a.layers && r >= a.offp[l + 1]) ++l;
+        const int q = r - (int)a.offp[l], width = a.w[l] + 1, o = q / width, i = q - o * width;
+        const int64_t in = e * P + a.off[l] + (int64_t)o * a.ip[l] + i;
+        if (to_pub) dst[t] = src[in];
+        else dst[in] = src[t];
+    }
 }
 
 // Augmented BF16 inputs Xa[e][b][ip] = (X[r][0..w0-1], 1, 0, ..) with r = idx[e][b] (or b), and
@@ -379,6 +488,7 @@ struct npf_mlp {
     int64_t idx_cap = 0;
     float *d_mu = nullptr, *d_sig = nullptr, *d_mean = nullptr, *d_spread = nullptr;
     int* d_fb = nullptr;
+    float* d_pub = nullptr;     // [E][Ppub] staging of weights or gradients in the public layout
     int64_t tcap = 0;   // floats of d_T
     int64_t mcap = 0;   // rows of d_mean / d_spread / d_fb
 };
@@ -416,7 +526,7 @@ void free_all(npf_mlp& m)
 {
     release_acts(m);
     cudaFree(m.W); cudaFree(m.M1); cudaFree(m.M2); cudaFree(m.G); cudaFree(m.Wb);
-    cudaFree(m.d_loss); cudaFree(m.d_X); cudaFree(m.d_T); cudaFree(m.d_idx);
+    cudaFree(m.d_loss); cudaFree(m.d_pub); cudaFree(m.d_X); cudaFree(m.d_T); cudaFree(m.d_idx);
     cudaFree(m.d_mu); cudaFree(m.d_sig); cudaFree(m.d_mean); cudaFree(m.d_spread); cudaFree(m.d_fb);
 }
 
@@ -536,25 +646,22 @@ Gemm weight_grad(const npf_mlp& m, int rows, int l)
 
 void sync(npf_mlp& m) { NPF_CUDA(cudaStreamSynchronize(m.s)); }
 
-// public [w_{l+1}][w_l + 1] per layer <-> internal [w_{l+1}][ip_l], member by member
-void to_internal(const npf_mlp& m, const float* pub, std::vector<float>& in)
+// d_pub <- the public layout of an internal array, or an internal array <- d_pub
+void relayout(npf_mlp& m, float* internal, bool to_pub)
 {
-    in.assign((size_t)m.E * m.P, 0.f);
-    for (int e = 0; e < m.E; ++e)
-        for (int l = 0; l < m.L; ++l)
-            for (int o = 0; o < m.w[l + 1]; ++o)
-                for (int i = 0; i <= m.w[l]; ++i)
-                    in[(size_t)e * m.P + m.off[l] + (size_t)o * m.ip[l] + i] =
-                        pub[(size_t)e * m.Ppub + m.offp[l] + (size_t)o * (m.w[l] + 1) + i];
-}
-void to_public(const npf_mlp& m, const std::vector<float>& in, float* pub)
-{
-    for (int e = 0; e < m.E; ++e)
-        for (int l = 0; l < m.L; ++l)
-            for (int o = 0; o < m.w[l + 1]; ++o)
-                for (int i = 0; i <= m.w[l]; ++i)
-                    pub[(size_t)e * m.Ppub + m.offp[l] + (size_t)o * (m.w[l] + 1) + i] =
-                        in[(size_t)e * m.P + m.off[l] + (size_t)o * m.ip[l] + i];
+    Layout a{};
+    a.layers = m.L;
+    for (int l = 0; l <= m.L; ++l) {
+        a.w[l] = m.w[l];
+        a.off[l] = l < m.L ? m.off[l] : m.P;
+        a.offp[l] = l < m.L ? m.offp[l] : m.Ppub;
+        if (l < m.L) a.ip[l] = m.ip[l];
+    }
+    if (!m.d_pub) m.d_pub = dalloc<float>(m.E * m.Ppub);
+    npf::LaunchScope ls(nullptr, "mlp_relayout", m.s);
+    k_relayout<<<grid_for(m.E * m.Ppub), 256, 0, m.s>>>(a, m.E, to_pub ? internal : m.d_pub,
+                                                      to_pub ? m.d_pub : internal, to_pub);
+    NPF_CUDA(cudaGetLastError());
 }
 
 void copy_out(void* dst, const void* src, size_t bytes, cudaStream_t s)
@@ -592,9 +699,6 @@ npf_mlp* npf_mlp_create(int ensemble, int layers, const int* widths, const float
             m->P += (int64_t)m->w[l + 1] * m->ip[l];
             m->Ppub += (int64_t)m->w[l + 1] * (m->w[l] + 1);
         }
-        std::vector<float> pub((size_t)ensemble * m->Ppub), in;
-        NPF_CUDA(cudaMemcpy(pub.data(), weights, pub.size() * sizeof(float), cudaMemcpyDefault));
-        to_internal(*m, pub.data(), in);
         const int64_t tot = (int64_t)ensemble * m->P;
         m->W = dalloc<float>(tot);
         m->M1 = dalloc<float>(tot);
@@ -602,9 +706,13 @@ npf_mlp* npf_mlp_create(int ensemble, int layers, const int* widths, const float
         m->G = dalloc<float>(tot);
         m->Wb = dalloc<__nv_bfloat16>(tot);
         m->d_loss = dalloc<double>(ensemble);
-        NPF_CUDA(cudaMemcpy(m->W, in.data(), (size_t)tot * sizeof(float), cudaMemcpyHostToDevice));
-        NPF_CUDA(cudaMemset(m->M1, 0, (size_t)tot * sizeof(float)));
-        NPF_CUDA(cudaMemset(m->M2, 0, (size_t)tot * sizeof(float)));
+        m->d_pub = dalloc<float>(ensemble * m->Ppub);
+        NPF_CUDA(cudaMemcpyAsync(m->d_pub, weights, (size_t)ensemble * m->Ppub * sizeof(float), cudaMemcpyDefault,
+                                 m->s));
+        NPF_CUDA(cudaMemsetAsync(m->W, 0, (size_t)tot * sizeof(float), m->s));
+        NPF_CUDA(cudaMemsetAsync(m->M1, 0, (size_t)tot * sizeof(float), m->s));
+        NPF_CUDA(cudaMemsetAsync(m->M2, 0, (size_t)tot * sizeof(float), m->s));
+        relayout(*m, m->W, false);
         {
             npf::LaunchScope ls(nullptr, "mlp_to_bf16", m->s);
             k_to_bf16<<<grid_for(tot), 256, 0, m->s>>>(tot, m->W, m->Wb);
@@ -625,11 +733,10 @@ int npf_mlp_get_weights(const npf_mlp* m, float* weights)
 {
     return run([&] {
         if (!m || !weights) npf::fail(NPF_ERR_ARG, "null argument");
-        std::vector<float> in((size_t)m->E * m->P), pub((size_t)m->E * m->Ppub);
-        NPF_CUDA(cudaStreamSynchronize(m->s));
-        NPF_CUDA(cudaMemcpy(in.data(), m->W, in.size() * sizeof(float), cudaMemcpyDeviceToHost));
-        to_public(*m, in, pub.data());
-        NPF_CUDA(cudaMemcpy(weights, pub.data(), pub.size() * sizeof(float), cudaMemcpyDefault));
+        npf_mlp& mm = const_cast<npf_mlp&>(*m);   // (the staging buffer; the weights stay)
+        relayout(mm, mm.W, true);
+        copy_out(weights, mm.d_pub, (size_t)mm.E * mm.Ppub * sizeof(float), mm.s);
+        sync(mm);
     });
 }
 
@@ -668,13 +775,11 @@ int npf_mlp_loss_grad(npf_mlp* m, int rows, const float* X, const float* T, floa
             g.C = m->G + m->off[l];
             gemm<EPI_F32, true, true>(*m, "mlp_weight_grad", g);
         }
-        std::vector<float> in((size_t)m->E * m->P), pub((size_t)m->E * m->Ppub);
         std::vector<double> l(m->E);
-        NPF_CUDA(cudaMemcpyAsync(in.data(), m->G, in.size() * sizeof(float), cudaMemcpyDeviceToHost, m->s));
+        relayout(*m, m->G, true);
+        copy_out(grads, m->d_pub, (size_t)m->E * m->Ppub * sizeof(float), m->s);
         NPF_CUDA(cudaMemcpyAsync(l.data(), m->d_loss, m->E * sizeof(double), cudaMemcpyDeviceToHost, m->s));
         sync(*m);
-        to_public(*m, in, pub.data());
-        NPF_CUDA(cudaMemcpy(grads, pub.data(), pub.size() * sizeof(float), cudaMemcpyDefault));
         std::vector<float> lf(l.begin(), l.end());
         NPF_CUDA(cudaMemcpy(loss, lf.data(), lf.size() * sizeof(float), cudaMemcpyDefault));
     });
@@ -708,7 +813,7 @@ int npf_mlp_train(npf_mlp* m, int rows, const float* X, const float* T, int epoc
             ad.g[l].C = reinterpret_cast<void*>(m->off[l]);
             ad.tile0[l + 1] = ad.tile0[l] + (ad.g[l].M + TM - 1) / TM * ((ad.g[l].N + TN - 1) / TN);
         }
-        for (int ep = 0; ep < epochs; ++ep) {
+        auto shuffle = [&] {
             for (int e = 0; e < m->E; ++e) {   // Fisher-Yates with splitmix64
                 int* p = perm.data() + (size_t)e * rows;
                 for (int r = 0; r < rows; ++r) p[r] = r;
@@ -717,6 +822,9 @@ int npf_mlp_train(npf_mlp* m, int rows, const float* X, const float* T, int epoc
                     std::swap(p[r], p[j]);
                 }
             }
+        };
+        if (epochs > 0) shuffle();
+        for (int ep = 0; ep < epochs; ++ep) {
             // the previous epoch's kernels may still read the index buffer
             NPF_CUDA(cudaStreamSynchronize(m->s));
             NPF_CUDA(cudaMemcpy(m->d_idx, perm.data(), perm.size() * sizeof(int), cudaMemcpyHostToDevice));
@@ -726,12 +834,13 @@ int npf_mlp_train(npf_mlp* m, int rows, const float* X, const float* T, int epoc
                 forward(*m, batch, true);
                 backward(*m, batch);
                 ++m->step;
-                ad.c1 = (float)(1.0 - std::pow((double)ad.b1, (double)m->step));
-                ad.c2 = (float)(1.0 - std::pow((double)ad.b2, (double)m->step));
+                ad.ic1 = (float)(1.0 / (1.0 - std::pow((double)ad.b1, (double)m->step)));
+                ad.ic2 = (float)(1.0 / (1.0 - std::pow((double)ad.b2, (double)m->step)));
                 npf::LaunchScope ls(nullptr, "mlp_grad_adam", m->s);
                 k_grad_adam<<<dim3((unsigned)ad.tile0[m->L], 1, (unsigned)m->E), 128, 0, m->s>>>(ad);
                 NPF_CUDA(cudaGetLastError());
             }
+            if (ep + 1 < epochs) shuffle();   // the next epoch's order, while this one's kernels run
             if (epoch_loss) {
                 std::vector<double> l(m->E);
                 NPF_CUDA(cudaMemcpyAsync(l.data(), m->d_loss, m->E * sizeof(double),
