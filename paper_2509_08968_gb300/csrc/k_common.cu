@@ -214,6 +214,60 @@ void launch_unpermute(Plan& p, const double2* in, double2* out, bool columns)
     NPF_CUDA(cudaGetLastError());
 }
 
+// max |V U - I| over the entries (NaN entries are passed over), as the bits of a non-negative double.
+__global__ void k_inverse_error(int n, const double2* __restrict__ V, const double2* __restrict__ U,
+                                unsigned long long* __restrict__ worst)
+{
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    double e = 0.0;
+    if (t < (int64_t)n * n) {
+        const int i = (int)(t / n), c = (int)(t % n);
+        double2 s = make_double2(0.0, 0.0);
+#pragma unroll 4
+        for (int j = 0; j < n; ++j) cfma(s, V[(int64_t)i * n + j], U[(int64_t)j * n + c]);
+        e = hypot(s.x - (c == i ? 1.0 : 0.0), s.y);
+        if (isnan(e)) e = 0.0;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) e = fmax(e, __shfl_xor_sync(0xffffffffu, e, o));
+    if (threadIdx.x % 32 == 0 && e > 0.0) atomicMax(worst, (unsigned long long)__double_as_longlong(e));
+}
+double inverse_error(Plan& p, const double2* V, const double2* U, double2* scratch)
+{
+    const int64_t nn = (int64_t)p.n * p.n;
+    NPF_CUDA(cudaMemsetAsync(scratch, 0, sizeof(double), p.stream));
+    {
+        LaunchScope ls(&p.prof, "inverse_error", p.stream);
+        k_inverse_error<<<(unsigned)((nn + 63) / 64), 64, 0, p.stream>>>(p.n, V, U, (unsigned long long*)scratch);
+        NPF_CUDA(cudaGetLastError());
+    }
+    double worst = 0.0;
+    NPF_CUDA(cudaMemcpyAsync(&worst, scratch, sizeof(double), cudaMemcpyDeviceToHost, p.stream));
+    NPF_CUDA(cudaStreamSynchronize(p.stream));
+    return worst;
+}
+
+// Modal data in the plan's mode order from the caller's: U's columns, V's rows (and V transposed).
+__global__ void k_order_modes(int n, const int* __restrict__ perm, const double2* __restrict__ Us,
+                              const double2* __restrict__ Vs, double2* __restrict__ U, double2* __restrict__ V,
+                              double2* __restrict__ Vt)
+{
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= (int64_t)n * n) return;
+    const int r = (int)(t / n), c = (int)(t % n);
+    U[t] = Us[(int64_t)r * n + perm[c]];
+    const double2 v = Vs[(int64_t)perm[r] * n + c];
+    V[t] = v;
+    Vt[(int64_t)c * n + r] = v;
+}
+void launch_order_modes(Plan& p, const double2* Us, const double2* Vs)
+{
+    const int64_t nn = (int64_t)p.n * p.n;
+    LaunchScope ls(&p.prof, "order_modes", p.stream);
+    k_order_modes<<<(unsigned)((nn + 255) / 256), 256, 0, p.stream>>>(p.n, p.d_perm, Us, Vs, p.d_U, p.d_V, p.d_Vt);
+    NPF_CUDA(cudaGetLastError());
+}
+
 // cnt[r*(n+1) + v] = C(n - v + r - 1, r): non-decreasing r-tuples with values in [v, n).
 void build_cnt_table(Plan& p)
 {

@@ -1847,69 +1847,6 @@ static int default_slices(const Plan& p)
     return p.slices ? p.slices : (p.precision == NPF_PREC_FP32 ? 4 : 6);
 }
 
-// Host slicing of x with exponent e into S balanced digits.
-static void host_digits(double x, int e, int S, int* d)
-{
-    if (e == EXP_NONE || x == 0.0) { for (int s = 0; s < S; ++s) d[s] = 0; return; }
-    long long W = std::llrint(std::ldexp(x, 7 + 8 * (S - 1) - e));
-    for (int s = S - 1; s >= 1; --s) {
-        const int lo = (int)((W + 128) & 255) - 128;
-        d[s] = lo;
-        W = (W - lo) >> 8;
-    }
-    d[0] = (int)W;
-}
-
-static uint16_t bf16_of_digit(int d, int s)
-{
-    const float f = std::ldexp((float)d, -8 * s);   // exact: |d| <= 128
-    uint32_t u;
-    std::memcpy(&u, &f, 4);
-    return (uint16_t)(u >> 16);
-}
-
-// Fixed planes [S][512][kw] of an n x n complex matrix accessed as get(kidx, col):
-// complex K (kw = 256, interleaved): Re-row col = [Re, -Im, ..], Im-row col = [Im, Re, ..];
-// real K (kw = 128): Re-row col = [Re ..], Im-row col = [Im ..]. Exponent per column.
-template <class F>
-static void build_fixed(int n, int S, bool complexK, F get, std::vector<uint16_t>& planes,
-                        std::vector<int>& ex)
-{
-    const int kw = complexK ? KP : NP;
-    planes.assign((size_t)S * 512 * kw, 0);
-    ex.assign(256, EXP_NONE);
-    for (int c = 0; c < n; ++c) {
-        double m = 0.0;
-        for (int k = 0; k < n; ++k) {
-            const double2 v = get(k, c);
-            m = std::max(m, std::max(std::fabs(v.x), std::fabs(v.y)));
-        }
-        int e = EXP_NONE;
-        if (m > 0) std::frexp(m, &e);
-        ex[c] = e;
-        for (int k = 0; k < n; ++k) {
-            const double2 v = get(k, c);
-            int dr[8], di[8];
-            host_digits(v.x, e, S, dr);
-            host_digits(v.y, e, S, di);
-            for (int s = 0; s < S; ++s) {
-                uint16_t* P = planes.data() + (size_t)s * 512 * kw;
-                uint16_t* re_row = P + (size_t)c * kw;
-                uint16_t* im_row = P + (size_t)(256 + c) * kw;
-                if (complexK) {
-                    re_row[2 * k] = bf16_of_digit(dr[s], s);
-                    re_row[2 * k + 1] = bf16_of_digit(-di[s], s);
-                    im_row[2 * k] = bf16_of_digit(di[s], s);
-                    im_row[2 * k + 1] = bf16_of_digit(dr[s], s);
-                } else {
-                    re_row[k] = bf16_of_digit(dr[s], s);
-                    im_row[k] = bf16_of_digit(di[s], s);
-                }
-            }
-        }
-    }
-}
-
 template <class T>
 static T* upload(const std::vector<T>& v)
 {
@@ -1980,44 +1917,96 @@ static void set_smem_attrs()
     done = true;
 }
 
-// Device copy of a host vector: a new buffer when `dst` is null, else overwritten in place.
-template <class D, class T>
-static void put(D*& dst, const std::vector<T>& v)
+// Fixed planes [S][512][kw] of an n x n complex matrix, a block per column c (k: the K index; entry
+// m[k][c], or m[c][k] when trans): complex K (kw = 256, interleaved): Re-row c = [Re, -Im, ..], Im-row
+// 256 + c = [Im, Re, ..]; real K (kw = 128): Re-row [Re ..], Im-row [Im ..]. Exponent per column.
+// Rows and K entries past n keep the zeros of the allocation.
+template <int S>
+__global__ void __launch_bounds__(128)
+    k_fixed_planes(const double2* __restrict__ m, int n, int trans, int complexK,
+                   __nv_bfloat16* __restrict__ planes, int* __restrict__ ex)
 {
-    if (!dst) {
-        dst = reinterpret_cast<D*>(upload(v));
-        return;
+    const int c = blockIdx.x, k = threadIdx.x;   // n <= 128: one K entry a thread
+    double2 v = make_double2(0.0, 0.0);
+    if (c < n && k < n) v = m[trans ? c * n + k : k * n + c];
+    __shared__ double red[128];
+    red[k] = fmax(fabs(v.x), fabs(v.y));
+    __syncthreads();
+    for (int w = 64; w > 0; w >>= 1) {
+        if (k < w) red[k] = fmax(red[k], red[k + w]);
+        __syncthreads();
     }
-    NPF_CUDA(cudaMemcpy(dst, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice));
+    int e = EXP_NONE;
+    if (red[0] > 0.0) frexp(red[0], &e);
+    if (k == 0) ex[c] = e;
+    if (c >= n || k >= n) return;
+    long long wr = 0, wi = 0;
+    if (e != EXP_NONE) {
+        const double sc = pow2d(7 + 8 * (S - 1) - e);
+        wr = __double2ll_rn(v.x * sc);
+        wi = __double2ll_rn(v.y * sc);
+    }
+    uint32_t w[S], wn[S];
+    digit_pairs<S>(wr, wi, w);        // (Re, Im)
+    digit_pairs<S>(wr, -wi, wn);      // (Re, -Im)
+    const int kw = complexK ? KP : NP;
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+        uint16_t* re = reinterpret_cast<uint16_t*>(planes) + ((size_t)s * 512 + c) * kw;
+        uint16_t* im = re + (size_t)256 * kw;
+        if (complexK) {
+            *reinterpret_cast<uint32_t*>(re + 2 * k) = wn[s];
+            *reinterpret_cast<uint32_t*>(im + 2 * k) = w[s] >> 16 | w[s] << 16;
+        } else {
+            re[k] = (uint16_t)w[s];
+            im[k] = (uint16_t)(w[s] >> 16);
+        }
+    }
+}
+
+// A complex matrix as double-float pairs.
+static __global__ void k_to_df(const double2* __restrict__ m, int count, float4* __restrict__ out)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= count) return;
+    const double2 v = m[t];
+    const float rh = (float)v.x, ih = (float)v.y;
+    out[t] = make_float4(rh, (float)(v.x - rh), ih, (float)(v.y - ih));
+}
+
+// One fixed matrix (buffers allocated on first use, then overwritten in place), on the plan's stream.
+static void fixed_matrix(Plan& p, int S, const double2* m, bool trans, bool complexK, __nv_bfloat16*& planes, int*& ex)
+{
+    const size_t bytes = (size_t)S * 512 * (complexK ? KP : NP) * sizeof(__nv_bfloat16);
+    if (!planes) {
+        NPF_CUDA(cudaMalloc(&planes, bytes));
+        NPF_CUDA(cudaMemsetAsync(planes, 0, bytes, p.stream));
+    }
+    if (!ex) NPF_CUDA(cudaMalloc(&ex, 256 * sizeof(int)));
+    LaunchScope ls(&p.prof, "split_fixed_planes", p.stream);
+    auto kern = S == 2 ? k_fixed_planes<2> : S == 3 ? k_fixed_planes<3> : S == 4 ? k_fixed_planes<4>
+              : S == 5 ? k_fixed_planes<5> : k_fixed_planes<6>;
+    kern<<<256, 128, 0, p.stream>>>(m, p.n, trans, complexK, planes, ex);
+    NPF_CUDA(cudaGetLastError());
+}
+
+static void to_df(Plan& p, const double2* m, float4*& out)
+{
+    const int count = p.n * p.n;
+    if (!out) NPF_CUDA(cudaMalloc(&out, (size_t)count * sizeof(float4)));
+    LaunchScope ls(&p.prof, "split_to_df", p.stream);
+    k_to_df<<<(count + 255) / 256, 256, 0, p.stream>>>(m, count, out);
+    NPF_CUDA(cudaGetLastError());
 }
 
 // Slices of Phi, Psi and Psi^T and the double-float Psi, from the plan's modal data.
 static void fill_fixed(Plan& p, SplitOperand* so)
 {
-    const int n = p.n, S = so->S;
-    std::vector<double2> U(n * n), V(n * n);
-    NPF_CUDA(cudaMemcpy(U.data(), p.d_U, U.size() * sizeof(double2), cudaMemcpyDeviceToHost));
-    NPF_CUDA(cudaMemcpy(V.data(), p.d_V, V.size() * sizeof(double2), cudaMemcpyDeviceToHost));
-    std::vector<uint16_t> planes;
-    std::vector<int> ex;
-    // Phi: K index a, column p: phi_{a p}
-    build_fixed(n, S, true, [&](int a, int c) { return U[(size_t)a * n + c]; }, planes, ex);
-    put(so->phi, planes);
-    put(so->phi_e, ex);
-    // Psi for the upper-index contraction: real K index j, column i: psi_{i j}
-    build_fixed(n, S, false, [&](int j, int i) { return V[(size_t)i * n + j]; }, planes, ex);
-    put(so->psir, planes);
-    put(so->psir_e, ex);
-    // Psi^T rows k for the reduction: complex K index p, row k: psi_{p k}
-    build_fixed(n, S, true, [&](int pidx, int k) { return V[(size_t)pidx * n + k]; }, planes, ex);
-    put(so->red, planes);
-    put(so->red_e, ex);
-    std::vector<float4> pdf((size_t)n * n);
-    for (size_t t = 0; t < pdf.size(); ++t) {
-        const float rh = (float)V[t].x, ih = (float)V[t].y;
-        pdf[t] = make_float4(rh, (float)(V[t].x - rh), ih, (float)(V[t].y - ih));
-    }
-    put(so->psi_df, pdf);
+    const int S = so->S;
+    fixed_matrix(p, S, p.d_U, false, true, so->phi, so->phi_e);      // K index a, column p: phi_{a p}
+    fixed_matrix(p, S, p.d_V, true, false, so->psir, so->psir_e);    // real K index j, column i: psi_{i j}
+    fixed_matrix(p, S, p.d_V, false, true, so->red, so->red_e);      // K index p, column k: psi_{p k}
+    to_df(p, p.d_V, so->psi_df);
 }
 
 static SplitOperand& prepare(Plan& p)
@@ -2039,20 +2028,8 @@ static SplitOperand& prepare(Plan& p)
 // of the reduction GEMM (rows k, complex K index p), its exponents, and W in double-float.
 static void prepare_weights(Plan& p, SplitOperand& so, const double2* dW)
 {
-    const int n = p.n, S = so.S;
-    std::vector<double2> W((size_t)n * n);
-    NPF_CUDA(cudaMemcpy(W.data(), dW, W.size() * sizeof(double2), cudaMemcpyDeviceToHost));
-    std::vector<uint16_t> planes;
-    std::vector<int> ex;
-    build_fixed(n, S, true, [&](int pidx, int k) { return W[(size_t)pidx * n + k]; }, planes, ex);
-    put(so.wred, planes);
-    put(so.wred_e, ex);
-    std::vector<float4> wdf((size_t)n * n);
-    for (size_t t = 0; t < wdf.size(); ++t) {
-        const float rh = (float)W[t].x, ih = (float)W[t].y;
-        wdf[t] = make_float4(rh, (float)(W[t].x - rh), ih, (float)(W[t].y - ih));
-    }
-    put(so.w_df, wdf);
+    fixed_matrix(p, so.S, dW, false, true, so.wred, so.wred_e);
+    to_df(p, dW, so.w_df);
 }
 
 // Slot rows of the order's tuples from the plan's eigenvalues.
@@ -2066,14 +2043,12 @@ static void fill_slots(Plan& p, SplitOperand& so, int N)
 }
 
 #ifndef NPF_SPLIT_LOW
-void split_refresh_modes(Plan& p)
+void split_refresh_modes(Plan& p)   // (the caller waits for the stream: a batch's graph runs on others)
 {
     if (!p.split) return;
     fill_fixed(p, p.split);   // same n and S: the buffers (and graphs) stay valid
-    bool any = false;
     for (int N = 2; N <= 4; ++N)
-        if (p.split->slot_nm[N] == p.nm) { fill_slots(p, *p.split, N); any = true; }
-    if (any) NPF_CUDA(cudaStreamSynchronize(p.stream));   // (a batch's graph runs on other streams)
+        if (p.split->slot_nm[N] == p.nm) fill_slots(p, *p.split, N);
 }
 #endif
 

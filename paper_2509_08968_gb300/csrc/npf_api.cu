@@ -117,29 +117,26 @@ void activate_staged(Plan& p)
 
 std::atomic<uint64_t> g_next_plan_id{0};
 
-// The caller's modal data (host copies) into the device buffers in the plan's mode order: device
-// mode j is the caller's mode perm[j] (identity without a subset).
-void upload_modes(Plan& p)
+// The caller's modal data (host copies; `staged`: U and V are in d_tmp and d_sum already) into the
+// device buffers in the plan's mode order: device mode j is the caller's mode perm[j] (identity
+// without a subset). Waits for the stream, since other streams (batches) read the buffers.
+void upload_modes(Plan& p, bool staged)
 {
     const int n = p.n;
     const size_t nn = (size_t)n * n;
     std::vector<int> perm(n);
     for (int j = 0; j < n; ++j) perm[j] = p.perm.empty() ? j : p.perm[j];
-    std::vector<double2> U(nn), V(nn), Vt(nn), lam(n);
-    for (int j = 0; j < n; ++j) {
-        lam[j] = p.h_lam[perm[j]];
-        for (int a = 0; a < n; ++a) {
-            U[(size_t)a * n + j] = p.h_U[(size_t)a * n + perm[j]];     // column j = mode perm[j]
-            V[(size_t)j * n + a] = p.h_V[(size_t)perm[j] * n + a];     // row j = mode perm[j]
-        }
+    std::vector<double2> lam(n);
+    for (int j = 0; j < n; ++j) lam[j] = p.h_lam[perm[j]];
+    if (!staged) {
+        copy_in(p.d_tmp, p.h_U.data(), nn * sizeof(double2), p.stream);
+        copy_in(p.d_sum, p.h_V.data(), nn * sizeof(double2), p.stream);
     }
-    for (int i = 0; i < n; ++i)
-        for (int k = 0; k < n; ++k) Vt[(size_t)k * n + i] = V[(size_t)i * n + k];
-    NPF_CUDA(cudaMemcpy(p.d_U, U.data(), nn * sizeof(double2), cudaMemcpyHostToDevice));
-    NPF_CUDA(cudaMemcpy(p.d_V, V.data(), nn * sizeof(double2), cudaMemcpyHostToDevice));
-    NPF_CUDA(cudaMemcpy(p.d_Vt, Vt.data(), nn * sizeof(double2), cudaMemcpyHostToDevice));
-    NPF_CUDA(cudaMemcpy(p.d_lam, lam.data(), n * sizeof(double2), cudaMemcpyHostToDevice));
-    NPF_CUDA(cudaMemcpy(p.d_perm, perm.data(), n * sizeof(int), cudaMemcpyHostToDevice));
+    copy_in(p.d_lam, lam.data(), n * sizeof(double2), p.stream);
+    copy_in(p.d_perm, perm.data(), n * sizeof(int), p.stream);
+    npf::launch_order_modes(p, p.d_tmp, p.d_sum);
+    npf::split_refresh_modes(p);   // tensor-core forms: slices of Phi and Psi, in place
+    NPF_CUDA(cudaStreamSynchronize(p.stream));
 }
 
 // Validate (max |V U - I| <= NPF_INVERSE_TOL) and copy the modal data into the plan's buffers.
@@ -147,40 +144,21 @@ void load_modes(Plan& p, const npf_c128* eigvals, const npf_c128* U, const npf_c
 {
     const int n = p.n;
     const size_t nn = (size_t)n * n;
-    // host copies for validation and the transposed Psi
-    std::vector<double2> hU(nn), hV(nn), hVt(nn);
+    // host copies first: for device sources this waits for the work that the legacy stream has queued
+    std::vector<double2> hU(nn), hV(nn), hl(n);
     NPF_CUDA(cudaMemcpy(hU.data(), U, nn * sizeof(double2), cudaMemcpyDefault));
     NPF_CUDA(cudaMemcpy(hV.data(), V, nn * sizeof(double2), cudaMemcpyDefault));
-    for (int i = 0; i < n; ++i)
-        for (int k = 0; k < n; ++k) hVt[(size_t)k * n + i] = hV[(size_t)i * n + k];
-    // max |V U - I|
-    double worst = 0.0;
-    {
-        std::vector<double2> row(n);
-        for (int i = 0; i < n; ++i) {
-            for (int c = 0; c < n; ++c) row[c] = make_double2(0, 0);
-            for (int j = 0; j < n; ++j) {
-                const double2 v = hV[(size_t)i * n + j];
-                const double2* u = &hU[(size_t)j * n];
-                for (int c = 0; c < n; ++c) {
-                    row[c].x += v.x * u[c].x - v.y * u[c].y;
-                    row[c].y += v.x * u[c].y + v.y * u[c].x;
-                }
-            }
-            for (int c = 0; c < n; ++c) {
-                const double re = row[c].x - (c == i ? 1.0 : 0.0);
-                worst = std::fmax(worst, std::hypot(re, row[c].y));
-            }
-        }
-    }
+    NPF_CUDA(cudaMemcpy(hl.data(), eigvals, n * sizeof(double2), cudaMemcpyDefault));
+    copy_in(p.d_tmp, hU.data(), nn * sizeof(double2), p.stream);
+    copy_in(p.d_sum, hV.data(), nn * sizeof(double2), p.stream);
+    const double worst = npf::inverse_error(p, p.d_sum, p.d_tmp, p.d_npf);
     if (!(worst <= NPF_INVERSE_TOL))
         npf::fail(NPF_ERR_NOT_INVERSE,
                   "max|V U - I| = " + std::to_string(worst) + " exceeds NPF_INVERSE_TOL");
     p.h_U = std::move(hU);
     p.h_V = std::move(hV);
-    p.h_lam.resize(n);
-    NPF_CUDA(cudaMemcpy(p.h_lam.data(), eigvals, n * sizeof(double2), cudaMemcpyDefault));
-    upload_modes(p);
+    p.h_lam = std::move(hl);
+    upload_modes(p, true);
 }
 
 
@@ -581,7 +559,6 @@ int npf_set_modes(npf_handle* h, const npf_c128* eigvals, const npf_c128* U, con
         Plan& p = h->p;
         NPF_CUDA(cudaStreamSynchronize(p.stream));
         load_modes(p, eigvals, U, V);
-        npf::split_refresh_modes(p);   // tensor-core forms: slices of Phi and Psi, in place
     });
 }
 
@@ -607,8 +584,7 @@ int npf_set_mode_subset(npf_handle* h, int m, const int* modes)
         NPF_CUDA(cudaStreamSynchronize(p.stream));
         p.perm = perm;
         p.nm = perm.empty() ? n : m;
-        upload_modes(p);
-        npf::split_refresh_modes(p);
+        upload_modes(p, false);
         ++p.gen;
     });
 }

@@ -174,6 +174,10 @@ void launch_axpy(Plan& p, double2* y, double a, const double2* x, double b, int6
 void launch_hadamard_t(Plan& p, double sign, const double2* Z, double2* out);   // out[k][i] = sign U[k][i] Z[i][k]
 // results back to the caller's mode order: columns (out[k][perm[j]] = in[k][j]) or rows
 void launch_unpermute(Plan& p, const double2* in, double2* out, bool columns);
+// max |V U - I|; scratch: one element
+double inverse_error(Plan& p, const double2* V, const double2* U, double2* scratch);
+// U, V and V transposed in the plan's mode order (d_perm) from the caller's order
+void launch_order_modes(Plan& p, const double2* Us, const double2* Vs);
 void build_cnt_table(Plan& p);
 void note_launches(int64_t k);   // k more kernels launched (graph replays)
 
