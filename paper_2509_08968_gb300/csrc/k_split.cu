@@ -20,10 +20,10 @@
 //
 // Dataflow of one order N (Algorithm 2). h and every intermediate are symmetric in their a's and in
 // their p's, so only sorted tuples are formed, stored in colexicographic rank:
-//   P1     : S[i][Q] = sum_j psi_{ij} A^j_Q on the packed (sorted) lower tuples Q (real rows Q,
-//            K = j), then per-i digit records of S (the upper index first: step 4 moved ahead,
-//            which the contraction order allows).
-//   expand : rows (i, sorted (a_1..a_{N-1})), K = a_N, digits of S^i_{sort(a)}
+//   P1     : S[i][Q] = sum_j psi_{ij} A^j_Q on the sorted lower tuples Q (real rows Q, K = j), V and
+//            the exponent per i (the upper index first: step 4 moved ahead, which the contraction
+//            order allows).
+//   expand : rows (i, sorted (a_1..a_{N-1})), K = a_N, digits of S^i_{sort(a)} gathered from V
 //   c = 1..N-2 : contract an a with Phi; V (the exact 64-bit accumulators) per
 //            (i, sorted p's, sorted a's), regathered into the digit rows
 //            (i, sorted p's, sorted a's less one), K = the remaining a, with exact row exponents
@@ -64,10 +64,13 @@ constexpr int ROW_THREADS = 64 + 32 * EPI_WARPS;
 // ---------------------------------------------------------------------------------------
 // Integer / double-float helpers
 // ---------------------------------------------------------------------------------------
-__device__ __forceinline__ int bitlen64(long long v)
+// Bit length of max(|v.x|, |v.y|) (one less for a negative power of two, which the top digit's range
+// [-128, 128] holds).
+__device__ __forceinline__ int bitlen(longlong2 v)
 {
-    const unsigned long long a = v < 0 ? (unsigned long long)(-v) : (unsigned long long)v;
-    return a ? 64 - __clzll(a) : 0;
+    const unsigned long long m = (unsigned long long)(v.x < 0 ? ~v.x : v.x) |
+                                 (unsigned long long)(v.y < 0 ? ~v.y : v.y);
+    return 64 - __clzll((long long)m);
 }
 
 // W = round(V * 2^sh) for |result| < 2^47.
@@ -329,23 +332,32 @@ __device__ __forceinline__ void load_levels(uint32_t taddr, int stride, uint32_t
     }
 }
 
-// Colexicographic ranks of sorted pairs and triples.
+// Colexicographic ranks of sorted pairs, triples and quadruples.
 __host__ __device__ __forceinline__ int rank2(int a, int b) { return b * (b + 1) / 2 + a; }   // a <= b
 __host__ __device__ __forceinline__ int rank3(int a, int b, int c)                            // a <= b <= c
 {
     return c * (c + 1) * (c + 2) / 6 + b * (b + 1) / 2 + a;
 }
+__host__ __device__ __forceinline__ int rank4(int a, int b, int c, int d)                     // a <= .. <= d <= 128
+{
+    return d * (d + 1) * (d + 2) / 6 * (d + 3) / 4 + rank3(a, b, c);
+}
 
 // ---------------------------------------------------------------------------------------
 // Input preparation (once per tensor): A^T digit planes for the upper-index contraction,
-// rows = packed lower tuples Q (exponent per Q over all j), K' = j (real).
+// rows = sorted lower tuples Q (exponent per Q over all j), K' = j (real). The packed tensor's
+// tuples are in lexicographic order; the rows go to their colexicographic rank, the order of every
+// later intermediate (a row is 256 bytes a plane, so the scatter costs nothing).
 // ---------------------------------------------------------------------------------------
 template <int S>
-__global__ void k_prep_at(const double* __restrict__ A, int64_t P, int n,
-                          __nv_bfloat16* __restrict__ planes, int64_t plane_stride,
-                          int* __restrict__ expQ)
+__global__ void k_prep_at(const double* __restrict__ A, int64_t P, int n, int N,
+                          const int64_t* __restrict__ cnt, __nv_bfloat16* __restrict__ planes,
+                          int64_t plane_stride, int* __restrict__ expQ)
 {
-    // one warp per Q row: lanes cover j = lane, lane+32, lane+64, lane+96
+    __shared__ int cn[5 * (NP + 1)];   // non-decreasing r-tuples in [v, n), r <= N
+    for (int t = threadIdx.x; t < (N + 1) * (n + 1); t += blockDim.x) cn[t] = (int)cnt[t];
+    __syncthreads();
+    // one warp per Q: lanes cover j = lane, lane+32, lane+64, lane+96
     const int64_t q = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
     const int lane = threadIdx.x % 32;
     if (q >= P) return;
@@ -357,11 +369,29 @@ __global__ void k_prep_at(const double* __restrict__ A, int64_t P, int n,
         v[t] = j < n ? A[(int64_t)j * P + q] : 0.0;
         m = fmax(m, fabs(v[t]));
     }
+    // the tuple of lexicographic rank q, an index at a time: the first index is >= x for the last
+    // cn[r][x] of the r-tuples from the previous index on
+    int64_t row = 0;
+    {
+        int rem = (int)q, prev = 0;
+        for (int pos = 0; pos < N; ++pos) {
+            const int* c = cn + (N - pos) * (n + 1);
+            int x = prev;
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const int w = lane + 32 * t;
+                x += __popc(__ballot_sync(0xffffffffu, w > prev && w < n && rem >= c[prev] - c[min(w, n)]));
+            }
+            rem -= c[prev] - c[x];
+            prev = x;
+            row += pos == 0 ? x : pos == 1 ? rank2(0, x) : pos == 2 ? rank3(0, 0, x) : rank4(0, 0, 0, x);
+        }
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
     int e = EXP_NONE;
     if (m > 0.0) frexp(m, &e);
-    if (lane == 0) expQ[q] = e;
+    if (lane == 0) expQ[row] = e;
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
         const int j = lane + 32 * t;
@@ -376,7 +406,7 @@ __global__ void k_prep_at(const double* __restrict__ A, int64_t P, int n,
             } else {
                 d = (int)W;
             }
-            reinterpret_cast<uint16_t*>(planes)[s * plane_stride + q * NP + j] =
+            reinterpret_cast<uint16_t*>(planes)[s * plane_stride + row * NP + j] =
                 (uint16_t)digit_bf16(d, s);
         }
     }
@@ -395,7 +425,7 @@ __global__ void k_prep_at(const double* __restrict__ A, int64_t P, int n,
 //   reduction              : rows (i, sorted (p_1..p_{N-1})), K = p_N
 // Each forms only new indices p <= the row's first p.
 // ---------------------------------------------------------------------------------------
-enum { EPI_F64T = 0, EPI_SLICE = 1, EPI_DIVIDE = 2, EPI_SLAB = 3, EPI_REDUCE = 4, EPI_V = 5 };
+enum { EPI_V = 0, EPI_SLICE = 1, EPI_DIVIDE = 2, EPI_SLAB = 3, EPI_REDUCE = 4 };
 
 // Tensor maps of one operand: every slice plane in one box (`all`), and the planes of levels
 // 0..2 only (`low`, the second pass of a tile with the level-3 hold).
@@ -425,6 +455,7 @@ struct RowArgs {
     // EPI_V: V (two 64-bit integers) at out_v[(new tuple) * R + row]; colmask: outer = (i, p), and
     // the new tuple (i, rank2(q, p)), else (i, q)
     longlong2* out_v;
+    int* emax;           // EPI_V: largest exponent of every column (merged by atomicMax), or nullptr
     // EPI_SLICE: rows (tuple t of nt sorted (p_3..p_N), a_1); output rows are the divide's slots, RS
     // per upper index
     int nt;
@@ -452,8 +483,7 @@ struct RowArgs {
     __nv_bfloat16* out_planes;
     int64_t out_plane_stride;
     int* out_exp;
-    double2* out_f64;    // EPI_F64T: out[q * ld_f64 + o]; EPI_SLAB: out[i * n + q]; EPI_REDUCE: Psi_N
-    int64_t ld_f64;
+    double2* out_f64;    // EPI_SLAB: out[i * n + q]; EPI_REDUCE: Psi_N
     // EPI_DIVIDE / EPI_SLAB / EPI_REDUCE
     const double2* lam;
     const float4* psi_df;    // the reduction weights W[p][k] (psi_{p k}) as double-float, at p*n + k
@@ -1265,21 +1295,16 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                         const int qc = qbase + cl;
                         const int eb = colEb[cl];
                         if (MODE == EPI_V) {
+                            longlong2 v = make_longlong2(0ll, 0ll);
                             if (row_in && qc < args.ncv && qc <= firstp) {
-                                longlong2 v;
                                 v.x = combine(rv[0][c], rv[1][c], rv[2][c], rv[3][c]);
                                 v.y = combine(iv[0][c], iv[1][c], iv[2][c], iv[3][c]);
                                 args.out_v[vbase + (int64_t)qc * args.R] = v;
                             }
-                            continue;
-                        }
-                        if (MODE == EPI_F64T) {
-                            if (qc < args.ncv) {
-                                const double sc = pow2d(ea + eb - VEXP);
-                                const long long Vr = combine(rv[0][c], rv[1][c], rv[2][c], rv[3][c]);
-                                const long long Vi = combine(iv[0][c], iv[1][c], iv[2][c], iv[3][c]);
-                                args.out_f64[(int64_t)qc * args.ld_f64 + o] =
-                                    make_double2((double)Vr * sc, (double)Vi * sc);
+                            if (args.emax) {
+                                const unsigned key = v.x | v.y ? (unsigned)(bitlen(v) + ea + eb - VEXP + 8192) : 0u;
+                                const unsigned wmax = __reduce_max_sync(0xffffffffu, key);
+                                if (lane == 0 && wmax) atomicMax(&colE[cl], (int)wmax);
                             }
                             continue;
                         }
@@ -1411,6 +1436,8 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
             }
             tc::fence_before_sync();
             epi_sync();
+            if (MODE == EPI_V && args.emax && et < bnc && qbase + et < args.ncv && colE[et])
+                atomicMax(&args.emax[qbase + et], colE[et] - 8192);
             if (trc && et == 0) trc[3] = global_ns();
             if (et == 0) tc::mbar_arrive(&tempty[set]);
             ++t;
@@ -1424,157 +1451,31 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
     }
 }
 
-// ---------------------------------------------------------------------------------------
-// Digit records of S^i_Q (per upper index i, exponent over all Q) for the dense expansion.
-// ---------------------------------------------------------------------------------------
-// The exponent of max_Q |S^i_Q| per upper index i: blocks (chunk, i) take strided slices of one
-// row and merge their maxima by an integer atomicMax on the frexp exponent (monotone in the
-// magnitude), so that each row spreads over several SMs. E holds EXP_NONE on entry (k_exp_init).
-static __global__ void k_exp_init(int* __restrict__ E, int n)
+// Start of a term: the output (zeroed unless the term is added to it), the exponents of S and the
+// error flag (nullptr: a batch's, zeroed once for all).
+static __global__ void k_term_init(double2* __restrict__ out, int64_t count, int* __restrict__ sE, int nm,
+                                   int* __restrict__ err)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) E[i] = EXP_NONE;
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < count) out[t] = make_double2(0.0, 0.0);
+    if (t < nm) sE[t] = EXP_NONE;
+    if (t == 0 && err) *err = 0;
 }
 
-static __global__ void k_s_exp(const double2* __restrict__ Sd, int64_t ld, int64_t P, int* __restrict__ E)
-{
-    const int i = blockIdx.y;
-    double m = 0.0;
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < P;
-         q += (int64_t)gridDim.x * blockDim.x) {
-        const double2 v = Sd[(int64_t)i * ld + q];
-        m = fmax(m, fmax(fabs(v.x), fabs(v.y)));
-    }
-    __shared__ double red[256];
-    red[threadIdx.x] = m;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + w]);
-        __syncthreads();
-    }
-    if (threadIdx.x == 0 && red[0] > 0.0) {
-        int e;
-        frexp(red[0], &e);
-        atomicMax(&E[i], e);
-    }
-}
-
-// rec[i*P + q] = 8 x uint32: (Re, Im) BF16 digit pairs of S^i_q for planes 0..S-1
-template <int S>
-__global__ void k_s_records(const double2* __restrict__ Sd, int64_t ld, int64_t P, int n,
-                            const int* __restrict__ E, uint4* __restrict__ rec)
-{
-    const int64_t tot = (int64_t)n * P;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < tot;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int i = (int)(idx / P);
-        const int64_t q = idx % P;
-        const int e = E[i];
-        uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        if (e != EXP_NONE) {
-            const double2 v = Sd[(int64_t)i * ld + q];
-            const double sc = pow2d(7 + 8 * (S - 1) - e);
-            uint32_t ww[S];
-            digit_pairs<S>(__double2ll_rn(v.x * sc), __double2ll_rn(v.y * sc), ww);
-#pragma unroll
-            for (int s = 0; s < S; ++s) w[s] = ww[s];
-        }
-        rec[idx * 2 + 0] = make_uint4(w[0], w[1], w[2], w[3]);
-        rec[idx * 2 + 1] = make_uint4(w[4], w[5], w[6], w[7]);
-    }
-}
-
-// Expansion: one warp per (upper index i, sorted (N-1)-tuple of a's, colexicographic rank). Lane t
-// covers a_N = lane + 32 t: the digit records S^i_{sort(tuple, a_N)} are gathered (rec holds the
-// packed, lexicographic order) into the first mode product's operand row. Layout: row
-// (i - i0) R + rank, 2^lg complex K entries a row of which kout are written (entries past n are
-// zeros: they meet the fixed matrix's zero rows, where stale bit patterns could be NaN).
-template <int S>
-__global__ void k_expand_sorted(const uint4* __restrict__ rec, int64_t P, int n, int N, int i0,
-                                int ib, int lg, int kout, const int64_t* __restrict__ cnt,
-                                const uint32_t* __restrict__ tuples, int64_t ntup, int64_t R,
-                                uint32_t* __restrict__ planes, int64_t plane_stride_u32)
-{
-    // the rank table (rows 0..N of C(n - v + r - 1, r), <= 5 x 129 entries) in shared memory:
-    // every gathered record's rank reads it, and from global memory its dependent loads made
-    // the kernel latency-bound
-    __shared__ int64_t s_cnt[5 * (NP + 1)];
-    for (int t = threadIdx.x; t < (N + 1) * (n + 1); t += blockDim.x) s_cnt[t] = cnt[t];
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int nd = N - 1;
-    for (int64_t item = warp; item < ntup * ib; item += nwarps) {
-        const int il = (int)(item / ntup);
-        const int64_t r0row = item - il * ntup;
-        const uint32_t pk = tuples[r0row];
-        int pre[3];
-#pragma unroll
-        for (int m = 0; m < 3; ++m) pre[m] = (int)((pk >> (8 * m)) & 255u);
-        // The four records' ranks first, then their eight loads back to back, so that a lane's
-        // gathers are in flight together. The sorted tuple is the prefix with a_N inserted at
-        // pos (the number of prefix values <= a_N); its rank is the telescoped count over the
-        // tuple, with every index a compile-time constant so that nothing goes to local memory.
-        int64_t qv[4];
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const int aN = lane + 32 * t;
-            qv[t] = -1;
-            if (aN < n) {
-                int pos = 0;
-#pragma unroll
-                for (int m = 0; m < 3; ++m) pos += (m < nd && pre[m] <= aN) ? 1 : 0;
-                int64_t r = 0;
-                int prev = 0;
-#pragma unroll
-                for (int m = 0; m < 4; ++m) {
-                    if (m < N) {
-                        const int sm = m < pos ? pre[m < 3 ? m : 2]
-                                               : (m == pos ? aN : pre[m >= 1 ? m - 1 : 0]);
-                        const int64_t* row = s_cnt + (N - m) * (n + 1);
-                        r += row[prev] - row[sm];
-                        prev = sm;
-                    }
-                }
-                qv[t] = r;
-            }
-        }
-        uint4 r0[4], r1[4];
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            r0[t] = make_uint4(0u, 0u, 0u, 0u);
-            r1[t] = make_uint4(0u, 0u, 0u, 0u);
-            if (qv[t] >= 0) {
-                r0[t] = rec[((int64_t)(i0 + il) * P + qv[t]) * 2 + 0];
-                r1[t] = rec[((int64_t)(i0 + il) * P + qv[t]) * 2 + 1];
-            }
-        }
-        uint32_t* dst = planes + (((int64_t)il * R + r0row) << lg) + lane;
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const uint32_t rr[8] = {r0[t].x, r0[t].y, r0[t].z, r0[t].w, r1[t].x, r1[t].y, r1[t].z, r1[t].w};
-            if (lane + 32 * t < kout)
-#pragma unroll
-                for (int s = 0; s < S; ++s) dst[s * plane_stride_u32 + 32 * t] = rr[s];
-        }
-    }
-}
-
-// Operand rows of the next mode product from a mode product's V (EPI_V): one warp per row
-// (outer, sorted M-tuple of a's), outer = (i, sorted tuple of p's). Lane t covers a = lane + 32 t:
-// it gathers V[outer][rank(sort(tuple, a))], and the row gets its exact exponent (the largest
-// bit length) and its digits. V is in units of 2^(ea + eb - VEXP) with eb of the newest p.
-//   ea: by upper index (M + 1 = N - 1: the first product's operand has one exponent per index) or
-//       (ea_row) by the source product's operand row, (i, p, rank) with p the tuple's other index
+// Operand rows of a mode product from the exact 64-bit values V of the stage before (EPI_V): one
+// warp per row (outer, sorted M-tuple of a's). Lane t covers a = lane + 32 t: it gathers
+// V[outer][rank(sort(tuple, a))] and writes its digits. V is in units of 2^(ea + eb - VEXP).
+//   SRC 0: V of the first mode product, outer = (i, p); ea by i, eb by p
+//   SRC 1: V of the second (order 4), outer = (i, p_3 <= p_4); ea by its operand row (i, p_4, rank),
+//          eb by p_3
+//   SRC 2: V of the upper contraction (M = N - 1), outer = i; ea by rank (the tensor's), eb by i, and
+//          the rows share the exponent rowE[i]; the others get their exact one (largest bit length)
 // Neighbouring rows gather neighbouring entries (colexicographic rank), so the warps of a block
-// share sectors. Bound: HBM writes (4 S bytes an entry against 16 read per source entry): 0.69 ms
-// per upper index and product at n = 120, order 4 (3.2 GB: 4.7 TB/s). It pays because the products
-// before it run on sorted a's only: 614 ms of mode products became 245 + 166 here.
-template <int S, int M>
+// share sectors. Bound: HBM writes (4 S bytes an entry against 16 read per source entry).
+template <int S, int M, int SRC>
 __global__ void __launch_bounds__(256)
     k_regather(const longlong2* __restrict__ V, int64_t Rsrc, int n, int nm, int nt, const uint32_t* __restrict__ ttup,
-               const int* __restrict__ ea, int ea_row, const int* __restrict__ eb, int lg, int kout,
+               const int* __restrict__ ea, const int* __restrict__ eb, const int* __restrict__ rowE, int lg, int kout,
                int nrows, int64_t Rdst, int64_t nouter, const uint32_t* __restrict__ tuples,
                uint32_t* __restrict__ planes, int64_t plane_stride_u32, int* __restrict__ out_exp)
 {
@@ -1585,17 +1486,23 @@ __global__ void __launch_bounds__(256)
         const int64_t outer = st / chunks;
         const int row = (int)(st - outer * chunks) * 8 + (int)(threadIdx.x >> 5);
         if (row >= nrows) continue;
-        const int64_t i = outer / nt;
-        const int t = (int)(outer - i * nt);
-        const uint32_t tp = ea_row ? ttup[t] : (uint32_t)t;  // the newest p in the low byte
-        const int q = (int)(tp & 255u);
-        const int e0 = eb[q] - VEXP + (ea_row ? 0 : ea[i]);
-        const int* earow = ea_row ? ea + (i * nm + (int)((tp >> 8) & 255u)) * Rsrc : nullptr;
-        int x = row, y = 0;
-        if (M == 2) {
+        int e0;
+        const int* earow = ea;
+        if (SRC == 2) {
+            e0 = eb[outer] - VEXP;
+        } else {
+            const int64_t i = outer / nt;
+            const int t = (int)(outer - i * nt);
+            const uint32_t tp = SRC == 1 ? ttup[t] : (uint32_t)t;   // the newest p in the low byte
+            e0 = eb[tp & 255u] - VEXP + (SRC == 0 ? ea[i] : 0);
+            if (SRC == 1) earow = ea + (i * nm + (int)((tp >> 8) & 255u)) * Rsrc;
+        }
+        int x = row, y = 0, z = 0;
+        if (M >= 2) {
             const uint32_t pk = tuples[row];
             x = (int)(pk & 255u);
             y = (int)((pk >> 8) & 255u);
+            z = (int)((pk >> 16) & 255u);
         }
         const longlong2* src = V + outer * Rsrc;
         longlong2 v[4];
@@ -1606,23 +1513,32 @@ __global__ void __launch_bounds__(256)
             v[k] = make_longlong2(0ll, 0ll);
             ex[k] = 0;
             if (a < n) {
-                const int rk = M == 1 ? (a <= x ? rank2(a, x) : rank2(x, a))
-                                      : (a <= x ? rank3(a, x, y) : a <= y ? rank3(x, a, y) : rank3(x, y, a));
+                int rk;
+                if (M == 0) rk = a;
+                else if (M == 1) rk = rank2(min(a, x), max(a, x));
+                else if (M == 2) {
+                    const int lo = min(a, x), hi = max(a, y);
+                    rk = rank3(lo, x + y + a - lo - hi, hi);
+                } else {
+                    const int lo = min(a, x), hi = max(a, z);
+                    const int p = a <= y ? max(a, x) : y, q = a <= y ? y : min(a, z);   // the middle two
+                    rk = rank4(lo, p, q, hi);
+                }
                 v[k] = src[rk];
-                if (ea_row) ex[k] = earow[rk];
+                if (SRC != 0) ex[k] = earow[rk];
             }
         }
-        int key = 0;
+        int E;
+        if (SRC == 2) {
+            E = rowE[outer];
+        } else {
+            int key = 0;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const unsigned long long m = (unsigned long long)(v[k].x < 0 ? ~v[k].x : v[k].x) |
-                                         (unsigned long long)(v[k].y < 0 ? ~v[k].y : v[k].y);
-            // bit length of max(|x|, |y|) (one less for a negative power of two, which the top
-            // digit's range [-128, 128] holds)
-            if (v[k].x | v[k].y) key = max(key, 64 - __clzll((long long)m) + ex[k] + e0 + 8192);
+            for (int k = 0; k < 4; ++k)
+                if (v[k].x | v[k].y) key = max(key, bitlen(v[k]) + ex[k] + e0 + 8192);
+            key = (int)__reduce_max_sync(0xffffffffu, (unsigned)key);
+            E = key ? key - 8192 : EXP_NONE;
         }
-        key = (int)__reduce_max_sync(0xffffffffu, (unsigned)key);
-        const int E = key ? key - 8192 : EXP_NONE;
         const int sh = e0 - E + 7 + 8 * (S - 1);
         const int64_t rowp = outer * Rdst + row;
         uint32_t* dst = planes + (rowp << lg) + lane;
@@ -1630,7 +1546,7 @@ __global__ void __launch_bounds__(256)
         for (int k = 0; k < 4; ++k) {
             if (lane + 32 * k < kout) {
                 uint32_t w[S];
-                if (key) {
+                if (E != EXP_NONE) {
                     digit_pairs<S>(shift_full(v[k].x, sh + ex[k]), shift_full(v[k].y, sh + ex[k]), w);
                 } else {
 #pragma unroll
@@ -1640,7 +1556,7 @@ __global__ void __launch_bounds__(256)
                 for (int s = 0; s < S; ++s) dst[s * plane_stride_u32 + 32 * k] = w[s];
             }
         }
-        if (lane == 0) out_exp[rowp] = E;
+        if (SRC != 2 && lane == 0) out_exp[rowp] = E;
     }
 }
 
@@ -1692,8 +1608,8 @@ static __global__ void k_slot_rows(int N, int64_t count, const uint32_t* __restr
 }
 
 // Zeros in the reduction rows' K entries that its tiles read but the divide does not write: from
-// the chunk of the tile's smallest p_{N-1} up to the row's own p_{N-1}, and from nm to the end of
-// the last chunk. kc: complex K entries a chunk. One thread per (upper index, row, 8th entry).
+// the chunk of the tile's smallest p_{N-1} up to the row's own p_{N-1}, and from nm to the operand's
+// inner extent. kc: complex K entries a chunk. One thread per (upper index, row, 8th entry).
 template <int S>
 __global__ void k_zero_heads(int N, int nm, int kc, int lg, int Q, int64_t RT, int nouter,
                              const uint32_t* __restrict__ tuples, uint32_t* __restrict__ planes,
@@ -1711,7 +1627,7 @@ __global__ void k_zero_heads(int N, int nm, int kc, int lg, int Q, int64_t RT, i
     for (int k = p0 / kc * kc + e; k < p; k += 8)
 #pragma unroll
         for (int s = 0; s < S; ++s) dst[s * plane_stride_u32 + k] = 0u;
-    const int end = min(1 << lg, (nm + kc - 1) / kc * kc);
+    const int end = min(1 << lg, (nm + 7) / 8 * 8);
     for (int k = nm + e; k < end; k += 8)
 #pragma unroll
         for (int s = 0; s < S; ++s) dst[s * plane_stride_u32 + k] = 0u;
@@ -1811,15 +1727,16 @@ static CUtensorMap encode_map(const void* base, int rank, const cuuint64_t* dims
 
 // Operands as the callers describe them: data planes [S][rows][inner] and fixed-matrix planes
 // [S][512][inner] (Re rows at 0.., Im rows at 256..), BF16.
-struct DataOp { const void* base; int64_t inner, rows; };
+struct DataOp { const void* base; int64_t inner, stride, rows; };   // stride: elements between rows
 struct FixedOp { const void* base; int64_t inner; };
 
-// Data operand as a 3-D tensor (inner, rows, plane); box {bk, 128 rows, planes}.
+// Data operand as a 3-D tensor (inner, rows, plane); box {bk, 128 rows, planes}. Past the inner
+// extent a box holds zeros.
 template <int S>
 static TMaps plane_maps(const DataOp& d, int bk)
 {
     const cuuint64_t dims[3] = {(cuuint64_t)d.inner, (cuuint64_t)d.rows, (cuuint64_t)S};
-    const cuuint64_t strides[2] = {(cuuint64_t)d.inner * 2, (cuuint64_t)(d.rows * d.inner * 2)};
+    const cuuint64_t strides[2] = {(cuuint64_t)d.stride * 2, (cuuint64_t)(d.rows * d.stride * 2)};
     const cuuint32_t box_all[3] = {(cuuint32_t)bk, (cuuint32_t)NP, (cuuint32_t)S};
     const cuuint32_t box_low[3] = {(cuuint32_t)bk, (cuuint32_t)NP, (cuuint32_t)pass_planes<S>(2)};
     return {encode_map(d.base, 3, dims, strides, box_all, bk),
@@ -1864,8 +1781,8 @@ static size_t dense_bytes(int n, int N, int S)
 }
 
 #ifndef NPF_SPLIT_LOW
-// A term is accepted when S, its records and the dense rows of one upper index fit the budget (the
-// sorted rows it forms take less).
+// A term is accepted when S, digit records of it (32 bytes an entry) and the dense rows of one upper
+// index fit the budget: the sorted rows it forms take less, and no records are kept.
 size_t split_min_bytes(const Plan& p, int N)
 {
     const int64_t P = p.packed_count[N], rows = (P + NP - 1) / NP * NP;
@@ -1907,7 +1824,6 @@ static void set_smem_attrs()
 {
     static bool done = false;
     if (done) return;
-    smem_attr<S, EPI_F64T, false>();   // packed-tuple rows: never sub-blocks
     smem_attr<S, EPI_SLICE, false>();
     smem_attr<S, EPI_SLICE, true>();
     smem_attr<S, EPI_DIVIDE, false>();
@@ -2160,7 +2076,7 @@ static void prepare_tensor(Plan& p, SplitOperand& so, int N)
     NPF_CUDA(cudaMemsetAsync(so.at[N], 0, (size_t)S * rows * NP * 2, p.stream));
     {
         LaunchScope ls(&p.prof, "split_prepare_tensor", p.stream);
-        k_prep_at<S><<<(unsigned)((P + 7) / 8), 256, 0, p.stream>>>(p.d_tensor[N], P, p.n, so.at[N],
+        k_prep_at<S><<<(unsigned)((P + 7) / 8), 256, 0, p.stream>>>(p.d_tensor[N], P, p.n, N, p.d_cnt, so.at[N],
                                                                     rows * NP, so.at_e[N]);
         NPF_CUDA(cudaGetLastError());
     }
@@ -2336,8 +2252,7 @@ static void launch_rows(Plan& p, const char* name, const DataOp& A, const FixedO
 
 static double factorial(int N) { double f = 1; for (int t = 2; t <= N; ++t) f *= t; return f; }
 
-// Device memory of one order: S (FP64, n x P), records (n x P x 32 B), and per upper index of a
-// batch two buffers that the stages alternate (A: the operands of the mode products and of the
+// Device memory of one order: V of S (16 bytes, n x P) and per upper index of a batch two buffers that the stages alternate (A: the operands of the mode products and of the
 // reduction, B: V and the divide's slots) plus the row exponents.
 template <int S>
 static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const double2* W, bool accumulate)
@@ -2352,7 +2267,6 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     if (N >= 2 && !slab) ensure_ptuples(p, so, N - 1);
     if (N == 4) ensure_ptuples(p, so, 2);
     int* const err = p.err_override ? p.err_override : so.err;   // a batch zeroes and checks its own
-    if (!p.err_override) NPF_CUDA(cudaMemsetAsync(err, 0, sizeof(int), p.stream));
     const int n = p.n;
     const int nm = p.nm;                 // modes in use (a critical-mode subset comes first)
     const int64_t P = p.packed_count[N];
@@ -2378,7 +2292,6 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     // ---- memory plan (Algorithm 1's rule on the upper-index space)
     const size_t row_bytes = (size_t)rad * 4 * S;
     const size_t s_bytes = (size_t)n * Prows * sizeof(double2);
-    const size_t rec_bytes = (size_t)n * P * 32;
     const size_t a_per = (size_t)std::max(std::max(R0, R1), std::max(R2, Qc)) * row_bytes;
     const size_t b_per = std::max((size_t)v_per * sizeof(longlong2), (size_t)RS * row_bytes);
     const size_t e_per = (size_t)(R1 + R2 + RS + Qc) * sizeof(int);
@@ -2386,15 +2299,14 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     const size_t budget = effective_budget(p);
     if (split_min_bytes(p, N) > budget)
         fail(NPF_ERR_OOM, "memory budget too small for one upper-index batch");
-    const int ib = (int)std::min<size_t>((size_t)nm, (budget - s_bytes - rec_bytes) / per_i);
+    const int ib = (int)std::min<size_t>((size_t)nm, (budget - s_bytes) / per_i);
     const int64_t Q2 = N == 4 && !slab ? npairs : 0;              // order 4: weights of the pairs
     const size_t wbytes = (size_t)Q2 * n * sizeof(float4);
     Arena& ar = p.scratch();
-    ar.reserve(s_bytes + rec_bytes + (size_t)ib * (a_per + b_per + e_per) + wbytes + 10 * 256 + 1024);
+    ar.reserve(s_bytes + (size_t)ib * (a_per + b_per + e_per) + wbytes + 10 * 256 + 1024);
     uint8_t* base = (uint8_t*)ar.base;
     auto take = [&](size_t bytes) { uint8_t* r = base; base += (bytes + 255) & ~(size_t)255; return r; };
-    double2* Sd = (double2*)take(s_bytes);
-    uint4* rec = (uint4*)take(rec_bytes);
+    longlong2* Sv = (longlong2*)take(s_bytes);
     int* sE = (int*)take(256 * sizeof(int));
     uint8_t* bufA = take((size_t)ib * a_per);
     uint8_t* bufB = take((size_t)ib * b_per);
@@ -2412,13 +2324,19 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
         wpre = wp;
     }
 
-    // a slab entry whose accumulator is exactly zero is not stored, so the slab starts at zero
-    if (!accumulate) launch_zero(p, d_out, (int64_t)n * n);
+    {
+        // (a slab entry whose accumulator is exactly zero is not stored, so the slab starts at zero)
+        LaunchScope ls(&p.prof, "split_term_init", p.stream);
+        const int64_t cells = accumulate ? 0 : (int64_t)n * n;
+        k_term_init<<<(unsigned)((std::max<int64_t>(cells, nm) + 255) / 256), 256, 0, p.stream>>>(
+            d_out, cells, sE, nm, p.err_override ? nullptr : err);
+        NPF_CUDA(cudaGetLastError());
+    }
 
     const FixedOp tPhi{so.phi, KP};
     const FixedOp tPsiR{so.psir, NP};
     const FixedOp tRed{W ? so.wred : so.red, KP};
-    const DataOp tAT{so.at[N], NP, Prows};
+    const DataOp tAT{so.at[N], NP, NP, Prows};
 
     RowArgs base0{};
     base0.n = n;
@@ -2442,44 +2360,37 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     if (slab)
         for (int m = 0; m < N - 1; ++m) base0.pre[m] = prefix[m];
 
-    // ---- P1: S[i][Q] = sum_j psi_ij A^j_Q (rows Q, real K = j)
+    // ---- P1: V of S[i][Q] = sum_j psi_ij A^j_Q (rows Q, real K = j), and its exponent per i
     {
         RowArgs a = base0;
         a.ea = so.at_e[N];
         a.eb = so.psir_e;
-        a.num_tiles = Prows / NP * a.ncol_tiles;
         a.R = Prows;
-        a.out_f64 = Sd;
-        a.ld_f64 = Prows;
-        launch_rows<S, EPI_F64T>(p, "split_upper_contraction", tAT, tPsiR, n, a);   // K = j < n
-    }
-    {
-        LaunchScope ls(&p.prof, "split_s_records", p.stream);
-        // a few blocks per upper index, so that the n rows fill the GPU
-        const int64_t per_row = std::max<int64_t>(1, std::min<int64_t>((2 * sm_count() + nm - 1) / nm,
-                                                                       (P + 255) / 256));
-        k_exp_init<<<(nm + 255) / 256, 256, 0, p.stream>>>(sE, nm);
-        k_s_exp<<<dim3((unsigned)per_row, (unsigned)nm), 256, 0, p.stream>>>(Sd, Prows, P, sE);
-        k_s_records<S><<<4096, 256, 0, p.stream>>>(Sd, Prows, P, nm, sE, rec);
-        NPF_CUDA(cudaGetLastError());
+        a.RB = (int)(Prows / NP);
+        a.num_tiles = Prows / NP * a.ncol_tiles;
+        a.out_v = Sv;
+        a.emax = sE;
+        launch_rows<S, EPI_V>(p, "split_upper_contraction", tAT, tPsiR, n, a);   // K = j < n
     }
 
-    // K entries a launch reads: whole chunks of its pipeline
-    auto chunked = [&](int bk) { return std::min(rad, (n + bk / 2 - 1) / (bk / 2) * (bk / 2)); };
-    const int kmode = chunked(RowCfg<S, EPI_SLICE>::BK), kdiv = chunked(RowCfg<S, EPI_DIVIDE>::BK);
-    const int kslab = chunked(RowCfg<S, EPI_SLAB>::BK);
+    // K entries written per row: whole 32-byte sectors, which the MMAs' last K step covers
+    const int kout = std::min(rad, (n + 7) / 8 * 8);
 
     const int rlo = std::max(0, p.row_lo);                       // upper-index rows to form
     const int rhi = p.row_hi < 0 ? nm : std::min(p.row_hi, nm);
     for (int i0 = rlo; i0 < rhi; i0 += ib) {
         const int cur = std::min(ib, rhi - i0);
-        auto operand = [&](const uint8_t* buf, int64_t R) { return DataOp{buf, 2 * rad, cur * R}; };
+        auto operand = [&](const uint8_t* buf, int64_t R) { return DataOp{buf, 2 * kout, 2 * rad, cur * R}; };
         auto plane = [&](int64_t R) { return cur * R * rad; };   // plane stride in complex entries
         {
             LaunchScope ls(&p.prof, "split_expand", p.stream);
-            k_expand_sorted<S><<<8192, 256, 0, p.stream>>>(rec, P, n, N, i0, cur, lg, kmode, p.d_cnt,
-                                                           so.atup[N - 1], so.natup[N - 1], R0,
-                                                           (uint32_t*)bufA, plane(R0));
+            auto kern = N == 1 ? k_regather<S, 0, 2> : N == 2 ? k_regather<S, 1, 2>
+                      : N == 3 ? k_regather<S, 2, 2> : k_regather<S, 3, 2>;
+            const int nrows = (int)so.natup[N - 1];
+            const unsigned grid = (unsigned)std::min<int64_t>((int64_t)cur * ((nrows + 7) / 8), 1 << 16);
+            kern<<<grid, 256, 0, p.stream>>>(Sv + (int64_t)i0 * Prows, Prows, n, nm, 1, nullptr, so.at_e[N],
+                                             so.psir_e + i0, sE + i0, lg, kout, nrows, R0, cur, so.atup[N - 1],
+                                             (uint32_t*)bufA, plane(R0), nullptr);
             NPF_CUDA(cudaGetLastError());
         }
         // ---- the first N - 2 mode products: V per sorted tuple, regathered into the next operand
@@ -2501,9 +2412,9 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
             const int64_t Rdst = pairs ? nrows : rad;
             LaunchScope ls(&p.prof, "split_regather", p.stream);
             const unsigned grid = (unsigned)std::min<int64_t>(outs * ((nrows + 7) / 8), 1 << 16);
-            auto kern = pairs ? k_regather<S, 2> : k_regather<S, 1>;
+            auto kern = pairs ? k_regather<S, 2, 0> : c == 1 ? k_regather<S, 1, 0> : k_regather<S, 1, 1>;
             kern<<<grid, 256, 0, p.stream>>>((const longlong2*)bufB, Ra, n, nm, (int)(outs / cur), base0.ttup,
-                                             c == 1 ? sE + i0 : E1, c == 2, so.phi_e, lg, kmode, nrows, Rdst,
+                                             c == 1 ? sE + i0 : E1, so.phi_e, nullptr, lg, kout, nrows, Rdst,
                                              outs, so.atup[2], (uint32_t*)bufA, outs * Rdst * rad,
                                              pairs ? E1 : E2);
             NPF_CUDA(cudaGetLastError());
@@ -2521,7 +2432,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
             a.RB = (int)((a.R + NP - 1) / NP);
             a.num_tiles = (int64_t)cur * a.RB * a.ncol_tiles;
             a.RS = RS;
-            a.kout = slab ? kslab : kdiv;
+            a.kout = kout;
             a.out_planes = (__nv_bfloat16*)bufB;
             a.out_plane_stride = 2 * plane(RS);
             a.out_exp = ES;
@@ -2581,7 +2492,8 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
         a.wpre = wpre;
         a.i0 = i0;
         a.out_f64 = d_out;
-        launch_rows<S, EPI_REDUCE>(p, "split_reduce", operand(bufA, Qc), tRed, 2 * nm, a);   // K = p_N < nm
+        const DataOp red{bufA, 2 * std::min(rad, (nm + 7) / 8 * 8), 2 * rad, cur * Qc};   // K = p_N < nm
+        launch_rows<S, EPI_REDUCE>(p, "split_reduce", red, tRed, 2 * nm, a);
     }
     if (p.err_override) return;   // the batch reads the shared flag after its graph has run
     int herr = 0;
