@@ -101,8 +101,10 @@ __device__ __forceinline__ uint32_t digit_bf16(int d, int s)
 // Balanced base-256 digits of W (|W| <= 2^(7 + 8(S-1))), packed as (Re, Im) BF16 pairs per
 // plane: plane s holds d_s * 2^(-8 s), d_0 the most significant digit. Adding 128 to every lower
 // digit (the constant OFF) turns them into plain bytes u = d + 128 in [0, 255] with no borrows,
-// and the top digit is the arithmetic shift of the sum. A byte becomes the float d * 2^(-8 s)
-// exactly through the bit pattern of 2^23 + u and one fused multiply-add.
+// and the top digit is the arithmetic shift of the sum. A byte's low seven bits are the mantissa of
+// the BF16 number (128 + (u & 127)) 2^(-8 s); subtracting 128 or 256 (u >= 128 or not) times 2^(-8 s)
+// leaves d 2^(-8 s) exactly, so a pair takes one byte permute, two logic operations and one packed
+// BF16 subtraction.
 template <int S>
 struct DigitOff {
     static constexpr long long value = (DigitOff<S - 1>::value << 8) | 128;
@@ -110,45 +112,28 @@ struct DigitOff {
 template <>
 struct DigitOff<0> { static constexpr long long value = 0; };
 
-__device__ __forceinline__ float byte_to_digit(uint32_t u, int s)
-{
-    // (2^23 + u) * 2^(-8s) - (2^23 + 128) * 2^(-8s) = (u - 128) * 2^(-8s), exact
-    const float sc = pow2f(-8 * s);
-    return fmaf(__uint_as_float(0x4B000000u | u), sc, -8388736.0f * sc);
-}
-
-// The float 2^23 + u for the byte u at position k (0..3) of x: one byte permute places the byte
-// under the exponent bits 0x4B (bytes 1 and 2 zero).
-__device__ __forceinline__ float byte_float(uint32_t x, int k)
-{
-    return __uint_as_float(__byte_perm(x, 0x4B000000u, 0x7440u | (uint32_t)k));
-}
-
 template <int S>
 __device__ __forceinline__ void digit_pairs(long long Wr, long long Wi, uint32_t (&out)[S])
 {
     constexpr long long OFF = DigitOff<S - 1>::value;   // 128 in each of the S-1 lower bytes
     const unsigned long long ur = (unsigned long long)(Wr + OFF);
     const unsigned long long ui = (unsigned long long)(Wi + OFF);
-    const uint32_t rlo = (uint32_t)ur, rhi = (uint32_t)(ur >> 32);
-    const uint32_t ilo = (uint32_t)ui, ihi = (uint32_t)(ui >> 32);
+    // top digits in [-128, 128]: exact in FP32, and their upper halves are the BF16 bits
+    const float fr = (float)(int)((long long)ur >> (8 * (S - 1)));
+    const float fi = (float)(int)((long long)ui >> (8 * (S - 1)));
+    out[0] = __byte_perm(__float_as_uint(fr), __float_as_uint(fi), 0x7632);
 #pragma unroll
-    for (int s = 0; s < S; ++s) {
+    for (int s = 1; s < S; ++s) {
         const int k = S - 1 - s;   // byte position from the least significant end
-        float fr, fi;
-        if (s == 0) {
-            const long long tr = (long long)(Wr + OFF) >> (8 * k);
-            const long long ti = (long long)(Wi + OFF) >> (8 * k);
-            fr = byte_to_digit((uint32_t)(tr + 128), 0);
-            fi = byte_to_digit((uint32_t)(ti + 128), 0);
-        } else {
-            // (2^23 + u) 2^(-8s) - (2^23 + 128) 2^(-8s) = (u - 128) 2^(-8s), exact
-            const float sc = pow2f(-8 * s);
-            fr = fmaf(k < 4 ? byte_float(rlo, k) : byte_float(rhi, k - 4), sc, -8388736.0f * sc);
-            fi = fmaf(k < 4 ? byte_float(ilo, k) : byte_float(ihi, k - 4), sc, -8388736.0f * sc);
-        }
-        // both are exact BF16 values: their upper halves are the BF16 bits (Re low, Im high)
-        out[s] = __byte_perm(__float_as_uint(fr), __float_as_uint(fi), 0x7632);
+        const uint32_t xr = (uint32_t)(k < 4 ? ur : ur >> 32), xi = (uint32_t)(k < 4 ? ui : ui >> 32);
+        // (Re byte, Im byte) in the low halves' low bytes (the other bytes are masked off)
+        const uint32_t p = __byte_perm(xr, xi, (unsigned)((k & 3) | ((k & 3) + 4) << 8));
+        const uint32_t one = 0x43004300u - 0x04000400u * (uint32_t)s;         // 128 * 2^(-8 s), twice
+        const uint32_t a = (p & 0x007F007Fu) | one;
+        const uint32_t c = (p & 0x00800080u) ^ (one + 0x00800080u);           // 256 or 128 times 2^(-8 s)
+        const __nv_bfloat162 d = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&a),
+                                         *reinterpret_cast<const __nv_bfloat162*>(&c));
+        out[s] = *reinterpret_cast<const uint32_t*>(&d);
     }
 }
 
@@ -1471,32 +1456,33 @@ static __global__ void k_term_init(double2* __restrict__ out, int64_t count, int
 //   SRC 2: V of the upper contraction (M = N - 1), outer = i; ea by rank (the tensor's), eb by i, and
 //          the rows share the exponent rowE[i]; the others get their exact one (largest bit length)
 // Neighbouring rows gather neighbouring entries (colexicographic rank), so the warps of a block
-// share sectors. Bound: HBM writes (4 S bytes an entry against 16 read per source entry).
+// share sectors. A block takes one outer index and a strided share of its rows, so that nothing
+// but the gather, the shifts and the digits is left per row: the kernel is bound by its
+// instructions (IPC 0.72 a scheduler) as much as by its HBM writes (4 S bytes an entry against 16 read
+// per source entry).
 template <int S, int M, int SRC>
 __global__ void __launch_bounds__(256)
     k_regather(const longlong2* __restrict__ V, int64_t Rsrc, int n, int nm, int nt, const uint32_t* __restrict__ ttup,
                const int* __restrict__ ea, const int* __restrict__ eb, const int* __restrict__ rowE, int lg, int kout,
-               int nrows, int64_t Rdst, int64_t nouter, const uint32_t* __restrict__ tuples,
+               int nrows, int64_t Rdst, unsigned parts, const uint32_t* __restrict__ tuples,
                uint32_t* __restrict__ planes, int64_t plane_stride_u32, int* __restrict__ out_exp)
 {
     const int lane = threadIdx.x & 31;
-    const int chunks = (nrows + 7) / 8;                      // 8 rows (one a warp) a step
-    const int64_t steps = nouter * chunks;
-    for (int64_t st = blockIdx.x; st < steps; st += gridDim.x) {
-        const int64_t outer = st / chunks;
-        const int row = (int)(st - outer * chunks) * 8 + (int)(threadIdx.x >> 5);
-        if (row >= nrows) continue;
-        int e0;
-        const int* earow = ea;
-        if (SRC == 2) {
-            e0 = eb[outer] - VEXP;
-        } else {
-            const int64_t i = outer / nt;
-            const int t = (int)(outer - i * nt);
-            const uint32_t tp = SRC == 1 ? ttup[t] : (uint32_t)t;   // the newest p in the low byte
-            e0 = eb[tp & 255u] - VEXP + (SRC == 0 ? ea[i] : 0);
-            if (SRC == 1) earow = ea + (i * nm + (int)((tp >> 8) & 255u)) * Rsrc;
-        }
+    const unsigned outer = blockIdx.x / parts;
+    int e0;
+    const int* earow = ea;
+    if (SRC == 2) {
+        e0 = eb[outer] - VEXP;
+    } else {
+        const unsigned i = outer / (unsigned)nt, t = outer - i * (unsigned)nt;
+        const uint32_t tp = SRC == 1 ? ttup[t] : t;          // the newest p in the low byte
+        e0 = eb[tp & 255u] - VEXP + (SRC == 0 ? ea[i] : 0);
+        if (SRC == 1) earow = ea + ((int64_t)i * nm + (int)((tp >> 8) & 255u)) * Rsrc;
+    }
+    const longlong2* src = V + outer * Rsrc;
+    const int Eall = SRC == 2 ? rowE[outer] : 0;
+    for (int row = (int)(blockIdx.x - outer * parts) * 8 + (int)(threadIdx.x >> 5); row < nrows;
+         row += (int)parts * 8) {
         int x = row, y = 0, z = 0;
         if (M >= 2) {
             const uint32_t pk = tuples[row];
@@ -1504,11 +1490,11 @@ __global__ void __launch_bounds__(256)
             y = (int)((pk >> 8) & 255u);
             z = (int)((pk >> 16) & 255u);
         }
-        const longlong2* src = V + outer * Rsrc;
         longlong2 v[4];
         int ex[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
+            if (32 * k >= n) break;
             const int a = lane + 32 * k;
             v[k] = make_longlong2(0ll, 0ll);
             ex[k] = 0;
@@ -1528,14 +1514,24 @@ __global__ void __launch_bounds__(256)
                 if (SRC != 0) ex[k] = earow[rk];
             }
         }
-        int E;
-        if (SRC == 2) {
-            E = rowE[outer];
-        } else {
+        int E = Eall;
+        if (SRC == 0) {
+            // one unit for all entries: the bit length of the OR of their magnitudes (the lowest bit
+            // as it is, so that a minus one counts)
+            unsigned long long m = 0ull;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (32 * k < n)
+                    m |= (unsigned long long)((v[k].x ^ (v[k].x >> 63)) | (v[k].y ^ (v[k].y >> 63)) |
+                                              ((v[k].x | v[k].y) & 1));
+            const unsigned hi = __reduce_or_sync(0xffffffffu, (unsigned)(m >> 32));
+            const unsigned lo = __reduce_or_sync(0xffffffffu, (unsigned)m);
+            E = hi | lo ? (hi ? 64 - __clz((int)hi) : 32 - __clz((int)lo)) + e0 : EXP_NONE;
+        } else if (SRC == 1) {
             int key = 0;
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                if (v[k].x | v[k].y) key = max(key, bitlen(v[k]) + ex[k] + e0 + 8192);
+                if (32 * k < n && (v[k].x | v[k].y)) key = max(key, bitlen(v[k]) + ex[k] + e0 + 8192);
             key = (int)__reduce_max_sync(0xffffffffu, (unsigned)key);
             E = key ? key - 8192 : EXP_NONE;
         }
@@ -1544,9 +1540,10 @@ __global__ void __launch_bounds__(256)
         uint32_t* dst = planes + (rowp << lg) + lane;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
+            if (32 * k >= kout) break;
             if (lane + 32 * k < kout) {
                 uint32_t w[S];
-                if (E != EXP_NONE) {
+                if (E != EXP_NONE && 32 * k < n) {
                     digit_pairs<S>(shift_full(v[k].x, sh + ex[k]), shift_full(v[k].y, sh + ex[k]), w);
                 } else {
 #pragma unroll
@@ -2252,6 +2249,14 @@ static void launch_rows(Plan& p, const char* name, const DataOp& A, const FixedO
 
 static double factorial(int N) { double f = 1; for (int t = 2; t <= N; ++t) f *= t; return f; }
 
+// Blocks that share one outer index of a regather: about eight rows a warp, more blocks when few.
+static unsigned regather_parts(int64_t outers, int nrows)
+{
+    const int64_t all = (nrows + 7) / 8;                         // one row a warp
+    const int64_t want = std::max<int64_t>((all + 7) / 8, (8 * sm_count() + outers - 1) / std::max<int64_t>(outers, 1));
+    return (unsigned)std::max<int64_t>(1, std::min(all, want));
+}
+
 // Device memory of one order: V of S (16 bytes, n x P) and per upper index of a batch two buffers that the stages alternate (A: the operands of the mode products and of the
 // reduction, B: V and the divide's slots) plus the row exponents.
 template <int S>
@@ -2387,10 +2392,10 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
             auto kern = N == 1 ? k_regather<S, 0, 2> : N == 2 ? k_regather<S, 1, 2>
                       : N == 3 ? k_regather<S, 2, 2> : k_regather<S, 3, 2>;
             const int nrows = (int)so.natup[N - 1];
-            const unsigned grid = (unsigned)std::min<int64_t>((int64_t)cur * ((nrows + 7) / 8), 1 << 16);
-            kern<<<grid, 256, 0, p.stream>>>(Sv + (int64_t)i0 * Prows, Prows, n, nm, 1, nullptr, so.at_e[N],
-                                             so.psir_e + i0, sE + i0, lg, kout, nrows, R0, cur, so.atup[N - 1],
-                                             (uint32_t*)bufA, plane(R0), nullptr);
+            const unsigned parts = regather_parts(cur, nrows);
+            kern<<<(unsigned)cur * parts, 256, 0, p.stream>>>(
+                Sv + (int64_t)i0 * Prows, Prows, n, nm, 1, nullptr, so.at_e[N], so.psir_e + i0, sE + i0, lg, kout,
+                nrows, R0, parts, so.atup[N - 1], (uint32_t*)bufA, plane(R0), nullptr);
             NPF_CUDA(cudaGetLastError());
         }
         // ---- the first N - 2 mode products: V per sorted tuple, regathered into the next operand
@@ -2411,12 +2416,12 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
             const int nrows = pairs ? (int)so.natup[2] : n;
             const int64_t Rdst = pairs ? nrows : rad;
             LaunchScope ls(&p.prof, "split_regather", p.stream);
-            const unsigned grid = (unsigned)std::min<int64_t>(outs * ((nrows + 7) / 8), 1 << 16);
+            const unsigned parts = regather_parts(outs, nrows);
             auto kern = pairs ? k_regather<S, 2, 0> : c == 1 ? k_regather<S, 1, 0> : k_regather<S, 1, 1>;
-            kern<<<grid, 256, 0, p.stream>>>((const longlong2*)bufB, Ra, n, nm, (int)(outs / cur), base0.ttup,
-                                             c == 1 ? sE + i0 : E1, so.phi_e, nullptr, lg, kout, nrows, Rdst,
-                                             outs, so.atup[2], (uint32_t*)bufA, outs * Rdst * rad,
-                                             pairs ? E1 : E2);
+            kern<<<(unsigned)outs * parts, 256, 0, p.stream>>>(
+                (const longlong2*)bufB, Ra, n, nm, (int)(outs / cur), base0.ttup, c == 1 ? sE + i0 : E1, so.phi_e,
+                nullptr, lg, kout, nrows, Rdst, parts, so.atup[2], (uint32_t*)bufA, outs * Rdst * rad,
+                pairs ? E1 : E2);
             NPF_CUDA(cudaGetLastError());
         }
         // ---- the last mode product (its output rows are the divide's slots)
