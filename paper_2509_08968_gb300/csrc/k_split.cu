@@ -59,7 +59,7 @@ constexpr int TMEM_COLS = 512;
 constexpr int kErrTimeout = 1;
 constexpr int VEXP = 44;       // value = V * 2^(e_a + e_b - VEXP), V in units of 2^-30 of L0
 constexpr int EPI_WARPS = 16;  // epilogue warps (four per TMEM lane quarter)
-constexpr int ROW_THREADS = 64 + 32 * EPI_WARPS;
+constexpr int ROW_THREADS = 64 + 32 * EPI_WARPS + 64;   // producer, MMA, epilogue, two set-up warps
 
 // ---------------------------------------------------------------------------------------
 // Integer / double-float helpers
@@ -220,25 +220,6 @@ __device__ __forceinline__ long long df_round_i64(dfl x)
     return ((long long)t << 24) + __float2int_rn(rem + x.lo);
 }
 
-// One row of the divide's operand (a slot): a sorted tuple (p_2 <= .. <= p_N). The table holds the
-// slots of one upper index (it does not depend on the index) and is refreshed with the modes.
-struct SlotRow {
-    double2 sigma;        // lambda_{p_2} + .. + lambda_{p_N}
-    tfl sr, si;           // sigma as exact triple-floats
-    dfl f_row, f_first;   // 1 / prod(run lengths)! of the tuple (f_first: the first run one longer)
-    float fmb;            // f_row in FP32 (exponent estimates)
-    int den, run1;        // prod(run lengths)!, length of the first run
-    int firstp;           // p_2, or -1 for a padding slot
-    int rbase;            // reduction row of (p_1, .., p_{N-1}) = rbase + p_1
-    int kpos;             // p_N, the K position in that row
-    int seg;              // segment within the 128-row tile; bit 8: the segment's first row
-    int pad;
-};
-// What the quotient reads per element, copied to shared memory (one per tile row).
-struct RowInfo {
-    tfl sr, si;
-    dfl f_row, f_first;
-};
 constexpr int SEGS = 8;   // segments a 128-row divide tile may hold
 
 // 1 / d for a small positive integer d as a double-float (relative error ~2^-46), without FP64.
@@ -294,26 +275,19 @@ __device__ __forceinline__ int f32_exponent(float x) { return ((__float_as_int(x
 template <int S>
 struct Lev { static constexpr int N = S < 4 ? S : 4; };
 
-// Load 4 columns of every used level of one accumulator group (levels `stride` columns apart);
-// with the level-3 hold (HOLD), level 3 comes from shared memory (`held`) instead of TMEM.
-template <int S, bool HOLD>
-__device__ __forceinline__ void load_levels(uint32_t taddr, int stride, uint32_t (&v)[4][4],
-                                            const float4* held)
+// Load UC (2 or 4) columns of every used level of one accumulator group (levels `stride` columns apart).
+template <int S, int UC>
+__device__ __forceinline__ void load_levels(uint32_t taddr, int stride, uint32_t (&v)[4][UC])
 {
 #pragma unroll
     for (int L = 0; L < 4; ++L) {
-        if (L < Lev<S>::N && !(HOLD && L == 3)) tc::tmem_ld4(taddr + L * stride, v[L]);
-        else if (!(HOLD && L == 3)) {
+        if (L < Lev<S>::N) {
+            if constexpr (UC == 4) tc::tmem_ld4(taddr + L * stride, v[L]);
+            else tc::tmem_ld2(taddr + L * stride, v[L]);
+        } else {
 #pragma unroll
-            for (int c = 0; c < 4; ++c) v[L][c] = 0u;
+            for (int c = 0; c < UC; ++c) v[L][c] = 0u;
         }
-    }
-    if (HOLD) {
-        const float4 h = *held;
-        v[3][0] = __float_as_uint(h.x);
-        v[3][1] = __float_as_uint(h.y);
-        v[3][2] = __float_as_uint(h.z);
-        v[3][3] = __float_as_uint(h.w);
     }
 }
 
@@ -412,12 +386,6 @@ __global__ void k_prep_at(const double* __restrict__ A, int64_t P, int n, int N,
 // ---------------------------------------------------------------------------------------
 enum { EPI_V = 0, EPI_SLICE = 1, EPI_DIVIDE = 2, EPI_SLAB = 3, EPI_REDUCE = 4 };
 
-// Tensor maps of one operand: every slice plane in one box (`all`), and the planes of levels
-// 0..2 only (`low`, the second pass of a tile with the level-3 hold).
-struct TMaps {
-    CUtensorMap all, low;
-};
-
 struct RowArgs {
     int kch;             // pipeline stages of K' (16 or 32 wide; K' past the operands' length is
                          // zero on both sides)
@@ -426,7 +394,7 @@ struct RowArgs {
     const int* ea;       // row exponents, by operand row or (ea_outer) by outer index
     int ea_outer;
     const int* eb;       // column exponents of the fixed matrix (256 entries)
-    int bnc;             // complex columns per tile (16, 32, 48 or 64)
+    int bnc;             // complex columns per tile (16 or 32)
     int ncol_tiles;
     int64_t num_tiles;
     int N;               // order
@@ -448,14 +416,21 @@ struct RowArgs {
     int64_t RS;
     const int* segbase;      // first slot of the segment (p_2, .., p_{N-1}), by its colex rank
     // EPI_DIVIDE, EPI_SLAB: the slots; EPI_DIVIDE writes reduction rows, RT per upper index
-    const SlotRow* srow;
+    // (smeta: {p_2 or -1 for a padding slot; reduction row less p_1; kpos | segment << 8 | the
+    // segment's first row << 12 | first run's length << 13 | prod(run lengths)! << 16}, kpos = p_N
+    // the K position in that row; ssum, ssig: lambda_{p_2} + .. + lambda_{p_N} as exact triple-floats
+    // [6][nslot] and in FP64)
+    const int4* smeta;
+    const float* ssum;
+    const double2* ssig;
+    int nslot;
     const uint32_t* stup;    // the slots' tuples, 8 bits per index (all ones: padding)
     const int* tpmax;        // largest p_2 of each tile's slots
     int64_t RT;
     // EPI_REDUCE: rows are the sorted tuples (p_1 <= .. <= p_{N-1}) in colexicographic rank
     const uint32_t* tuples;  // 8 bits per index
-    const float4* wpre;      // prod_{m <= N-2} W[p_m][k] per sorted (N-2)-tuple (colex rank) and k,
-                             // as double-float complex
+    const float4* wpre;      // W[p_1][k] W[p_2][k] at k * ldw + the pair's colex rank (orders 3 and 4), as
+    int64_t ldw;             // double-float complex: the 32 rows of a warp read one run
     const int* tiles;        // the tiles that run (nullptr: every tile, skipped ones tested)
     const unsigned* ntiles_run;   // their count
     int kout;            // K entries written per row of the next operand (whole chunks of it)
@@ -471,7 +446,7 @@ struct RowArgs {
     double2* out_f64;    // EPI_SLAB: out[i * n + q]; EPI_REDUCE: Psi_N
     // EPI_DIVIDE / EPI_SLAB / EPI_REDUCE
     const double2* lam;
-    const float4* psi_df;    // the reduction weights W[p][k] (psi_{p k}) as double-float, at p*n + k
+    const float4* psi_df;    // the reduction weights W[p][k] (psi_{p k}) as double-float, at k*n + p
     int i0;
     double invfact, eps;
     int divide;
@@ -491,51 +466,47 @@ __device__ __forceinline__ unsigned long long global_ns()
     return t;
 }
 
-// Pipeline of one k_rows variant. With four levels, the divide and reduction tiles run in two
-// passes with the level-3 hold (their epilogues outlast their MMAs, so the overlap pays): stages of
-// one 16-wide K' step (32-byte swizzle) to make room for the 64 KB hold. The other modes run one
-// pass over stages of two K' steps (64-byte swizzle): their MMA phase already moves operands as
-// fast as TMA refills shared memory, and a second pass would re-read planes 0..2.
-template <int S, int MODE>
-struct Pipe {
-    static constexpr bool two = Lev<S>::N == 4 && (MODE == EPI_DIVIDE || MODE == EPI_REDUCE);
-    // K' elements per stage: 16 (32-byte rows) where the 64 KB hold leaves three 48 KB stages,
-    // 32 (64-byte rows) otherwise
-    static constexpr int BK = two ? 16 : 32;
-    static constexpr int KS = BK / KSTEP;        // MMA K steps per stage
-    // K steps per stage of the second pass, which reads planes 0..2 only: as many as the
-    // stage's S plane slots hold, so the ring keeps as many bytes in flight as in the first pass
-    static constexpr int P2 = two ? S / 3 : 1;
-};
-
+// Pipeline of one k_rows variant: every launch runs one pass over K through a ring of stages. The
+// divide and the reduction, whose tables need room, take five stages of one 16-wide K' step (32-byte
+// rows and swizzle), the others three stages of two steps (64-byte rows).
 template <int S, int MODE>
 struct RowCfg {
-    static constexpr int BK = Pipe<S, MODE>::BK;
+    static constexpr bool big_tables = MODE == EPI_DIVIDE || MODE == EPI_REDUCE;
+    static constexpr int BK = big_tables ? 16 : 32;            // K' elements per stage
+    static constexpr int KS = BK / KSTEP;                      // MMA K steps per stage
     static constexpr int A_TILE = NP * BK * 2;                 // 4 or 8 KB
-    // fixed-matrix rows of a stage: up to 128 in the two-pass modes, 64 in the one-pass modes, whose
-    // tiles are at most 32 complex columns wide (three 72 KB stages at six slices instead of two of
-    // 96 KB: the mode products wait for staging, not for the tensor core; n = 120, orders 3 + 4:
-    // 659 -> 614 ms a call)
-    static constexpr int BROWS = Pipe<S, MODE>::two ? NP : 64;
-    static constexpr int B_TILE = BROWS * BK * 2;
+    static constexpr int B_TILE = 64 * BK * 2;                 // at most 32 complex columns
     static constexpr int STAGE_BYTES = S * (A_TILE + B_TILE);
-    // level-3 hold: [4 column groups][HSLOT float4 slots][128 rows]; a thread holds the Re and Im
-    // level-3 values of its column units (up to 4 at 64 columns)
-    static constexpr int HSLOT = 8;
-    static constexpr int HOLD_BYTES = Pipe<S, MODE>::two ? 4 * HSLOT * NP * 16 : 0;
-    // barriers, column tables, reduction partials and row tables, and 1 KB of alignment slack
-    // (the other epilogues use only the barriers, the column tables and the output rows)
-    static constexpr int TABLES = MODE == EPI_DIVIDE || MODE == EPI_REDUCE ? 14 * 1024 : 4 * 1024;
-    static_assert(2 * 8 * 8 + 5 * 8 + 8 <= 256, "barriers fit the first 256 bytes of the tables");
+    // tables (offsets from a 1 KB boundary after the stages): barriers and the TMEM slot in the
+    // first 256 bytes, column exponent keys by tile parity ([4 sub-blocks][32], the divide's
+    // [SEGS][32]), reciprocals of small integers, then the tile tables
+    // (two buffers, filled by the set-up warps)
+    static constexpr int COLE = 256, COLE_N = MODE == EPI_DIVIDE ? SEGS * 32 : 128;
+    static constexpr int RCP = 256 + 2048;
+    static constexpr int TILE = RCP + 256;
+    // one tile's tables
+    static constexpr int META = 0;       // int[8]
+    static constexpr int QINFO = 32;     // int4[4 lane quarters]
+    static constexpr int COLEB = 96;     // int[32] fixed-matrix column exponents
+    static constexpr int ROWM = 256;     // int4[128 rows]
+    static constexpr int SROWQ = ROWM + 2048;        // EPI_SLICE: int[4 sub-blocks][32] output slots
+    static constexpr int LAMF = ROWM + 2048;         // EPI_DIVIDE: float2[32] lambda_q - lambda_i
+    static constexpr int LAMT = LAMF + 256;          //   the same as exact triple-floats, tfl[32][2]
+    static constexpr int SIG = LAMT + 64 * 12;       //   float[6][128] the rows' sigma as triple-floats
+    static constexpr int TILE_BYTES = MODE == EPI_DIVIDE ? SIG + 6 * NP * 4 : MODE == EPI_SLICE ? SROWQ + 512 : SROWQ;
+    static constexpr int TABLES = TILE + 2 * TILE_BYTES + 1024;   // and 1 KB of alignment slack
     static constexpr int SMEM_MAX = 227 * 1024;
-    static constexpr int STAGES_FIT = (SMEM_MAX - TABLES - HOLD_BYTES) / STAGE_BYTES;
+    static constexpr int STAGES_FIT = (SMEM_MAX - TABLES) / STAGE_BYTES;
     static constexpr int STAGES = STAGES_FIT < 8 ? STAGES_FIT : 8;
-    static constexpr int SMEM = STAGES * STAGE_BYTES + HOLD_BYTES + TABLES;
+    static constexpr int SMEM = STAGES * STAGE_BYTES + TABLES;
+    static_assert((2 * 8 + 8) * 8 + 8 <= 256, "barriers fit the first 256 bytes of the tables");
+    static_assert(2 * COLE_N * 4 <= 2048, "keys");
+    static_assert(COLEB + 128 <= ROWM, "tile tables");
     static_assert(STAGES >= 3, "pipeline stages");
     static_assert(SMEM <= SMEM_MAX, "shared memory");
 };
 
-// Position of a tile (tiles are ordered row block major).
+// Position of a tile (column tile fastest, but for the reduction).
 struct TilePos {
     int ct;         // column tile
     int outer;      // upper index of the launch (RB > 0)
@@ -547,6 +518,14 @@ __device__ __forceinline__ TilePos tile_pos(const RowArgs& a, int64_t tile)
     const unsigned t = (unsigned)tile;   // (launch_rows bounds the tile count to 2^31)
     const unsigned rb = a.lgncol >= 0 ? t >> a.lgncol : t / (unsigned)a.ncol_tiles;
     TilePos p;
+    if (a.kfrom) {   // the reduction: row block fastest, then column tile, then upper index
+        const unsigned g = t / (unsigned)a.RB;
+        p.outer = (int)(g / (unsigned)a.ncol_tiles);
+        p.ct = (int)(g - (unsigned)p.outer * (unsigned)a.ncol_tiles);
+        p.rr0 = (int)(t - g * (unsigned)a.RB) * NP;
+        p.row0 = (int64_t)p.outer * a.R + p.rr0;
+        return p;
+    }
     p.ct = (int)(t - rb * (unsigned)a.ncol_tiles);
     if (a.RB > 0) {
         p.outer = (int)(rb / (unsigned)a.RB);
@@ -574,7 +553,6 @@ __device__ __forceinline__ int tile_pmax(const RowArgs& a, int lg, const TilePos
 // lg: the row radix (a compile-time 7 in the kernels without sub-blocks)
 __device__ __forceinline__ bool tile_skipped(const RowArgs& a, int lg, const TilePos& p)
 {
-    if (p.ct * a.bnc >= a.ncv) return true;                // every column is padding
     if (a.tpmax) return p.ct * a.bnc > a.tpmax[p.rr0 / NP];   // slots: columns p_1 <= p_2
     return a.colmask && p.ct * a.bnc > tile_pmax(a, lg, p);
 }
@@ -598,90 +576,61 @@ __device__ __forceinline__ void mbar_drain(uint64_t* bar, uint32_t parity)
     }
 }
 
-// Whether the slice pair (s, u) belongs to a pass (PASS 0: every pair; 1: level 3; 2: levels 0..2).
-__host__ __device__ constexpr bool pair_in_pass(int pass, int s, int u)
-{
-    return pass == 0 || (pass == 1) == (s + u >= 3);
-}
-
-template <bool ACC>
-__device__ __forceinline__ void mma_col(int col, uint32_t leader, uint32_t d, uint32_t a, uint32_t b,
+__device__ __forceinline__ void mma_col(int col, uint32_t acc, uint32_t leader, uint32_t d, uint32_t a, uint32_t b,
                                         uint32_t hi, uint32_t idesc)
 {
-    if (col == 1) tc::mma_bf16_lohi<ACC, 1>(leader, d, a, b, hi, idesc);
-    else if (col == 2) tc::mma_bf16_lohi<ACC, 2>(leader, d, a, b, hi, idesc);
-    else if (col == 3) tc::mma_bf16_lohi<ACC, 3>(leader, d, a, b, hi, idesc);
-    else tc::mma_bf16_lohi<ACC, 0>(leader, d, a, b, hi, idesc);
+    if (col == 1) tc::mma_bf16_lohi<1>(acc, leader, d, a, b, hi, idesc);
+    else if (col == 2) tc::mma_bf16_lohi<2>(acc, leader, d, a, b, hi, idesc);
+    else if (col == 3) tc::mma_bf16_lohi<3>(acc, leader, d, a, b, hi, idesc);
+    else tc::mma_bf16_lohi<0>(acc, leader, d, a, b, hi, idesc);
 }
 
-// One K' step of MMAs: the slice pairs (s, u), s + u < S, of one pass into their level
-// accumulators. PASS 0: every pair (no hold); PASS 1: the level-3 pairs (s + u >= 3); PASS 2: the
-// pairs of levels 0..2. FIRST: the step opens the pass, so each level's first MMA overwrites
+// One K step of MMAs: the slice pairs (s, u), s + u < S, into their level accumulators (level L at TMEM
+// column tmem + L * lstride). acc = 0: the step opens the tile, so each level's first MMA overwrites
 // instead of accumulating. The loops unroll into straight-line MMAs with constant descriptor
-// offsets (start address / 16 in the low half).
-// Level L accumulates at TMEM column tmem + L * lstride.
-// NKS: MMA K steps issued from the stage (32-byte K offsets within a 64-byte swizzled row; 1 when
-// the stage's second half is padding). The descriptor's swizzle matches the stage width.
-// The MMAs that share a data plane s and K step run back to back over the fixed-matrix planes u,
-// with the data tile held in the tensor core's collector buffer: shared memory delivers each
-// data tile once per (s, K step) instead of once per pair (M = N = 128 MMAs otherwise read 8 KB
-// of operands per 64 cycles, which the measured MMA rate showed to be the limit).
-template <int S, int MODE, int PASS, bool FIRST, int NKS>
-__device__ __forceinline__ void issue_kstep(uint32_t leader, uint32_t tmem, uint32_t lstride,
+// offsets (start address / 16 in the low half); one copy of them serves every step, since all roles
+// of the kernel share the instruction cache.
+// The MMAs that share a data plane s run back to back over the fixed-matrix planes u, with the data
+// tile held in the tensor core's collector buffer: 36 cycles an MMA at N = 64 (48 without, where
+// shared memory delivers the 4 KB data tile every time).
+template <int S, int MODE>
+__device__ __forceinline__ void issue_kstep(uint32_t acc, uint32_t leader, uint32_t tmem, uint32_t lstride,
                                             uint32_t a_lo, uint32_t b_lo, uint32_t b_plane16,
                                             uint32_t idesc)
 {
     using C = RowCfg<S, MODE>;
     constexpr uint32_t hi = C::BK == 32 ? tc::kSdescSw64Hi : tc::kSdescSw32Hi;
-    bool first[4] = {FIRST, FIRST, FIRST, FIRST};
+    bool first[4] = {true, true, true, true};
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-        int nu = 0;   // pairs of this pass on data plane s
+        const uint32_t ao = a_lo + (uint32_t)((s * C::A_TILE) >> 4);
 #pragma unroll
-        for (int u = 0; u < S - s; ++u) nu += pair_in_pass(PASS, s, u) ? 1 : 0;
-#pragma unroll
-        for (int ks = 0; ks < NKS; ++ks) {
-            const uint32_t ao = a_lo + (uint32_t)((s * C::A_TILE + ks * 32) >> 4);
-            int j = 0;
-#pragma unroll
-            for (int u = 0; u < S - s; ++u) {
-                if (!pair_in_pass(PASS, s, u)) continue;
-                const int L = s + u < 3 ? s + u : 3;
-                const uint32_t bo = b_lo + (uint32_t)u * b_plane16 + (uint32_t)(ks * 2);
-                // collector: fill on the first MMA of the run, release on the last
-                const int col = nu == 1 ? 0 : j == 0 ? 1 : j == nu - 1 ? 3 : 2;
-                if (first[L]) mma_col<false>(col, leader, tmem + L * lstride, ao, bo, hi, idesc);
-                else mma_col<true>(col, leader, tmem + L * lstride, ao, bo, hi, idesc);
-                first[L] = false;
-                ++j;
-            }
+        for (int u = 0; u < S - s; ++u) {
+            const int L = s + u < 3 ? s + u : 3;
+            // collector: fill on the first MMA of the run, release on the last
+            const int col = S - s == 1 ? 0 : u == 0 ? 1 : u == S - s - 1 ? 3 : 2;
+            mma_col(col, first[L] ? acc : 1u, leader, tmem + L * lstride, ao, b_lo + (uint32_t)u * b_plane16, hi, idesc);
+            first[L] = false;
         }
     }
 }
 
-// Planes a pass reads (level 3 needs every plane; levels 0..2 only planes 0..2).
-template <int S>
-__host__ __device__ constexpr int pass_planes(int pass) { return pass == 2 ? (S < 3 ? S : 3) : S; }
-
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, %0;" ::"r"(32 * EPI_WARPS) : "memory"); }
+// epi_sync that also tells whether any epilogue thread brought `f`.
+__device__ __forceinline__ bool epi_any(bool f)
+{
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %1, 0;\n\t"
+        "bar.red.or.pred q, 1, %2, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"(f ? 1 : 0), "r"(32 * EPI_WARPS)
+        : "memory");
+    return r != 0;
+}
 
-// Persistent row GEMM: one CTA per SM walks the tiles blockIdx.x, +gridDim.x, ... Roles:
-//   warp 0 (one lane): TMA producer over a ring of STAGES shared-memory stages (16 or 32 K'
-//                      each) that runs across tiles, so the next tile's operands stream in during
-//                      this tile's epilogue;
-//   warp 1           : MMA issuer (the warp runs the loop, one elected lane issues). The four
-//                      level accumulators of a 128 x bnc-complex tile take 8 bnc TMEM columns.
-//                      One-pass modes at bnc <= 32 alternate two accumulator sets, so the next
-//                      tile's MMAs run during this tile's epilogue; at bnc = 64 they fill TMEM and
-//                      wait for it. The divide and the reduction (four levels) run two passes
-//                      over K: first the 15 level-3 slice pairs (S = 6), then the 6 pairs of
-//                      levels 0..2. The epilogue copies level 3 to a shared-memory hold as soon as
-//                      the tile is complete, so the next tile's level-3 pass (most of its MMAs)
-//                      overlaps the rest of this tile's epilogue; only the levels-0..2 pass waits
-//                      for it;
-//   warps 2..17      : epilogue (lane quarter = warp % 4, column group = (warp - 2) / 4). Values
-//                      needed twice (a column exponent before slicing) are read from TMEM twice
-//                      instead of being staged in shared memory.
 // The tiles of a launch that run (tile_skipped false), compacted: each block scans 256
 // consecutive tiles and appends the running ones in order at a position taken with one atomic.
 // The persistent kernel then walks this list: a skipped tile cost each of its roles a decode
@@ -708,54 +657,61 @@ static __global__ void k_tile_list(RowArgs a, int lg, int* __restrict__ list, un
     if (run) list[base + wsum[warp] + __popc(bal & ((1u << lane) - 1u))] = (int)tile;
 }
 
-static_assert(sizeof(tfl) == 12 && 6144 + 128 * sizeof(tfl) <= 7680, "table layout");
-static_assert(7680 + 128 * sizeof(RowInfo) + 1024 <= 14 * 1024, "tables and alignment slack");
-static_assert(1536 + 4 * 64 * 4 + 1024 <= 4 * 1024, "re-slicing tables and alignment slack");
-static_assert(1536 + SEGS * 64 * 4 <= 5632, "the divide's segment exponents lie in the partials' place");
-
+// Persistent row GEMM: one CTA per SM walks the tiles blockIdx.x, +gridDim.x, ... Roles:
+//   warp 0 (one lane): TMA producer over a ring of STAGES shared-memory stages that runs across
+//                      tiles, so the next tile's operands stream in during this tile's epilogue;
+//   warp 1           : MMA issuer (the warp runs the loop, one elected lane issues). The four
+//                      level accumulators of a 128 x bnc-complex tile take 8 bnc <= 256 TMEM columns;
+//                      tiles alternate two sets, so the next tile's MMAs run during this tile's
+//                      epilogue;
+//   warps 2..17      : epilogue (lane quarter = warp % 4, column group = (warp - 2) / 4). Values
+//                      needed twice (a column exponent before slicing) are read from TMEM twice
+//                      instead of being staged in shared memory;
+//   warps 18, 19     : set-up: the next tile's tables (row exponents and indices, eigenvalue sums,
+//                      output rows) into the other of two buffers. Chains of dependent global loads,
+//                      they took 2 to 7 us a tile in front of the epilogue.
+// Bound per 32-column tile of a mode product at n = 120: shared memory (MMA operand reads 1.08 MB and TMA
+// writes 0.59 MB at 128 bytes a clock: 6.3 us; MMAs 5.4 us) of 7.1 us measured; below n = 64 and in
+// the divide and the reduction the epilogue. 32-column tiles in every mode: an epilogue and the next
+// tile's MMAs overlap, which one 64-column tile with all 512 TMEM columns (and a level-3 hold in
+// shared memory) allowed in part only: divide at n = 120, order 3, 1.83 -> 1.45 ms a call (24 us a
+// 64-column tile before, 13 us a 32-column one now, of which the kept columns are fewer).
 template <int S, int MODE, bool SUBB>
 __global__ void __launch_bounds__(ROW_THREADS, 1)
-    k_rows(const __grid_constant__ TMaps tmA, const __grid_constant__ TMaps tmB, RowArgs args)
+    k_rows(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, RowArgs args)
 {
     using C = RowCfg<S, MODE>;
-    constexpr bool TWO = Pipe<S, MODE>::two;
     constexpr int BKm = C::BK;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t* stage_base = smem;
-    float4* hold = (float4*)(smem + C::STAGES * C::STAGE_BYTES);   // level-3 hold (S >= 4)
-    // tables at fixed offsets from a 1 KB boundary: barriers and the TMEM slot in the first
-    // 256 bytes (at most 2 x 8 + 5 barriers), then each table 16-byte aligned
-    uint8_t* tables = smem + C::STAGES * C::STAGE_BYTES + C::HOLD_BYTES;
+    uint8_t* tables = smem + C::STAGES * C::STAGE_BYTES;
     uint64_t* full = (uint64_t*)tables;
     uint64_t* empty = full + C::STAGES;
     uint64_t* tfull = empty + C::STAGES;       // [2] MMA -> epilogue: accumulators complete
-    uint64_t* tempty = tfull + 2;              // [2] epilogue -> MMA: levels 0..2 (all, no hold) read
-    uint64_t* t3empty = tempty + 2;            // epilogue -> MMA: level 3 copied to the hold
-    uint32_t* tmem_slot = (uint32_t*)(t3empty + 1);
-    int* stop = (int*)(tmem_slot + 1);
-    // column exponent keys: [4 sub-blocks][64], or the divide's [SEGS][64] in the partials' place
-    int* colE = (int*)(tables + (MODE == EPI_DIVIDE ? 1536 : 256));
-    int* colEb = (int*)(tables + 1280);        // 64 fixed-matrix column exponents
-    int* srowq = (int*)(tables + 1536);        // EPI_SLICE, last: [4 sub-blocks][64] output slots
-    float4* red = (float4*)(tables + 1536);    // [4 lane quarters][64 columns] reduction partials
-    int* qpin = (int*)(tables + 5632);         // EPI_REDUCE: p_{N-1} of each lane quarter's rows, or -1
-    float2* lamf = (float2*)(tables + 5632);   // 64 lambda_q in FP32 (exponent estimates)
-    tfl* lamt = (tfl*)(tables + 6144);         // 64 x (Re, Im) lambda_q as exact triple-floats
-    RowInfo* rowinfo = (RowInfo*)(tables + 7680);   // [128]
+    uint64_t* tempty = tfull + 2;              // [2] epilogue -> MMA: accumulators read
+    uint64_t* sfull = tempty + 2;              // [2] set-up -> epilogue: tables filled
+    uint64_t* sempty = sfull + 2;              // [2] epilogue -> set-up: tables read
+    uint32_t* tmem_slot = (uint32_t*)(sempty + 2);
+    int* colE_all = (int*)(tables + C::COLE);
+    dfl* rcp = (dfl*)(tables + C::RCP);        // 1 / d, 1 <= d <= 24
 
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int bnc = args.bnc;
     const int bnr = 2 * bnc;
     const uint32_t b_bytes_tile = (uint32_t)bnr * BKm * 2;
-    const int64_t ntiles = args.num_tiles;
     // tiles walked by every role: the running-tile list when there is one
-    const int64_t nloop = args.tiles ? (int64_t)*(volatile const unsigned*)args.ntiles_run : ntiles;
-    // TMEM accumulator sets: two when one tile's levels fit in half of TMEM (single-pass modes,
-    // 2 * bnc <= 64 real columns a level), so that the MMAs of the next tile run during this
-    // tile's epilogue; tile t uses set t % nset, its levels lstride columns apart
-    const int nset = (!TWO && Lev<S>::N * bnr <= TMEM_COLS / 2) ? 2 : 1;
-    const uint32_t lstride = nset == 2 ? (uint32_t)bnr : 128u;
+    const int64_t nloop = args.tiles ? (int64_t)*(volatile const unsigned*)args.ntiles_run : args.num_tiles;
+    auto tile_at = [&](int64_t k) -> int64_t {
+        return k >= nloop ? 0 : args.tiles ? (int64_t)args.tiles[k] : k;
+    };
+    // The reduction takes consecutive tiles (row blocks of one upper index and column tile), so that its
+    // epilogue can sum over them in registers; the others take every gridDim.x-th.
+    const int64_t per = (nloop + gridDim.x - 1) / gridDim.x;
+    const int64_t kbeg = MODE == EPI_REDUCE ? per * blockIdx.x : blockIdx.x;
+    const int64_t kend = MODE == EPI_REDUCE ? min(nloop, kbeg + per) : nloop;
+    const int64_t kstep = MODE == EPI_REDUCE ? 1 : gridDim.x;
+    const uint32_t lstride = (uint32_t)bnr;    // TMEM columns between levels
     const int lg = SUBB ? args.lg : 7;         // row radix 2^lg (sub-blocks only below 128)
 
     if (threadIdx.x == 0) {
@@ -766,18 +722,20 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
         for (int b = 0; b < 2; ++b) {
             tc::mbar_init(&tfull[b], 1);
             tc::mbar_init(&tempty[b], 1);
+            tc::mbar_init(&sfull[b], 2);       // one arrival per set-up warp
+            tc::mbar_init(&sempty[b], 1);
         }
-        tc::mbar_init(t3empty, EPI_WARPS);     // one arrival per epilogue warp
         tc::fence_mbar_init();
-        tc::tma_prefetch(&tmA.all);
-        tc::tma_prefetch(&tmA.low);
-        tc::tma_prefetch(&tmB.all);
-        tc::tma_prefetch(&tmB.low);
+        tc::tma_prefetch(&tmA);
+        tc::tma_prefetch(&tmB);
     }
     if (warp == 1) {
         tc::tmem_alloc(tmem_slot, TMEM_COLS);
         tc::tmem_relinquish();
     }
+    if (MODE != EPI_REDUCE)
+        for (int e = threadIdx.x; e < 2 * C::COLE_N; e += ROW_THREADS) colE_all[e] = 0;
+    if (MODE == EPI_DIVIDE && threadIdx.x >= 1 && threadIdx.x <= 24) rcp[threadIdx.x] = rcp_small(threadIdx.x);
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
@@ -785,39 +743,28 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
 
     if (warp == 0) {
         if (lane == 0) {
-            // ---------------- TMA producer: per tile one pass over the K' steps with every plane
-            // (no hold), or two: level 3 (every plane), then levels 0..2 (planes 0..2)
+            // ---------------- TMA producer: per tile the K' steps with every plane
             uint32_t it = 0;
             bool alive = true;
-            for (int64_t k = blockIdx.x; k < nloop && alive; k += gridDim.x) {
-                const int64_t tile = args.tiles ? (int64_t)args.tiles[k] : k;
-                const TilePos tp = tile_pos(args, tile);
-                if (!args.tiles && tile_skipped(args, lg, tp)) continue;
+            int64_t next = tile_at(kbeg);
+            for (int64_t k = kbeg; k < kend && alive; k += kstep) {
+                const TilePos tp = tile_pos(args, next);
+                next = tile_at(k + kstep);
                 const int64_t row0 = tp.row0;
                 const int bc = tp.ct * bnc;
-                const int k0 = first_chunk(args, tp, BKm);
-                for (int pass = TWO ? 1 : 0; pass <= (TWO ? 2 : 0) && alive; ++pass) {
-                    const int np = pass_planes<S>(pass);
-                    const int kstride = pass == 2 ? Pipe<S, MODE>::P2 : 1;
-                    for (int kc = k0; kc < args.kch; kc += kstride, ++it) {
-                        const int st = (int)(it % C::STAGES);
-                        const uint32_t ph = (it / C::STAGES) & 1;
-                        if (!tc::mbar_wait(&empty[st], ph ^ 1, args.err, kErrTimeout)) {
-                            alive = false;
-                            break;
-                        }
-                        uint8_t* sA = stage_base + st * C::STAGE_BYTES;
-                        uint8_t* sB = sA + S * C::A_TILE;
-                        const int nks = min(kstride, args.kch - kc);   // K steps in this stage
-                        tc::mbar_arrive_expect_tx(&full[st], nks * np * (C::A_TILE + b_bytes_tile));
-                        // A: [step][plane][128 rows][16]; B: [step][plane][Re rows, Im rows][16]
-                        for (int j = 0; j < nks; ++j) {
-                            tc::tma_load_3d(sA + j * np * C::A_TILE, pass == 2 ? &tmA.low : &tmA.all,
-                                            (kc + j) * BKm, (int)row0, 0, &full[st]);
-                            tc::tma_load_4d(sB + j * np * b_bytes_tile, pass == 2 ? &tmB.low : &tmB.all,
-                                            (kc + j) * BKm, bc, 0, 0, &full[st]);
-                        }
+                for (int kc = first_chunk(args, tp, BKm); kc < args.kch; ++kc, ++it) {
+                    const int st = (int)(it % C::STAGES);
+                    const uint32_t ph = (it / C::STAGES) & 1;
+                    if (!tc::mbar_wait(&empty[st], ph ^ 1, args.err, kErrTimeout)) {
+                        alive = false;
+                        break;
                     }
+                    uint8_t* sA = stage_base + st * C::STAGE_BYTES;
+                    uint8_t* sB = sA + S * C::A_TILE;
+                    tc::mbar_arrive_expect_tx(&full[st], S * (C::A_TILE + b_bytes_tile));
+                    // A: [plane][128 rows][BK]; B: [plane][Re rows, Im rows][BK]
+                    tc::tma_load_3d(sA, &tmA, kc * BKm, (int)row0, 0, &full[st]);
+                    tc::tma_load_4d(sB, &tmB, kc * BKm, bc, 0, 0, &full[st]);
                 }
             }
             if (!alive) {
@@ -828,93 +775,186 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
             }
         }
     } else if (warp == 1) {
-        {
-            // ---------------- MMA issuer: slice pairs (s, t), s + t < S, accumulated by level.
-            // With the hold, the level-3 pass of a tile starts once the epilogue has copied the
-            // previous tile's level 3 out of TMEM, and the pass of levels 0..2 once the epilogue
-            // has finished the previous tile.
-            // The whole warp runs this loop (waits made warp-uniform by a vote), so that the
-            // descriptor arithmetic stays uniform; one elected lane issues the MMAs and commits.
-            // Issued from a one-lane branch, each MMA cost ~75 cycles whatever its N.
-            const uint32_t leader = tc::elect_one();
-            const uint32_t idesc = tc::idesc_bf16_f32(128, bnr);
-            const uint32_t b16 = b_bytes_tile >> 4;   // B plane stride in 16-byte units
-            uint32_t it = 0, t = 0;
-            bool alive = true;
-            for (int64_t k = blockIdx.x; k < nloop && alive; k += gridDim.x) {
-                const int64_t tile = args.tiles ? (int64_t)args.tiles[k] : k;
-                const TilePos tp = tile_pos(args, tile);
-                if (!args.tiles && tile_skipped(args, lg, tp)) continue;
-                const int k0 = first_chunk(args, tp, BKm);
-                const int set = nset == 2 ? (int)(t & 1) : 0;
-                const uint32_t use = nset == 2 ? t >> 1 : t;     // earlier tiles on this set
-                const uint32_t tm = tmem + (uint32_t)set * (TMEM_COLS / 2);
-                for (int pass = TWO ? 1 : 0; pass <= (TWO ? 2 : 0) && alive; ++pass) {
-                    uint64_t* gate = pass == 1 ? t3empty : &tempty[set];
-                    if (!__all_sync(0xffffffffu, tc::mbar_wait(gate, (use & 1) ^ 1, args.err, kErrTimeout))) {
-                        alive = false;
-                        break;
-                    }
-                    tc::fence_after_sync();
-                    const int kstride = pass == 2 ? Pipe<S, MODE>::P2 : 1;
-                    for (int kc = k0; kc < args.kch; kc += kstride, ++it) {
-                        const int st = (int)(it % C::STAGES);
-                        const uint32_t ph = (it / C::STAGES) & 1;
-                        if (!__all_sync(0xffffffffu, tc::mbar_wait(&full[st], ph, args.err, kErrTimeout))) {
-                            alive = false;
-                            break;
-                        }
-                        tc::fence_after_sync();
-                        const uint32_t aBase = tc::smem_u32(stage_base + st * C::STAGE_BYTES);
-                        const uint32_t a_lo = tc::sdesc_sw64_lo(aBase);
-                        const uint32_t b_lo = tc::sdesc_sw64_lo(aBase + S * C::A_TILE);
-                        if constexpr (TWO) {
-                            // KS MMA K steps a chunk (1 at 16-wide chunks; 2 at 32-wide ones, 1
-                            // for a last chunk that is half padding)
-                            constexpr int KSm = Pipe<S, MODE>::KS;
-                            if (pass == 1) {
-                                const bool half = KSm > 1 && kc == args.kch - 1 && args.klast == 1;
-                                if (kc == k0) {
-                                    if (half) issue_kstep<S, MODE, 1, true, 1>(leader, tm, lstride, a_lo, b_lo, b16, idesc);
-                                    else issue_kstep<S, MODE, 1, true, KSm>(leader, tm, lstride, a_lo, b_lo, b16, idesc);
-                                } else {
-                                    if (half) issue_kstep<S, MODE, 1, false, 1>(leader, tm, lstride, a_lo, b_lo, b16, idesc);
-                                    else issue_kstep<S, MODE, 1, false, KSm>(leader, tm, lstride, a_lo, b_lo, b16, idesc);
-                                }
-                            } else {
-                                constexpr int np2 = pass_planes<S>(2);
-                                const int nks = min(kstride, args.kch - kc);
-                                for (int j = 0; j < nks; ++j) {
-                                    const uint32_t aj = a_lo + (uint32_t)(j * np2 * C::A_TILE / 16);
-                                    const uint32_t bj = b_lo + (uint32_t)(j * np2) * b16;
-                                    const bool half = KSm > 1 && kc + j == args.kch - 1 && args.klast == 1;
-                                    const bool first = kc == k0 && j == 0;
-                                    if (first) {
-                                        if (half) issue_kstep<S, MODE, 2, true, 1>(leader, tm, lstride, aj, bj, b16, idesc);
-                                        else issue_kstep<S, MODE, 2, true, KSm>(leader, tm, lstride, aj, bj, b16, idesc);
-                                    } else {
-                                        if (half) issue_kstep<S, MODE, 2, false, 1>(leader, tm, lstride, aj, bj, b16, idesc);
-                                        else issue_kstep<S, MODE, 2, false, KSm>(leader, tm, lstride, aj, bj, b16, idesc);
-                                    }
-                                }
-                            }
-                        } else {
-                            const bool half = kc == args.kch - 1 && args.klast == 1;
-                            if (kc == k0) {
-                                if (half) issue_kstep<S, MODE, 0, true, 1>(leader, tm, lstride, a_lo, b_lo, b16, idesc);
-                                else issue_kstep<S, MODE, 0, true, Pipe<S, MODE>::KS>(leader, tm, lstride, a_lo, b_lo, b16, idesc);
-                            } else {
-                                if (half) issue_kstep<S, MODE, 0, false, 1>(leader, tm, lstride, a_lo, b_lo, b16, idesc);
-                                else issue_kstep<S, MODE, 0, false, Pipe<S, MODE>::KS>(leader, tm, lstride, a_lo, b_lo, b16, idesc);
-                            }
-                        }
-                        tc::mma_commit(leader, &empty[st]);
+        // ---------------- MMA issuer: slice pairs (s, t), s + t < S, accumulated by level.
+        // The whole warp runs this loop (waits made warp-uniform by a vote), so that the
+        // descriptor arithmetic stays uniform; one elected lane issues the MMAs and commits.
+        // Nothing here depends on the tile but the reduction's first chunk: a value carried from one
+        // tile to the next (a prefetched index) made every MMA's operands per-lane values and the
+        // mode products 10% slower.
+        const uint32_t leader = tc::elect_one();
+        const uint32_t idesc = tc::idesc_bf16_f32(128, bnr);
+        const uint32_t b16 = b_bytes_tile >> 4;   // B plane stride in 16-byte units
+        uint32_t it = 0, t = 0;
+        bool alive = true;
+        for (int64_t k = kbeg; k < kend && alive; k += kstep) {
+            const int k0 = MODE == EPI_REDUCE ? first_chunk(args, tile_pos(args, tile_at(k)), BKm) : 0;
+            const int set = (int)(t & 1);
+            const uint32_t use = t >> 1;                     // earlier tiles on this set
+            // (the address comes from shared memory: taken from lane 0 it is known to be uniform)
+            const uint32_t tm = __shfl_sync(0xffffffffu, tmem + (uint32_t)set * (TMEM_COLS / 2), 0);
+            if (!__all_sync(0xffffffffu, tc::mbar_wait(&tempty[set], (use & 1) ^ 1, args.err, kErrTimeout))) {
+                alive = false;
+                break;
+            }
+            tc::fence_after_sync();
+            for (int kc = k0; kc < args.kch; ++kc, ++it) {
+                const int st = (int)(it % C::STAGES);
+                const uint32_t ph = (it / C::STAGES) & 1;
+                if (!__all_sync(0xffffffffu, tc::mbar_wait(&full[st], ph, args.err, kErrTimeout))) {
+                    alive = false;
+                    break;
+                }
+                tc::fence_after_sync();
+                const uint32_t aBase = tc::smem_u32(stage_base + st * C::STAGE_BYTES);
+                const uint32_t a_lo = tc::sdesc_sw64_lo(aBase);
+                const uint32_t b_lo = tc::sdesc_sw64_lo(aBase + S * C::A_TILE);
+                // 32-byte K offsets within a swizzled row; the last stage's second step may be padding
+                const int steps = kc == args.kch - 1 ? min(C::KS, args.klast) : C::KS;
+#pragma unroll 1
+                for (int ks = 0; ks < steps; ++ks)
+                    issue_kstep<S, MODE>(kc == k0 && ks == 0 ? 0u : 1u, leader, tm, lstride, a_lo + (uint32_t)(ks * 2),
+                                         b_lo + (uint32_t)(ks * 2), b16, idesc);
+                tc::mma_commit(leader, &empty[st]);
+            }
+            if (!alive) break;
+            if (!args.stall) tc::mma_commit(leader, &tfull[set]);
+            ++t;
+        }
+    } else if (warp >= 2 + EPI_WARPS) {
+        // ---------------- set-up warps: the tables of a tile, one tile ahead of the epilogue
+        const int st = threadIdx.x - 32 * (2 + EPI_WARPS);   // 0 .. 63
+        const int N = args.N;
+        uint32_t t = 0;
+        bool alive = true;
+        int64_t next = tile_at(kbeg);
+        for (int64_t k = kbeg; k < kend && alive; k += kstep) {
+            const int64_t tile = next;
+            const TilePos tp = tile_pos(args, tile);
+            next = tile_at(k + kstep);
+            const int buf = (int)(t & 1);
+            uint8_t* tb = tables + C::TILE + buf * C::TILE_BYTES;
+            unsigned long long* trc = args.trace ? args.trace + tile * 6 : nullptr;
+            alive = __all_sync(0xffffffffu, tc::mbar_wait_idle(&sempty[buf], ((t >> 1) & 1) ^ 1, args.err, kErrTimeout));
+            const unsigned long long t0 = trc ? global_ns() : 0ull;
+            const int qbase = tp.ct * bnc;
+            // every global load first: behind a store to the tables each would wait for the one before
+            // (rows st and st + 64; the rows 32 w .. + 31 of one warp and round are one lane quarter)
+            int ea[2], sea[2] = {0, 0};
+            uint32_t tup[2] = {0u, 0u};
+            int4 sm[2];
+            float sg[2][6];
+            bool row_in[2];
+            int vcols = min(bnc, args.ncv - qbase);
+            const int ebv = st < 32 && st < bnc ? args.eb[qbase + st] : 0;
+            const int err = st == 0 && (t & 7) == 0 ? *(volatile int*)args.err : 0;
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int r = st + 64 * j, rr = tp.rr0 + r;
+                const int64_t o = tp.row0 + r;
+                row_in[j] = args.RB == 0 || rr < args.R;          // (a last block reads past its index)
+                ea[j] = row_in[j] ? __ldg(args.ea + (args.ea_outer ? (args.RB > 0 ? (int64_t)tp.outer : o) : o)) : 0;
+                if (MODE == EPI_SLICE && N >= 4 && (rr >> lg) < args.nt) tup[j] = __ldg(args.ttup + (rr >> lg));
+                if (MODE == EPI_SLAB && N >= 2) tup[j] = __ldg(args.stup + rr);
+                if (MODE == EPI_REDUCE && row_in[j]) tup[j] = __ldg(args.tuples + rr);
+                if (MODE == EPI_DIVIDE) {                         // (the tables cover whole tiles)
+                    sm[j] = __ldg(args.smeta + rr);
+#pragma unroll
+                    for (int m = 0; m < 6; ++m) sg[j][m] = __ldg(args.ssum + (int64_t)m * args.nslot + rr);
+                }
+            }
+            double2 lq = make_double2(0.0, 0.0);
+            if (MODE == EPI_DIVIDE) {
+                vcols = min(vcols, __ldg(args.tpmax + tp.rr0 / NP) - qbase + 1);
+                // lambda_q - lambda_i, so that D = sigma_row + (lambda_q - lambda_i) needs no FP64
+                // per element (FP64 runs at a small fraction of the FP32 rate)
+                if (st >= 32 && st - 32 < bnc && qbase + st - 32 < args.ncv)
+                    lq = csub(args.lam[qbase + st - 32], args.lam[args.i0 + tp.outer]);
+            } else if ((MODE == EPI_SLICE || MODE == EPI_V) && args.colmask) {
+                vcols = min(vcols, tile_pmax(args, lg, tp) - qbase + 1);
+            }
+            if (MODE == EPI_SLICE) {
+                // output slot of (p_2 = q, the sub-block's shared p's); order 2: slot q
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const int tt = (tp.rr0 >> lg) + (st >> 5) + 2 * j, q = qbase + (st & 31);
+                    sea[j] = N >= 3 ? 0 : q;
+                    if (N >= 3 && (st >> 5) + 2 * j < (NP >> lg) && tt < args.nt) {
+                        const uint32_t pp = N == 3 ? (uint32_t)tt : __ldg(args.ttup + tt);
+                        const int p3 = (int)(pp & 255u), p4 = (int)((pp >> 8) & 255u);
+                        if (q <= p3) sea[j] = N == 3 ? __ldg(args.segbase + q) + p3 - q
+                                                     : __ldg(args.segbase + rank2(q, p3)) + p4 - p3;
                     }
                 }
-                if (!alive) break;
-                if (!args.stall) tc::mma_commit(leader, &tfull[set]);
-                ++t;
             }
+            if (st == 0) {
+                // columns of this tile that any row uses: below the modes in use and, with the
+                // sorted-tuple mask, at most the largest leading p of the tile's rows. Columns past
+                // them are neither read nor written, so the column groups split only the used ones.
+                int* meta = (int*)(tb + C::META);
+                meta[0] = qbase;
+                meta[1] = max(vcols, 0);
+                meta[2] = tp.outer;
+                meta[3] = tp.rr0;
+                meta[4] = !alive || err != 0;   // (another role's error is picked up every 8 tiles)
+            }
+            if (st < 32) ((int*)(tb + C::COLEB))[st] = ebv;
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int r = st + 64 * j;
+                int4 rm = make_int4(ea[j], NP, 0, 0);             // .y: the new index is <= it (-1: no row)
+                if (MODE == EPI_V) {
+                    if (args.colmask) rm.y = tp.outer % args.nm;
+                    if (!row_in[j]) rm.y = -1;
+                } else if (MODE == EPI_SLICE) {
+                    const int tt = (tp.rr0 + r) >> lg;            // row (p_3..p_N, a_1)
+                    if (N == 3) rm.y = tt;
+                    if (N >= 4) rm.y = (int)(tup[j] & 255u);
+                    if (!row_in[j] || tt >= args.nt) rm.y = -1;
+                } else if (MODE == EPI_DIVIDE) {
+                    rm.y = sm[j].x;
+                    rm.z = sm[j].y;
+                    rm.w = sm[j].z;
+#pragma unroll
+                    for (int m = 0; m < 6; ++m) ((float*)(tb + C::SIG))[m * NP + r] = sg[j][m];
+                    const bool ok = sm[j].x >= 0;
+                    const int seg = (sm[j].z >> 8) & 15;
+                    const int hi = __reduce_max_sync(0xffffffffu, sm[j].x);
+                    const int lo = __reduce_min_sync(0xffffffffu, ok ? seg : SEGS);
+                    const int up = __reduce_max_sync(0xffffffffu, ok ? seg : -1);
+                    if (lane == 0) ((int4*)(tb + C::QINFO))[r / 32] = make_int4(hi, lo, up, 0);
+                } else if (MODE == EPI_SLAB) {
+                    const bool ok = N >= 2 ? tup[j] != 0xFFFFFFFFu : tp.row0 + r < args.nouter;
+                    rm.y = !ok ? -1 : N >= 2 ? (int)(tup[j] & 255u) : NP;
+                    rm.z = (int)tup[j];
+                } else {
+                    // the row's last index p_{N-1} and the rank of its pair (p_1, p_2)
+                    const int p0 = (int)(tup[j] & 255u), p1 = (int)((tup[j] >> 8) & 255u);
+                    const int pin = (int)((tup[j] >> (8 * (N - 2))) & 255u);
+                    rm.z = !row_in[j] || N < 3 ? -1 : rank2(p0, p1);
+                    rm.y = row_in[j] ? pin : -1;
+                    // rows in colex order mostly share p_{N-1}: its weight is then applied once to the
+                    // quarter's sum instead of to every element
+                    const int hi = __reduce_max_sync(0xffffffffu, rm.y);
+                    const int lo = __reduce_min_sync(0xffffffffu, row_in[j] ? pin : NP);
+                    if (lane == 0)
+                        ((int4*)(tb + C::QINFO))[r / 32] = make_int4(N >= 4 && hi >= 0 && hi == lo ? hi : -1, 0, 0, 0);
+                }
+                ((int4*)(tb + C::ROWM))[r] = rm;
+            }
+            if (MODE == EPI_DIVIDE && st >= 32) {
+                const int c = st - 32;
+                ((float2*)(tb + C::LAMF))[c] = make_float2((float)lq.x, (float)lq.y);
+                ((tfl*)(tb + C::LAMT))[2 * c] = to_tfl(lq.x);
+                ((tfl*)(tb + C::LAMT))[2 * c + 1] = to_tfl(lq.y);
+            }
+            if (MODE == EPI_SLICE) {
+#pragma unroll
+                for (int j = 0; j < 2; ++j) ((int*)(tb + C::SROWQ))[32 * ((st >> 5) + 2 * j) + (st & 31)] = sea[j];
+            }
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&sfull[buf]);
+            if (trc && st == 0) trc[5] = global_ns() - t0;
+            ++t;
         }
     } else {
         // ---------------- epilogue
@@ -925,176 +965,107 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
         const uint32_t trow0 = tmem + ((uint32_t)(q4 * 32) << 16);
         constexpr int NGRP = EPI_WARPS / 4;                 // column groups per lane quarter
         const int N = args.N, n = args.n;
-        uint32_t t = 0;
-        for (int64_t k = blockIdx.x; k < nloop; k += gridDim.x) {
-            const int64_t tile = args.tiles ? (int64_t)args.tiles[k] : k;
-            const TilePos tp = tile_pos(args, tile);
-            if (!args.tiles && tile_skipped(args, lg, tp)) continue;
-            unsigned long long* trc = args.trace ? args.trace + tile * 6 : nullptr;
-            const int qbase = tp.ct * bnc;
-            const int64_t o = tp.row0 + rl;                   // row of the operand
-            // (RB = 0: packed tuples, and order-1 slabs, whose rows are the outer indices)
-            const int64_t outer = args.RB > 0 ? (int64_t)tp.outer : o;
-            const int rr = tp.rr0 + rl;
-            const bool row_in = args.RB == 0 || rr < args.R;  // (a last block reads past its index)
-            const int ea = row_in ? args.ea[args.ea_outer ? outer : o] : 0;
-            const int sb = rl >> lg;                          // sub-block of the tile (warp-uniform)
-            // columns of this tile that any row uses: below the modes in use and, with the
-            // sorted-tuple mask, at most the largest leading p of the tile's rows. Columns
-            // past them are neither read nor written (the rows they would fill are never used),
-            // so the column groups split only the used ones, in units of 4.
-            int vcols = min(bnc, args.ncv - qbase);
-            if (MODE == EPI_DIVIDE) {
-                vcols = min(vcols, args.tpmax[tp.rr0 / NP] - qbase + 1);
-            } else if ((MODE == EPI_SLICE || MODE == EPI_V) && args.colmask) {
-                vcols = min(vcols, tile_pmax(args, lg, tp) - qbase + 1);
-            }
-            const int units = (max(vcols, 0) + 3) / 4;
-            const int cbeg = 4 * ((grp * units) / NGRP);
-            const int cols = 4 * (((grp + 1) * units) / NGRP) - cbeg;
-
-            // The divide's and the slab's rows are slots: their tuple (p_2, .., p_N).
-            int dg[8];
-            bool row_ok = row_in;
-            int firstp = NP;                                  // the new index is <= firstp
-            int warpp = NP;                                   // largest firstp of the warp's rows
-            int rbase = 0, kpos = 0, seg = 0, run1 = 1;
-            bool segfirst = false;
-            float fmb = 1.0f;
-            if (MODE == EPI_DIVIDE) {
-                const SlotRow& sr = args.srow[rr];            // (the table covers whole tiles)
-                firstp = sr.firstp;
-                row_ok = firstp >= 0;
-                rbase = sr.rbase;
-                kpos = sr.kpos;
-                seg = sr.seg & 255;
-                segfirst = (sr.seg & 256) != 0;
-                run1 = sr.run1;
-                fmb = sr.fmb;
-                warpp = __reduce_max_sync(0xffffffffu, firstp);
-                if (grp == 2) {
-                    RowInfo ri;
-                    ri.sr = sr.sr;
-                    ri.si = sr.si;
-                    ri.f_row = sr.f_row;
-                    ri.f_first = sr.f_first;
-                    rowinfo[rl] = ri;
-                }
-            } else if (MODE == EPI_SLAB) {
-                const uint32_t tup = N >= 2 ? args.stup[rr] : 0u;
+        const int sb = rl >> lg;                            // sub-block of the tile (warp-uniform)
+        // EPI_REDUCE: running sums of this thread's rows (a warp's columns are at most 8: 32 over four
+        // groups), the p_{N-1} whose weight they still lack (-1: none), and where they belong
+        dfl sr[8], si[8];
+        int red_w = -1, red_outer = -1, red_q = 0, red_cols = 0, red_c0 = 0;
 #pragma unroll
-                for (int m = 0; m < 8; ++m) dg[m] = m < N - 1 ? (int)((tup >> (8 * (m & 3))) & 255u) : 0;
-                row_ok = N >= 2 ? tup != 0xFFFFFFFFu : outer < args.nouter;
-                if (N >= 2) firstp = row_ok ? dg[0] : -1;
-            } else if (MODE == EPI_SLICE) {
-                // row (p_3..p_N, a_1)
-                const int tt = rr >> lg;
-                row_ok = tt < args.nt;
-                if (N == 3) firstp = tt;
-                if (N >= 4) firstp = row_ok ? (int)(args.ttup[tt] & 255u) : 0;
-                kpos = rl & ((1 << lg) - 1);                  // K position in the next operand's row
-            } else if (MODE == EPI_V && args.colmask) {
-                firstp = (int)(tp.outer % args.nm);
-            }
-            int64_t vbase = 0;                                // EPI_V: V of the new index 0
-            if (MODE == EPI_V)
-                vbase = (args.colmask ? (int64_t)(tp.outer / args.nm) * rank2(0, args.nm) + rank2(0, firstp)
-                                      : (int64_t)tp.outer * args.nm) * args.R + rr;
-            // Per-tile tables. Column exponents; the divide's columns: lambda_q - lambda_i (FP32
-            // and as exact triple-floats), so that D = sigma_row + (lambda_q - lambda_i) needs no
-            // FP64 per row (FP64 runs at a small fraction of the FP32 rate); the last mode
-            // product's output slots.
-            if (trc && et == 0) trc[5] = global_ns();         // set-up starts
-            if (MODE == EPI_DIVIDE) colE[et] = 0;
-            else if (et < 256) colE[et] = 0;
-            if (et < 64) colEb[et] = args.eb[qbase + et];
-            if (MODE == EPI_DIVIDE && et >= 128 && et < 192) {
-                const int c = et - 128;
-                const int q = qbase + c;
-                const double2 lq = q < args.ncv ? csub(args.lam[q], args.lam[args.i0 + (int)outer])
-                                                : make_double2(0.0, 0.0);
-                lamf[c] = make_float2((float)lq.x, (float)lq.y);
-                lamt[2 * c] = to_tfl(lq.x);
-                lamt[2 * c + 1] = to_tfl(lq.y);
-            }
-            if (MODE == EPI_SLICE && et >= 256) {
-                // output slot of (p_2 = q, the sub-block's shared p's); order 2: slot q
-                const int b = (et - 256) >> 6, c = et & 63, q = qbase + c;
-                const int tt = (tp.rr0 >> lg) + b;
-                int slot = q;
-                if (N >= 3) {
-                    slot = 0;
-                    if (tt < args.nt) {
-                        const uint32_t pp = N == 3 ? (uint32_t)tt : args.ttup[tt];
-                        const int p3 = (int)(pp & 255u), p4 = (int)((pp >> 8) & 255u);
-                        if (q <= p3) slot = N == 3 ? args.segbase[q] + p3 - q
-                                                   : args.segbase[rank2(q, p3)] + p4 - p3;
+        for (int c = 0; c < 8; ++c) { sr[c] = {0.f, 0.f}; si[c] = {0.f, 0.f}; }
+        // -sum over the warp's 32 rows, times the missing weight, into Psi_N[i][k]: exchanges with the
+        // lanes 16, 8 and 4 apart halve the columns a lane carries (8 -> 4 -> 2 -> 1), those 2 and 1
+        // apart finish them. Once per run of tiles instead of once a tile, with two barriers and FP64
+        // products: the reduction's epilogue took 11.6 us per 64 columns and tile.
+        auto flush = [&] {
+            if (red_outer >= 0) {
+#pragma unroll
+                for (int step = 0; step < 3; ++step) {
+                    const int off = 16 >> step, half = 4 >> step;
+                    const bool up = (lane & off) != 0;
+#pragma unroll
+                    for (int j = 0; j < half; ++j) {
+                        const dfl tr = up ? sr[j] : sr[j + half], ti = up ? si[j] : si[j + half];
+                        const dfl mr = up ? sr[j + half] : sr[j], mi = up ? si[j + half] : si[j];
+                        sr[j] = df_add(mr, dfl{__shfl_xor_sync(0xffffffffu, tr.hi, off),
+                                               __shfl_xor_sync(0xffffffffu, tr.lo, off)});
+                        si[j] = df_add(mi, dfl{__shfl_xor_sync(0xffffffffu, ti.hi, off),
+                                               __shfl_xor_sync(0xffffffffu, ti.lo, off)});
                     }
                 }
-                srowq[64 * b + c] = slot;
+#pragma unroll
+                for (int off = 2; off > 0; off >>= 1) {
+                    sr[0] = df_add(sr[0], dfl{__shfl_xor_sync(0xffffffffu, sr[0].hi, off),
+                                              __shfl_xor_sync(0xffffffffu, sr[0].lo, off)});
+                    si[0] = df_add(si[0], dfl{__shfl_xor_sync(0xffffffffu, si[0].hi, off),
+                                              __shfl_xor_sync(0xffffffffu, si[0].lo, off)});
+                }
+                // the column by the lane's bits 16, 8 and 4
+                const int col = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
+                const int qc = red_q + red_c0 + col;
+                if ((lane & 3) == 0 && col < red_cols && qc < args.ncv &&
+                    (sr[0].hi != 0.f || si[0].hi != 0.f)) {
+                    double2 v = make_double2(df_to_d(sr[0]), df_to_d(si[0]));
+                    if (red_w >= 0) {
+                        const float4 x = __ldg(args.psi_df + qc * n + red_w);
+                        v = cmul(v, make_double2((double)x.x + (double)x.y, (double)x.z + (double)x.w));
+                    }
+                    const int64_t at = (int64_t)(args.i0 + red_outer) * n + qc;
+                    atomicAdd(&args.out_f64[at].x, -v.x);
+                    atomicAdd(&args.out_f64[at].y, -v.y);
+                }
             }
-            // sigma of the row's p's minus lambda_i in FP64 (slabs, and the FP64 quotient)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) { sr[c] = {0.f, 0.f}; si[c] = {0.f, 0.f}; }
+        };
+        uint32_t t = 0;
+        for (int64_t k = kbeg; k < kend; k += kstep) {
+            const int buf = (int)(t & 1);
+            unsigned long long* trc = args.trace ? args.trace + (args.tiles ? (int64_t)args.tiles[k] : k) * 6 : nullptr;
+            uint8_t* tb = tables + C::TILE + buf * C::TILE_BYTES;
+            const int* meta = (const int*)(tb + C::META);
+            const bool got = tc::mbar_wait(&sfull[buf], (t >> 1) & 1, args.err, kErrTimeout);
+            if (epi_any(!got || meta[4] != 0)) break;       // uniform over the epilogue warps
+            const int qbase = meta[0], vcols = meta[1], outer0 = meta[2], rr = meta[3] + rl;
+            const int* colEb = (const int*)(tb + C::COLEB);
+            int* colE = colE_all + buf * C::COLE_N;         // this tile's keys; the other tile parity's
+            if (MODE != EPI_REDUCE)                         // are cleared for the next tile
+                for (int e = et; e < C::COLE_N; e += 32 * EPI_WARPS) colE_all[(buf ^ 1) * C::COLE_N + e] = 0;
+            const int units = (vcols + 3) / 4;
+            const int cbeg = 4 * ((grp * units) / NGRP);
+            const int cols = 4 * (((grp + 1) * units) / NGRP) - cbeg;
+            const int4 rm = ((const int4*)(tb + C::ROWM))[rl];
+            const int ea = rm.x, firstp = rm.y;             // the new index is <= firstp
+            const bool row_ok = firstp >= 0;
+            const int kpos = MODE == EPI_DIVIDE ? rm.w & 255 : rl & ((1 << lg) - 1);   // K position in the next row
+            const int seg = (rm.w >> 8) & 15, run1 = (rm.w >> 13) & 7, den = (rm.w >> 16) & 255;
+            const int* qinfo = (const int*)(tb + C::QINFO) + 4 * q4;
+            const tfl* lamt = (const tfl*)(tb + C::LAMT);
+            const float2* lamf = (const float2*)(tb + C::LAMF);
+            const float* sig = (const float*)(tb + C::SIG) + rl;
+            const int* srowq = (const int*)(tb + C::SROWQ) + 32 * sb;
+            int64_t vbase = 0;                              // EPI_V: V of the new index 0
+            if (MODE == EPI_V)
+                vbase = (args.colmask ? (int64_t)(outer0 / args.nm) * rank2(0, args.nm) + rank2(0, max(firstp, 0))
+                                      : (int64_t)outer0 * args.nm) * args.R + rr;
+            // sum of the row's eigenvalues minus lambda_i in FP64 (slabs, and the FP64 quotient)
             double2 sigma = make_double2(0.0, 0.0);
+            const int i_row = args.i0 + (MODE == EPI_SLAB && args.RB == 0 ? rr + (int)(tile_at(k) / args.ncol_tiles) * NP : outer0);
             if (MODE == EPI_SLAB && row_ok) {
 #pragma unroll
-                for (int m = 0; m < 7; ++m)
-                    if (m < N - 1) sigma = cadd(sigma, args.lam[dg[m]]);
-                sigma = csub(sigma, args.lam[args.i0 + (int)outer]);
+                for (int m = 0; m < 3; ++m)
+                    if (m < N - 1) sigma = cadd(sigma, args.lam[((unsigned)rm.z >> (8 * m)) & 255u]);
+                sigma = csub(sigma, args.lam[i_row]);
             }
             if (MODE == EPI_DIVIDE && args.fp64_quotient && row_ok)
-                sigma = csub(args.srow[rr].sigma, args.lam[args.i0 + (int)outer]);
-            // EPI_REDUCE: the row's last index p_{N-1} and the rank of its prefix
-            int pin = 0, pre = -1;
-            bool uni = false;
-            if (MODE == EPI_REDUCE) {
-                if (row_ok) {
-                    const uint32_t tup = args.tuples[rr];
-                    const int p0 = (int)(tup & 255u), p1 = (int)((tup >> 8) & 255u);
-                    pin = (int)((tup >> (8 * (N - 2))) & 255u);
-                    if (N == 3) pre = p0;
-                    if (N >= 4) pre = p1 * (p1 + 1) / 2 + p0;
-                }
-                // rows in colex order mostly share p_{N-1}: its weight is then applied once to the
-                // quarter's sum instead of to every element
-                const int hi = __reduce_max_sync(0xffffffffu, row_ok ? pin : -1);
-                const int lo = __reduce_min_sync(0xffffffffu, row_ok ? pin : NP);
-                uni = N >= 3 && hi >= 0 && hi == lo;
-                if (grp == 0 && lane == 0) qpin[q4] = uni ? hi : -1;
-            }
-            // another role's error is picked up every 8 tiles (the waits see it at once)
-            if (et == 0 && (t & 7) == 0) *stop = *(volatile int*)args.err;
-            epi_sync();
-            if (*stop) break;                                // uniform over the epilogue warps
+                sigma = csub(args.ssig[rr], args.lam[i_row]);
             if (trc && et == 0) {
                 trc[0] = global_ns();
                 trc[4] = blockIdx.x + 1;
             }
             // warp-uniform (the epilogue's shuffles and TMEM loads are warp-collective)
-            const int set = nset == 2 ? (int)(t & 1) : 0;
-            const uint32_t use = nset == 2 ? t >> 1 : t;
-            const uint32_t trow = trow0 + (uint32_t)set * (TMEM_COLS / 2);
-            const bool ok = __all_sync(0xffffffffu, tc::mbar_wait(&tfull[set], use & 1, args.err, kErrTimeout));
+            const uint32_t trow = trow0 + (uint32_t)buf * (TMEM_COLS / 2);
+            const bool ok = __all_sync(0xffffffffu, tc::mbar_wait(&tfull[buf], (t >> 1) & 1, args.err, kErrTimeout));
             tc::fence_after_sync();
-            // this thread's level-3 slots of the hold: Re columns of unit u at slot u, Im at
-            // HSLOT / 2 + u
-            constexpr int HS2 = C::HSLOT / 2;
-            float4* held = hold + ((size_t)grp * C::HSLOT * NP + rl);
-            if (TWO && ok) {
-                // level 3 out of TMEM first, so that the next tile's level-3 MMAs can start
-                for (int u = 0; u < cols / 4; ++u) {
-                    uint32_t r3[4], i3[4];
-                    tc::tmem_ld4(trow + 3 * lstride + cbeg + 4 * u, r3);
-                    tc::tmem_ld4(trow + bnc + 3 * lstride + cbeg + 4 * u, i3);
-                    tc::tmem_wait_ld();
-                    held[(size_t)u * NP] = make_float4(__uint_as_float(r3[0]), __uint_as_float(r3[1]),
-                                                       __uint_as_float(r3[2]), __uint_as_float(r3[3]));
-                    held[(size_t)(HS2 + u) * NP] = make_float4(__uint_as_float(i3[0]), __uint_as_float(i3[1]),
-                                                             __uint_as_float(i3[2]), __uint_as_float(i3[3]));
-                }
-                tc::fence_before_sync();
-                __syncwarp();
-                if (lane == 0) tc::mbar_arrive(t3empty);
-            }
             if (trc && et == 0) trc[1] = global_ns();         // accumulators complete
 
             // h of one element in native FP64 (EPI_SLAB, and EPI_DIVIDE with fp64_quotient):
@@ -1102,7 +1073,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
             // clamped denominator
             auto quotient = [&](long long Vr, long long Vi, int eb, int qc) -> double2 {
                 double f = args.invfact;                      // 1 / N!, or 1 / prod(run lengths)!
-                if (MODE == EPI_DIVIDE) f = 1.0 / (double)(args.srow[rr].den * (qc == firstp ? run1 + 1 : 1));
+                if (MODE == EPI_DIVIDE) f = 1.0 / (double)(den * (qc == firstp ? run1 + 1 : 1));
                 const double sc = pow2d(ea + eb - VEXP) * f;
                 double2 h = make_double2((double)Vr * sc, (double)Vi * sc);
                 if (args.divide) {
@@ -1125,16 +1096,11 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                 // lower bound of the clamped |D| (FP32 error of the sum bounded by 4 ulp of its
                 // terms).
                 float2 sf = make_float2(0.f, 0.f);
-                int seg0 = 0, seg1 = 0;                       // segments of this warp's rows
-                if (MODE == EPI_DIVIDE) {
-                    sf = make_float2(rowinfo[rl].sr.a, rowinfo[rl].si.a);
-                    seg0 = __reduce_min_sync(0xffffffffu, row_ok ? seg : SEGS);
-                    seg1 = __reduce_max_sync(0xffffffffu, row_ok ? seg : -1);
-                }
+                if (MODE == EPI_DIVIDE) sf = make_float2(sig[0], sig[3 * NP]);
                 if (ok) {
                     constexpr float deep = deep_level_bound(S);
                     for (int c4 = cbeg; c4 < cbeg + cols; c4 += 4) {
-                        if (MODE == EPI_DIVIDE && qbase + c4 > warpp) break;   // no row of the warp
+                        if (MODE == EPI_DIVIDE && qbase + c4 > qinfo[0]) break;   // no row of the warp
                         uint32_t rv[2][4], iv[2][4];   // levels 0 and 1 only
                         tc::tmem_ld4(trow + c4, rv[0]);
                         tc::tmem_ld4(trow + c4 + lstride, rv[1]);
@@ -1152,13 +1118,13 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                             const float bi = level_bound01(iv[0][c], iv[1][c], deep);
                             unsigned key = 0;
                             if (MODE == EPI_SLICE) {
-                                const bool valid = row_ok && kpos < n && qc < args.ncv && qc <= firstp;
+                                const bool valid = kpos < n && qc < args.ncv && qc <= firstp;
                                 // bitlen(V) <= exponent(bound) + 30
                                 const float bm = fmaxf(br, bi);
                                 if (valid && bm > 0.f)
                                     key = (unsigned)(f32_exponent(bm) + 30 + ea + eb - VEXP + 8192);
                                 const unsigned wmax = __reduce_max_sync(0xffffffffu, key);
-                                if (lane == 0 && wmax) atomicMax(&colE[64 * sb + cl], (int)wmax);
+                                if (lane == 0 && wmax) atomicMax(&colE[32 * sb + cl], (int)wmax);
                             } else {
                                 if (qc < args.ncv && qc <= firstp && (br > 0.f || bi > 0.f)) {
                                     float lb = 1.0f;
@@ -1169,14 +1135,14 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                                                                     fabsf(lq.x) + fabsf(lq.y));
                                         lb = fmaxf(sqrtf(fmaf(dx, dx, dy * dy)) - del, (float)args.eps);
                                     }
-                                    const float fm = qc == firstp ? fmb / (float)(run1 + 1) : fmb;
+                                    const float fm = rcp[den * (qc == firstp ? run1 + 1 : 1)].hi;
                                     const float hm = sqrtf(fmaf(br, br, bi * bi)) * fm / lb *
                                                      (1.0f + 0.0009765625f);
                                     key = (unsigned)(f32_exponent(hm) + 30 + ea + eb - VEXP + 8192);
                                 }
-                                for (int g = seg0; g <= seg1; ++g) {
+                                for (int g = qinfo[1]; g <= qinfo[2]; ++g) {
                                     const unsigned wmax = __reduce_max_sync(0xffffffffu, seg == g ? key : 0u);
-                                    if (lane == 0 && wmax) atomicMax(&colE[64 * g + cl], (int)wmax);
+                                    if (lane == 0 && wmax) atomicMax(&colE[32 * g + cl], (int)wmax);
                                 }
                             }
                         }
@@ -1187,101 +1153,83 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
             }
 
             if (MODE == EPI_REDUCE && ok) {
-                // G[c'][k] times the weights of the row's p's in double-float, summed over the
-                // warp's 32 rows by a transposing butterfly: the first two exchanges halve the
-                // columns each lane carries (4 -> 2 -> 1), the last three finish one column per
-                // lane group
-                const bool b4 = (lane & 16) != 0, b3 = (lane & 8) != 0;
-                for (int c4 = cbeg; c4 < cbeg + cols; c4 += 4) {
-                    uint32_t rv[4][4], iv[4][4];
-                    const int u = (c4 - cbeg) / 4;
-                    load_levels<S, TWO>(trow + c4, lstride, rv, held + (size_t)u * NP);
-                    load_levels<S, TWO>(trow + bnc + c4, lstride, iv, held + (size_t)(HS2 + u) * NP);
+                // G[c'][k] times the weights of the row's p's in double-float, summed by each thread over
+                // the tiles of one (upper index, column tile) whose rows in this quarter share p_{N-1}
+                const int pin = max(firstp, 0), pre = rm.z;
+                const bool uni = qinfo[0] >= 0;
+                const int wp = qinfo[0];
+                if (wp != red_w || outer0 != red_outer || qbase != red_q) {
+                    flush();
+                    red_w = wp;
+                    red_outer = outer0;
+                    red_q = qbase;
+                    red_cols = cols;
+                    red_c0 = cbeg;
+                }
+                // two columns a round, the sums rotating through the first two registers (an unrolled
+                // body of eight elements does not fit the instruction cache beside the other roles)
+#pragma unroll 1
+                for (int h = 0; h < 4; ++h) {
+                    const int c2 = cbeg + 2 * h;
+                    uint32_t rv[4][2], iv[4][2];
+                    load_levels<S, 2>(trow + min(c2, bnc - 2), lstride, rv);
+                    load_levels<S, 2>(trow + bnc + min(c2, bnc - 2), lstride, iv);
                     tc::tmem_wait_ld();
-                    dfl pr[4], pi[4];
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const int cl = c4 + c;
+                    for (int c = 0; c < 2; ++c) {
+                        const int cl = c2 + c;
                         const int qc = qbase + cl;
-                        pr[c] = {0.f, 0.f};
-                        pi[c] = {0.f, 0.f};
                         const dfl vr = level_sum_df(rv[0][c], rv[1][c], rv[2][c], rv[3][c]);
                         const dfl vi = level_sum_df(iv[0][c], iv[1][c], iv[2][c], iv[3][c]);
-                        if (row_ok && qc < args.ncv && (vr.hi != 0.f || vi.hi != 0.f)) {
-                            const int sc = ea + colEb[cl] - VEXP + 30;
-                            const dfl gr = {ldexpf(vr.hi, sc), ldexpf(vr.lo, sc)};
-                            const dfl gi = {ldexpf(vi.hi, sc), ldexpf(vi.lo, sc)};
-                            // prod_{m <= N-2} W[p_m][k], and W[p_{N-1}][k] unless it is left to the sum
-                            const float4 w = pre >= 0 ? args.wpre[(int64_t)pre * n + qc]
-                                                      : args.psi_df[(int64_t)pin * n + qc];
+                        if (row_ok && 2 * h < cols && qc < args.ncv && (vr.hi != 0.f || vi.hi != 0.f)) {
+                            const int sc = ea + colEb[cl] - VEXP + 30, s1 = max(-126, min(126, sc));
+                            const float f = pow2f(s1);
+                            dfl gr = {vr.hi * f, vr.lo * f}, gi = {vi.hi * f, vi.lo * f};
+                            if (sc != s1) {   // (values near the ends of FP32's range)
+                                gr = {ldexpf(gr.hi, sc - s1), ldexpf(gr.lo, sc - s1)};
+                                gi = {ldexpf(gi.hi, sc - s1), ldexpf(gi.lo, sc - s1)};
+                            }
+                            // order 3: the whole weight W[p_1][k] W[p_2][k]; order 4: that, and
+                            // W[p_3][k] unless it is left to the sum
+                            const float4 w = pre >= 0 ? __ldg(args.wpre + (int64_t)qc * args.ldw + pre)
+                                                      : __ldg(args.psi_df + qc * n + pin);
                             dfl wr = {w.x, w.y}, wi = {w.z, w.w};
-                            if (pre >= 0 && !uni) {
-                                const float4 x = args.psi_df[(int64_t)pin * n + qc];
+                            if (N >= 4 && !uni) {
+                                const float4 x = __ldg(args.psi_df + qc * n + pin);
                                 const dfl xr = {x.x, x.y}, xi = {x.z, x.w};
                                 const dfl tr = df_add(df_mul(wr, xr), df_neg(df_mul(wi, xi)));
                                 wi = df_add(df_mul(wr, xi), df_mul(wi, xr));
                                 wr = tr;
                             }
-                            pr[c] = df_add(df_mul(gr, wr), df_neg(df_mul(gi, wi)));
-                            pi[c] = df_add(df_mul(gr, wi), df_mul(gi, wr));
+                            sr[c] = df_add(sr[c], df_add(df_mul(gr, wr), df_neg(df_mul(gi, wi))));
+                            si[c] = df_add(si[c], df_add(df_mul(gr, wi), df_mul(gi, wr)));
                         }
                     }
-                    // exchange 1 (lanes 16 apart): keep columns {0,1} or {2,3}, send the others
-                    dfl kr[2], ki[2];
+                    const dfl r0 = sr[0], r1 = sr[1], i0 = si[0], i1 = si[1];
 #pragma unroll
-                    for (int j = 0; j < 2; ++j) {
-                        const dfl sr = b4 ? pr[j] : pr[j + 2], si = b4 ? pi[j] : pi[j + 2];
-                        const dfl mr = b4 ? pr[j + 2] : pr[j], mi = b4 ? pi[j + 2] : pi[j];
-                        const dfl rr2 = {__shfl_xor_sync(0xffffffffu, sr.hi, 16),
-                                         __shfl_xor_sync(0xffffffffu, sr.lo, 16)};
-                        const dfl ri2 = {__shfl_xor_sync(0xffffffffu, si.hi, 16),
-                                         __shfl_xor_sync(0xffffffffu, si.lo, 16)};
-                        kr[j] = df_add(mr, rr2);
-                        ki[j] = df_add(mi, ri2);
-                    }
-                    // exchange 2 (lanes 8 apart): keep one of the two
-                    dfl ar, ai;
-                    {
-                        const dfl sr = b3 ? kr[0] : kr[1], si = b3 ? ki[0] : ki[1];
-                        const dfl mr = b3 ? kr[1] : kr[0], mi = b3 ? ki[1] : ki[0];
-                        const dfl rr2 = {__shfl_xor_sync(0xffffffffu, sr.hi, 8),
-                                         __shfl_xor_sync(0xffffffffu, sr.lo, 8)};
-                        const dfl ri2 = {__shfl_xor_sync(0xffffffffu, si.hi, 8),
-                                         __shfl_xor_sync(0xffffffffu, si.lo, 8)};
-                        ar = df_add(mr, rr2);
-                        ai = df_add(mi, ri2);
-                    }
-#pragma unroll
-                    for (int off = 4; off > 0; off >>= 1) {
-                        const dfl orr = {__shfl_xor_sync(0xffffffffu, ar.hi, off),
-                                         __shfl_xor_sync(0xffffffffu, ar.lo, off)};
-                        const dfl oi = {__shfl_xor_sync(0xffffffffu, ai.hi, off),
-                                        __shfl_xor_sync(0xffffffffu, ai.lo, off)};
-                        ar = df_add(ar, orr);
-                        ai = df_add(ai, oi);
-                    }
-                    if ((lane & 7) == 0)   // lanes 0, 8, 16, 24 hold columns 0, 1, 2, 3
-                        red[q4 * 64 + c4 + (b4 ? 2 : 0) + (b3 ? 1 : 0)] =
-                            make_float4(ar.hi, ar.lo, ai.hi, ai.lo);
+                    for (int c = 0; c < 6; ++c) { sr[c] = sr[c + 2]; si[c] = si[c + 2]; }
+                    sr[6] = r0; sr[7] = r1; si[6] = i0; si[7] = i1;
                 }
             }
             if (MODE != EPI_REDUCE && ok) {
                 // pass 2 (or the only pass): outputs
-                for (int c4 = cbeg; c4 < cbeg + cols; c4 += 4) {
-                    if (MODE == EPI_DIVIDE && qbase + c4 > warpp) break;
-                    uint32_t rv[4][4], iv[4][4];
-                    const int u = (c4 - cbeg) / 4;
-                    load_levels<S, TWO>(trow + c4, lstride, rv, held + (size_t)u * NP);
-                    load_levels<S, TWO>(trow + bnc + c4, lstride, iv, held + (size_t)(HS2 + u) * NP);
+                constexpr int UC = MODE == EPI_DIVIDE ? 2 : 4;   // columns a round (instruction cache)
+#pragma unroll 1
+                for (int c4 = cbeg; c4 < cbeg + cols; c4 += UC) {
+                    if (MODE == EPI_DIVIDE && qbase + c4 > qinfo[0]) break;
+                    uint32_t rv[4][UC], iv[4][UC];
+                    load_levels<S, UC>(trow + c4, lstride, rv);
+                    load_levels<S, UC>(trow + bnc + c4, lstride, iv);
                     tc::tmem_wait_ld();
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
+                    for (int c = 0; c < UC; ++c) {
                         const int cl = c4 + c;
                         const int qc = qbase + cl;
                         const int eb = colEb[cl];
+                        const bool valid = qc < args.ncv && qc <= firstp;
                         if (MODE == EPI_V) {
                             longlong2 v = make_longlong2(0ll, 0ll);
-                            if (row_in && qc < args.ncv && qc <= firstp) {
+                            if (valid) {
                                 v.x = combine(rv[0][c], rv[1][c], rv[2][c], rv[3][c]);
                                 v.y = combine(iv[0][c], iv[1][c], iv[2][c], iv[3][c]);
                                 args.out_v[vbase + (int64_t)qc * args.R] = v;
@@ -1293,7 +1241,6 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                             }
                             continue;
                         }
-                        const bool valid = row_ok && qc < args.ncv && qc <= firstp;
                         if (MODE == EPI_SLAB) {
                             // store h^i_{pre, q} when the multiset (q, row p's) minus pre is {extra}
                             const long long Vr = combine(rv[0][c], rv[1][c], rv[2][c], rv[3][c]);
@@ -1302,7 +1249,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                             const double2 h = quotient(Vr, Vi, eb, qc);
                             int tt[8];
                             tt[0] = qc;
-                            for (int m = 0; m < N - 1; ++m) tt[m + 1] = dg[m];
+                            for (int m = 0; m < N - 1; ++m) tt[m + 1] = (int)(((unsigned)rm.z >> (8 * m)) & 255u);
                             int used[8] = {0, 0, 0, 0, 0, 0, 0, 0};
                             int matched = 0, extra = -1, nextra = 0;
                             for (int a = 0; a < N; ++a) {
@@ -1313,14 +1260,14 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                                 else { extra = tt[a]; ++nextra; }
                             }
                             if (matched == N - 1 && nextra == 1)
-                                args.out_f64[(int64_t)(args.i0 + outer) * n + extra] = h;
+                                args.out_f64[(int64_t)i_row * n + extra] = h;
                             continue;
                         }
                         uint32_t w[S];
                         if (MODE == EPI_SLICE) {
                             if (!valid || kpos >= args.kout) continue;   // unused rows and entries
-                            const int64_t rowp = outer * args.RS + srowq[64 * sb + cl];
-                            const int key = colE[64 * sb + cl];
+                            const int64_t rowp = (int64_t)outer0 * args.RS + srowq[cl];
+                            const int key = colE[32 * sb + cl];
                             const int E = key ? key - 8192 : EXP_NONE;
                             if (key == 0 || kpos >= n) {
 #pragma unroll
@@ -1340,8 +1287,8 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                         }
                         // EPI_DIVIDE: reduction row (p_1 = q, .., p_{N-1}), K = p_N
                         if (!valid) continue;
-                        const int64_t rowp = outer * args.RT + rbase + qc;
-                        const int key = colE[64 * seg + cl];
+                        const int64_t rowp = (int64_t)outer0 * args.RT + rm.z + qc;
+                        const int key = colE[32 * seg + cl];
                         const int E = key ? key - 8192 : EXP_NONE;
                         if (key == 0) {
 #pragma unroll
@@ -1359,8 +1306,8 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                             const dfl vi = level_sum_df(iv[0][c], iv[1][c], iv[2][c], iv[3][c]);
                             dfl Dr = {1.f, 0.f}, Di = {0.f, 0.f};
                             if (args.divide) {
-                                Dr = tfl_sum(rowinfo[rl].sr, lamt[2 * cl]);
-                                Di = tfl_sum(rowinfo[rl].si, lamt[2 * cl + 1]);
+                                Dr = tfl_sum(tfl{sig[0], sig[NP], sig[2 * NP]}, lamt[2 * cl]);
+                                Di = tfl_sum(tfl{sig[3 * NP], sig[4 * NP], sig[5 * NP]}, lamt[2 * cl + 1]);
                             }
                             dfl m2 = df_add(df_mul(Dr, Dr), df_mul(Di, Di));
                             if (args.divide && m2.hi < args.eps2f) {   // Alg. 2 step 9
@@ -1370,52 +1317,20 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                             }
                             const float r0 = __frcp_rn(m2.hi);
                             const dfl e1 = df_add(dfl{1.f, 0.f}, df_neg(df_mul(m2, dfl{r0, 0.f})));
-                            const dfl rcp = df_add(dfl{r0, 0.f}, df_mul(dfl{r0, 0.f}, e1));
-                            const dfl rf = df_mul(rcp, qc == firstp ? rowinfo[rl].f_first
-                                                                    : rowinfo[rl].f_row);
+                            const dfl inv = df_add(dfl{r0, 0.f}, df_mul(dfl{r0, 0.f}, e1));
+                            const dfl rf = df_mul(inv, rcp[den * (qc == firstp ? run1 + 1 : 1)]);
                             const dfl nr = df_add(df_mul(vr, Dr), df_mul(vi, Di));
                             const dfl ni = df_add(df_mul(vi, Dr), df_neg(df_mul(vr, Di)));
-                            const int k = ea + eb - VEXP + 30 + 7 + 8 * (S - 1) - E;
+                            const int e = ea + eb - VEXP + 30 + 7 + 8 * (S - 1) - E;
                             const dfl qr = df_mul(nr, rf), qi = df_mul(ni, rf);
-                            digit_pairs<S>(df_round_i64(dfl{ldexpf(qr.hi, k), ldexpf(qr.lo, k)}),
-                                           df_round_i64(dfl{ldexpf(qi.hi, k), ldexpf(qi.lo, k)}), w);
+                            digit_pairs<S>(df_round_i64(dfl{ldexpf(qr.hi, e), ldexpf(qr.lo, e)}),
+                                           df_round_i64(dfl{ldexpf(qi.hi, e), ldexpf(qi.lo, e)}), w);
                         }
                         uint32_t* dst = reinterpret_cast<uint32_t*>(args.out_planes) + (rowp << args.lgout) + kpos;
 #pragma unroll
                         for (int s = 0; s < S; ++s) dst[s * (args.out_plane_stride / 2)] = w[s];
                         // the row's first entry holds p_N = p_{N-1} (order 2: p_2 = p_1 = q)
-                        if (N >= 3 ? segfirst : kpos == qc) args.out_exp[rowp] = E;
-                    }
-                }
-            }
-            if (MODE == EPI_REDUCE) {
-                // the four lane quarters' partials of every column, their common weight
-                // W[p_{N-1}][k] where it was left out, and -sum into Psi_N[i][k]
-                epi_sync();
-                const int cl = et;
-                const int qc = qbase + cl;
-                if (ok && cl < bnc && qc < args.ncv) {
-                    dfl ar = {0.f, 0.f}, ai = {0.f, 0.f};
-                    double2 v = make_double2(0.0, 0.0);
-                    for (int pp = 0; pp < 4; ++pp) {
-                        const float4 g = red[pp * 64 + cl];
-                        ar = df_add(ar, dfl{g.x, g.y});
-                        ai = df_add(ai, dfl{g.z, g.w});
-                        const int wp = qpin[pp];
-                        if (pp < 3 && qpin[pp + 1] == wp) continue;   // same weight: one product
-                        double2 s = make_double2(df_to_d(ar), df_to_d(ai));
-                        if (wp >= 0) {
-                            const float4 x = args.psi_df[(int64_t)wp * n + qc];
-                            s = cmul(s, make_double2((double)x.x + (double)x.y, (double)x.z + (double)x.w));
-                        }
-                        v = cadd(v, s);
-                        ar = {0.f, 0.f};
-                        ai = {0.f, 0.f};
-                    }
-                    if (v.x != 0.0 || v.y != 0.0) {
-                        const int64_t at = (int64_t)(args.i0 + tp.outer) * n + qc;
-                        atomicAdd(&args.out_f64[at].x, -v.x);
-                        atomicAdd(&args.out_f64[at].y, -v.y);
+                        if (N >= 3 ? (rm.w & 4096) != 0 : kpos == qc) args.out_exp[rowp] = E;
                     }
                 }
             }
@@ -1424,9 +1339,13 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
             if (MODE == EPI_V && args.emax && et < bnc && qbase + et < args.ncv && colE[et])
                 atomicMax(&args.emax[qbase + et], colE[et] - 8192);
             if (trc && et == 0) trc[3] = global_ns();
-            if (et == 0) tc::mbar_arrive(&tempty[set]);
+            if (et == 0) {
+                tc::mbar_arrive(&tempty[buf]);
+                tc::mbar_arrive(&sempty[buf]);
+            }
             ++t;
         }
+        if (MODE == EPI_REDUCE) flush();
     }
     tc::fence_before_sync();
     __syncthreads();
@@ -1557,22 +1476,19 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-// Slot rows (SlotRow) of the tuples tup[0, count): eigenvalue sums, run lengths and the place in
-// the reduction's operand.
-static __global__ void k_slot_rows(int N, int64_t count, const uint32_t* __restrict__ tup,
+// The divide's slots (RowArgs: smeta, ssum, ssig) of the tuples tup[0, count): eigenvalue sums, run
+// lengths and the place in the reduction's operand. They do not depend on the upper index.
+static __global__ void k_slot_rows(int N, int count, const uint32_t* __restrict__ tup,
                                    const int* __restrict__ segs, const double2* __restrict__ lam,
-                                   SlotRow* __restrict__ out)
+                                   int4* __restrict__ meta, float* __restrict__ sum, double2* __restrict__ sig)
 {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= count) return;
-    SlotRow r{};
-    r.firstp = -1;
-    r.den = 1;
-    r.run1 = 1;
+    int4 r = make_int4(-1, 0, 1 << 13 | 1 << 16, 0);
+    double2 sg = make_double2(0.0, 0.0);
     const uint32_t t = tup[idx];
     if (t != 0xFFFFFFFFu) {
         int d[3];
-        double2 sg = make_double2(0.0, 0.0);
         const int np = N - 1;
         for (int m = 0; m < 3; ++m) {
             d[m] = (int)((t >> (8 * m)) & 255u);
@@ -1587,21 +1503,20 @@ static __global__ void k_slot_rows(int N, int64_t count, const uint32_t* __restr
             for (int u = 2; u <= run; ++u) den *= u;
             run = 1;
         }
-        r.sigma = sg;
-        r.sr = to_tfl(sg.x);
-        r.si = to_tfl(sg.y);
-        r.den = den;
-        r.run1 = r1;
-        r.fmb = 1.0f / (float)den;
-        r.f_row = rcp_small(den);
-        r.f_first = rcp_small(den * (r1 + 1));
-        r.firstp = d[0];
-        r.kpos = d[np - 1];
-        if (N == 3) r.rbase = d[0] * (d[0] + 1) / 2;
-        if (N == 4) r.rbase = d[1] * (d[1] + 1) * (d[1] + 2) / 6 + d[0] * (d[0] + 1) / 2;
-        r.seg = segs[idx];
+        r.x = d[0];
+        if (N == 3) r.y = rank2(0, d[0]);
+        if (N == 4) r.y = rank3(0, d[0], d[1]);
+        r.z = d[np - 1] | segs[idx] << 8 | r1 << 13 | den << 16;
     }
-    out[idx] = r;
+    meta[idx] = r;
+    sig[idx] = sg;
+    const tfl a = to_tfl(sg.x), b = to_tfl(sg.y);
+    sum[idx] = a.a;
+    sum[count + idx] = a.b;
+    sum[2 * count + idx] = a.c;
+    sum[3 * count + idx] = b.a;
+    sum[4 * count + idx] = b.b;
+    sum[5 * count + idx] = b.c;
 }
 
 // Zeros in the reduction rows' K entries that its tiles read but the divide does not write: from
@@ -1630,20 +1545,20 @@ __global__ void k_zero_heads(int N, int nm, int kc, int lg, int Q, int64_t RT, i
         for (int s = 0; s < S; ++s) dst[s * plane_stride_u32 + k] = 0u;
 }
 
-// Prefix weights of the compact reduction: out[t][k] = prod_{m < M} W[p_m][k] for the t-th sorted
+// Prefix weights of the reduction: out[k][t] = prod_{m < M} W[p_m][k] for the t-th sorted
 // M-tuple (p_0..p_{M-1}) (8 bits per index in tup[t]), FP64 products stored as double-float
-// complex (Re hi, Re lo, Im hi, Im lo).
+// complex (Re hi, Re lo, Im hi, Im lo). M = 1: W transposed.
 static __global__ void k_prefix_weights(int M, int n, int64_t count, const uint32_t* __restrict__ tup,
                                  const double2* __restrict__ W, float4* __restrict__ out)
 {
     const int64_t tot = count * n;
     for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < tot;
          idx += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t t = idx / n;
-        const int k = (int)(idx % n);
+        const int k = (int)(idx / count);
+        const int64_t t = idx - k * count;
         double2 w = make_double2(1.0, 0.0);
         for (int m = 0; m < M; ++m) {
-            const int pm = (int)((tup[t] >> (8 * m)) & 255u);
+            const int pm = M == 1 ? (int)t : (int)((tup[t] >> (8 * m)) & 255u);
             w = cmul(w, W[(int64_t)pm * n + k]);
         }
         const float rh = (float)w.x, ih = (float)w.y;
@@ -1675,7 +1590,9 @@ struct SplitOperand {
     // per order, for the modes in use: the divide's slots (128 a tile) and the tables around them
     int slot_nm[kMaxOrder + 1] = {};          // modes the tables were built for (0: none)
     int slot_tiles[kMaxOrder + 1] = {};
-    SlotRow* srow[kMaxOrder + 1] = {};
+    int4* smeta[kMaxOrder + 1] = {};
+    float* ssum[kMaxOrder + 1] = {};
+    double2* ssig[kMaxOrder + 1] = {};
     uint32_t* stup[kMaxOrder + 1] = {};
     int* sseg[kMaxOrder + 1] = {};
     int* stpmax[kMaxOrder + 1] = {};
@@ -1730,28 +1647,24 @@ struct FixedOp { const void* base; int64_t inner; };
 // Data operand as a 3-D tensor (inner, rows, plane); box {bk, 128 rows, planes}. Past the inner
 // extent a box holds zeros.
 template <int S>
-static TMaps plane_maps(const DataOp& d, int bk)
+static CUtensorMap plane_map(const DataOp& d, int bk)
 {
     const cuuint64_t dims[3] = {(cuuint64_t)d.inner, (cuuint64_t)d.rows, (cuuint64_t)S};
     const cuuint64_t strides[2] = {(cuuint64_t)d.stride * 2, (cuuint64_t)(d.rows * d.stride * 2)};
-    const cuuint32_t box_all[3] = {(cuuint32_t)bk, (cuuint32_t)NP, (cuuint32_t)S};
-    const cuuint32_t box_low[3] = {(cuuint32_t)bk, (cuuint32_t)NP, (cuuint32_t)pass_planes<S>(2)};
-    return {encode_map(d.base, 3, dims, strides, box_all, bk),
-            encode_map(d.base, 3, dims, strides, box_low, bk)};
+    const cuuint32_t box[3] = {(cuuint32_t)bk, (cuuint32_t)NP, (cuuint32_t)S};
+    return encode_map(d.base, 3, dims, strides, box, bk);
 }
 
 // Fixed matrix as a 4-D tensor (inner, row within the half, half, plane); box {bk, bnc, 2,
 // planes}, so a plane's tile is its bnc Re rows followed by its bnc Im rows.
 template <int S>
-static TMaps fixed_maps(const FixedOp& f, int bnc, int bk)
+static CUtensorMap fixed_map(const FixedOp& f, int bnc, int bk)
 {
     const cuuint64_t dims[4] = {(cuuint64_t)f.inner, 256, 2, (cuuint64_t)S};
     const cuuint64_t strides[3] = {(cuuint64_t)f.inner * 2, (cuuint64_t)(256 * f.inner * 2),
                                    (cuuint64_t)(512 * f.inner * 2)};
-    const cuuint32_t box_all[4] = {(cuuint32_t)bk, (cuuint32_t)bnc, 2, (cuuint32_t)S};
-    const cuuint32_t box_low[4] = {(cuuint32_t)bk, (cuuint32_t)bnc, 2, (cuuint32_t)pass_planes<S>(2)};
-    return {encode_map(f.base, 4, dims, strides, box_all, bk),
-            encode_map(f.base, 4, dims, strides, box_low, bk)};
+    const cuuint32_t box[4] = {(cuuint32_t)bk, (cuuint32_t)bnc, 2, (cuuint32_t)S};
+    return encode_map(f.base, 4, dims, strides, box, bk);
 }
 
 static int default_slices(const Plan& p)
@@ -1799,7 +1712,7 @@ void split_release(Plan& p)
     for (int N = 0; N <= kMaxOrder; ++N) { cudaFree(so->at[N]); cudaFree(so->at_e[N]); }
     cudaFree(so->wred); cudaFree(so->wred_e); cudaFree(so->w_df);
     for (int N = 0; N <= kMaxOrder; ++N) {
-        cudaFree(so->srow[N]); cudaFree(so->stup[N]); cudaFree(so->sseg[N]);
+        cudaFree(so->smeta[N]); cudaFree(so->ssum[N]); cudaFree(so->ssig[N]); cudaFree(so->stup[N]); cudaFree(so->sseg[N]);
         cudaFree(so->stpmax[N]); cudaFree(so->segbase[N]);
     }
     for (int M = 0; M < 4; ++M) { cudaFree(so->ptup[M]); cudaFree(so->atup[M]); }
@@ -1877,16 +1790,6 @@ __global__ void __launch_bounds__(128)
     }
 }
 
-// A complex matrix as double-float pairs.
-static __global__ void k_to_df(const double2* __restrict__ m, int count, float4* __restrict__ out)
-{
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= count) return;
-    const double2 v = m[t];
-    const float rh = (float)v.x, ih = (float)v.y;
-    out[t] = make_float4(rh, (float)(v.x - rh), ih, (float)(v.y - ih));
-}
-
 // One fixed matrix (buffers allocated on first use, then overwritten in place), on the plan's stream.
 static void fixed_matrix(Plan& p, int S, const double2* m, bool trans, bool complexK, __nv_bfloat16*& planes, int*& ex)
 {
@@ -1903,12 +1806,13 @@ static void fixed_matrix(Plan& p, int S, const double2* m, bool trans, bool comp
     NPF_CUDA(cudaGetLastError());
 }
 
+// The reduction's weights transposed, in double-float.
 static void to_df(Plan& p, const double2* m, float4*& out)
 {
     const int count = p.n * p.n;
     if (!out) NPF_CUDA(cudaMalloc(&out, (size_t)count * sizeof(float4)));
     LaunchScope ls(&p.prof, "split_to_df", p.stream);
-    k_to_df<<<(count + 255) / 256, 256, 0, p.stream>>>(m, count, out);
+    k_prefix_weights<<<(count + 255) / 256, 256, 0, p.stream>>>(1, p.n, p.n, nullptr, m, out);
     NPF_CUDA(cudaGetLastError());
 }
 
@@ -1945,13 +1849,13 @@ static void prepare_weights(Plan& p, SplitOperand& so, const double2* dW)
     to_df(p, dW, so.w_df);
 }
 
-// Slot rows of the order's tuples from the plan's eigenvalues.
+// The slot tables of the order from the plan's eigenvalues.
 static void fill_slots(Plan& p, SplitOperand& so, int N)
 {
-    const int64_t count = (int64_t)so.slot_tiles[N] * NP;
+    const int count = so.slot_tiles[N] * NP;
     LaunchScope ls(&p.prof, "split_slot_rows", p.stream);
-    k_slot_rows<<<(unsigned)((count + 127) / 128), 128, 0, p.stream>>>(N, count, so.stup[N], so.sseg[N],
-                                                                      p.d_lam, so.srow[N]);
+    k_slot_rows<<<(unsigned)((count + 127) / 128), 128, 0, p.stream>>>(N, count, so.stup[N], so.sseg[N], p.d_lam,
+                                                                      so.smeta[N], so.ssum[N], so.ssig[N]);
     NPF_CUDA(cudaGetLastError());
 }
 
@@ -2004,9 +1908,9 @@ static void ensure_atuples(Plan& p, SplitOperand& so, int M)   // over the state
 static void ensure_slots(Plan& p, SplitOperand& so, int N)
 {
     if (so.slot_nm[N] == p.nm) return;
-    cudaFree(so.srow[N]); cudaFree(so.stup[N]); cudaFree(so.sseg[N]); cudaFree(so.stpmax[N]);
+    cudaFree(so.smeta[N]); cudaFree(so.ssum[N]); cudaFree(so.ssig[N]); cudaFree(so.stup[N]); cudaFree(so.sseg[N]); cudaFree(so.stpmax[N]);
     cudaFree(so.segbase[N]);
-    so.srow[N] = nullptr; so.stup[N] = nullptr; so.sseg[N] = nullptr; so.stpmax[N] = nullptr;
+    so.smeta[N] = nullptr; so.ssum[N] = nullptr; so.ssig[N] = nullptr; so.stup[N] = nullptr; so.sseg[N] = nullptr; so.stpmax[N] = nullptr;
     so.segbase[N] = nullptr;
     so.slot_nm[N] = 0;
     const int nm = p.nm;
@@ -2040,7 +1944,7 @@ static void ensure_slots(Plan& p, SplitOperand& so, int N)
                 const uint32_t pn = (uint32_t)(N == 2 ? r : x.p3 + r);
                 tup[pos] = N == 2 ? pn : N == 3 ? (uint32_t)x.p2 | pn << 8
                                                 : (uint32_t)x.p2 | (uint32_t)x.p3 << 8 | pn << 16;
-                seg[pos] = k | (r == 0 ? 256 : 0);
+                seg[pos] = k | (r == 0 ? 16 : 0);
             }
         }
     }
@@ -2049,7 +1953,9 @@ static void ensure_slots(Plan& p, SplitOperand& so, int N)
     so.sseg[N] = upload(seg);
     so.stpmax[N] = upload(tpmax);
     so.segbase[N] = upload(base);
-    NPF_CUDA(cudaMalloc(&so.srow[N], tup.size() * sizeof(SlotRow)));
+    NPF_CUDA(cudaMalloc(&so.smeta[N], tup.size() * sizeof(int4)));
+    NPF_CUDA(cudaMalloc(&so.ssum[N], tup.size() * 6 * sizeof(float)));
+    NPF_CUDA(cudaMalloc(&so.ssig[N], tup.size() * sizeof(double2)));
     so.slot_nm[N] = nm;
     fill_slots(p, so, N);
 }
@@ -2126,7 +2032,7 @@ static void trace_report(const char* name, const std::vector<unsigned long long>
         d[1].push_back(r[2] ? (double)(r[2] - r[1]) : 0.0);      // column-exponent pass
         d[2].push_back((double)(r[3] - (r[2] ? r[2] : r[1])));   // output pass
         cta[r[4]].push_back({r[0], r[3]});
-        if (r[5]) d[4].push_back((double)(r[0] - r[5]));        // the tile's set-up
+        if (r[5]) d[4].push_back((double)r[5]);                 // the tile's set-up (beside other tiles)
     }
     // between a CTA's tiles: skipped tiles, the per-tile tables and the error-flag read
     double busy = 0.0;
@@ -2171,27 +2077,11 @@ static void launch_rows(Plan& p, const char* name, const DataOp& A, const FixedO
                         RowArgs a)
 {
     constexpr int bk = RowCfg<S, MODE>::BK;
-    if (Pipe<S, MODE>::two && a.bnc < 64) {
-        // the divide's and the reduction's two-pass tiles keep one TMEM accumulator set and the
-        // level-3 hold, so a narrower tile only adds MMA issues (an M = 128 MMA costs ~55 cycles
-        // at N <= 64, 64 at N = 128): they run 64 complex columns wide (or the whole radix)
-        // whatever the tuned width
-        const int rad = a.bnc * a.ncol_tiles;
-        const int wide = rad < 64 ? rad : 64;
-        a.num_tiles = a.num_tiles / a.ncol_tiles * (rad / wide);
-        a.ncol_tiles = rad / wide;
-        a.bnc = wide;
-    }
-    if (!Pipe<S, MODE>::two && a.bnc > 32) {   // one-pass stages hold 32 columns (see RowCfg)
-        a.num_tiles = a.num_tiles / a.ncol_tiles * (a.bnc * a.ncol_tiles / 32);
-        a.ncol_tiles = a.bnc * a.ncol_tiles / 32;
-        a.bnc = 32;
-    }
     a.kch = (kprime + bk - 1) / bk;            // K' past kprime holds zeros on both sides
     a.lgncol = (a.ncol_tiles & (a.ncol_tiles - 1)) == 0 ? __builtin_ctz((unsigned)a.ncol_tiles) : -1;
     a.klast = (kprime + KSTEP - 1) / KSTEP - (bk / KSTEP) * (a.kch - 1);
-    const TMaps tA = plane_maps<S>(A, bk);
-    const TMaps tB = fixed_maps<S>(B, a.bnc, bk);
+    const CUtensorMap tA = plane_map<S>(A, bk);
+    const CUtensorMap tB = fixed_map<S>(B, a.bnc, bk);
     if (a.num_tiles >= (int64_t)1 << 31) fail(NPF_ERR_UNSUPPORTED, "too many tiles in one launch");
     if (a.colmask) {
         // the running tiles, listed on the device (stream order puts the list before the launch);
@@ -2270,18 +2160,17 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     for (int M = N >= 4 ? 2 : std::max(N - 1, 0); M <= N - 1; ++M) ensure_atuples(p, so, M);
     if (N >= 2) ensure_slots(p, so, N);
     if (N >= 2 && !slab) ensure_ptuples(p, so, N - 1);
-    if (N == 4) ensure_ptuples(p, so, 2);
+    if (N >= 3) ensure_ptuples(p, so, 2);
     int* const err = p.err_override ? p.err_override : so.err;   // a batch zeroes and checks its own
     const int n = p.n;
     const int nm = p.nm;                 // modes in use (a critical-mode subset comes first)
-    const int64_t P = p.packed_count[N];
     const int64_t Prows = so.at_rows[N];
     // K extent of an operand row: the radix 2^lg >= n
     const int lg = n <= 32 ? 5 : n <= 64 ? 6 : 7;
     const int rad = 1 << lg;
     // complex columns per tile (the slab path runs untuned: 32 when the plan autotunes); the mode
-    // products run at most 32 columns, the divide and the reduction 64 (launch_rows)
-    const int bnc = std::min(p.tile_n > 0 ? (p.tile_n == 48 ? 32 : p.tile_n) : 32, rad);
+    // tiles are at most 32 wide (launch_rows)
+    const int bnc = p.tile_n == 16 ? 16 : 32;
 
     // ---- rows per upper index of every stage
     const int64_t npairs = (int64_t)nm * (nm + 1) / 2;
@@ -2304,9 +2193,9 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     const size_t budget = effective_budget(p);
     if (split_min_bytes(p, N) > budget)
         fail(NPF_ERR_OOM, "memory budget too small for one upper-index batch");
-    const int ib = (int)std::min<size_t>((size_t)nm, (budget - s_bytes) / per_i);
-    const int64_t Q2 = N == 4 && !slab ? npairs : 0;              // order 4: weights of the pairs
+    const int64_t Q2 = N >= 3 && !slab ? npairs : 0;              // weights of the pairs (less than records)
     const size_t wbytes = (size_t)Q2 * n * sizeof(float4);
+    const int ib = (int)std::min<size_t>((size_t)nm, (budget - s_bytes - wbytes) / per_i);
     Arena& ar = p.scratch();
     ar.reserve(s_bytes + (size_t)ib * (a_per + b_per + e_per) + wbytes + 10 * 256 + 1024);
     uint8_t* base = (uint8_t*)ar.base;
@@ -2319,12 +2208,13 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     int* E2 = (int*)take((size_t)ib * R2 * sizeof(int));
     int* ES = (int*)take((size_t)ib * RS * sizeof(int));
     int* ER = (int*)take((size_t)ib * Qc * sizeof(int));
-    // order 3: the prefix weight is W itself (the double-float copy); order 4: pairs' products
-    const float4* wpre = W ? so.w_df : so.psi_df;
-    if (N == 4 && !slab) {
+    // orders 3 and 4: products of the weights of two indices
+    const float4* wpre = nullptr;
+    if (Q2 > 0) {
         float4* wp = (float4*)take(wbytes);
         LaunchScope ls(&p.prof, "split_prefix_weights", p.stream);
-        k_prefix_weights<<<1024, 256, 0, p.stream>>>(N - 2, n, Q2, so.ptup[2], W ? W : p.d_V, wp);
+        k_prefix_weights<<<(unsigned)std::min<int64_t>((Q2 * n + 255) / 256, 4096), 256, 0, p.stream>>>(
+            2, n, Q2, so.ptup[2], W ? W : p.d_V, wp);
         NPF_CUDA(cudaGetLastError());
         wpre = wp;
     }
@@ -2358,7 +2248,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     base0.eps2f = (float)(p.eps * p.eps);
     base0.err = err;
     base0.bnc = bnc;
-    base0.ncol_tiles = rad / bnc;
+    base0.ncol_tiles = (nm + bnc - 1) / bnc;
     base0.lg = 7;
     base0.segbase = N >= 2 ? so.segbase[N] : nullptr;
     base0.ttup = N == 4 ? so.ptup[2] : nullptr;
@@ -2454,7 +2344,10 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
                 a.R = RS;
                 a.RB = so.slot_tiles[N];
                 a.num_tiles = (int64_t)cur * a.RB * a.ncol_tiles;
-                a.srow = so.srow[N];
+                a.smeta = so.smeta[N];
+                a.ssum = so.ssum[N];
+                a.ssig = so.ssig[N];
+                a.nslot = so.slot_tiles[N] * NP;
                 a.stup = so.stup[N];
             } else {                                             // order 1: a row per upper index
                 a.ea = sE + i0;
@@ -2487,6 +2380,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
         // ---- reduction: rows (i, p_1 <= .. <= p_{N-1}), K = p_N, columns k (Psi^T)
         RowArgs a = base0;
         a.ncv = n;                         // columns: states k
+        a.ncol_tiles = (n + bnc - 1) / bnc;
         a.kfrom = 1;                       // K = p_N >= the tile's smallest p_{N-1}
         a.ea = ER;
         a.eb = W ? so.wred_e : so.red_e;
@@ -2495,6 +2389,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
         a.num_tiles = (int64_t)cur * a.RB * a.ncol_tiles;
         a.tuples = so.ptup[N - 1];
         a.wpre = wpre;
+        a.ldw = Q2;
         a.i0 = i0;
         a.out_f64 = d_out;
         const DataOp red{bufA, 2 * std::min(rad, (nm + 7) / 8 * 8), 2 * rad, cur * Qc};   // K = p_N < nm

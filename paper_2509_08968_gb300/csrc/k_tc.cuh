@@ -59,8 +59,27 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity)
 // the kernel has recorded an error.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* err, int code)
 {
+    if (mbar_try_wait(bar, parity)) return true;   // (reading the clock is slow)
     const unsigned long long t0 = wall_ns();
     for (long long it = 0; it < kWaitLimit; ++it) {
+        if (mbar_try_wait(bar, parity)) return true;
+        if ((it & 1023) == 1023) {
+            if (*(volatile int*)err) return false;
+            if (wall_ns() - t0 > kWaitNs) break;
+        }
+    }
+    atomicCAS(err, 0, code);
+    return false;
+}
+
+// The same for a role with time to spare: sleeps between polls, which otherwise take shared-memory
+// bandwidth and issue slots from the others.
+__device__ __forceinline__ bool mbar_wait_idle(uint64_t* bar, uint32_t parity, int* err, int code)
+{
+    if (mbar_try_wait(bar, parity)) return true;
+    const unsigned long long t0 = wall_ns();
+    for (long long it = 0; it < kWaitLimit; ++it) {
+        __nanosleep(256);
         if (mbar_try_wait(bar, parity)) return true;
         if ((it & 1023) == 1023) {
             if (*(volatile int*)err) return false;
@@ -149,6 +168,13 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4])
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(taddr));
 }
+// The same for 2 columns.
+__device__ __forceinline__ void tmem_ld2(uint32_t taddr, uint32_t (&r)[2])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];"
+                 : "=r"(r[0]), "=r"(r[1])
+                 : "r"(taddr));
+}
 __device__ __forceinline__ void tmem_wait_ld()
 {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
@@ -169,9 +195,9 @@ __device__ __forceinline__ uint32_t elect_one()
 
 // D[tmem] (+)= A[smem] * B[smem]^T, BF16 inputs, FP32 accumulation. The whole issuing warp runs
 // the call (its descriptor arithmetic stays warp-uniform) and the lane with `leader` != 0 issues
-// the MMA. The shared-memory descriptors are given as 32-bit halves (low: start address and
-// leading offset, high: stride offset, version, layout) and the accumulate flag is fixed, so that
-// a loop of MMAs over one stage costs a 32-bit add per operand and the instruction.
+// the MMA (acc = 0: it overwrites D). The shared-memory descriptors are given as 32-bit halves (low:
+// start address and leading offset, high: stride offset, version, layout), so that a loop of MMAs over
+// one stage costs a 32-bit add per operand and the instruction.
 // COL keeps the A operand in the tensor core's collector buffer across consecutive MMAs that read
 // the same A tile: 1 fills it (reading A from shared memory), 2 reads it from the buffer, 3 reads
 // it from the buffer and releases it; 0 reads A from shared memory only.
@@ -182,11 +208,11 @@ __device__ __forceinline__ uint32_t elect_one()
                  "setp.ne.b32 p, %5, 0;\n\t"                                                     \
                  "setp.ne.b32 q, %6, 0;\n\t"                                                     \
                  "@q tcgen05.mma.cta_group::1.kind::f16" QUAL " [%0], da, db, %4, p;\n\t}"         \
-                 ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "n"(ACC ? 1 : 0),     \
+                 ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(acc),     \
                  "r"(leader)                                                                    \
                  : "memory")
-template <bool ACC, int COL>
-__device__ __forceinline__ void mma_bf16_lohi(uint32_t leader, uint32_t d_tmem, uint32_t a_lo,
+template <int COL>
+__device__ __forceinline__ void mma_bf16_lohi(uint32_t acc, uint32_t leader, uint32_t d_tmem, uint32_t a_lo,
                                               uint32_t b_lo, uint32_t hi, uint32_t idesc)
 {
     if constexpr (COL == 0) NPF_MMA("");
