@@ -58,6 +58,7 @@ __global__ void __launch_bounds__(128)
     k_chain_upper(int n, int ilo, int rows, int64_t P, const double* __restrict__ A,
                   const double2* __restrict__ V, double2* __restrict__ S, unsigned* __restrict__ count)
 {
+    pdl_wait();
     if (blockIdx.x == 0 && blockIdx.y == 0)
         for (int r = threadIdx.x; r < rows; r += blockDim.x) count[r] = 0u;
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -117,13 +118,15 @@ __global__ void __launch_bounds__(THREADS) k_chain(ChainArgs a)
     const int row = blockIdx.y, i = a.ilo + row;
     const double2* Si = a.S + (int64_t)row * a.P;
 
-    for (int t = tid; t < (N + 1) * (n + 1); t += THREADS) cn[t] = (int)a.cnt[t];
     for (int k = tid; k < n; k += THREADS) psi[k] = make_double2(0.0, 0.0);
     if (N >= 3)
         for (int y = tid; y < n; y += THREADS)
             for (int x = 0; x <= y; ++x) tab[tri(y) + x] = (unsigned)x | (unsigned)y << 8;
     __syncthreads();
     unsigned* tab3 = tab + tri(n);
+    pdl_wait();   // (the tables above need no global memory)
+    for (int t = tid; t < (N + 1) * (n + 1); t += THREADS) cn[t] = (int)a.cnt[t];
+    __syncthreads();
     if (N == 4) {
         for (int z = 0; z < n; ++z)
             for (int t = tid; t < tri(z + 1); t += THREADS) tab3[tet(z) + t] = tab[t] | (unsigned)z << 16;
@@ -298,8 +301,7 @@ void launch(Plan& p, const ChainArgs& a, int rows)
     const size_t bytes = smem_bytes(N, a.n, a.nm);
     NPF_CUDA(cudaFuncSetAttribute(k_chain<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
     LaunchScope ls(&p.prof, "fp64_chain", p.stream);
-    k_chain<N><<<dim3((unsigned)(a.nm * a.chunks), (unsigned)rows), THREADS, bytes, p.stream>>>(a);
-    NPF_CUDA(cudaGetLastError());
+    launch_dependent(k_chain<N>, dim3((unsigned)(a.nm * a.chunks), (unsigned)rows), dim3(THREADS), bytes, p.stream, a);
 }
 
 }  // namespace
@@ -346,9 +348,8 @@ void chain_term(Plan& p, int N, double2* d_out, const double2* W, bool accumulat
     a.accumulate = accumulate;
     {
         LaunchScope ls(&p.prof, "fp64_chain_upper", p.stream);
-        k_chain_upper<<<dim3((unsigned)((a.P + 127) / 128), (unsigned)((rows + 3) / 4)), 128, 0, p.stream>>>(
-            n, lo, rows, a.P, p.d_tensor[N], p.d_V, S, a.count);
-        NPF_CUDA(cudaGetLastError());
+        launch_dependent(k_chain_upper, dim3((unsigned)((a.P + 127) / 128), (unsigned)((rows + 3) / 4)), dim3(128), 0,
+                         p.stream, n, lo, rows, a.P, p.d_tensor[N], p.d_V, S, a.count);
     }
     if (N == 2) launch<2>(p, a, rows);
     else if (N == 3) launch<3>(p, a, rows);

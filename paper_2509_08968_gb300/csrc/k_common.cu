@@ -97,6 +97,7 @@ void Arena::reserve(size_t bytes)
 {
     if (bytes <= cap) return;
     if (frozen) fail(NPF_ERR_OOM, "scratch would have to grow while work is recorded into a graph");
+    if (base) NPF_CUDA(cudaDeviceSynchronize());   // work in flight may still use the smaller block
     release();
     void* ptr = nullptr;
     cudaError_t e = cudaMalloc(&ptr, bytes);
@@ -120,6 +121,7 @@ void Arena::release()
 __global__ void k_finish(int n, const double2* __restrict__ U, const double2* __restrict__ V,
                          const double2* __restrict__ S, double2* __restrict__ out)
 {
+    pdl_wait();
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (int64_t)n * n) return;
     const int k = (int)(idx / n), i = (int)(idx % n);
@@ -132,8 +134,8 @@ void launch_finish(Plan& p, const double2* d_sum, double2* d_npf)
 {
     const int64_t tot = (int64_t)p.n * p.n;
     LaunchScope ls(&p.prof, "npf_finish", p.stream);
-    k_finish<<<(unsigned)((tot + 255) / 256), 256, 0, p.stream>>>(p.n, p.d_U, p.d_V, d_sum, d_npf);
-    NPF_CUDA(cudaGetLastError());
+    launch_dependent(k_finish, dim3((unsigned)((tot + 255) / 256)), dim3(256), 0, p.stream, p.n, p.d_U, p.d_V, d_sum,
+                     d_npf);
 }
 
 __global__ void k_zero(double2* d, int64_t count)

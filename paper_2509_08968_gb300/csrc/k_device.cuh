@@ -7,6 +7,12 @@
 
 namespace npf {
 
+// Programmatic dependent launch (launch_dependent): a kernel so launched may be set up before the one
+// in front of it in the stream has ended; it reads and writes global memory only after pdl_wait,
+// which returns when that one has ended and its writes are visible. (No kernel triggers its
+// successor early: blocks that wait for a long kernel made large systems 12% slower.)
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
 __device__ __forceinline__ double2 cmul(double2 a, double2 b)

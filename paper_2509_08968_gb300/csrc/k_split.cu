@@ -639,6 +639,7 @@ static __global__ void k_tile_list(RowArgs a, int lg, int* __restrict__ list, un
 {
     __shared__ unsigned wsum[8];
     __shared__ unsigned base;
+    pdl_wait();
     const int64_t tile = (int64_t)blockIdx.x * 256 + threadIdx.x;
     bool run = false;
     if (tile < a.num_tiles) {
@@ -700,18 +701,6 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
     const int bnc = args.bnc;
     const int bnr = 2 * bnc;
     const uint32_t b_bytes_tile = (uint32_t)bnr * BKm * 2;
-    // tiles walked by every role: the running-tile list when there is one
-    const int64_t nloop = args.tiles ? (int64_t)*(volatile const unsigned*)args.ntiles_run : args.num_tiles;
-    auto tile_at = [&](int64_t k) -> int64_t {
-        return k >= nloop ? 0 : args.tiles ? (int64_t)args.tiles[k] : k;
-    };
-    // The reduction takes consecutive tiles (row blocks of one upper index and column tile), so that its
-    // epilogue can sum over them in registers; the others take every gridDim.x-th.
-    const int64_t per = (nloop + gridDim.x - 1) / gridDim.x;
-    const int64_t kbeg = MODE == EPI_REDUCE ? per * blockIdx.x : blockIdx.x;
-    const int64_t kend = MODE == EPI_REDUCE ? min(nloop, kbeg + per) : nloop;
-    const int64_t kstep = MODE == EPI_REDUCE ? 1 : gridDim.x;
-    const uint32_t lstride = (uint32_t)bnr;    // TMEM columns between levels
     const int lg = SUBB ? args.lg : 7;         // row radix 2^lg (sub-blocks only below 128)
 
     if (threadIdx.x == 0) {
@@ -740,6 +729,20 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = *tmem_slot;
+    pdl_wait();   // (no global memory before)
+
+    // tiles walked by every role: the running-tile list when there is one
+    const int64_t nloop = args.tiles ? (int64_t)*(volatile const unsigned*)args.ntiles_run : args.num_tiles;
+    auto tile_at = [&](int64_t k) -> int64_t {
+        return k >= nloop ? 0 : args.tiles ? (int64_t)args.tiles[k] : k;
+    };
+    // The reduction takes consecutive tiles (row blocks of one upper index and column tile), so that its
+    // epilogue can sum over them in registers; the others take every gridDim.x-th.
+    const int64_t per = (nloop + gridDim.x - 1) / gridDim.x;
+    const int64_t kbeg = MODE == EPI_REDUCE ? per * blockIdx.x : blockIdx.x;
+    const int64_t kend = MODE == EPI_REDUCE ? min(nloop, kbeg + per) : nloop;
+    const int64_t kstep = MODE == EPI_REDUCE ? 1 : gridDim.x;
+    const uint32_t lstride = (uint32_t)bnr;    // TMEM columns between levels
 
     if (warp == 0) {
         if (lane == 0) {
@@ -1355,15 +1358,75 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
     }
 }
 
-// Start of a term: the output (zeroed unless the term is added to it), the exponents of S and the
-// error flag (nullptr: a batch's, zeroed once for all).
-static __global__ void k_term_init(double2* __restrict__ out, int64_t count, int* __restrict__ sE, int nm,
-                                   int* __restrict__ err)
+// Zeros in the reduction rows' K entries that its tiles read but the divide does not write: from
+// the chunk of the tile's smallest p_{N-1} up to the row's own p_{N-1}, and from nm to the operand's
+// inner extent. kc: complex K entries a chunk. t: one of 8 threads a row.
+template <int S>
+__device__ __forceinline__ void zero_head(int64_t t, int N, int nm, int kc, int lg, int Q, const uint32_t* __restrict__ tuples,
+                                          uint32_t* __restrict__ planes, int64_t plane_stride_u32)
 {
+    const int e = (int)(t & 7);
+    const int64_t row = t >> 3;
+    const int outer = (int)(row / Q), r = (int)(row - (int64_t)outer * Q);
+    const int sh = 8 * (N - 2);
+    const int p = (int)((tuples[r] >> sh) & 255u);
+    const int p0 = (int)((tuples[r & ~(NP - 1)] >> sh) & 255u);
+    uint32_t* dst = planes + (row << lg);
+    for (int k = p0 / kc * kc + e; k < p; k += 8)
+#pragma unroll
+        for (int s = 0; s < S; ++s) dst[s * plane_stride_u32 + k] = 0u;
+    const int end = min(1 << lg, (nm + 7) / 8 * 8);
+    for (int k = nm + e; k < end; k += 8)
+#pragma unroll
+        for (int s = 0; s < S; ++s) dst[s * plane_stride_u32 + k] = 0u;
+}
+
+template <int S>
+__global__ void k_zero_heads(int N, int nm, int kc, int lg, int Q, int nouter, const uint32_t* __restrict__ tuples,
+                             uint32_t* __restrict__ planes, int64_t plane_stride_u32)
+{
+    pdl_wait();
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < count) out[t] = make_double2(0.0, 0.0);
-    if (t < nm) sE[t] = EXP_NONE;
-    if (t == 0 && err) *err = 0;
+    if (t < (int64_t)Q * nouter * 8) zero_head<S>(t, N, nm, kc, lg, Q, tuples, planes, plane_stride_u32);
+}
+
+// Start of a term: the output (zeroed unless the term is added to it), the exponents of S, the error
+// flag (nullptr: a batch's, or one that holds earlier orders), and where they exist the pairs' weights
+// wpre[k][t] = W[p_1][k] W[p_2][k] (FP64 products as double-float complex) and the reduction rows'
+// heads (when their buffer is the reduction's own).
+struct TermInit {
+    double2* out;
+    int64_t cells;
+    int* sE;
+    int n, nm;
+    int* err;
+    const double2* W;
+    const uint32_t* pairs;
+    int64_t npairs;
+    float4* wpre;
+    int64_t heads;           // threads for the heads (8 a row), 0: none
+    int N, kc, lg, Q;
+    const uint32_t* tuples;
+    uint32_t* planes;
+    int64_t plane_stride_u32;
+};
+template <int S>
+__global__ void k_term_init(const __grid_constant__ TermInit a)
+{
+    pdl_wait();
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t t = t0; t < a.cells; t += step) a.out[t] = make_double2(0.0, 0.0);
+    if (t0 < a.nm) a.sE[t0] = EXP_NONE;
+    if (t0 == 0 && a.err) *a.err = 0;
+    for (int64_t t = t0; t < a.npairs * a.n; t += step) {
+        const int k = (int)(t / a.npairs);
+        const uint32_t p = a.pairs[t - k * a.npairs];
+        const double2 w = cmul(a.W[(int64_t)(p & 255u) * a.n + k], a.W[(int64_t)((p >> 8) & 255u) * a.n + k]);
+        const float rh = (float)w.x, ih = (float)w.y;
+        a.wpre[t] = make_float4(rh, (float)(w.x - rh), ih, (float)(w.y - ih));
+    }
+    for (int64_t t = t0; t < a.heads; t += step)
+        zero_head<S>(t, a.N, a.nm, a.kc, a.lg, a.Q, a.tuples, a.planes, a.plane_stride_u32);
 }
 
 // Operand rows of a mode product from the exact 64-bit values V of the stage before (EPI_V): one
@@ -1388,6 +1451,7 @@ __global__ void __launch_bounds__(256)
 {
     const int lane = threadIdx.x & 31;
     const unsigned outer = blockIdx.x / parts;
+    pdl_wait();
     int e0;
     const int* earow = ea;
     if (SRC == 2) {
@@ -1519,51 +1583,14 @@ static __global__ void k_slot_rows(int N, int count, const uint32_t* __restrict_
     sum[5 * count + idx] = b.c;
 }
 
-// Zeros in the reduction rows' K entries that its tiles read but the divide does not write: from
-// the chunk of the tile's smallest p_{N-1} up to the row's own p_{N-1}, and from nm to the operand's
-// inner extent. kc: complex K entries a chunk. One thread per (upper index, row, 8th entry).
-template <int S>
-__global__ void k_zero_heads(int N, int nm, int kc, int lg, int Q, int64_t RT, int nouter,
-                             const uint32_t* __restrict__ tuples, uint32_t* __restrict__ planes,
-                             int64_t plane_stride_u32)
+// W transposed, as double-float complex (Re hi, Re lo, Im hi, Im lo).
+static __global__ void k_to_df(int n, const double2* __restrict__ W, float4* __restrict__ out)
 {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int e = (int)(idx & 7);
-    const int64_t row = idx >> 3;
-    if (row >= (int64_t)Q * nouter) return;
-    const int outer = (int)(row / Q), r = (int)(row - (int64_t)outer * Q);
-    const int sh = 8 * (N - 2);
-    const int p = (int)((tuples[r] >> sh) & 255u);
-    const int p0 = (int)((tuples[r & ~(NP - 1)] >> sh) & 255u);
-    uint32_t* dst = planes + (((int64_t)outer * RT + r) << lg);
-    for (int k = p0 / kc * kc + e; k < p; k += 8)
-#pragma unroll
-        for (int s = 0; s < S; ++s) dst[s * plane_stride_u32 + k] = 0u;
-    const int end = min(1 << lg, (nm + 7) / 8 * 8);
-    for (int k = nm + e; k < end; k += 8)
-#pragma unroll
-        for (int s = 0; s < S; ++s) dst[s * plane_stride_u32 + k] = 0u;
-}
-
-// Prefix weights of the reduction: out[k][t] = prod_{m < M} W[p_m][k] for the t-th sorted
-// M-tuple (p_0..p_{M-1}) (8 bits per index in tup[t]), FP64 products stored as double-float
-// complex (Re hi, Re lo, Im hi, Im lo). M = 1: W transposed.
-static __global__ void k_prefix_weights(int M, int n, int64_t count, const uint32_t* __restrict__ tup,
-                                 const double2* __restrict__ W, float4* __restrict__ out)
-{
-    const int64_t tot = count * n;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < tot;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int k = (int)(idx / count);
-        const int64_t t = idx - k * count;
-        double2 w = make_double2(1.0, 0.0);
-        for (int m = 0; m < M; ++m) {
-            const int pm = M == 1 ? (int)t : (int)((tup[t] >> (8 * m)) & 255u);
-            w = cmul(w, W[(int64_t)pm * n + k]);
-        }
-        const float rh = (float)w.x, ih = (float)w.y;
-        out[idx] = make_float4(rh, (float)(w.x - rh), ih, (float)(w.y - ih));
-    }
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n * n) return;
+    const double2 w = W[(t % n) * n + t / n];
+    const float rh = (float)w.x, ih = (float)w.y;
+    out[t] = make_float4(rh, (float)(w.x - rh), ih, (float)(w.y - ih));
 }
 
 // =======================================================================================
@@ -1812,7 +1839,7 @@ static void to_df(Plan& p, const double2* m, float4*& out)
     const int count = p.n * p.n;
     if (!out) NPF_CUDA(cudaMalloc(&out, (size_t)count * sizeof(float4)));
     LaunchScope ls(&p.prof, "split_to_df", p.stream);
-    k_prefix_weights<<<(count + 255) / 256, 256, 0, p.stream>>>(1, p.n, p.n, nullptr, m, out);
+    k_to_df<<<(count + 255) / 256, 256, 0, p.stream>>>(p.n, m, out);
     NPF_CUDA(cudaGetLastError());
 }
 
@@ -2083,12 +2110,14 @@ static void launch_rows(Plan& p, const char* name, const DataOp& A, const FixedO
     const CUtensorMap tA = plane_map<S>(A, bk);
     const CUtensorMap tB = fixed_map<S>(B, a.bnc, bk);
     if (a.num_tiles >= (int64_t)1 << 31) fail(NPF_ERR_UNSUPPORTED, "too many tiles in one launch");
-    if (a.colmask) {
-        // the running tiles, listed on the device (stream order puts the list before the launch);
-        // without a column mask every tile runs
+    if (a.colmask && a.num_tiles > 8 * sm_count()) {
+        // the running tiles, listed on the device (stream order puts the list before the launch).
+        // Without a column mask, or with a few tiles a CTA only (where the list's two launches cost
+        // more than the MMAs of the masked tiles: 6 us against 2 to 4), every tile runs
         SplitOperand& so = *p.split;
         if (!so.tile_list || so.tile_cap < a.num_tiles) {
             if (p.capturing) fail(NPF_ERR_CUDA, "tile list would grow during graph capture");
+            NPF_CUDA(cudaStreamSynchronize(p.stream));
             cudaFree(so.tile_list);
             cudaFree(so.tile_count);
             so.tile_list = nullptr;
@@ -2099,9 +2128,8 @@ static void launch_rows(Plan& p, const char* name, const DataOp& A, const FixedO
         }
         NPF_CUDA(cudaMemsetAsync(so.tile_count, 0, sizeof(unsigned), p.stream));
         LaunchScope ls(&p.prof, "split_tile_list", p.stream);
-        k_tile_list<<<(unsigned)((a.num_tiles + 255) / 256), 256, 0, p.stream>>>(a, a.lg, so.tile_list,
-                                                                                so.tile_count);
-        NPF_CUDA(cudaGetLastError());
+        launch_dependent(k_tile_list, dim3((unsigned)((a.num_tiles + 255) / 256)), dim3(256), 0, p.stream, a, a.lg,
+                         so.tile_list, so.tile_count);
         a.tiles = so.tile_list;
         a.ntiles_run = so.tile_count;
     }
@@ -2118,15 +2146,15 @@ static void launch_rows(Plan& p, const char* name, const DataOp& A, const FixedO
         // an odd stride keeps each CTA from seeing only one column tile (the column tiles of a
         // row tile differ in cost under the sorted-tuple masks)
         int64_t grid = std::min<int64_t>(a.num_tiles, sm_count());
-        if (grid > 1 && a.ncol_tiles > 1 && grid % 2 == 0) grid -= 1;
-        const unsigned g = (unsigned)std::max<int64_t>(grid, 1);
+        if (grid < a.num_tiles && a.ncol_tiles > 1 && grid % 2 == 0) grid -= 1;
+        const dim3 g((unsigned)std::max<int64_t>(grid, 1)), b(ROW_THREADS);
+        constexpr size_t smem = RowCfg<S, MODE>::SMEM;
         if constexpr (MODE == EPI_SLICE) {
-            if (a.lg < 7) k_rows<S, MODE, true><<<g, ROW_THREADS, RowCfg<S, MODE>::SMEM, p.stream>>>(tA, tB, a);
-            else k_rows<S, MODE, false><<<g, ROW_THREADS, RowCfg<S, MODE>::SMEM, p.stream>>>(tA, tB, a);
+            if (a.lg < 7) launch_dependent(k_rows<S, MODE, true>, g, b, smem, p.stream, tA, tB, a);
+            else launch_dependent(k_rows<S, MODE, false>, g, b, smem, p.stream, tA, tB, a);
         } else {
-            k_rows<S, MODE, false><<<g, ROW_THREADS, RowCfg<S, MODE>::SMEM, p.stream>>>(tA, tB, a);
+            launch_dependent(k_rows<S, MODE, false>, g, b, smem, p.stream, tA, tB, a);
         }
-        NPF_CUDA(cudaGetLastError());
     }
     if (tracing) {
         std::vector<unsigned long long> h((size_t)a.num_tiles * 6);
@@ -2190,43 +2218,66 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     const size_t b_per = std::max((size_t)v_per * sizeof(longlong2), (size_t)RS * row_bytes);
     const size_t e_per = (size_t)(R1 + R2 + RS + Qc) * sizeof(int);
     const size_t per_i = std::min(dense_bytes(n, N, S), a_per + b_per + e_per);
-    const size_t budget = effective_budget(p);
-    if (split_min_bytes(p, N) > budget)
-        fail(NPF_ERR_OOM, "memory budget too small for one upper-index batch");
     const int64_t Q2 = N >= 3 && !slab ? npairs : 0;              // weights of the pairs (less than records)
     const size_t wbytes = (size_t)Q2 * n * sizeof(float4);
-    const int ib = (int)std::min<size_t>((size_t)nm, (budget - s_bytes - wbytes) / per_i);
+    const int rlo = std::max(0, p.row_lo);                       // upper-index rows to form
+    const int rhi = p.row_hi < 0 ? nm : std::min(p.row_hi, nm);
+    // One batch of a small system: the reduction's rows get a buffer of their own, so that the first
+    // launch can clear their heads.
+    const size_t red_bytes = (size_t)nm * Qc * row_bytes;
+    const size_t all_bytes = s_bytes + (size_t)nm * (a_per + b_per + e_per) + wbytes + 10 * 256 + 1024;
     Arena& ar = p.scratch();
-    ar.reserve(s_bytes + (size_t)ib * (a_per + b_per + e_per) + wbytes + 10 * 256 + 1024);
+    bool own_red = !slab && red_bytes <= ((size_t)64 << 20);
+    int ib = nm;
+    // (scratch that holds everything already needs no look at the free memory)
+    if (p.mem_budget || ar.cap < all_bytes + (own_red ? red_bytes : 0)) {
+        const size_t budget = effective_budget(p);
+        if (split_min_bytes(p, N) > budget)
+            fail(NPF_ERR_OOM, "memory budget too small for one upper-index batch");
+        ib = (int)std::min<size_t>((size_t)nm, (budget - s_bytes - wbytes) / per_i);
+        own_red &= ib == nm && all_bytes + red_bytes <= budget;
+    }
+    ar.reserve(s_bytes + (size_t)ib * (a_per + b_per + e_per) + wbytes + (own_red ? red_bytes : 0) + 10 * 256 + 1024);
     uint8_t* base = (uint8_t*)ar.base;
     auto take = [&](size_t bytes) { uint8_t* r = base; base += (bytes + 255) & ~(size_t)255; return r; };
     longlong2* Sv = (longlong2*)take(s_bytes);
     int* sE = (int*)take(256 * sizeof(int));
     uint8_t* bufA = take((size_t)ib * a_per);
     uint8_t* bufB = take((size_t)ib * b_per);
+    uint8_t* bufR = own_red ? take(red_bytes) : bufA;            // reduction rows
     int* E1 = (int*)take((size_t)ib * R1 * sizeof(int));
     int* E2 = (int*)take((size_t)ib * R2 * sizeof(int));
     int* ES = (int*)take((size_t)ib * RS * sizeof(int));
     int* ER = (int*)take((size_t)ib * Qc * sizeof(int));
-    // orders 3 and 4: products of the weights of two indices
-    const float4* wpre = nullptr;
-    if (Q2 > 0) {
-        float4* wp = (float4*)take(wbytes);
-        LaunchScope ls(&p.prof, "split_prefix_weights", p.stream);
-        k_prefix_weights<<<(unsigned)std::min<int64_t>((Q2 * n + 255) / 256, 4096), 256, 0, p.stream>>>(
-            2, n, Q2, so.ptup[2], W ? W : p.d_V, wp);
-        NPF_CUDA(cudaGetLastError());
-        wpre = wp;
-    }
-
+    float4* wpre = (float4*)take(wbytes);
+    constexpr int kred = RowCfg<S, EPI_REDUCE>::BK / 2;          // complex K entries of a reduction chunk
     {
         // (a slab entry whose accumulator is exactly zero is not stored, so the slab starts at zero)
         LaunchScope ls(&p.prof, "split_term_init", p.stream);
-        const int64_t cells = accumulate ? 0 : (int64_t)n * n;
-        k_term_init<<<(unsigned)((std::max<int64_t>(cells, nm) + 255) / 256), 256, 0, p.stream>>>(
-            d_out, cells, sE, nm, p.err_override ? nullptr : err);
-        NPF_CUDA(cudaGetLastError());
+        TermInit a{};
+        a.out = d_out;
+        a.cells = accumulate ? 0 : (int64_t)n * n;
+        a.sE = sE;
+        a.n = n;
+        a.nm = nm;
+        a.err = p.err_override || (p.defer_err && p.err_live) ? nullptr : err;
+        a.W = W ? W : p.d_V;
+        a.pairs = so.ptup[2];
+        a.npairs = Q2;
+        a.wpre = wpre;
+        a.heads = own_red ? Qc * (rhi - rlo) * 8 : 0;
+        a.N = N;
+        a.kc = kred;
+        a.lg = lg;
+        a.Q = (int)Qc;
+        a.tuples = N >= 2 ? so.ptup[N - 1] : nullptr;
+        a.planes = (uint32_t*)bufR;
+        a.plane_stride_u32 = (int64_t)(rhi - rlo) * Qc * rad;
+        const int64_t work = std::max(std::max<int64_t>((int64_t)n * n, Q2 * n), a.heads);
+        launch_dependent(k_term_init<S>, dim3((unsigned)std::min<int64_t>((work + 255) / 256, 4096)), dim3(256), 0,
+                         p.stream, a);
     }
+    p.err_live = true;
 
     const FixedOp tPhi{so.phi, KP};
     const FixedOp tPsiR{so.psir, NP};
@@ -2271,8 +2322,6 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     // K entries written per row: whole 32-byte sectors, which the MMAs' last K step covers
     const int kout = std::min(rad, (n + 7) / 8 * 8);
 
-    const int rlo = std::max(0, p.row_lo);                       // upper-index rows to form
-    const int rhi = p.row_hi < 0 ? nm : std::min(p.row_hi, nm);
     for (int i0 = rlo; i0 < rhi; i0 += ib) {
         const int cur = std::min(ib, rhi - i0);
         auto operand = [&](const uint8_t* buf, int64_t R) { return DataOp{buf, 2 * kout, 2 * rad, cur * R}; };
@@ -2283,10 +2332,9 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
                       : N == 3 ? k_regather<S, 2, 2> : k_regather<S, 3, 2>;
             const int nrows = (int)so.natup[N - 1];
             const unsigned parts = regather_parts(cur, nrows);
-            kern<<<(unsigned)cur * parts, 256, 0, p.stream>>>(
-                Sv + (int64_t)i0 * Prows, Prows, n, nm, 1, nullptr, so.at_e[N], so.psir_e + i0, sE + i0, lg, kout,
-                nrows, R0, parts, so.atup[N - 1], (uint32_t*)bufA, plane(R0), nullptr);
-            NPF_CUDA(cudaGetLastError());
+            launch_dependent(kern, dim3((unsigned)cur * parts), dim3(256), 0, p.stream, Sv + (int64_t)i0 * Prows, Prows,
+                             n, nm, 1, nullptr, so.at_e[N], so.psir_e + i0, sE + i0, lg, kout, nrows, R0, parts,
+                             so.atup[N - 1], (uint32_t*)bufA, plane(R0), nullptr);
         }
         // ---- the first N - 2 mode products: V per sorted tuple, regathered into the next operand
         for (int c = 1; c <= N - 2; ++c) {
@@ -2308,11 +2356,9 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
             LaunchScope ls(&p.prof, "split_regather", p.stream);
             const unsigned parts = regather_parts(outs, nrows);
             auto kern = pairs ? k_regather<S, 2, 0> : c == 1 ? k_regather<S, 1, 0> : k_regather<S, 1, 1>;
-            kern<<<(unsigned)outs * parts, 256, 0, p.stream>>>(
-                (const longlong2*)bufB, Ra, n, nm, (int)(outs / cur), base0.ttup, c == 1 ? sE + i0 : E1, so.phi_e,
-                nullptr, lg, kout, nrows, Rdst, parts, so.atup[2], (uint32_t*)bufA, outs * Rdst * rad,
-                pairs ? E1 : E2);
-            NPF_CUDA(cudaGetLastError());
+            launch_dependent(kern, dim3((unsigned)outs * parts), dim3(256), 0, p.stream, (const longlong2*)bufB, Ra, n,
+                             nm, (int)(outs / cur), base0.ttup, c == 1 ? sE + i0 : E1, so.phi_e, nullptr, lg, kout,
+                             nrows, Rdst, parts, so.atup[2], (uint32_t*)bufA, outs * Rdst * rad, pairs ? E1 : E2);
         }
         // ---- the last mode product (its output rows are the divide's slots)
         if (N >= 2) {
@@ -2364,18 +2410,15 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
             a.tpmax = so.stpmax[N];
             a.RT = Qc;
             a.lgout = lg;
-            a.out_planes = (__nv_bfloat16*)bufA;
+            a.out_planes = (__nv_bfloat16*)bufR;
             a.out_plane_stride = 2 * plane(Qc);
             a.out_exp = ER;
             launch_rows<S, EPI_DIVIDE>(p, "split_mode_divide", op, tPhi, 2 * n, a);
         }
-        {
+        if (!own_red) {
             LaunchScope ls(&p.prof, "split_zero_heads", p.stream);
-            const int64_t tot = Qc * cur * 8;
-            k_zero_heads<S><<<(unsigned)((tot + 255) / 256), 256, 0, p.stream>>>(
-                N, nm, RowCfg<S, EPI_REDUCE>::BK / 2, lg, (int)Qc, Qc, cur, so.ptup[N - 1],
-                (uint32_t*)bufA, plane(Qc));
-            NPF_CUDA(cudaGetLastError());
+            launch_dependent(k_zero_heads<S>, dim3((unsigned)((Qc * cur * 8 + 255) / 256)), dim3(256), 0, p.stream, N, nm,
+                             kred, lg, (int)Qc, cur, so.ptup[N - 1], (uint32_t*)bufR, plane(Qc));
         }
         // ---- reduction: rows (i, p_1 <= .. <= p_{N-1}), K = p_N, columns k (Psi^T)
         RowArgs a = base0;
@@ -2392,15 +2435,24 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
         a.ldw = Q2;
         a.i0 = i0;
         a.out_f64 = d_out;
-        const DataOp red{bufA, 2 * std::min(rad, (nm + 7) / 8 * 8), 2 * rad, cur * Qc};   // K = p_N < nm
+        const DataOp red{bufR, 2 * std::min(rad, (nm + 7) / 8 * 8), 2 * rad, cur * Qc};   // K = p_N < nm
         launch_rows<S, EPI_REDUCE>(p, "split_reduce", red, tRed, 2 * nm, a);
     }
-    if (p.err_override) return;   // the batch reads the shared flag after its graph has run
+    if (p.err_override || p.defer_err) return;   // the batch, or the entry point, reads the flag at its end
+    split_check(p);
+}
+
+#ifndef NPF_SPLIT_LOW
+void split_check(Plan& p)
+{
+    if (!p.err_live || !p.split) return;
+    p.err_live = false;
     int herr = 0;
-    NPF_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, p.stream));
+    NPF_CUDA(cudaMemcpyAsync(&herr, p.split->err, sizeof(int), cudaMemcpyDeviceToHost, p.stream));
     NPF_CUDA(cudaStreamSynchronize(p.stream));
     if (herr) fail(NPF_ERR_TIMEOUT, "a tensor-core pipeline wait gave up");
 }
+#endif
 
 // The 2..5-slice runs live in a second translation unit (k_split_low.cu, these sources compiled
 // with NPF_SPLIT_LOW), so that the kernel instantiations of the two halves build in parallel.

@@ -60,6 +60,18 @@ void sync(Plan& p)
     p.prof.flush();
 }
 
+// The terms of one entry point leave the tensor-core error flag to done(), one wait for all of them.
+struct DeferCheck {
+    Plan& p;
+    explicit DeferCheck(Plan& p_) : p(p_) { p.defer_err = true; p.err_live = false; }
+    void done()
+    {
+        npf::split_check(p);   // waits for the stream when a tensor-core term ran
+        sync(p);
+    }
+    ~DeferCheck() { p.defer_err = false; p.err_live = false; }
+};
+
 void free_plan(Plan& p)
 {
     cudaFree(p.d_lam);
@@ -214,13 +226,17 @@ int tuned_tile(Plan& p, int N)
 
 // -sum_p h^i_p prod_m W[p_m][k] into out (W = nullptr: the left eigenvectors, i.e. Psi_N).
 // Small systems: the tensor-core forms run the FP64 chain too (k_chain.cu), two launches an order
-// instead of eight to ten. Time of one call, orders 2 / 3 / 4, chain against tensor-core path:
-// n = 40 / 20 / 12: 122 / 118 / 131 us against 161 / 157 / 177; n = 48 / 24 / 14: 183 / 193 / 266
-// against 168 / 168 / 211 (its work grows as n^4 / n^5 / n^6 on the FP64 pipe). Options that choose
-// how the tensor-core path works keep it, and a budget too small for it is refused as before.
+// instead of six (order 2) to ten. Time of one call, orders 2 / 3 / 4, chain against tensor-core
+// path: n = 24 / 16 / 10: 57 / 69 / 83 us against 67 / 82 / 85; n = 26 / 18 / 11: 74 / 93 / 105
+// against 67 / 83 / 90 (its work grows as n^4 / n^5 / n^6 on the FP64 pipe). In a batch, whose
+// streams hide each other's launches but share that pipe, the lines lie lower: 64 systems of n in
+// [4, 12] at order 2: 883 us against 1060, in [12, 24] 1348 against 1160; [4, 10] at order 3: 968
+// against 1146, [10, 16] 1534 against 1319. Options that choose how the tensor-core path works keep
+// it, and a budget too small for it is refused as before.
 bool small_system(const Plan& p, int N)
 {
-    constexpr int limit[5] = {0, 0, 44, 22, 12};
+    constexpr int alone[5] = {0, 0, 25, 16, 10}, batched[5] = {0, 0, 12, 10, 8};
+    const int* limit = p.shared_arena ? batched : alone;
     if (N < 2 || N > 4 || p.n > limit[N] || p.slices || p.tile_n != 32 || p.fp64_quotient || p.debug_stall)
         return false;
     if (p.mem_budget && npf::split_min_bytes(p, N) > p.mem_budget)
@@ -669,10 +685,11 @@ int npf_compute_prefetch(npf_handle* h, int order, npf_c128* out, int count, con
         // stream; the staging buffers held the tensors replaced at the last activation, whose
         // readers finished before that call returned
         for (int t = 0; t < count; ++t) stage_tensor(p, orders[t], coeffs[t]);
+        DeferCheck check(p);
         compute_npf(p, order);
         NPF_CUDA(cudaMemcpyAsync(out, p.d_npf, (size_t)p.n * p.n * sizeof(double2),
                                  cudaMemcpyDefault, p.stream));
-        sync(p);
+        check.done();
     });
 }
 
@@ -703,6 +720,7 @@ int npf_interaction(npf_handle* h, int order, double delta, npf_c128* out)
         if (order < 1 || order > p.Nmax) npf::fail(NPF_ERR_ARG, "order must be in [1, N_max]");
         if (!(delta > 0.0)) npf::fail(NPF_ERR_ARG, "delta must be > 0");
         activate_staged(p);
+        DeferCheck check(p);
         const int64_t nn = (int64_t)p.n * p.n;
         // z(0) = delta Psi + sum_M delta^M Psi_M (Eq. 7; Eq. 9's corrected coordinates), kept in
         // d_sum; the per-order results go to d_npf as scratch before the copies
@@ -724,7 +742,6 @@ int npf_interaction(npf_handle* h, int order, double delta, npf_c128* out)
         // pN1[k][i] = phi_ki z^i(0)
         npf::launch_hadamard_t(p, 1.0, z, p.d_npf);
         emit(out);
-        sync(p);
         for (int M = 2; M <= order; ++M) {
             npf_c128* dst = out + (int64_t)(M - 1) * nn;
             if (!p.d_tensor[M]) {
@@ -736,8 +753,8 @@ int npf_interaction(npf_handle* h, int order, double delta, npf_c128* out)
                 npf::launch_hadamard_t(p, -1.0, p.d_psiN[M], p.d_npf);
             }
             emit(dst);
-            sync(p);
         }
+        check.done();
     });
 }
 
@@ -779,6 +796,7 @@ int npf_get_term(npf_handle* h, int order, npf_c128* out)
         activate_staged(p);
         if (!p.d_tensor[order])
             npf::fail(NPF_ERR_MISSING_TENSOR, "no tensor set for order " + std::to_string(order));
+        DeferCheck check(p);
         compute_term(p, order, p.d_psiN[order]);
         const double2* res = p.d_psiN[order];
         if (p.permuted()) {   // rows i back to the caller's mode order
@@ -787,7 +805,7 @@ int npf_get_term(npf_handle* h, int order, npf_c128* out)
         }
         NPF_CUDA(cudaMemcpyAsync(out, res, (size_t)p.n * p.n * sizeof(double2),
                                  cudaMemcpyDefault, p.stream));
-        sync(p);
+        check.done();
     });
 }
 

@@ -63,6 +63,24 @@ struct Arena {
     void release();
 };
 
+// Launch that may overlap the end of the kernel in front of it (the kernel begins with pdl_wait): the
+// launch latency, block start and set-up of a chain of short kernels hide behind one another.
+template <class... P, class... A>
+void launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    NPF_CUDA(cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...));
+}
+
 struct SplitOperand;  // per-precision prepared matrices (defined in the split unit)
 
 // ----------------------------------------------------------------------------------------
@@ -116,6 +134,8 @@ struct Plan {
     bool capturing = false;         // work is being recorded into a CUDA graph: no host syncs
     Arena* shared_arena = nullptr;  // scratch shared by the plans issued on one stream
     int* err_override = nullptr;    // device error flag shared by a batch (checked by the batch)
+    // tensor-core error flag checked once at the end of an entry point instead of after every order
+    bool defer_err = false, err_live = false;
     Arena& scratch() { return shared_arena ? *shared_arena : arena; }
 
     // prefetched tensors (npf_compute_prefetch): copied on up_stream into d_stage while the plan
@@ -151,6 +171,7 @@ void chain_term(Plan& p, int N, double2* d_out, const double2* W, bool accumulat
 // ----------------------------------------------------------------------------------------
 void split_term(Plan& p, int N, double2* d_out, const double2* W = nullptr, bool accumulate = false);
 void split_slab(Plan& p, int N, const int* prefix, double2* d_out);
+void split_check(Plan& p);   // waits for the stream; throws if a deferred term's pipeline wait gave up
 size_t split_min_bytes(const Plan& p, int N);   // smallest budget a term is accepted with
 void split_release(Plan& p);
 void split_prepare_tensor(Plan& p, int N);   // digit planes of a newly uploaded tensor

@@ -22,8 +22,8 @@ def npf():
     return m
 
 
-@pytest.mark.parametrize("n,N", [(1, 2), (2, 3), (3, 4), (44, 2), (45, 2), (22, 3), (23, 3), (12, 4), (13, 4),
-                                 (40, 3), (21, 4)])
+@pytest.mark.parametrize("n,N", [(1, 2), (2, 3), (3, 4), (25, 2), (26, 2), (16, 3), (17, 3), (10, 4), (11, 4),
+                                 (45, 2), (40, 3), (21, 4)])
 def test_both_sides_of_the_rule(npf, n, N):
     lam, U, V, A = _odd_system(n, N, 70 * n + N)
     ref = oracle.psiN(A, n, N, U, V, lam, p1_block=8)
@@ -39,7 +39,7 @@ def test_both_sides_of_the_rule(npf, n, N):
                 assert rel_fro(p.term(N), ref0) < tol
 
 
-@pytest.mark.parametrize("n,N", [(9, 2), (11, 3), (7, 4)])
+@pytest.mark.parametrize("n,N", [(9, 2), (13, 2), (9, 3), (11, 3), (7, 4), (9, 4)])
 def test_rows_subset_weights_and_batch(npf, n, N):
     lam, U, V, A = _odd_system(n, N, 80 * n + N)
     sysm = SimpleNamespace(n=n, lam=lam, U=U, V=V, tensors={N: A})
@@ -55,8 +55,8 @@ def test_rows_subset_weights_and_batch(npf, n, N):
         outs = [np.empty((n, n), np.complex128) for _ in range(2)]
         for _ in range(3):   # eager, recorded, replayed
             npf.batch_compute([p, q], [N, N], outs)
-            for o in outs:
-                assert rel_fro(o, U * (V + ref).T) < 1e-12
+            for o, tol in zip(outs, (1e-10, 1e-12)):   # (in a batch p leaves the chain at smaller n)
+                assert rel_fro(o, U * (V + ref).T) < tol
         modes = [0, n - 1, 2]
         p.set_mode_subset(modes)
         assert rel_fro(p.term(N), oracle.psiN_subset(A, n, N, U, V, lam, modes)) < 1e-12
