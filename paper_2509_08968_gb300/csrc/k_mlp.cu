@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "../../include/npf_mlp.h"
+#include "k_device.cuh"
 #include "npf_internal.h"
 
 namespace npf {
@@ -209,6 +210,7 @@ __global__ void __launch_bounds__(128) k_gemm(const __grid_constant__ Gemm g)
     __shared__ __align__(16) __nv_bfloat16 sA[STAGES * STAGE], sB[STAGES * STAGE];
     const int e = blockIdx.z, m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
     float acc[2][4][4];
+    pdl_wait();
     gemm_tile<AT, BT>(g, e, m0, n0, sA, sB, acc);
     if (EPI == EPI_RELU_BF16 || EPI == EPI_MASK_BF16) {
         // hidden widths are multiples of 16: a thread's column pairs are whole
@@ -285,6 +287,7 @@ __global__ void __launch_bounds__(128) k_grad_adam(const __grid_constant__ AdamS
     const int t = (int)blockIdx.x - s.tile0[l], nt = (g.N + TN - 1) / TN;
     const int e = blockIdx.z, m0 = t / nt * TM, n0 = t % nt * TN;
     float acc[2][4][4];
+    pdl_wait();
     gemm_tile<true, true>(g, e, m0, n0, sA, sB, acc);
     // the gradient tile through shared memory, so that the state moves in coalesced 16-byte accesses
     constexpr int LDG = TN + 4;
@@ -369,6 +372,7 @@ __global__ void k_gather(int E, int Bn, int w0, int ip, int wo, const float* __r
                          int64_t idx_stride, int64_t cap, __nv_bfloat16* __restrict__ Xa,
                          float* __restrict__ Tb)
 {
+    pdl_wait();
     const int64_t nx = (int64_t)E * Bn * ip, nt = T ? (int64_t)E * Bn * wo : 0;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nx + nt;
          t += (int64_t)gridDim.x * blockDim.x) {
@@ -419,6 +423,7 @@ __global__ void k_ens_stats(int E, int wo, int64_t cap, const float* __restrict_
 {
     const int r = blockIdx.x;
     float worst = 0.f;
+    pdl_wait();
     for (int o = threadIdx.x; o < wo; o += blockDim.x) {
         double s1 = 0.0, s2 = 0.0;
         for (int e = 0; e < E; ++e) {
@@ -576,8 +581,7 @@ void gemm(npf_mlp& m, const char* name, const Gemm& g)
 {
     npf::LaunchScope ls(nullptr, name, m.s);
     dim3 grid((unsigned)((g.N + TN - 1) / TN), (unsigned)((g.M + TM - 1) / TM), (unsigned)m.E);
-    k_gemm<EPI, AT, BT><<<grid, 128, 0, m.s>>>(g);
-    NPF_CUDA(cudaGetLastError());
+    npf::launch_dependent(k_gemm<EPI, AT, BT>, grid, dim3(128), 0, m.s, g);
 }
 
 void gather(npf_mlp& m, int rows, const float* dX, const float* dT, const int* idx,
@@ -585,9 +589,7 @@ void gather(npf_mlp& m, int rows, const float* dX, const float* dT, const int* i
 {
     npf::LaunchScope ls(nullptr, "mlp_gather", m.s);
     const int64_t tot = (int64_t)m.E * rows * (m.ip[0] + (dT ? m.w[m.L] : 0));
-    k_gather<<<grid_for(tot), 256, 0, m.s>>>(m.E, rows, m.w[0], m.ip[0], m.w[m.L], dX, dT, idx,
-                                             idx_stride, m.cap, m.H[0], m.Tb);
-    NPF_CUDA(cudaGetLastError());
+    npf::launch_dependent(k_gather, dim3(grid_for(tot)), dim3(256), 0, m.s, m.E, rows, m.w[0], m.ip[0], m.w[m.L], dX, dT, idx, idx_stride, m.cap, m.H[0], m.Tb);
 }
 
 // loss: the last layer's epilogue forms the output's error and the loss instead of storing Y
@@ -837,8 +839,7 @@ int npf_mlp_train(npf_mlp* m, int rows, const float* X, const float* T, int epoc
                 ad.ic1 = (float)(1.0 / (1.0 - std::pow((double)ad.b1, (double)m->step)));
                 ad.ic2 = (float)(1.0 / (1.0 - std::pow((double)ad.b2, (double)m->step)));
                 npf::LaunchScope ls(nullptr, "mlp_grad_adam", m->s);
-                k_grad_adam<<<dim3((unsigned)ad.tile0[m->L], 1, (unsigned)m->E), 128, 0, m->s>>>(ad);
-                NPF_CUDA(cudaGetLastError());
+                npf::launch_dependent(k_grad_adam, dim3((unsigned)ad.tile0[m->L], 1, (unsigned)m->E), dim3(128), 0, m->s, ad);
             }
             if (ep + 1 < epochs) shuffle();   // the next epoch's order, while this one's kernels run
             if (epoch_loss) {
@@ -883,10 +884,7 @@ int npf_mlp_predict(npf_mlp* m, int rows, const float* X, const float* mu, const
         forward(*m, rows, false);
         {
             npf::LaunchScope ls(nullptr, "mlp_ensemble_gate", m->s);
-            k_ens_stats<<<rows, 128, 0, m->s>>>(m->E, wo, m->cap, m->Y, m->d_mu, m->d_sig,
-                                                (float)spread_limit, m->d_mean, m->d_spread,
-                                                m->d_fb);
-            NPF_CUDA(cudaGetLastError());
+            npf::launch_dependent(k_ens_stats, dim3(rows), dim3(128), 0, m->s, m->E, wo, m->cap, m->Y, m->d_mu, m->d_sig, (float)spread_limit, m->d_mean, m->d_spread, m->d_fb);
         }
         copy_out(mean, m->d_mean, (size_t)rows * wo * sizeof(float), m->s);
         copy_out(spread, m->d_spread, (size_t)rows * sizeof(float), m->s);
