@@ -1624,6 +1624,11 @@ struct SplitOperand {
     int* sseg[kMaxOrder + 1] = {};
     int* stpmax[kMaxOrder + 1] = {};
     int* segbase[kMaxOrder + 1] = {};
+    // reduction rows of the last term (Plan::keep_red): planes, exponents, their bytes
+    uint8_t* kept[kMaxOrder + 1] = {};
+    int* kept_e[kMaxOrder + 1] = {};
+    size_t kept_bytes[kMaxOrder + 1] = {};
+    bool kept_ok[kMaxOrder + 1] = {};
     // sorted M-tuples over the modes in use in colexicographic order, 8 bits per index
     uint32_t* ptup[4] = {};
     int64_t nptup[4] = {};
@@ -1718,6 +1723,12 @@ static size_t dense_bytes(int n, int N, int S)
 }
 
 #ifndef NPF_SPLIT_LOW
+void split_drop_kept(Plan& p)
+{
+    if (!p.split) return;
+    for (bool& ok : p.split->kept_ok) ok = false;
+}
+
 // A term is accepted when S, digit records of it (32 bytes an entry) and the dense rows of one upper
 // index fit the budget: the sorted rows it forms take less, and no records are kept.
 size_t split_min_bytes(const Plan& p, int N)
@@ -1741,6 +1752,7 @@ void split_release(Plan& p)
     for (int N = 0; N <= kMaxOrder; ++N) {
         cudaFree(so->smeta[N]); cudaFree(so->ssum[N]); cudaFree(so->ssig[N]); cudaFree(so->stup[N]); cudaFree(so->sseg[N]);
         cudaFree(so->stpmax[N]); cudaFree(so->segbase[N]);
+        cudaFree(so->kept[N]); cudaFree(so->kept_e[N]);
     }
     for (int M = 0; M < 4; ++M) { cudaFree(so->ptup[M]); cudaFree(so->atup[M]); }
     cudaFree(so->err);
@@ -2003,7 +2015,8 @@ static void prepare_tensor(Plan& p, SplitOperand& so, int N)
         NPF_CUDA(cudaMalloc(&so.at[N], (size_t)S * rows * NP * 2));
         NPF_CUDA(cudaMalloc(&so.at_e[N], (size_t)rows * sizeof(int)));
     }
-    NPF_CUDA(cudaMemsetAsync(so.at[N], 0, (size_t)S * rows * NP * 2, p.stream));
+    if (rows > P)   // the padding rows of every plane (k_prep_at writes the others whole)
+        NPF_CUDA(cudaMemset2DAsync(so.at[N] + P * NP, (size_t)rows * NP * 2, 0, (size_t)(rows - P) * NP * 2, S, p.stream));
     {
         LaunchScope ls(&p.prof, "split_prepare_tensor", p.stream);
         k_prep_at<S><<<(unsigned)((P + 7) / 8), 256, 0, p.stream>>>(p.d_tensor[N], P, p.n, N, p.d_cnt, so.at[N],
@@ -2228,6 +2241,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     const size_t all_bytes = s_bytes + (size_t)nm * (a_per + b_per + e_per) + wbytes + 10 * 256 + 1024;
     Arena& ar = p.scratch();
     bool own_red = !slab && red_bytes <= ((size_t)64 << 20);
+    bool keep = !slab && p.keep_red && rhi - rlo == nm && red_bytes <= ((size_t)256 << 20);
     int ib = nm;
     // (scratch that holds everything already needs no look at the free memory)
     if (p.mem_budget || ar.cap < all_bytes + (own_red ? red_bytes : 0)) {
@@ -2236,7 +2250,22 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
             fail(NPF_ERR_OOM, "memory budget too small for one upper-index batch");
         ib = (int)std::min<size_t>((size_t)nm, (budget - s_bytes - wbytes) / per_i);
         own_red &= ib == nm && all_bytes + red_bytes <= budget;
+        keep &= ib == nm && all_bytes + red_bytes <= budget;
     }
+    // kept rows: up to 256 MB an order, in a buffer of the plan that a repeated call finds again
+    if (keep) {
+        const size_t eb = (size_t)nm * Qc * sizeof(int);
+        if (so.kept_bytes[N] != red_bytes + eb) {
+            if (so.kept[N]) NPF_CUDA(cudaStreamSynchronize(p.stream));
+            cudaFree(so.kept[N]); cudaFree(so.kept_e[N]);
+            so.kept[N] = nullptr; so.kept_e[N] = nullptr; so.kept_bytes[N] = 0;
+            NPF_CUDA(cudaMalloc(&so.kept[N], red_bytes));
+            NPF_CUDA(cudaMalloc(&so.kept_e[N], eb));
+            so.kept_bytes[N] = red_bytes + eb;
+        }
+        own_red = false;   // (no room in the scratch for it)
+    }
+    const bool again = keep && W && so.kept_ok[N];   // only the reduction is left to do
     ar.reserve(s_bytes + (size_t)ib * (a_per + b_per + e_per) + wbytes + (own_red ? red_bytes : 0) + 10 * 256 + 1024);
     uint8_t* base = (uint8_t*)ar.base;
     auto take = [&](size_t bytes) { uint8_t* r = base; base += (bytes + 255) & ~(size_t)255; return r; };
@@ -2244,11 +2273,11 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     int* sE = (int*)take(256 * sizeof(int));
     uint8_t* bufA = take((size_t)ib * a_per);
     uint8_t* bufB = take((size_t)ib * b_per);
-    uint8_t* bufR = own_red ? take(red_bytes) : bufA;            // reduction rows
+    uint8_t* bufR = keep ? so.kept[N] : own_red ? take(red_bytes) : bufA;   // reduction rows
     int* E1 = (int*)take((size_t)ib * R1 * sizeof(int));
     int* E2 = (int*)take((size_t)ib * R2 * sizeof(int));
     int* ES = (int*)take((size_t)ib * RS * sizeof(int));
-    int* ER = (int*)take((size_t)ib * Qc * sizeof(int));
+    int* ER = keep ? so.kept_e[N] : (int*)take((size_t)ib * Qc * sizeof(int));
     float4* wpre = (float4*)take(wbytes);
     constexpr int kred = RowCfg<S, EPI_REDUCE>::BK / 2;          // complex K entries of a reduction chunk
     {
@@ -2265,7 +2294,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
         a.pairs = so.ptup[2];
         a.npairs = Q2;
         a.wpre = wpre;
-        a.heads = own_red ? Qc * (rhi - rlo) * 8 : 0;
+        a.heads = own_red || (keep && !again) ? Qc * (rhi - rlo) * 8 : 0;
         a.N = N;
         a.kc = kred;
         a.lg = lg;
@@ -2307,7 +2336,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
         for (int m = 0; m < N - 1; ++m) base0.pre[m] = prefix[m];
 
     // ---- P1: V of S[i][Q] = sum_j psi_ij A^j_Q (rows Q, real K = j), and its exponent per i
-    {
+    if (!again) {
         RowArgs a = base0;
         a.ea = so.at_e[N];
         a.eb = so.psir_e;
@@ -2326,7 +2355,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
         const int cur = std::min(ib, rhi - i0);
         auto operand = [&](const uint8_t* buf, int64_t R) { return DataOp{buf, 2 * kout, 2 * rad, cur * R}; };
         auto plane = [&](int64_t R) { return cur * R * rad; };   // plane stride in complex entries
-        {
+        if (!again) {
             LaunchScope ls(&p.prof, "split_expand", p.stream);
             auto kern = N == 1 ? k_regather<S, 0, 2> : N == 2 ? k_regather<S, 1, 2>
                       : N == 3 ? k_regather<S, 2, 2> : k_regather<S, 3, 2>;
@@ -2337,7 +2366,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
                              so.atup[N - 1], (uint32_t*)bufA, plane(R0), nullptr);
         }
         // ---- the first N - 2 mode products: V per sorted tuple, regathered into the next operand
-        for (int c = 1; c <= N - 2; ++c) {
+        for (int c = 1; c <= N - 2 && !again; ++c) {
             const int64_t Ra = arows(N - c), outers = c == 1 ? cur : (int64_t)cur * nm;
             RowArgs a = base0;
             a.ea = c == 1 ? sE + i0 : E1;
@@ -2361,7 +2390,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
                              nrows, Rdst, parts, so.atup[2], (uint32_t*)bufA, outs * Rdst * rad, pairs ? E1 : E2);
         }
         // ---- the last mode product (its output rows are the divide's slots)
-        if (N >= 2) {
+        if (N >= 2 && !again) {
             RowArgs a = base0;
             a.lg = lg;
             a.ea = N == 2 ? sE + i0 : E2;
@@ -2380,7 +2409,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
             launch_rows<S, EPI_SLICE>(p, "split_mode_product", operand(bufA, a.R), tPhi, 2 * n, a);
         }
         // ---- the last contraction: divide, or the slab's entries
-        {
+        if (!again) {
             RowArgs a = base0;
             a.eb = so.phi_e;
             a.i0 = i0;
@@ -2415,7 +2444,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
             a.out_exp = ER;
             launch_rows<S, EPI_DIVIDE>(p, "split_mode_divide", op, tPhi, 2 * n, a);
         }
-        if (!own_red) {
+        if (!own_red && !keep) {
             LaunchScope ls(&p.prof, "split_zero_heads", p.stream);
             launch_dependent(k_zero_heads<S>, dim3((unsigned)((Qc * cur * 8 + 255) / 256)), dim3(256), 0, p.stream, N, nm,
                              kred, lg, (int)Qc, cur, so.ptup[N - 1], (uint32_t*)bufR, plane(Qc));
@@ -2437,6 +2466,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
         a.out_f64 = d_out;
         const DataOp red{bufR, 2 * std::min(rad, (nm + 7) / 8 * 8), 2 * rad, cur * Qc};   // K = p_N < nm
         launch_rows<S, EPI_REDUCE>(p, "split_reduce", red, tRed, 2 * nm, a);
+        so.kept_ok[N] = keep;
     }
     if (p.err_override || p.defer_err) return;   // the batch, or the entry point, reads the flag at its end
     split_check(p);

@@ -72,6 +72,13 @@ struct DeferCheck {
     ~DeferCheck() { p.defer_err = false; p.err_live = false; }
 };
 
+// The terms of one entry point share their reduction rows (Plan::keep_red).
+struct KeepReduction {
+    Plan& p;
+    explicit KeepReduction(Plan& p_) : p(p_) { npf::split_drop_kept(p); p.keep_red = true; }
+    ~KeepReduction() { p.keep_red = false; npf::split_drop_kept(p); }
+};
+
 void free_plan(Plan& p)
 {
     cudaFree(p.d_lam);
@@ -721,6 +728,7 @@ int npf_interaction(npf_handle* h, int order, double delta, npf_c128* out)
         if (!(delta > 0.0)) npf::fail(NPF_ERR_ARG, "delta must be > 0");
         activate_staged(p);
         DeferCheck check(p);
+        KeepReduction keep(p);
         const int64_t nn = (int64_t)p.n * p.n;
         // z(0) = delta Psi + sum_M delta^M Psi_M (Eq. 7; Eq. 9's corrected coordinates), kept in
         // d_sum; the per-order results go to d_npf as scratch before the copies

@@ -136,6 +136,10 @@ struct Plan {
     int* err_override = nullptr;    // device error flag shared by a batch (checked by the batch)
     // tensor-core error flag checked once at the end of an entry point instead of after every order
     bool defer_err = false, err_live = false;
+    // mode interactions reduce every order's divided entries twice, against Psi and against z(0):
+    // keep_red asks a tensor-core term that runs in one batch to keep its reduction rows, which a
+    // later term of the same call with other weights then starts from
+    bool keep_red = false;
     Arena& scratch() { return shared_arena ? *shared_arena : arena; }
 
     // prefetched tensors (npf_compute_prefetch): copied on up_stream into d_stage while the plan
@@ -171,6 +175,7 @@ void chain_term(Plan& p, int N, double2* d_out, const double2* W, bool accumulat
 // ----------------------------------------------------------------------------------------
 void split_term(Plan& p, int N, double2* d_out, const double2* W = nullptr, bool accumulate = false);
 void split_slab(Plan& p, int N, const int* prefix, double2* d_out);
+void split_drop_kept(Plan& p);   // reduction rows kept by keep_red are no longer valid
 void split_check(Plan& p);   // waits for the stream; throws if a deferred term's pipeline wait gave up
 size_t split_min_bytes(const Plan& p, int N);   // smallest budget a term is accepted with
 void split_release(Plan& p);

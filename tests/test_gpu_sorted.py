@@ -4,6 +4,7 @@ the sizes where their tables have remainders: odd n, one mode, segments of lengt
 several short segments, n just past a row radix, a mode subset of odd size, batches of a few upper
 indices, the FP32 form and a slab. Tolerances are the library's bars for the forms (1e-10, 1e-5)."""
 from math import comb
+from types import SimpleNamespace
 
 import numpy as np
 import pytest
@@ -84,3 +85,27 @@ def test_few_upper_indices_and_new_modes(npf, n, N):
         with pytest.raises(npf.NpfError) as e:
             p.term(N)
         assert e.value.status == npf.NPF_ERR_OOM
+
+
+@pytest.mark.parametrize("n", [27, 35])
+def test_interaction_shares_the_divided_entries(npf, n):
+    """Mode interactions reduce each order twice from one set of divided entries when it runs in one
+    batch: against the oracle, again after new modal data, and with a budget of few upper indices,
+    where nothing is kept."""
+    def system(seed):
+        lam, U, V, A3 = _odd_system(n, 3, seed)
+        return SimpleNamespace(n=n, lam=lam, U=U, V=V,
+                               tensors={2: S.random_packed_tensor_dense_fill(n, 2, 5), 3: A3})
+    one, two = system(3), system(4)
+    two.tensors = one.tensors
+    with npf.Plan(one.lam, one.U, one.V, 3) as p:
+        for N, t in one.tensors.items():
+            p.set_tensor(N, t)
+        for s in (one, two):
+            ref = oracle.interaction_npfs(s, 3, 0.1)
+            p.set_modes(s.lam, s.U, s.V)
+            for _ in range(2):
+                assert rel_fro(p.interaction(3, 0.1), ref) < 1e-10
+            assert rel_fro(p.term(3), oracle.psiN(s.tensors[3], n, 3, s.U, s.V, s.lam, p1_block=8)) < 1e-10
+        p.set_option(npf.OPT_MEM_BUDGET, 60e6 if n > 32 else 20e6)
+        assert rel_fro(p.interaction(3, 0.1), ref) < 1e-10
