@@ -11,7 +11,8 @@
 // epilogue recombines V = (L0 + L1 + L2) * 2^30 + rint(L3 * 2^30) exactly in 64-bit integers
 // (|V| <= 2^53, resolution 2^-30 of the L0 unit); the value is V * 2^(e_a + e_b - VEXP),
 // VEXP = 14 + 30. It then re-slices V for the next contraction (integer arithmetic, new exponent
-// shared by the next operand's K-row), or divides by the resonance denominator in native FP64.
+// shared by the next operand's K-row), keeps V itself for a regather, or divides by the resonance
+// denominator.
 //
 // Complex operands interleave (Re, Im) along K': row = [Re x_0, Im x_0, Re x_1, Im x_1, ...]
 // (K' = 256 for 128 complex entries). A fixed complex matrix W is stored as Re-row p =
@@ -163,19 +164,6 @@ __device__ __forceinline__ dfl two_sum(float a, float b)
     const float s = a + b;
     const float bb = s - a;
     return {s, (a - (s - bb)) + (b - bb)};
-}
-// V * 2^sc as a double-float (relative error ~2^-48) for |V| < 2^53. V is split into three
-// 21-bit pieces that are exact floats, so only 32-bit conversions are used: 64-bit integer <->
-// float conversions are slow on this GPU.
-__device__ __forceinline__ dfl df_from_i64(long long V, int sc)
-{
-    const int v2 = (int)(V >> 42);
-    const int v1 = (int)((V >> 21) & 0x1FFFFF);
-    const int v0 = (int)(V & 0x1FFFFF);
-    const dfl a = two_sum((float)v2 * 4398046511104.0f, (float)v1 * 2097152.0f);   // 2^42, 2^21
-    const dfl b = two_sum(a.hi, (float)v0);
-    const dfl r = df_norm(b.hi, b.lo + a.lo);
-    return {ldexpf(r.hi, sc), ldexpf(r.lo, sc)};
 }
 __device__ __forceinline__ double df_to_d(dfl a) { return (double)a.hi + (double)a.lo; }
 __device__ __forceinline__ dfl to_dfl(double x)
@@ -2155,7 +2143,7 @@ static void launch_rows(Plan& p, const char* name, const DataOp& A, const FixedO
     }
     {
         LaunchScope ls(&p.prof, name, p.stream);
-        // persistent: one CTA per SM (the shared memory allows one), tiles strided over CTAs
+        // persistent: one CTA per SM (the shared memory allows one), tiles strided over CTAs;
         // an odd stride keeps each CTA from seeing only one column tile (the column tiles of a
         // row tile differ in cost under the sorted-tuple masks)
         int64_t grid = std::min<int64_t>(a.num_tiles, sm_count());
@@ -2188,8 +2176,9 @@ static unsigned regather_parts(int64_t outers, int nrows)
     return (unsigned)std::max<int64_t>(1, std::min(all, want));
 }
 
-// Device memory of one order: V of S (16 bytes, n x P) and per upper index of a batch two buffers that the stages alternate (A: the operands of the mode products and of the
-// reduction, B: V and the divide's slots) plus the row exponents.
+// Device memory of one order: V of S (16 bytes, n x P) and per upper index of a batch two buffers
+// that the stages alternate (A: the operands of the mode products and of the reduction, B: V and the
+// divide's slots) plus the row exponents.
 template <int S>
 static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const double2* W, bool accumulate)
 {
@@ -2209,8 +2198,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     // K extent of an operand row: the radix 2^lg >= n
     const int lg = n <= 32 ? 5 : n <= 64 ? 6 : 7;
     const int rad = 1 << lg;
-    // complex columns per tile (the slab path runs untuned: 32 when the plan autotunes); the mode
-    // tiles are at most 32 wide (launch_rows)
+    // complex columns per tile: two accumulator sets of 32 fill TMEM, so the wider settings run 32 too
     const int bnc = p.tile_n == 16 ? 16 : 32;
 
     // ---- rows per upper index of every stage
@@ -2241,7 +2229,8 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     const size_t all_bytes = s_bytes + (size_t)nm * (a_per + b_per + e_per) + wbytes + 10 * 256 + 1024;
     Arena& ar = p.scratch();
     bool own_red = !slab && red_bytes <= ((size_t)64 << 20);
-    bool keep = !slab && p.keep_red && rhi - rlo == nm && red_bytes <= ((size_t)256 << 20);
+    // (under a budget of the caller's nothing is kept beside the scratch)
+    bool keep = !slab && p.keep_red && !p.mem_budget && rhi - rlo == nm && red_bytes <= ((size_t)256 << 20);
     int ib = nm;
     // (scratch that holds everything already needs no look at the free memory)
     if (p.mem_budget || ar.cap < all_bytes + (own_red ? red_bytes : 0)) {
@@ -2259,11 +2248,17 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
             if (so.kept[N]) NPF_CUDA(cudaStreamSynchronize(p.stream));
             cudaFree(so.kept[N]); cudaFree(so.kept_e[N]);
             so.kept[N] = nullptr; so.kept_e[N] = nullptr; so.kept_bytes[N] = 0;
-            NPF_CUDA(cudaMalloc(&so.kept[N], red_bytes));
-            NPF_CUDA(cudaMalloc(&so.kept_e[N], eb));
-            so.kept_bytes[N] = red_bytes + eb;
+            so.kept_ok[N] = false;
+            if (cudaMalloc(&so.kept[N], red_bytes) != cudaSuccess || cudaMalloc(&so.kept_e[N], eb) != cudaSuccess) {
+                cudaGetLastError();   // no room: the rows are formed again for every weight matrix
+                cudaFree(so.kept[N]);
+                so.kept[N] = nullptr; so.kept_e[N] = nullptr;
+                keep = false;
+            } else {
+                so.kept_bytes[N] = red_bytes + eb;
+            }
         }
-        own_red = false;   // (no room in the scratch for it)
+        if (keep) own_red = false;   // (no room in the scratch for it)
     }
     const bool again = keep && W && so.kept_ok[N];   // only the reduction is left to do
     ar.reserve(s_bytes + (size_t)ib * (a_per + b_per + e_per) + wbytes + (own_red ? red_bytes : 0) + 10 * 256 + 1024);

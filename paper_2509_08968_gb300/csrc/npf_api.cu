@@ -190,7 +190,7 @@ void load_modes(Plan& p, const npf_c128* eigvals, const npf_c128* U, const npf_c
 using TuneKey = std::array<int, 5>;
 std::mutex g_tune_mu;
 std::map<TuneKey, int> g_tuned;
-constexpr int kTileCandidates[4] = {16, 32, 48, 64};
+constexpr int kTileCandidates[2] = {16, 32};   // (48 and 64 run 32-column tiles)
 
 TuneKey tune_key(const Plan& p, int N) { return {p.n, N, p.precision, p.slices, p.divide}; }
 
@@ -205,7 +205,7 @@ int tuned_tile(Plan& p, int N)
     NPF_CUDA(cudaEventCreate(&e0));
     NPF_CUDA(cudaEventCreate(&e1));
     float best = std::numeric_limits<float>::infinity();
-    int best_tile = 64;
+    int best_tile = 32;
     try {
         for (int t : kTileCandidates) {
             p.tile_n = t;
