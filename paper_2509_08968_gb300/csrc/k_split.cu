@@ -1417,9 +1417,10 @@ __global__ void k_term_init(const __grid_constant__ TermInit a)
         zero_head<S>(t, a.N, a.nm, a.kc, a.lg, a.Q, a.tuples, a.planes, a.plane_stride_u32);
 }
 
-// Operand rows of a mode product from the exact 64-bit values V of the stage before (EPI_V): one
-// warp per row (outer, sorted M-tuple of a's). Lane t covers a = lane + 32 t: it gathers
-// V[outer][rank(sort(tuple, a))] and writes its digits. V is in units of 2^(ea + eb - VEXP).
+// Operand rows of a mode product from the exact 64-bit values V of the stage before (EPI_V): a warp
+// takes RW rows (outer, sorted M-tuple of a's) at a time, CH chunks of 32 entries a row: lane t
+// covers a = t, t + 32, .. It gathers V[outer][rank(sort(tuple, a))] and writes its digits. V is in
+// units of 2^(ea + eb - VEXP).
 //   SRC 0: V of the first mode product, outer = (i, p); ea by i, eb by p
 //   SRC 1: V of the second (order 4), outer = (i, p_3 <= p_4); ea by its operand row (i, p_4, rank),
 //          eb by p_3
@@ -1427,10 +1428,13 @@ __global__ void k_term_init(const __grid_constant__ TermInit a)
 //          the rows share the exponent rowE[i]; the others get their exact one (largest bit length)
 // Neighbouring rows gather neighbouring entries (colexicographic rank), so the warps of a block
 // share sectors. A block takes one outer index and a strided share of its rows, so that nothing
-// but the gather, the shifts and the digits is left per row: the kernel is bound by its
-// instructions (IPC 0.72 a scheduler) as much as by its HBM writes (4 S bytes an entry against 16 read
-// per source entry).
-template <int S, int M, int SRC>
+// but the gather, the shifts and the digits is left per row: a rank is one of M + 1 row constants
+// plus a binomial of the lane's a, kept in registers, and a plane's address a 32-bit offset from the
+// block's. Computing whole ranks and 64-bit addresses per entry, a row a warp: 5.50 against 4.51 ms at
+// n = 60, order 4; 1.16 against 1.10 at n = 120, order 3 (6.65 GB: 6.0 TB/s). What bounds it is mixed:
+// HBM writes (4 S bytes an entry against 16 read per source entry) at n = 120, the scattered half of
+// the gathers and the integer instructions (IPC 0.65 a scheduler) below.
+template <int S, int M, int SRC, int CH, int RW>
 __global__ void __launch_bounds__(256)
     k_regather(const longlong2* __restrict__ V, int64_t Rsrc, int n, int nm, int nt, const uint32_t* __restrict__ ttup,
                const int* __restrict__ ea, const int* __restrict__ eb, const int* __restrict__ rowE, int lg, int kout,
@@ -1439,6 +1443,14 @@ __global__ void __launch_bounds__(256)
 {
     const int lane = threadIdx.x & 31;
     const unsigned outer = blockIdx.x / parts;
+    int au[CH], bin2[CH], bin3[CH], bin4[CH];                // a; rank of (0, a), (0, 0, a), (0, 0, 0, a)
+#pragma unroll
+    for (int c = 0; c < CH; ++c) {
+        au[c] = lane + 32 * c;
+        bin2[c] = rank2(0, au[c]);
+        bin3[c] = M >= 2 ? rank3(0, 0, au[c]) : 0;
+        bin4[c] = M >= 3 ? rank4(0, 0, 0, au[c]) : 0;
+    }
     pdl_wait();
     int e0;
     const int* earow = ea;
@@ -1451,80 +1463,87 @@ __global__ void __launch_bounds__(256)
         if (SRC == 1) earow = ea + ((int64_t)i * nm + (int)((tp >> 8) & 255u)) * Rsrc;
     }
     const longlong2* src = V + outer * Rsrc;
+    uint32_t* dst[S];
+#pragma unroll
+    for (int s = 0; s < S; ++s) dst[s] = planes + s * plane_stride_u32 + ((int64_t)outer * Rdst << lg);
+    int* oexp = SRC == 2 ? nullptr : out_exp + outer * Rdst;
     const int Eall = SRC == 2 ? rowE[outer] : 0;
-    for (int row = (int)(blockIdx.x - outer * parts) * 8 + (int)(threadIdx.x >> 5); row < nrows;
-         row += (int)parts * 8) {
-        int x = row, y = 0, z = 0;
-        if (M >= 2) {
-            const uint32_t pk = tuples[row];
-            x = (int)(pk & 255u);
-            y = (int)((pk >> 8) & 255u);
-            z = (int)((pk >> 16) & 255u);
-        }
-        longlong2 v[4];
-        int ex[4];
+    const int step = (int)parts * 8 * RW;
+    for (int row = ((int)(blockIdx.x - outer * parts) * 8 + (int)(threadIdx.x >> 5)) * RW; row < nrows; row += step) {
+        longlong2 v[RW][CH];
+        int ex[RW][CH], E[RW];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            if (32 * k >= n) break;
-            const int a = lane + 32 * k;
-            v[k] = make_longlong2(0ll, 0ll);
-            ex[k] = 0;
-            if (a < n) {
-                int rk;
-                if (M == 0) rk = a;
-                else if (M == 1) rk = rank2(min(a, x), max(a, x));
-                else if (M == 2) {
-                    const int lo = min(a, x), hi = max(a, y);
-                    rk = rank3(lo, x + y + a - lo - hi, hi);
-                } else {
-                    const int lo = min(a, x), hi = max(a, z);
-                    const int p = a <= y ? max(a, x) : y, q = a <= y ? y : min(a, z);   // the middle two
-                    rk = rank4(lo, p, q, hi);
+        for (int j = 0; j < RW; ++j) {
+            const int r = min(row + j, nrows - 1);           // (a last round repeats its last row)
+            int x = r, y = 0, z = 0;
+            if (M >= 2) {
+                const uint32_t pk = tuples[r];
+                x = (int)(pk & 255u);
+                y = (int)((pk >> 8) & 255u);
+                z = (int)((pk >> 16) & 255u);
+            }
+            // rank less the part of a: a below x, between x and y, between y and z, above
+            const int last = M >= 3 ? rank4(0, 0, 0, z) : M == 2 ? rank3(0, 0, y) : rank2(0, x);
+            const int c0 = M >= 3 ? last + rank3(0, x, y) : M == 2 ? last + rank2(0, x) : last;
+            const int c1 = M >= 3 ? last + rank3(0, 0, y) + x : M == 2 ? last + x : x;
+            const int c2 = M >= 3 ? last + rank2(x, y) : rank2(x, y);
+            const int c3 = rank3(x, y, z);
+#pragma unroll
+            for (int c = 0; c < CH; ++c) {
+                v[j][c] = make_longlong2(0ll, 0ll);
+                ex[j][c] = 0;
+                const int a = au[c];
+                if (a < n) {
+                    int rk = a;
+                    if (M == 1) rk = a <= x ? c0 + a : c1 + bin2[c];
+                    if (M == 2) rk = a <= x ? c0 + a : a <= y ? c1 + bin2[c] : c2 + bin3[c];
+                    if (M == 3) rk = a <= x ? c0 + a : a <= y ? c1 + bin2[c] : a <= z ? c2 + bin3[c] : c3 + bin4[c];
+                    v[j][c] = src[rk];
+                    if (SRC != 0) ex[j][c] = earow[rk];
                 }
-                v[k] = src[rk];
-                if (SRC != 0) ex[k] = earow[rk];
             }
         }
-        int E = Eall;
-        if (SRC == 0) {
-            // one unit for all entries: the bit length of the OR of their magnitudes (the lowest bit
-            // as it is, so that a minus one counts)
-            unsigned long long m = 0ull;
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (32 * k < n)
-                    m |= (unsigned long long)((v[k].x ^ (v[k].x >> 63)) | (v[k].y ^ (v[k].y >> 63)) |
-                                              ((v[k].x | v[k].y) & 1));
-            const unsigned hi = __reduce_or_sync(0xffffffffu, (unsigned)(m >> 32));
-            const unsigned lo = __reduce_or_sync(0xffffffffu, (unsigned)m);
-            E = hi | lo ? (hi ? 64 - __clz((int)hi) : 32 - __clz((int)lo)) + e0 : EXP_NONE;
-        } else if (SRC == 1) {
-            int key = 0;
+        for (int j = 0; j < RW; ++j) {
+            E[j] = Eall;
+            if (SRC == 0) {
+                // one unit for all entries: the bit length of the OR of their magnitudes (the lowest
+                // bit as it is, so that a minus one counts)
+                unsigned long long m = 0ull;
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (32 * k < n && (v[k].x | v[k].y)) key = max(key, bitlen(v[k]) + ex[k] + e0 + 8192);
-            key = (int)__reduce_max_sync(0xffffffffu, (unsigned)key);
-            E = key ? key - 8192 : EXP_NONE;
-        }
-        const int sh = e0 - E + 7 + 8 * (S - 1);
-        const int64_t rowp = outer * Rdst + row;
-        uint32_t* dst = planes + (rowp << lg) + lane;
+                for (int c = 0; c < CH; ++c)
+                    m |= (unsigned long long)((v[j][c].x ^ (v[j][c].x >> 63)) | (v[j][c].y ^ (v[j][c].y >> 63)) |
+                                              ((v[j][c].x | v[j][c].y) & 1));
+                const unsigned hi = __reduce_or_sync(0xffffffffu, (unsigned)(m >> 32));
+                const unsigned lo = __reduce_or_sync(0xffffffffu, (unsigned)m);
+                E[j] = hi | lo ? (hi ? 64 - __clz((int)hi) : 32 - __clz((int)lo)) + e0 : EXP_NONE;
+            } else if (SRC == 1) {
+                int key = 0;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            if (32 * k >= kout) break;
-            if (lane + 32 * k < kout) {
-                uint32_t w[S];
-                if (E != EXP_NONE && 32 * k < n) {
-                    digit_pairs<S>(shift_full(v[k].x, sh + ex[k]), shift_full(v[k].y, sh + ex[k]), w);
-                } else {
-#pragma unroll
-                    for (int s = 0; s < S; ++s) w[s] = 0u;
-                }
-#pragma unroll
-                for (int s = 0; s < S; ++s) dst[s * plane_stride_u32 + 32 * k] = w[s];
+                for (int c = 0; c < CH; ++c)
+                    if (v[j][c].x | v[j][c].y) key = max(key, bitlen(v[j][c]) + ex[j][c] + e0 + 8192);
+                key = (int)__reduce_max_sync(0xffffffffu, (unsigned)key);
+                E[j] = key ? key - 8192 : EXP_NONE;
             }
+            if (RW > 1 && row + j >= nrows) break;
+            const int sh = e0 - E[j] + 7 + 8 * (S - 1);
+            const uint32_t at = ((uint32_t)(row + j) << lg) + (uint32_t)lane;
+#pragma unroll
+            for (int c = 0; c < CH; ++c) {
+                if (au[c] < kout) {
+                    uint32_t w[S];
+                    if (E[j] != EXP_NONE) {
+                        digit_pairs<S>(shift_full(v[j][c].x, sh + ex[j][c]), shift_full(v[j][c].y, sh + ex[j][c]), w);
+                    } else {
+#pragma unroll
+                        for (int s = 0; s < S; ++s) w[s] = 0u;
+                    }
+#pragma unroll
+                    for (int s = 0; s < S; ++s) dst[s][at + 32 * c] = w[s];
+                }
+            }
+            if (SRC != 2 && lane == 0) oexp[row + j] = E[j];
         }
-        if (SRC != 2 && lane == 0) out_exp[rowp] = E;
     }
 }
 
@@ -2168,10 +2187,24 @@ static void launch_rows(Plan& p, const char* name, const DataOp& A, const FixedO
 
 static double factorial(int N) { double f = 1; for (int t = 2; t <= N; ++t) f *= t; return f; }
 
-// Blocks that share one outer index of a regather: about eight rows a warp, more blocks when few.
-static unsigned regather_parts(int64_t outers, int nrows)
+// The regather's variant: 32-entry chunks of a row (CH), and the rows that a warp takes at a time (RW),
+// so that three to six gathers are in flight. Twice as many rows were slower (n = 60, order 4: 4.51
+// against 4.88 ms; n = 120, order 3: 1.10 against 1.20), one row less slower at n = 60 and 75.
+static constexpr int regather_rows(int ch) { return ch == 1 ? 4 : ch <= 3 ? 2 : 1; }
+template <int S, int M, int SRC>
+static decltype(&k_regather<S, M, SRC, 4, regather_rows(4)>) regather_kernel(int n)
 {
-    const int64_t all = (nrows + 7) / 8;                         // one row a warp
+    return n <= 32   ? k_regather<S, M, SRC, 1, regather_rows(1)>
+           : n <= 64 ? k_regather<S, M, SRC, 2, regather_rows(2)>
+           : n <= 96 ? k_regather<S, M, SRC, 3, regather_rows(3)>
+                     : k_regather<S, M, SRC, 4, regather_rows(4)>;
+}
+
+// Blocks that share one outer index of a regather: about eight rounds a warp, more blocks when few.
+static unsigned regather_parts(int64_t outers, int nrows, int n)
+{
+    const int rows = 8 * regather_rows((n + 31) / 32);           // a round's
+    const int64_t all = (nrows + rows - 1) / rows;               // one round a warp
     const int64_t want = std::max<int64_t>((all + 7) / 8, (8 * sm_count() + outers - 1) / std::max<int64_t>(outers, 1));
     return (unsigned)std::max<int64_t>(1, std::min(all, want));
 }
@@ -2352,10 +2385,10 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
         auto plane = [&](int64_t R) { return cur * R * rad; };   // plane stride in complex entries
         if (!again) {
             LaunchScope ls(&p.prof, "split_expand", p.stream);
-            auto kern = N == 1 ? k_regather<S, 0, 2> : N == 2 ? k_regather<S, 1, 2>
-                      : N == 3 ? k_regather<S, 2, 2> : k_regather<S, 3, 2>;
+            auto kern = N == 1 ? regather_kernel<S, 0, 2>(n) : N == 2 ? regather_kernel<S, 1, 2>(n)
+                      : N == 3 ? regather_kernel<S, 2, 2>(n) : regather_kernel<S, 3, 2>(n);
             const int nrows = (int)so.natup[N - 1];
-            const unsigned parts = regather_parts(cur, nrows);
+            const unsigned parts = regather_parts(cur, nrows, n);
             launch_dependent(kern, dim3((unsigned)cur * parts), dim3(256), 0, p.stream, Sv + (int64_t)i0 * Prows, Prows,
                              n, nm, 1, nullptr, so.at_e[N], so.psir_e + i0, sE + i0, lg, kout, nrows, R0, parts,
                              so.atup[N - 1], (uint32_t*)bufA, plane(R0), nullptr);
@@ -2378,8 +2411,8 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
             const int nrows = pairs ? (int)so.natup[2] : n;
             const int64_t Rdst = pairs ? nrows : rad;
             LaunchScope ls(&p.prof, "split_regather", p.stream);
-            const unsigned parts = regather_parts(outs, nrows);
-            auto kern = pairs ? k_regather<S, 2, 0> : c == 1 ? k_regather<S, 1, 0> : k_regather<S, 1, 1>;
+            const unsigned parts = regather_parts(outs, nrows, n);
+            auto kern = pairs ? regather_kernel<S, 2, 0>(n) : c == 1 ? regather_kernel<S, 1, 0>(n) : regather_kernel<S, 1, 1>(n);
             launch_dependent(kern, dim3((unsigned)outs * parts), dim3(256), 0, p.stream, (const longlong2*)bufB, Ra, n,
                              nm, (int)(outs / cur), base0.ttup, c == 1 ? sE + i0 : E1, so.phi_e, nullptr, lg, kout,
                              nrows, Rdst, parts, so.atup[2], (uint32_t*)bufA, outs * Rdst * rad, pairs ? E1 : E2);

@@ -65,6 +65,18 @@ def test_subset_odd_sizes(npf, n, N, m):
         assert rel_fro(p.term(N), full) < 1e-12
 
 
+@pytest.mark.parametrize("n,N,m", [(32, 4, 3), (33, 4, 3), (64, 3, 4), (96, 3, 3), (97, 3, 3)])
+def test_regather_chunks(npf, n, N, m):
+    """Sizes on both sides of the regather's variants (1 to 4 chunks of 32 entries a row)."""
+    lam, U, V, A = _odd_system(n, N, 60 * n + N)
+    modes = np.random.default_rng(n).permutation(n)[:m]
+    ref = oracle.psiN_subset(A, n, N, U, V, lam, modes)
+    with npf.Plan(lam, U, V, N) as p:
+        p.set_tensor(N, A)
+        p.set_mode_subset(modes)
+        assert rel_fro(p.term(N), ref) < 1e-10
+
+
 @pytest.mark.parametrize("n,N", [(9, 3), (11, 4), (35, 3)])
 def test_few_upper_indices_and_new_modes(npf, n, N):
     """Batches of a few upper indices, and modal data replaced in a plan whose tables exist."""
