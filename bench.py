@@ -294,7 +294,7 @@ def main():
     ap.add_argument("--cpu-sample", type=float, default=0.0, help=argparse.SUPPRESS)
     ap.add_argument("--no-e2e", action="store_true")
     ap.add_argument("--tile-n", type=int, default=0,
-                    help="complex columns per tensor-core tile (16/32/48/64; 0 = library default)")
+                    help="complex columns per tensor-core tile (16 or 32; 48 and 64 run 32; 0 = library default)")
     ap.add_argument("--modes", type=int, default=0,
                     help="critical-mode subset: the m least-damped modes (0 = all modes)")
     ap.add_argument("--mem-budget", type=float, default=0.0,
@@ -407,7 +407,7 @@ def main():
     roof = None
     if prof:
         name, (cnt, tot_ms) = max(prof.items(), key=lambda kv: kv[1][1])
-        work, kind = algorithmic_work_per_step(name, n, args.precision, m_modes)
+        work, kind = formed_work_per_step(name, n, args.precision, m_modes)
         if work is not None:
             per_launch = work * args.steps / cnt
             avg_ms = tot_ms / cnt
@@ -652,10 +652,10 @@ def run_batch(args, world, rank, local, dist):
     for s, N in systems:
         n = s.n
         f = n * comb(n + N - 1, N) * n * 4
-        f += sum(n * comb(n + c - 1, c) * a_part(n, N, c) * n * 8 for c in range(1, N))
+        f += sum(n * comb(n + c - 1, c) * comb(n + N - c - 1, N - c) * n * 8 for c in range(1, N))
         f += n * comb(n + N - 1, N) * n * 8 + n * comb(n + N - 1, N) * n * 8
         f *= pairs
-        t = args.tile_n or npf.tuned_tile(n, N, args.precision) or 64
+        t = min(args.tile_n or npf.tuned_tile(n, N, args.precision) or 32, 32)
         tiles[f"n{n}o{N}"] = t
         # padded tile shape: the row radix (32 / 64 / 128 >= n) per innermost row index, K' in
         # chunks of 32, t columns
@@ -821,11 +821,11 @@ def a_part(n, N, c):
 
 
 def algorithmic_work_per_step(name, n, precision, m=None):
-    """Algorithmic work of every launch of `name` in one step, as (amount, kind).
+    """Algorithmic work of every launch of `name` in one step, as (amount, kind), for an
+    implementation that sorts the p's and at most a pair of the a's; formed_work_per_step counts
+    what the library's kernels form.
 
-    Tensor kernels (kind "flops"): executed BF16 tensor flops of the work the symmetric method
-    needs -- only non-decreasing lower-index tuples are formed, indices unpadded (n, not 128);
-    a complex multiply-add over K is 8 real flops, times the slice pairs. Per order N with
+    Tensor kernels (kind "flops"): BF16 tensor flops, indices unpadded (n, not 128); a complex multiply-add over K is 8 real flops, times the slice pairs. Per order N with
     C(m, r) = binomial:
       split_upper_contraction : C(n+N-1,N) packed tuples x n (i) x n (j) x 4 (real x complex)
       split_mode_product      : sum_{c=1..N-1} n (i) x C(n+c-1,c) (sorted p's) x A_c (a's)
@@ -859,6 +859,28 @@ def algorithmic_work_per_step(name, n, precision, m=None):
         else:
             return None, None
     return tot, ("bytes" if name == "split_expand" else "flops")
+
+
+def formed_work_per_step(name, n, precision, m=None):
+    """The work of `name` on the tuples the library forms, as (amount, kind): every intermediate
+    holds sorted p's and sorted a's, C(r + k - 1, k) of the k-tuples over r. Rooflines use it.
+
+      split_mode_product : sum_{c=1..N-1} n (i) x C(n+c-1,c) (p's) x C(n+N-c-1,N-c) (a's) x n (K) x 8
+      split_expand, split_regather (bytes): 16 a sorted entry read, 4 S an entry of every row
+                           (sorted a's less one, K = the remaining a) written
+    The other kernels' work is algorithmic_work_per_step's."""
+    from math import comb
+    m = n if m is None else m
+    srt = lambda r, k: comb(r + k - 1, k)
+    if name == "split_mode_product":
+        return PAIRS[precision] * sum(m * srt(m, c) * srt(n, N - c) * n * 8
+                                      for N in ORDERS for c in range(1, N)), "flops"
+    if name in ("split_expand", "split_regather"):
+        # the upper contraction's output (c = 0), or those of the mode products c = 1 .. N - 2
+        return sum(m * srt(m, c) * (16 * srt(n, N - c) + 4 * SLICES[precision] * srt(n, N - c - 1) * n)
+                   for N in ORDERS for c in ((0,) if name == "split_expand" else range(1, N - 1))), "bytes"
+    return algorithmic_work_per_step(name, n, precision, m)
+
 
 
 if __name__ == "__main__":
