@@ -165,6 +165,20 @@ __device__ __forceinline__ dfl two_sum(float a, float b)
     const float bb = s - a;
     return {s, (a - (s - bb)) + (b - bb)};
 }
+// a b + c d as the exact leading sum s + e of the two products' leading parts, with the rest (their
+// rounding errors and the cross terms; error a few 2^-47 of |a b| + |c d|) in e, not normalised: 16
+// operations where two df_mul and a df_add take 27.
+__device__ __forceinline__ dfl df_dot2(dfl a, dfl b, dfl c, dfl d)
+{
+    const float p = a.hi * b.hi, q = c.hi * d.hi;
+    float e = fmaf(a.hi, b.hi, -p) + fmaf(c.hi, d.hi, -q);
+    e = fmaf(a.hi, b.lo, e);
+    e = fmaf(a.lo, b.hi, e);
+    e = fmaf(c.hi, d.lo, e);
+    e = fmaf(c.lo, d.hi, e);
+    const dfl s = two_sum(p, q);
+    return {s.hi, s.lo + e};
+}
 __device__ __forceinline__ double df_to_d(dfl a) { return (double)a.hi + (double)a.lo; }
 __device__ __forceinline__ dfl to_dfl(double x)
 {
@@ -1162,6 +1176,16 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
 #pragma unroll 1
                 for (int h = 0; h < 4; ++h) {
                     const int c2 = cbeg + 2 * h;
+                    // the weights of these columns, asked for before the accumulators (of a valid row and
+                    // column in any case): 1.44 -> 1.17 ms a call at n = 120, order 3 (n = 60, order 4: 1.72
+                    // -> 1.62); a round ahead of them spilled registers (1.73). Order 3: the whole weight W[p_1][k] W[p_2][k]; order 4: that,
+                    // and W[p_3][k] unless it is left to the sum
+                    float4 w4[2];
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        const int qa = min(qbase + c2 + c, args.ncv - 1);
+                        w4[c] = pre >= 0 ? __ldg(args.wpre + (int64_t)qa * args.ldw + pre) : __ldg(args.psi_df + qa * n + pin);
+                    }
                     uint32_t rv[4][2], iv[4][2];
                     load_levels<S, 2>(trow + min(c2, bnc - 2), lstride, rv);
                     load_levels<S, 2>(trow + bnc + min(c2, bnc - 2), lstride, iv);
@@ -1180,20 +1204,16 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                                 gr = {ldexpf(gr.hi, sc - s1), ldexpf(gr.lo, sc - s1)};
                                 gi = {ldexpf(gi.hi, sc - s1), ldexpf(gi.lo, sc - s1)};
                             }
-                            // order 3: the whole weight W[p_1][k] W[p_2][k]; order 4: that, and
-                            // W[p_3][k] unless it is left to the sum
-                            const float4 w = pre >= 0 ? __ldg(args.wpre + (int64_t)qc * args.ldw + pre)
-                                                      : __ldg(args.psi_df + qc * n + pin);
-                            dfl wr = {w.x, w.y}, wi = {w.z, w.w};
+                            dfl wr = {w4[c].x, w4[c].y}, wi = {w4[c].z, w4[c].w};
                             if (N >= 4 && !uni) {
                                 const float4 x = __ldg(args.psi_df + qc * n + pin);
                                 const dfl xr = {x.x, x.y}, xi = {x.z, x.w};
-                                const dfl tr = df_add(df_mul(wr, xr), df_neg(df_mul(wi, xi)));
-                                wi = df_add(df_mul(wr, xi), df_mul(wi, xr));
+                                const dfl tr = df_dot2(wr, xr, df_neg(wi), xi);
+                                wi = df_dot2(wr, xi, wi, xr);
                                 wr = tr;
                             }
-                            sr[c] = df_add(sr[c], df_add(df_mul(gr, wr), df_neg(df_mul(gi, wi))));
-                            si[c] = df_add(si[c], df_add(df_mul(gr, wi), df_mul(gi, wr)));
+                            sr[c] = df_add(sr[c], df_dot2(gr, wr, df_neg(gi), wi));
+                            si[c] = df_add(si[c], df_dot2(gr, wi, gi, wr));
                         }
                     }
                     const dfl r0 = sr[0], r1 = sr[1], i0 = si[0], i1 = si[1];
@@ -1300,7 +1320,8 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                                 Dr = tfl_sum(tfl{sig[0], sig[NP], sig[2 * NP]}, lamt[2 * cl]);
                                 Di = tfl_sum(tfl{sig[3 * NP], sig[4 * NP], sig[5 * NP]}, lamt[2 * cl + 1]);
                             }
-                            dfl m2 = df_add(df_mul(Dr, Dr), df_mul(Di, Di));
+                            dfl m2 = df_dot2(Dr, Dr, Di, Di);      // (no cancellation: one step normalises)
+                            m2 = df_norm(m2.hi, m2.lo);
                             if (args.divide && m2.hi < args.eps2f) {   // Alg. 2 step 9
                                 Dr = to_dfl(args.eps);
                                 Di = {0.f, 0.f};
@@ -1310,8 +1331,8 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                             const dfl e1 = df_add(dfl{1.f, 0.f}, df_neg(df_mul(m2, dfl{r0, 0.f})));
                             const dfl inv = df_add(dfl{r0, 0.f}, df_mul(dfl{r0, 0.f}, e1));
                             const dfl rf = df_mul(inv, rcp[den * (qc == firstp ? run1 + 1 : 1)]);
-                            const dfl nr = df_add(df_mul(vr, Dr), df_mul(vi, Di));
-                            const dfl ni = df_add(df_mul(vi, Dr), df_neg(df_mul(vr, Di)));
+                            const dfl nr = df_dot2(vr, Dr, vi, Di);
+                            const dfl ni = df_dot2(vi, Dr, df_neg(vr), Di);
                             const int e = ea + eb - VEXP + 30 + 7 + 8 * (S - 1) - E;
                             const dfl qr = df_mul(nr, rf), qi = df_mul(ni, rf);
                             digit_pairs<S>(df_round_i64(dfl{ldexpf(qr.hi, e), ldexpf(qr.lo, e)}),
