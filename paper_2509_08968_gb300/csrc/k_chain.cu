@@ -18,7 +18,7 @@
 // (k_fp64.cu) it does a third of the operations at order 3: n = 60, orders 2 and 3, 28.4 -> 9.1 ms
 // (2.1 of them for tail blocks and latency); n = 8, order 3, 184 -> 59 us. Against the tensor-core
 // chain (eight launches and more an order) it is two launches, which is what small systems wait
-// for: n = 10, orders 2 and 3, 243 -> 58 us. One block per (i, p_N) keeps 24 n^2 bytes at order 3, so
+// for: n = 10, orders 2 and 3, 243 -> 62 us. One block per (i, p_N) keeps 24 n^2 bytes at order 3, so
 // that two blocks share an SM up to n = 66.
 #include <algorithm>
 

@@ -508,7 +508,7 @@ struct RowCfg {
     static_assert(SMEM <= SMEM_MAX, "shared memory");
 };
 
-// Position of a tile (column tile fastest, but for the reduction).
+// Position of a tile (column tile fastest).
 struct TilePos {
     int ct;         // column tile
     int outer;      // upper index of the launch (RB > 0)
@@ -520,11 +520,10 @@ __device__ __forceinline__ TilePos tile_pos(const RowArgs& a, int64_t tile)
     const unsigned t = (unsigned)tile;   // (launch_rows bounds the tile count to 2^31)
     const unsigned rb = a.lgncol >= 0 ? t >> a.lgncol : t / (unsigned)a.ncol_tiles;
     TilePos p;
-    if (a.kfrom) {   // the reduction: row block fastest, then column tile, then upper index
-        const unsigned g = t / (unsigned)a.RB;
-        p.outer = (int)(g / (unsigned)a.ncol_tiles);
-        p.ct = (int)(g - (unsigned)p.outer * (unsigned)a.ncol_tiles);
-        p.rr0 = (int)(t - g * (unsigned)a.RB) * NP;
+    if (a.kfrom) {   // the reduction: `tile` is a row block, the block's column tile changes every 32 of them
+        p.outer = (int)(t / (unsigned)a.RB);
+        p.ct = (int)((blockIdx.x + (t >> 5)) % (unsigned)a.ncol_tiles);
+        p.rr0 = (int)(t - (unsigned)p.outer * (unsigned)a.RB) * NP;
         p.row0 = (int64_t)p.outer * a.R + p.rr0;
         return p;
     }
@@ -673,11 +672,12 @@ static __global__ void k_tile_list(RowArgs a, int lg, int* __restrict__ list, un
 //   warps 18, 19     : set-up: the next tile's tables (row exponents and indices, eigenvalue sums,
 //                      output rows) into the other of two buffers. Chains of dependent global loads,
 //                      they took 2 to 7 us a tile in front of the epilogue.
-// Bound per 32-column tile of a mode product at n = 120: shared memory (MMA operand reads 1.08 MB and TMA
-// writes 0.59 MB at 128 bytes a clock: 6.3 us; MMAs 5.4 us) of 7.1 us measured; below n = 64 and in
-// the divide and the reduction the epilogue. 32-column tiles in every mode: an epilogue and the next
+// Bound per 32-column tile of a mode product at n = 120: 7.1 us, 5.4 of them its 315 MMAs (without any
+// TMA load the launches take 2.64 ms instead of 3.06); shared memory carries 1.08 MB of MMA operand
+// reads and 0.59 MB of TMA writes meanwhile (6.3 us at 128 bytes a clock). Below n = 64 and in the
+// divide and the reduction the epilogue bounds it. 32-column tiles in every mode: an epilogue and the next
 // tile's MMAs overlap, which one 64-column tile with all 512 TMEM columns (and a level-3 hold in
-// shared memory) allowed in part only: divide at n = 120, order 3, 1.83 -> 1.45 ms a call (24 us a
+// shared memory) allowed in part only: divide at n = 120, order 3, 1.83 -> 1.45 ms a call (1.39 now) (24 us a
 // 64-column tile before, 13 us a 32-column one now, of which the kept columns are fewer).
 template <int S, int MODE, bool SUBB>
 __global__ void __launch_bounds__(ROW_THREADS, 1)
@@ -738,11 +738,15 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
     auto tile_at = [&](int64_t k) -> int64_t {
         return k >= nloop ? 0 : args.tiles ? (int64_t)args.tiles[k] : k;
     };
-    // The reduction takes consecutive tiles (row blocks of one upper index and column tile), so that its
-    // epilogue can sum over them in registers; the others take every gridDim.x-th.
-    const int64_t per = (nloop + gridDim.x - 1) / gridDim.x;
-    const int64_t kbeg = MODE == EPI_REDUCE ? per * blockIdx.x : blockIdx.x;
-    const int64_t kend = MODE == EPI_REDUCE ? min(nloop, kbeg + per) : nloop;
+    // The reduction takes consecutive row blocks, so that its epilogue can sum over them in registers. The
+    // ncol_tiles blocks of a group walk the same row blocks side by side, each on another column tile (in
+    // turn, since the last one is narrower), so that the rows are read from HBM once: with each column
+    // tile walked by itself they were read once for each (1.7 GB in 338 us at n = 120, order 3, 34 upper
+    // indices). The other modes take every gridDim.x-th tile.
+    const int64_t nred = args.num_tiles / args.ncol_tiles, groups = gridDim.x / (unsigned)args.ncol_tiles;
+    const int64_t per = (nred + groups - 1) / max(groups, (int64_t)1);
+    const int64_t kbeg = MODE == EPI_REDUCE ? per * (blockIdx.x / (unsigned)args.ncol_tiles) : blockIdx.x;
+    const int64_t kend = MODE == EPI_REDUCE ? min(nred, kbeg + per) : nloop;
     const int64_t kstep = MODE == EPI_REDUCE ? 1 : gridDim.x;
     const uint32_t lstride = (uint32_t)bnr;    // TMEM columns between levels
 
@@ -838,7 +842,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
             next = tile_at(k + kstep);
             const int buf = (int)(t & 1);
             uint8_t* tb = tables + C::TILE + buf * C::TILE_BYTES;
-            unsigned long long* trc = args.trace ? args.trace + tile * 6 : nullptr;
+            unsigned long long* trc = args.trace ? args.trace + (MODE == EPI_REDUCE ? tile * args.ncol_tiles + tp.ct : tile) * 6 : nullptr;
             alive = __all_sync(0xffffffffu, tc::mbar_wait_idle(&sempty[buf], ((t >> 1) & 1) ^ 1, args.err, kErrTimeout));
             const unsigned long long t0 = trc ? global_ns() : 0ull;
             const int qbase = tp.ct * bnc;
@@ -1025,7 +1029,10 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
         uint32_t t = 0;
         for (int64_t k = kbeg; k < kend; k += kstep) {
             const int buf = (int)(t & 1);
-            unsigned long long* trc = args.trace ? args.trace + (args.tiles ? (int64_t)args.tiles[k] : k) * 6 : nullptr;
+            unsigned long long* trc = nullptr;
+            if (args.trace)
+                trc = args.trace + 6 * (MODE == EPI_REDUCE ? k * args.ncol_tiles + tile_pos(args, k).ct
+                                        : args.tiles       ? (int64_t)args.tiles[k] : k);
             uint8_t* tb = tables + C::TILE + buf * C::TILE_BYTES;
             const int* meta = (const int*)(tb + C::META);
             const bool got = tc::mbar_wait(&sfull[buf], (t >> 1) & 1, args.err, kErrTimeout);
@@ -2187,7 +2194,9 @@ static void launch_rows(Plan& p, const char* name, const DataOp& A, const FixedO
         // an odd stride keeps each CTA from seeing only one column tile (the column tiles of a
         // row tile differ in cost under the sorted-tuple masks)
         int64_t grid = std::min<int64_t>(a.num_tiles, sm_count());
-        if (grid < a.num_tiles && a.ncol_tiles > 1 && grid % 2 == 0) grid -= 1;
+        if (MODE == EPI_REDUCE)   // whole groups of a block per column tile
+            grid = std::max<int64_t>(1, std::min<int64_t>(a.num_tiles, sm_count()) / a.ncol_tiles) * a.ncol_tiles;
+        else if (grid < a.num_tiles && a.ncol_tiles > 1 && grid % 2 == 0) grid -= 1;
         const dim3 g((unsigned)std::max<int64_t>(grid, 1)), b(ROW_THREADS);
         constexpr size_t smem = RowCfg<S, MODE>::SMEM;
         if constexpr (MODE == EPI_SLICE) {
