@@ -65,6 +65,17 @@ def test_subset_odd_sizes(npf, n, N, m):
         assert rel_fro(p.term(N), full) < 1e-12
 
 
+@pytest.mark.parametrize("n,N,tile", [(5, 3, 16), (70, 3, 16), (90, 2, 16), (100, 2, 16), (75, 2, 32)])
+def test_reduction_groups(npf, n, N, tile):
+    """One to seven column tiles, of which the last is narrower: the blocks of a reduction group."""
+    lam, U, V, A = _odd_system(n, N, 70 * n + N)
+    ref = oracle.psiN(A, n, N, U, V, lam, p1_block=8)
+    with npf.Plan(lam, U, V, N) as p:
+        p.set_option(npf.OPT_TILE_N, tile)
+        p.set_tensor(N, A)
+        assert rel_fro(p.term(N), ref) < 1e-10
+
+
 @pytest.mark.parametrize("n,N,m", [(32, 4, 3), (33, 4, 3), (64, 3, 4), (96, 3, 3), (97, 3, 3)])
 def test_regather_chunks(npf, n, N, m):
     """Sizes on both sides of the regather's variants (1 to 4 chunks of 32 entries a row)."""
