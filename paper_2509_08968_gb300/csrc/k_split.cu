@@ -389,6 +389,7 @@ __global__ void k_prep_at(const double* __restrict__ A, int64_t P, int n, int N,
 enum { EPI_V = 0, EPI_SLICE = 1, EPI_DIVIDE = 2, EPI_SLAB = 3, EPI_REDUCE = 4 };
 
 struct RowArgs {
+    int arows;           // rows of a data tile that are loaded (a multiple of 8; 128 but in EPI_SLICE)
     int kch;             // pipeline stages of K' (16 or 32 wide; K' past the operands' length is
                          // zero on both sides)
     int klast;           // 16-wide steps in the last stage (1 or 2 for 32-wide stages): the rest
@@ -596,7 +597,7 @@ __device__ __forceinline__ void mma_col(int col, uint32_t acc, uint32_t leader, 
 // shared memory delivers the 4 KB data tile every time).
 template <int S, int MODE>
 __device__ __forceinline__ void issue_kstep(uint32_t acc, uint32_t leader, uint32_t tmem, uint32_t lstride,
-                                            uint32_t a_lo, uint32_t b_lo, uint32_t b_plane16,
+                                            uint32_t a_lo, uint32_t a_plane16, uint32_t b_lo, uint32_t b_plane16,
                                             uint32_t idesc)
 {
     using C = RowCfg<S, MODE>;
@@ -604,7 +605,7 @@ __device__ __forceinline__ void issue_kstep(uint32_t acc, uint32_t leader, uint3
     bool first[4] = {true, true, true, true};
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-        const uint32_t ao = a_lo + (uint32_t)((s * C::A_TILE) >> 4);
+        const uint32_t ao = a_lo + (uint32_t)s * a_plane16;
 #pragma unroll
         for (int u = 0; u < S - s; ++u) {
             const int L = s + u < 3 ? s + u : 3;
@@ -703,6 +704,10 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
     const int bnc = args.bnc;
     const int bnr = 2 * bnc;
     const uint32_t b_bytes_tile = (uint32_t)bnr * BKm * 2;
+    // A tile of the last mode product at radix 128 loads the rows a_1 < arows only; the MMAs read the
+    // next plane's for the others (still in the stage), whose results no one uses. At n = 75, FP32 form,
+    // order 4, the padding was 41% of the rows: mode products 20.3 -> 17.5 ms.
+    const uint32_t a_bytes_tile = MODE == EPI_SLICE && !SUBB ? (uint32_t)args.arows * BKm * 2 : (uint32_t)C::A_TILE;
     const int lg = SUBB ? args.lg : 7;         // row radix 2^lg (sub-blocks only below 128)
 
     if (threadIdx.x == 0) {
@@ -770,7 +775,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                     }
                     uint8_t* sA = stage_base + st * C::STAGE_BYTES;
                     uint8_t* sB = sA + S * C::A_TILE;
-                    tc::mbar_arrive_expect_tx(&full[st], S * (C::A_TILE + b_bytes_tile));
+                    tc::mbar_arrive_expect_tx(&full[st], S * (a_bytes_tile + b_bytes_tile));
                     // A: [plane][128 rows][BK]; B: [plane][Re rows, Im rows][BK]
                     tc::tma_load_3d(sA, &tmA, kc * BKm, (int)row0, 0, &full[st]);
                     tc::tma_load_4d(sB, &tmB, kc * BKm, bc, 0, 0, &full[st]);
@@ -792,7 +797,8 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
         // mode products 10% slower.
         const uint32_t leader = tc::elect_one();
         const uint32_t idesc = tc::idesc_bf16_f32(128, bnr);
-        const uint32_t b16 = b_bytes_tile >> 4;   // B plane stride in 16-byte units
+        const uint32_t a16 = a_bytes_tile >> 4;   // plane strides in 16-byte units
+        const uint32_t b16 = b_bytes_tile >> 4;
         uint32_t it = 0, t = 0;
         bool alive = true;
         for (int64_t k = kbeg; k < kend && alive; k += kstep) {
@@ -821,7 +827,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                 const int steps = kc == args.kch - 1 ? min(C::KS, args.klast) : C::KS;
 #pragma unroll 1
                 for (int ks = 0; ks < steps; ++ks)
-                    issue_kstep<S, MODE>(kc == k0 && ks == 0 ? 0u : 1u, leader, tm, lstride, a_lo + (uint32_t)(ks * 2),
+                    issue_kstep<S, MODE>(kc == k0 && ks == 0 ? 0u : 1u, leader, tm, lstride, a_lo + (uint32_t)(ks * 2), a16,
                                          b_lo + (uint32_t)(ks * 2), b16, idesc);
                 tc::mma_commit(leader, &empty[st]);
             }
@@ -1714,14 +1720,14 @@ static CUtensorMap encode_map(const void* base, int rank, const cuuint64_t* dims
 struct DataOp { const void* base; int64_t inner, stride, rows; };   // stride: elements between rows
 struct FixedOp { const void* base; int64_t inner; };
 
-// Data operand as a 3-D tensor (inner, rows, plane); box {bk, 128 rows, planes}. Past the inner
+// Data operand as a 3-D tensor (inner, rows, plane); box {bk, box_rows, planes}. Past the inner
 // extent a box holds zeros.
 template <int S>
-static CUtensorMap plane_map(const DataOp& d, int bk)
+static CUtensorMap plane_map(const DataOp& d, int bk, int box_rows)
 {
     const cuuint64_t dims[3] = {(cuuint64_t)d.inner, (cuuint64_t)d.rows, (cuuint64_t)S};
     const cuuint64_t strides[2] = {(cuuint64_t)d.stride * 2, (cuuint64_t)(d.rows * d.stride * 2)};
-    const cuuint32_t box[3] = {(cuuint32_t)bk, (cuuint32_t)NP, (cuuint32_t)S};
+    const cuuint32_t box[3] = {(cuuint32_t)bk, (cuuint32_t)box_rows, (cuuint32_t)S};
     return encode_map(d.base, 3, dims, strides, box, bk);
 }
 
@@ -2158,7 +2164,8 @@ static void launch_rows(Plan& p, const char* name, const DataOp& A, const FixedO
     a.kch = (kprime + bk - 1) / bk;            // K' past kprime holds zeros on both sides
     a.lgncol = (a.ncol_tiles & (a.ncol_tiles - 1)) == 0 ? __builtin_ctz((unsigned)a.ncol_tiles) : -1;
     a.klast = (kprime + KSTEP - 1) / KSTEP - (bk / KSTEP) * (a.kch - 1);
-    const CUtensorMap tA = plane_map<S>(A, bk);
+    a.arows = MODE == EPI_SLICE && a.lg == 7 ? std::min(NP, (a.n + 7) / 8 * 8) : NP;
+    const CUtensorMap tA = plane_map<S>(A, bk, a.arows);
     const CUtensorMap tB = fixed_map<S>(B, a.bnc, bk);
     if (a.num_tiles >= (int64_t)1 << 31) fail(NPF_ERR_UNSUPPORTED, "too many tiles in one launch");
     if (a.colmask && a.num_tiles > 8 * sm_count()) {
