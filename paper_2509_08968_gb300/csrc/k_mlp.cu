@@ -30,7 +30,7 @@ constexpr int kMaxLayers = 8;
 constexpr int LDN = TK + 8, LDT = TM + 8;
 constexpr int STAGE = TM * LDN > TK * LDT ? TM * LDN : TK * LDT;
 
-enum { EPI_F32 = 0, EPI_RELU_BF16 = 1, EPI_MASK_BF16 = 2, EPI_LOSS = 3, EPI_ADAM = 4 };
+enum { EPI_F32 = 0, EPI_RELU_BF16 = 1, EPI_MASK_BF16 = 2, EPI_LOSS = 3 };
 
 // C[e] = op(A[e]) op(B[e]) over M x N with inner dimension K.
 //   A element (m, k): AT == 0 -> A[m * lda + k], AT == 1 -> A[k * lda + m]
@@ -52,14 +52,14 @@ struct Gemm {
     double* loss;                // EPI_LOSS: per member, += sum (Y - T)^2 / (M N)
 };
 
-// EPI_ADAM: the weight gradients of every layer in one launch, each tile updating its weights.
+// The weight gradients of every layer in one launch, each tile updating its weights.
 struct AdamStep {
     int layers;
     int tile0[kMaxLayers + 1];   // first tile of a layer
     Gemm g[kMaxLayers];          // C: offset of the layer's block in the parameter arrays, in floats
     float *W, *M1, *M2;
     __nv_bfloat16* Wb;
-    float lr, b1, b2, eps, ic1, ic2;   // ic: 1 / (1 - b^step)
+    float lr, b1, b2, eps, c1, c2;   // c: 1 - b^step
 };
 
 // D (16x8, FP32) += A (16x16, BF16, row-major fragment) * B (16x8, BF16, column fragment).
@@ -315,13 +315,21 @@ __global__ void __launch_bounds__(128) k_grad_adam(const __grid_constant__ AdamS
         m1[j] = *reinterpret_cast<const float4*>(s.M1 + o);
         m2[j] = *reinterpret_cast<const float4*>(s.M2 + o);
     }
-    // Reciprocals of the bias corrections from the host, and no operand that is zero in a division or
-    // square root (units that never fire have zero moments, and zeros take the slow branch of both:
-    // 150 instructions an element, 26 us a launch). sqrt(1e-36) = 1e-18 does not change eps = 1e-8.
+    // The products fused with sums are spelled out, so that the trained weights do not depend on the
+    // compiler's choice. Rounded divisions and square root, but none of a zero: units that never fire have
+    // zero moments, and zeros take the slow branch of both (150 instructions an element, 26 us a launch).
+    // Products with reciprocals of the corrections and of the denominator take 1.61 instead of 1.95 ms for
+    // 32 steps of the 4-256-256-256-64 ensemble of five, but a last place in a weight flips BF16 roundings in
+    // the steps behind it (trained weights 1.4e-3 apart).
+    auto quot = [](float x, float d) {
+        const float q = (x == 0.f ? 1.f : x) / d;
+        return x == 0.f ? x : q;
+    };
     auto adam = [&](float gr, float& x, float& a, float& v) {
-        a = s.b1 * a + (1.f - s.b1) * gr;
-        v = s.b2 * v + (1.f - s.b2) * gr * gr;
-        x = x - s.lr * (a * s.ic1) * __frcp_rn(sqrtf(fmaxf(v * s.ic2, 1e-36f)) + s.eps);
+        a = fmaf(1.f - s.b1, gr, s.b1 * a);
+        v = fmaf((1.f - s.b2) * gr, gr, s.b2 * v);
+        const float vh = quot(v, s.c2), r = sqrtf(vh == 0.f ? 1.f : vh);
+        x = x - quot(s.lr * quot(a, s.c1), (vh == 0.f ? 0.f : r) + s.eps);
     };
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -836,8 +844,8 @@ int npf_mlp_train(npf_mlp* m, int rows, const float* X, const float* T, int epoc
                 forward(*m, batch, true);
                 backward(*m, batch);
                 ++m->step;
-                ad.ic1 = (float)(1.0 / (1.0 - std::pow((double)ad.b1, (double)m->step)));
-                ad.ic2 = (float)(1.0 / (1.0 - std::pow((double)ad.b2, (double)m->step)));
+                ad.c1 = (float)(1.0 - std::pow((double)ad.b1, (double)m->step));
+                ad.c2 = (float)(1.0 - std::pow((double)ad.b2, (double)m->step));
                 npf::LaunchScope ls(nullptr, "mlp_grad_adam", m->s);
                 npf::launch_dependent(k_grad_adam, dim3((unsigned)ad.tile0[m->L], 1, (unsigned)m->E), dim3(128), 0, m->s, ad);
             }

@@ -32,3 +32,37 @@ def test_one_adam_step(widths, rows):
     assert np.abs(got - want)[sure].max() < lr * 3e-3
     assert np.abs(got - W).max() <= lr * 1.001
     assert abs(hist[0] - loss.mean()) < 1e-5 * loss.mean()
+
+
+def _fma(a, b, c):
+    """a b + c with one rounding to FP32 (long double holds the product exactly)."""
+    x = np.longdouble
+    return (a.astype(x) * np.asarray(b, x) + c.astype(x)).astype(np.float32)
+
+
+@pytest.mark.parametrize("widths,rows", [([4, 48, 9], 1), ([5, 16, 32, 13], 64), ([4, 256, 64], 33)])
+def test_adam_steps_are_exact(widths, rows):
+    """Adam's arithmetic bit for bit: FP32, every operation rounded to nearest, the moments' new terms
+    fused with their sums, two true divisions by the bias corrections. With equal rows the order of a
+    batch does not matter, so each step's gradient is npf_mlp_loss_grad's."""
+    from paper_2509_08968_gb300 import build
+    build.build()
+    from paper_2509_08968_gb300.mlp import Mlp
+    from paper_2509_08968_gb300.surrogate import init_weights
+    rng = np.random.default_rng(7 + rows)
+    w = init_weights(widths, 2, 6)
+    X = np.repeat(rng.uniform(-1, 1, (1, widths[0])).astype(np.float32), rows, 0)
+    T = np.repeat(rng.standard_normal((1, widths[-1])).astype(np.float32), rows, 0)
+    f = np.float32
+    b1, b2, one = f(0.9), f(0.999), f(1.0)
+    m, v = np.zeros_like(w), np.zeros_like(w)
+    with Mlp(widths, w) as net:
+        for k in range(1, 5):
+            _, g = net.loss_grad(X, T)
+            assert (g == 0).any() and (g != 0).any()
+            net.train(X, T, 1, rows, 1e-2, seed=k)
+            m, v = _fma(g, one - b1, b1 * m), _fma((one - b2) * g, g, b2 * v)
+            c1, c2 = f(1.0 - float(b1) ** k), f(1.0 - float(b2) ** k)
+            w = w - f(1e-2) * (m / c1) / (np.sqrt(v / c2) + f(1e-8))
+            got = net.weights()
+            assert w.dtype == np.float32 and np.array_equal(got, w), k
