@@ -60,15 +60,12 @@ void sync(Plan& p)
     p.prof.flush();
 }
 
-// The terms of one entry point leave the tensor-core error flag to done(), one wait for all of them.
+// The terms of one entry point leave the tensor-core error flag to done(), one wait for all of them,
+// before anything is copied to the caller (a call that fails writes nothing to its outputs).
 struct DeferCheck {
     Plan& p;
     explicit DeferCheck(Plan& p_) : p(p_) { p.defer_err = true; p.err_live = false; }
-    void done()
-    {
-        npf::split_check(p);   // waits for the stream when a tensor-core term ran
-        sync(p);
-    }
+    void done() { npf::split_check(p); }   // waits for the stream when a tensor-core term ran
     ~DeferCheck() { p.defer_err = false; p.err_live = false; }
 };
 
@@ -506,15 +503,16 @@ void batch_run(int count, npf_handle* const* plans, const int* orders, npf_c128*
     it->second.stamp = ++pool.clock;
     NPF_CUDA(cudaGraphLaunch(it->second.exec, pool.origin));
     npf::note_launches(it->second.kernels);
+    int herr = 0;
+    NPF_CUDA(cudaMemcpyAsync(&herr, pool.d_err, sizeof(int), cudaMemcpyDeviceToHost, pool.origin));
+    NPF_CUDA(cudaStreamSynchronize(pool.origin));
+    if (herr) npf::fail(NPF_ERR_TIMEOUT, "a tensor-core pipeline wait gave up inside the batch");
     for (int b = 0; b < count; ++b) {
         const Plan& p = plans[b]->p;
         NPF_CUDA(cudaMemcpyAsync(outs[b], p.d_npf, (size_t)p.n * p.n * sizeof(double2),
                                  cudaMemcpyDefault, pool.origin));
     }
-    int herr = 0;
-    NPF_CUDA(cudaMemcpyAsync(&herr, pool.d_err, sizeof(int), cudaMemcpyDeviceToHost, pool.origin));
     NPF_CUDA(cudaStreamSynchronize(pool.origin));
-    if (herr) npf::fail(NPF_ERR_TIMEOUT, "a tensor-core pipeline wait gave up inside the batch");
 }
 
 }  // namespace
@@ -694,9 +692,10 @@ int npf_compute_prefetch(npf_handle* h, int order, npf_c128* out, int count, con
         for (int t = 0; t < count; ++t) stage_tensor(p, orders[t], coeffs[t]);
         DeferCheck check(p);
         compute_npf(p, order);
+        check.done();
         NPF_CUDA(cudaMemcpyAsync(out, p.d_npf, (size_t)p.n * p.n * sizeof(double2),
                                  cudaMemcpyDefault, p.stream));
-        check.done();
+        sync(p);
     });
 }
 
@@ -731,14 +730,17 @@ int npf_interaction(npf_handle* h, int order, double delta, npf_c128* out)
         KeepReduction keep(p);
         const int64_t nn = (int64_t)p.n * p.n;
         // z(0) = delta Psi + sum_M delta^M Psi_M (Eq. 7; Eq. 9's corrected coordinates), kept in
-        // d_sum; the per-order results go to d_npf as scratch before the copies
+        // d_sum; then T_M[i][k], the order-M reduction against the weights W = z(0), in place of Psi_M
         double2* z = p.d_sum;
         for (int M = 2; M <= order; ++M)
             if (p.d_tensor[M]) compute_term(p, M, p.d_psiN[M]);
         npf::launch_axpy(p, z, delta, p.d_V, 0.0, nn);
         for (int M = 2; M <= order; ++M)
             if (p.d_tensor[M]) npf::launch_axpy(p, z, std::pow(delta, M), p.d_psiN[M], 1.0, nn);
-        // results leave in the caller's mode order (columns i)
+        for (int M = 2; M <= order; ++M)
+            if (p.d_tensor[M]) compute_term(p, M, p.d_psiN[M], z);
+        check.done();
+        // results (formed in d_npf) leave in the caller's mode order (columns i)
         auto emit = [&](npf_c128* dst) {
             const double2* res = p.d_npf;
             if (p.permuted()) {
@@ -747,22 +749,16 @@ int npf_interaction(npf_handle* h, int order, double delta, npf_c128* out)
             }
             NPF_CUDA(cudaMemcpyAsync(dst, res, nn * sizeof(double2), cudaMemcpyDefault, p.stream));
         };
-        // pN1[k][i] = phi_ki z^i(0)
+        // pN1[k][i] = phi_ki z^i(0); pNM[k][i] = phi_ki sum_p hM^i_p prod_m z^{p_m}(0) (Eq. 8)
+        // = -phi_ki T_M[i][k]
         npf::launch_hadamard_t(p, 1.0, z, p.d_npf);
         emit(out);
         for (int M = 2; M <= order; ++M) {
-            npf_c128* dst = out + (int64_t)(M - 1) * nn;
-            if (!p.d_tensor[M]) {
-                NPF_CUDA(cudaMemsetAsync(p.d_npf, 0, nn * sizeof(double2), p.stream));
-            } else {
-                // pNM[k][i] = phi_ki sum_p hM^i_p prod_m z^{p_m}(0) (Eq. 8) = -phi_ki T[i][k]
-                // with T the order-M reduction against the weights W = z(0)
-                compute_term(p, M, p.d_psiN[M], z);
-                npf::launch_hadamard_t(p, -1.0, p.d_psiN[M], p.d_npf);
-            }
-            emit(dst);
+            if (p.d_tensor[M]) npf::launch_hadamard_t(p, -1.0, p.d_psiN[M], p.d_npf);
+            else NPF_CUDA(cudaMemsetAsync(p.d_npf, 0, nn * sizeof(double2), p.stream));
+            emit(out + (int64_t)(M - 1) * nn);
         }
-        check.done();
+        sync(p);
     });
 }
 
@@ -806,6 +802,7 @@ int npf_get_term(npf_handle* h, int order, npf_c128* out)
             npf::fail(NPF_ERR_MISSING_TENSOR, "no tensor set for order " + std::to_string(order));
         DeferCheck check(p);
         compute_term(p, order, p.d_psiN[order]);
+        check.done();
         const double2* res = p.d_psiN[order];
         if (p.permuted()) {   // rows i back to the caller's mode order
             npf::launch_unpermute(p, res, p.d_tmp, false);
@@ -813,7 +810,7 @@ int npf_get_term(npf_handle* h, int order, npf_c128* out)
         }
         NPF_CUDA(cudaMemcpyAsync(out, res, (size_t)p.n * p.n * sizeof(double2),
                                  cudaMemcpyDefault, p.stream));
-        check.done();
+        sync(p);
     });
 }
 
