@@ -299,7 +299,8 @@ template <int N>
 void launch(Plan& p, const ChainArgs& a, int rows)
 {
     const size_t bytes = smem_bytes(N, a.n, a.nm);
-    NPF_CUDA(cudaFuncSetAttribute(k_chain<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    // (a constant: the attribute is the function's, and other threads launch it for other sizes)
+    NPF_CUDA(cudaFuncSetAttribute(k_chain<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem));
     LaunchScope ls(&p.prof, "fp64_chain", p.stream);
     launch_dependent(k_chain<N>, dim3((unsigned)(a.nm * a.chunks), (unsigned)rows), dim3(THREADS), bytes, p.stream, a);
 }

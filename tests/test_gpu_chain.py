@@ -2,6 +2,7 @@
 systems of the tensor-core forms, on both sides of the sizes where the route changes, with odd n,
 row ranges, a mode subset, no divide, weights other than Psi, batches and a budget that leaves
 the general path. Tolerance: 1e-12 for FP64 sums of at most 40^4 terms (the FP64 bar of the library)."""
+import threading
 from types import SimpleNamespace
 
 import numpy as np
@@ -74,3 +75,41 @@ def test_budget_below_the_chain_uses_the_general_path(npf):
         with pytest.raises(npf.NpfError) as e:
             p.term(N)
         assert e.value.status == npf.NPF_ERR_OOM
+
+
+def test_sizes_side_by_side(npf):
+    """The chain's shared memory grows with n (54 KB at n = 45, 2 KB at n = 8, order 3): launches of one
+    size do not change what another may have, be it in another thread or in a recorded batch."""
+    N = 3
+    systems = [_odd_system(n, N, 90 + n) for n in (45, 8)]
+    refs = [oracle.psiN(A, len(lam), N, U, V, lam, p1_block=8) for lam, U, V, A in systems]
+    plans = []
+    for lam, U, V, A in systems:
+        plans.append(npf.Plan(lam, U, V, N, precision="fp64"))
+        plans[-1].set_tensor(N, A)
+    outs = [np.empty(r.shape, np.complex128) for r in refs]
+    for _ in range(3):   # eager, recorded, replayed
+        npf.batch_compute(plans, [N, N], outs)
+        for (lam, U, V, A), r, o in zip(systems, refs, outs):
+            assert rel_fro(o, U * (V + r).T) < 1e-12
+    errors, stop = [], threading.Event()
+
+    def small():
+        try:
+            while not stop.is_set():
+                plans[1].term(N)
+        except npf.NpfError as e:
+            errors.append(e)
+
+    t = threading.Thread(target=small)
+    t.start()
+    try:
+        for _ in range(300):
+            got = plans[0].term(N)
+    finally:
+        stop.set()
+        t.join()
+        for p in plans:
+            p.close()
+    assert not errors
+    assert rel_fro(got, refs[0]) < 1e-12
