@@ -64,9 +64,19 @@ void sync(Plan& p)
 // before anything is copied to the caller (a call that fails writes nothing to its outputs).
 struct DeferCheck {
     Plan& p;
+    bool finished = false;
     explicit DeferCheck(Plan& p_) : p(p_) { p.defer_err = true; p.err_live = false; }
-    void done() { npf::split_check(p); }   // waits for the stream when a tensor-core term ran
-    ~DeferCheck() { p.defer_err = false; p.err_live = false; }
+    void done()
+    {
+        npf::split_check(p);   // waits for the stream when a tensor-core term ran
+        finished = true;
+    }
+    ~DeferCheck()
+    {
+        if (!finished) cudaStreamSynchronize(p.stream);   // a failed call: earlier terms may still run
+        p.defer_err = false;
+        p.err_live = false;
+    }
 };
 
 // The terms of one entry point share their reduction rows (Plan::keep_red).
@@ -470,10 +480,15 @@ void batch_run(int count, npf_handle* const* plans, const int* orders, npf_c128*
             const size_t budget = (size_t)(0.8 * (double)(fr + held) / kWorkers);
             void* bases[kWorkers];
             for (int w = 0; w < kWorkers; ++w) bases[w] = pool.arena[w].base;
-            for (int b = 0; b < count; ++b) {
-                const int w = worker[b];
-                PlanRoute r(plans[b]->p, pool.ws[w], &pool.arena[w], budget, false, nullptr);
-                compute_npf(plans[b]->p, orders[b]);
+            try {
+                for (int b = 0; b < count; ++b) {
+                    const int w = worker[b];
+                    PlanRoute r(plans[b]->p, pool.ws[w], &pool.arena[w], budget, false, nullptr);
+                    compute_npf(plans[b]->p, orders[b]);
+                }
+            } catch (...) {   // the systems before the failed one may still run
+                for (int w = 0; w < kWorkers; ++w) cudaStreamSynchronize(pool.ws[w]);
+                throw;
             }
             for (int w = 0; w < kWorkers; ++w) NPF_CUDA(cudaStreamSynchronize(pool.ws[w]));
             bool moved = false;
