@@ -328,7 +328,7 @@ void chain_term(Plan& p, int N, double2* d_out, const double2* W, bool accumulat
     if (!accumulate && rows < n) launch_zero(p, d_out, (int64_t)n * n);   // the other rows
     if (rows <= 0) return;
     Arena& ar = p.scratch();
-    ar.reserve(chain_scratch(p, N, rows));
+    ar.reserve(chain_scratch(p, N, rows), p.stream);
     ChainArgs a{};
     a.n = n;
     a.nm = p.nm;

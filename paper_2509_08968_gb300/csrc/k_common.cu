@@ -93,11 +93,13 @@ LaunchScope::~LaunchScope()
 }
 
 // ---------------------------------------------------------------------------------------
-void Arena::reserve(size_t bytes)
+void Arena::reserve(size_t bytes, cudaStream_t s)
 {
     if (bytes <= cap) return;
     if (frozen) fail(NPF_ERR_OOM, "scratch would have to grow while work is recorded into a graph");
-    if (base) NPF_CUDA(cudaDeviceSynchronize());   // work in flight may still use the smaller block
+    // work in flight may still use the smaller block (the whole device may not be waited for: another
+    // thread may be recording a batch)
+    if (base) NPF_CUDA(cudaStreamSynchronize(s));
     release();
     void* ptr = nullptr;
     cudaError_t e = cudaMalloc(&ptr, bytes);

@@ -215,7 +215,7 @@ void fp64_term(Plan& p, int N, double2* d_out, const double2* W, bool accumulate
         return;
     }
     Arena& ar = p.scratch();
-    ar.reserve(per_nb * nb);
+    ar.reserve(per_nb * nb, p.stream);
     double2* bufA = (double2*)ar.base;
     double2* bufB = bufA + (size_t)nb * nN;
     double2* bufC = bufB + (size_t)nb * nN;
@@ -278,13 +278,13 @@ void fp64_slab(Plan& p, int N, const int* prefix, double2* d_out)
     const int n = p.n;
     const int64_t nN1 = ipow64(n, N - 1);
     Arena& ar = p.scratch();
-    ar.reserve(2 * (size_t)n * nN1 * sizeof(double2));
+    ar.reserve(2 * (size_t)n * nN1 * sizeof(double2), p.stream);
     double2* X = (double2*)ar.base;
     double2* Y = X + (size_t)n * nN1;
     DivideArgs none = divide_args(p, N);
     if (N == 1) {
         // order 1: X[p][j] = sum_a A1[j][a] phi_{a p}, then h[i][p] = sum_j psi_ij X[p][j] / D
-        ar.reserve((size_t)n * n * sizeof(double2));
+        ar.reserve((size_t)n * n * sizeof(double2), p.stream);
         X = (double2*)ar.base;
         {
             LaunchScope ls(&p.prof, "fp64_first_contraction", p.stream);

@@ -2334,7 +2334,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
         if (keep) own_red = false;   // (no room in the scratch for it)
     }
     const bool again = keep && W && so.kept_ok[N];   // only the reduction is left to do
-    ar.reserve(s_bytes + (size_t)ib * (a_per + b_per + e_per) + wbytes + (own_red ? red_bytes : 0) + 10 * 256 + 1024);
+    ar.reserve(s_bytes + (size_t)ib * (a_per + b_per + e_per) + wbytes + (own_red ? red_bytes : 0) + 10 * 256 + 1024, p.stream);
     uint8_t* base = (uint8_t*)ar.base;
     auto take = [&](size_t bytes) { uint8_t* r = base; base += (bytes + 255) & ~(size_t)255; return r; };
     longlong2* Sv = (longlong2*)take(s_bytes);

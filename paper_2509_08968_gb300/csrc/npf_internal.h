@@ -59,7 +59,7 @@ struct Arena {
     void* base = nullptr;
     size_t cap = 0;
     bool frozen = false;   // set while work is recorded into a CUDA graph: growing fails
-    void reserve(size_t bytes);
+    void reserve(size_t bytes, cudaStream_t s);   // s: the stream that uses it
     void release();
 };
 
