@@ -679,6 +679,15 @@ void copy_out(void* dst, const void* src, size_t bytes, cudaStream_t s)
     NPF_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, s));
 }
 
+// Weights or gradients (d_pub) to the caller behind what the legacy stream has queued on a device
+// destination.
+void hand_out(npf_mlp& m, float* dst)
+{
+    sync(m);
+    NPF_CUDA(cudaMemcpy(dst, m.d_pub, (size_t)m.E * m.Ppub * sizeof(float), cudaMemcpyDefault));
+    NPF_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
+}
+
 }  // namespace
 
 extern "C" {
@@ -717,8 +726,9 @@ npf_mlp* npf_mlp_create(int ensemble, int layers, const int* widths, const float
         m->Wb = dalloc<__nv_bfloat16>(tot);
         m->d_loss = dalloc<double>(ensemble);
         m->d_pub = dalloc<float>(ensemble * m->Ppub);
-        NPF_CUDA(cudaMemcpyAsync(m->d_pub, weights, (size_t)ensemble * m->Ppub * sizeof(float), cudaMemcpyDefault,
-                                 m->s));
+        // (blocking: for device weights it waits for what the legacy stream has queued)
+        NPF_CUDA(cudaMemcpy(m->d_pub, weights, (size_t)ensemble * m->Ppub * sizeof(float), cudaMemcpyDefault));
+        NPF_CUDA(cudaStreamSynchronize(cudaStreamLegacy));   // (between device buffers it returns at once)
         NPF_CUDA(cudaMemsetAsync(m->W, 0, (size_t)tot * sizeof(float), m->s));
         NPF_CUDA(cudaMemsetAsync(m->M1, 0, (size_t)tot * sizeof(float), m->s));
         NPF_CUDA(cudaMemsetAsync(m->M2, 0, (size_t)tot * sizeof(float), m->s));
@@ -745,8 +755,7 @@ int npf_mlp_get_weights(const npf_mlp* m, float* weights)
         if (!m || !weights) npf::fail(NPF_ERR_ARG, "null argument");
         npf_mlp& mm = const_cast<npf_mlp&>(*m);   // (the staging buffer; the weights stay)
         relayout(mm, mm.W, true);
-        copy_out(weights, mm.d_pub, (size_t)mm.E * mm.Ppub * sizeof(float), mm.s);
-        sync(mm);
+        hand_out(mm, weights);
     });
 }
 
@@ -787,9 +796,8 @@ int npf_mlp_loss_grad(npf_mlp* m, int rows, const float* X, const float* T, floa
         }
         std::vector<double> l(m->E);
         relayout(*m, m->G, true);
-        copy_out(grads, m->d_pub, (size_t)m->E * m->Ppub * sizeof(float), m->s);
         NPF_CUDA(cudaMemcpyAsync(l.data(), m->d_loss, m->E * sizeof(double), cudaMemcpyDeviceToHost, m->s));
-        sync(*m);
+        hand_out(*m, grads);
         std::vector<float> lf(l.begin(), l.end());
         NPF_CUDA(cudaMemcpy(loss, lf.data(), lf.size() * sizeof(float), cudaMemcpyDefault));
     });
