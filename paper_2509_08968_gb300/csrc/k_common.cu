@@ -218,7 +218,7 @@ void launch_unpermute(Plan& p, const double2* in, double2* out, bool columns)
     NPF_CUDA(cudaGetLastError());
 }
 
-// max |V U - I| over the entries (NaN entries are passed over), as the bits of a non-negative double.
+// max |V U - I| over the entries (infinity when one is NaN), as the bits of a non-negative double.
 __global__ void k_inverse_error(int n, const double2* __restrict__ V, const double2* __restrict__ U,
                                 unsigned long long* __restrict__ worst)
 {
@@ -230,7 +230,7 @@ __global__ void k_inverse_error(int n, const double2* __restrict__ V, const doub
 #pragma unroll 4
         for (int j = 0; j < n; ++j) cfma(s, V[(int64_t)i * n + j], U[(int64_t)j * n + c]);
         e = hypot(s.x - (c == i ? 1.0 : 0.0), s.y);
-        if (isnan(e)) e = 0.0;
+        if (isnan(e)) e = __longlong_as_double(0x7FF0000000000000ll);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) e = fmax(e, __shfl_xor_sync(0xffffffffu, e, o));

@@ -92,3 +92,21 @@ def test_error_codes(npf):
     with pytest.raises(npf.NpfError) as e:
         npf.Plan(sysm.lam, sysm.U, bad, 2)
     assert e.value.status == npf.NPF_ERR_NOT_INVERSE
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf, 1j * np.nan])
+def test_modal_data_that_are_no_numbers_are_refused(npf, value):
+    """A NaN or infinity in U or V makes entries of V U - I NaN: no inverse, and a refused set_modes
+    leaves the plan as it was."""
+    sysm = S.config_small(0, orders=(2,))
+    with npf.Plan(sysm.lam, sysm.U, sysm.V, 2, precision="fp64") as p:
+        p.set_tensor(2, sysm.tensors[2])
+        before = p.compute(2)
+        for name in ("U", "V"):
+            m = {"U": sysm.U.copy(), "V": sysm.V.copy()}
+            m[name][3, 4] = value
+            for call in (lambda: npf.Plan(sysm.lam, m["U"], m["V"], 2), lambda: p.set_modes(sysm.lam, m["U"], m["V"])):
+                with pytest.raises(npf.NpfError) as e:
+                    call()
+                assert e.value.status == npf.NPF_ERR_NOT_INVERSE
+        assert np.array_equal(p.compute(2), before)
