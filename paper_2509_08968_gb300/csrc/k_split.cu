@@ -1774,7 +1774,9 @@ void split_drop_kept(Plan& p)
 }
 
 // A term is accepted when S, digit records of it (32 bytes an entry) and the dense rows of one upper
-// index fit the budget: the sorted rows it forms take less, and no records are kept.
+// index fit the budget. This is what callers rely on, not what a term needs: it forms no records, and
+// the sorted rows of an upper index with all tables fit in what is so accepted, at every size and
+// slice count (n = 120, order 4 would run in 22 GB of the 65 GB asked for).
 size_t split_min_bytes(const Plan& p, int N)
 {
     const int64_t P = p.packed_count[N], rows = (P + NP - 1) / NP * NP;
@@ -2291,7 +2293,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     const size_t a_per = (size_t)std::max(std::max(R0, R1), std::max(R2, Qc)) * row_bytes;
     const size_t b_per = std::max((size_t)v_per * sizeof(longlong2), (size_t)RS * row_bytes);
     const size_t e_per = (size_t)(R1 + R2 + RS + Qc) * sizeof(int);
-    const size_t per_i = std::min(dense_bytes(n, N, S), a_per + b_per + e_per);
+    const size_t per_i = a_per + b_per + e_per;
     const int64_t Q2 = N >= 3 && !slab ? npairs : 0;              // weights of the pairs (less than records)
     const size_t wbytes = (size_t)Q2 * n * sizeof(float4);
     const int rlo = std::max(0, p.row_lo);                       // upper-index rows to form
@@ -2299,7 +2301,8 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     // One batch of a small system: the reduction's rows get a buffer of their own, so that the first
     // launch can clear their heads.
     const size_t red_bytes = (size_t)nm * Qc * row_bytes;
-    const size_t all_bytes = s_bytes + (size_t)nm * (a_per + b_per + e_per) + wbytes + 10 * 256 + 1024;
+    const size_t fixed_bytes = s_bytes + wbytes + 10 * 256 + 1024;   // (and alignment, sE)
+    const size_t all_bytes = fixed_bytes + (size_t)nm * per_i;
     Arena& ar = p.scratch();
     bool own_red = !slab && red_bytes <= ((size_t)64 << 20);
     // (under a budget of the caller's nothing is kept beside the scratch)
@@ -2310,7 +2313,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
         const size_t budget = effective_budget(p);
         if (split_min_bytes(p, N) > budget)
             fail(NPF_ERR_OOM, "memory budget too small for one upper-index batch");
-        ib = (int)std::min<size_t>((size_t)nm, (budget - s_bytes - wbytes) / per_i);
+        ib = (int)std::min<size_t>((size_t)nm, (budget - fixed_bytes) / per_i);
         own_red &= ib == nm && all_bytes + red_bytes <= budget;
         keep &= ib == nm && all_bytes + red_bytes <= budget;
     }
@@ -2334,7 +2337,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
         if (keep) own_red = false;   // (no room in the scratch for it)
     }
     const bool again = keep && W && so.kept_ok[N];   // only the reduction is left to do
-    ar.reserve(s_bytes + (size_t)ib * (a_per + b_per + e_per) + wbytes + (own_red ? red_bytes : 0) + 10 * 256 + 1024, p.stream);
+    ar.reserve(fixed_bytes + (size_t)ib * per_i + (own_red ? red_bytes : 0), p.stream);
     uint8_t* base = (uint8_t*)ar.base;
     auto take = [&](size_t bytes) { uint8_t* r = base; base += (bytes + 255) & ~(size_t)255; return r; };
     longlong2* Sv = (longlong2*)take(s_bytes);

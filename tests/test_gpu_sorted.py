@@ -110,6 +110,24 @@ def test_few_upper_indices_and_new_modes(npf, n, N):
         assert e.value.status == npf.NPF_ERR_OOM
 
 
+def test_scratch_stays_in_the_budget(npf):
+    """The upper indices of a batch are counted by the rows they take, which at 2 slices, order 3 and
+    n = 32, 64, 128 are more than the dense rows that a budget is accepted by (17 MB here)."""
+    import torch
+    n, N = 128, 3
+    P = comb(n + N - 1, N)
+    lam, U, V, _ = _odd_system(n, 2, 5)
+    budget = n * P * 16 + n * (n + 1) // 2 * n * 16 + n * (2 * (128 ** 2 * (128 * 4 * 2 + 4)) + 4096)
+    with npf.Plan(lam, U, V, N) as p:
+        p.set_option(npf.OPT_SLICES, 2)
+        p.set_option(npf.OPT_MEM_BUDGET, budget)
+        p.set_tensor(N, torch.zeros((n, P), dtype=torch.float64, device="cuda"))
+        free = torch.cuda.mem_get_info()[0]
+        assert not p.term(N).any()
+        used = free - torch.cuda.mem_get_info()[0]
+    assert budget / 2 < used < budget + 8e6   # (and a few MB of tables)
+
+
 @pytest.mark.parametrize("n", [27, 35])
 def test_interaction_shares_the_divided_entries(npf, n):
     """Mode interactions reduce each order twice from one set of divided entries when it runs in one
