@@ -189,7 +189,10 @@ int npf_get_term(npf_handle* h, int order, npf_c128* out);
  * tensor), out[0][k*n + i] = pN1 = phi_ki z^i(0) and, for M = 2..order,
  * out[M-1][k*n + i] = pNM = phi_ki sum_p hM^i_p z^{p_1}(0) .. z^{p_M}(0) (Eq. 8; zero when order M
  * has no tensor). Summed over i and M they reproduce x^k(0) = delta up to O(delta^3) (Eq. 6).
- * out: [order][n][n], host or device. The plan's Psi_M terms and NPF buffer are overwritten. */
+ * out: [order][n][n], host or device. The plan's Psi_M terms and NPF buffer are overwritten. With
+ * mem_budget = 0 the plan keeps a workspace of up to 256 MB an order for the divided entries, within
+ * its 80% of the device memory; a call that needs scratch, a batch's first pass or a memory budget
+ * gives it back. */
 int npf_interaction(npf_handle* h, int order, double delta, npf_c128* out);
 
 /* The NPF of Algorithm 2 step 20 from given correction terms: out[k*n + i] =

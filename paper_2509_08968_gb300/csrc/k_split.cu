@@ -1668,7 +1668,8 @@ struct SplitOperand {
     int* sseg[kMaxOrder + 1] = {};
     int* stpmax[kMaxOrder + 1] = {};
     int* segbase[kMaxOrder + 1] = {};
-    // reduction rows of the last term (Plan::keep_red): planes, exponents, their bytes
+    // reduction rows of the last term (Plan::keep_red): planes, exponents, their bytes. Workspace of the
+    // plan: within the budget, and given back when another call asks for scratch
     uint8_t* kept[kMaxOrder + 1] = {};
     int* kept_e[kMaxOrder + 1] = {};
     size_t kept_bytes[kMaxOrder + 1] = {};
@@ -1766,7 +1767,22 @@ static size_t dense_bytes(int n, int N, int S)
     return 2 * ((size_t)ipow64(rad, N - 1) * ((size_t)rad * 4 * S + 4)) + 4096;
 }
 
+static void free_kept(SplitOperand& so, int N)
+{
+    if (so.kept[N]) cudaFree(so.kept[N]);
+    if (so.kept_e[N]) cudaFree(so.kept_e[N]);
+    so.kept[N] = nullptr;
+    so.kept_e[N] = nullptr;
+    so.kept_bytes[N] = 0;
+    so.kept_ok[N] = false;
+}
+
 #ifndef NPF_SPLIT_LOW
+void split_give_back(Plan& p)
+{
+    for (int N = 0; p.split && N <= kMaxOrder; ++N) free_kept(*p.split, N);
+}
+
 void split_drop_kept(Plan& p)
 {
     if (!p.split) return;
@@ -1798,7 +1814,7 @@ void split_release(Plan& p)
     for (int N = 0; N <= kMaxOrder; ++N) {
         cudaFree(so->smeta[N]); cudaFree(so->ssum[N]); cudaFree(so->ssig[N]); cudaFree(so->stup[N]); cudaFree(so->sseg[N]);
         cudaFree(so->stpmax[N]); cudaFree(so->segbase[N]);
-        cudaFree(so->kept[N]); cudaFree(so->kept_e[N]);
+        free_kept(*so, N);
     }
     for (int M = 0; M < 4; ++M) { cudaFree(so->ptup[M]); cudaFree(so->atup[M]); }
     cudaFree(so->err);
@@ -2310,25 +2326,29 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     int ib = nm;
     // (scratch that holds everything already needs no look at the free memory)
     if (p.mem_budget || ar.cap < all_bytes + (own_red ? red_bytes : 0)) {
-        const size_t budget = effective_budget(p);
+        // (a call that records may not free: its first, eager pass has done so)
+        size_t held = 0;
+        for (int M = 0; M <= kMaxOrder; ++M) {
+            if (!p.keep_red && !p.capturing) free_kept(so, M);
+            held += so.kept_bytes[M];
+        }
+        size_t budget = effective_budget(p);
+        if (!p.mem_budget) budget -= std::min(budget, held / 5);   // (80% of free, scratch and kept, less kept)
         if (split_min_bytes(p, N) > budget)
             fail(NPF_ERR_OOM, "memory budget too small for one upper-index batch");
         ib = (int)std::min<size_t>((size_t)nm, (budget - fixed_bytes) / per_i);
         own_red &= ib == nm && all_bytes + red_bytes <= budget;
         keep &= ib == nm && all_bytes + red_bytes <= budget;
     }
-    // kept rows: up to 256 MB an order, in a buffer of the plan that a repeated call finds again
+    // kept rows: up to 256 MB an order, in a buffer of the plan that a repeated interaction finds again
     if (keep) {
         const size_t eb = (size_t)nm * Qc * sizeof(int);
         if (so.kept_bytes[N] != red_bytes + eb) {
             if (so.kept[N]) NPF_CUDA(cudaStreamSynchronize(p.stream));
-            cudaFree(so.kept[N]); cudaFree(so.kept_e[N]);
-            so.kept[N] = nullptr; so.kept_e[N] = nullptr; so.kept_bytes[N] = 0;
-            so.kept_ok[N] = false;
+            free_kept(so, N);
             if (cudaMalloc(&so.kept[N], red_bytes) != cudaSuccess || cudaMalloc(&so.kept_e[N], eb) != cudaSuccess) {
                 cudaGetLastError();   // no room: the rows are formed again for every weight matrix
-                cudaFree(so.kept[N]);
-                so.kept[N] = nullptr; so.kept_e[N] = nullptr;
+                free_kept(so, N);
                 keep = false;
             } else {
                 so.kept_bytes[N] = red_bytes + eb;

@@ -475,6 +475,7 @@ void batch_run(int count, npf_handle* const* plans, const int* orders, npf_c128*
             // first sighting of this list: run it eagerly (tile tuning, operand preparation,
             // scratch sizing); its outputs are the result. A list seen again is recorded.
             size_t fr = 0, tot = 0, held = 0;
+            for (int b = 0; b < count; ++b) npf::split_give_back(plans[b]->p);
             NPF_CUDA(cudaMemGetInfo(&fr, &tot));
             for (int w = 0; w < kWorkers; ++w) held += pool.arena[w].cap;
             const size_t budget = (size_t)(0.8 * (double)(fr + held) / kWorkers);

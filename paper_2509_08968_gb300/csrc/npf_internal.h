@@ -176,6 +176,7 @@ void chain_term(Plan& p, int N, double2* d_out, const double2* W, bool accumulat
 void split_term(Plan& p, int N, double2* d_out, const double2* W = nullptr, bool accumulate = false);
 void split_slab(Plan& p, int N, const int* prefix, double2* d_out);
 void split_drop_kept(Plan& p);   // reduction rows kept by keep_red are no longer valid
+void split_give_back(Plan& p);   // frees their buffers
 void split_check(Plan& p);   // waits for the stream; throws if a deferred term's pipeline wait gave up
 size_t split_min_bytes(const Plan& p, int N);   // smallest budget a term is accepted with
 void split_release(Plan& p);

@@ -150,3 +150,27 @@ def test_interaction_shares_the_divided_entries(npf, n):
             assert rel_fro(p.term(3), oracle.psiN(s.tensors[3], n, 3, s.U, s.V, s.lam, p1_block=8)) < 1e-10
         p.set_option(npf.OPT_MEM_BUDGET, 60e6 if n > 32 else 20e6)
         assert rel_fro(p.interaction(3, 0.1), ref) < 1e-10
+
+
+def test_interaction_gives_its_workspace_back(npf):
+    """The divided entries that an interaction keeps (168 MB at n = 60, order 3) are workspace: another
+    call that needs scratch, a batch's first pass and a caller's budget each free them; a recorded
+    batch goes on, and the next interaction is right again."""
+    import torch
+    s = S.config_n60(0, orders=(3,))
+    ref = oracle.interaction_npfs(s, 3, 0.1)
+    term = oracle.psiN(s.tensors[3], 60, 3, s.U, s.V, s.lam, p1_block=4)
+    free = lambda: torch.cuda.mem_get_info()[0]
+    outs = [np.empty((60, 60), np.complex128)]
+    with npf.Plan(s.lam, s.U, s.V, 4) as p:
+        p.set_tensor(3, s.tensors[3])
+        assert rel_fro(p.interaction(3, 0.1), ref) < 1e-10
+        kept = free()
+        p.set_option(npf.OPT_MEM_BUDGET, 1.5e9)
+        assert rel_fro(p.term(3), term) < 1e-10
+        assert free() - kept > 150e6
+        p.set_option(npf.OPT_MEM_BUDGET, 0)
+        for k in range(3):   # eager (gives back), recorded beside a kept workspace, replayed
+            assert rel_fro(p.interaction(3, 0.1), ref) < 1e-10
+            npf.batch_compute([p], [3], outs)
+            assert rel_fro(outs[0], s.U * (s.V + term).T) < 1e-10
