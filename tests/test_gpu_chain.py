@@ -9,7 +9,7 @@ import numpy as np
 import pytest
 
 import oracle
-from tests._util import rel_fro
+from tests._util import ran, rel_fro
 from tests.test_gpu_sorted import _odd_system
 
 pytestmark = pytest.mark.gpu
@@ -31,8 +31,11 @@ def test_both_sides_of_the_rule(npf, n, N):
     for precision, tol in (("fp64", 1e-12), ("split_bf16", 1e-10), ("fp32", 1e-5)):
         with npf.Plan(lam, U, V, N, precision=precision) as p:
             p.set_tensor(N, A)
+            p.set_option(npf.OPT_PROFILE, 1)
             got = p.term(N)
             assert rel_fro(got, ref) < tol
+            chain = precision == "fp64" or n <= {2: 25, 3: 16, 4: 10}[N]
+            assert ("fp64_chain" in ran(p)) == chain
             if precision == "fp64":
                 assert np.array_equal(got, p.term(N))   # fixed order of summation
                 p.set_option(npf.OPT_DIVIDE, 0)

@@ -4,7 +4,7 @@ import pytest
 
 import npf_synth as S
 import oracle
-from tests._util import make_plan, rel_fro
+from tests._util import ROUTES, assert_route, make_plan, rel_fro, set_route
 
 pytestmark = pytest.mark.gpu
 TOL = {"split_bf16": 1e-10, "fp64": 1e-12}
@@ -18,13 +18,16 @@ def npf():
     return m
 
 
+@pytest.mark.parametrize("route", ROUTES)
 @pytest.mark.parametrize("prec", ["split_bf16", "fp64"])
 @pytest.mark.parametrize("delta", [0.05, 1.0])
-def test_small_system(npf, prec, delta):
+def test_small_system(npf, prec, delta, route):
     sysm = S.config_small(2, orders=(2, 3))
     ref = oracle.interaction_npfs(sysm, 3, delta)
     with make_plan(npf, sysm, 3, prec) as p:
+        set_route(npf, p, route, prec)
         got = p.interaction(3, delta)
+        assert_route(p, route, prec)
     for M in range(3):
         assert rel_fro(got[M], ref[M]) < TOL[prec], (M, rel_fro(got[M], ref[M]))
 
@@ -38,10 +41,13 @@ def test_n60_order3_split(npf):
         assert rel_fro(got[M], ref[M]) < TOL["split_bf16"], (M, rel_fro(got[M], ref[M]))
 
 
-def test_missing_order_is_zero(npf):
+@pytest.mark.parametrize("route", ROUTES)
+def test_missing_order_is_zero(npf, route):
     sysm = S.config_small(0, orders=(3,))
     ref = oracle.interaction_npfs(sysm, 3, 0.2)
     with make_plan(npf, sysm, 3, "split_bf16") as p:
+        set_route(npf, p, route)
         got = p.interaction(3, 0.2)
+        assert_route(p, route)
     assert np.all(got[1] == 0)
     assert rel_fro(got[2], ref[2]) < 1e-10 and rel_fro(got[0], ref[0]) < 1e-10

@@ -7,7 +7,7 @@ import pytest
 
 import npf_synth as S
 import oracle
-from tests._util import rel_fro
+from tests._util import ROUTES, assert_route, rel_fro, set_route
 
 pytestmark = pytest.mark.gpu
 
@@ -26,14 +26,17 @@ def _system(n, N, seed):
     return sysm
 
 
+@pytest.mark.parametrize("route", ROUTES)
 @pytest.mark.parametrize("n,N", [(10, 2), (30, 2), (34, 2), (64, 2), (66, 2),
                                  (10, 3), (34, 3), (12, 4)])
-def test_radix_boundaries_match_oracle(npf, n, N):
+def test_radix_boundaries_match_oracle(npf, n, N, route):
     sysm = _system(n, N, 1000 + n)
     ref = oracle.psiN(sysm.tensors[N], n, N, sysm.U, sysm.V, sysm.lam, p1_block=8)
     with npf.Plan(sysm.lam, sysm.U, sysm.V, N) as p:
+        set_route(npf, p, route)
         p.set_tensor(N, sysm.tensors[N])
         assert rel_fro(p.term(N), ref) < 1e-10
+        assert_route(p, route)
 
 
 @pytest.mark.parametrize("n,N", [(30, 2), (34, 3)])
@@ -69,15 +72,18 @@ def test_autotuned_plan_term_and_slab(npf):
         assert rel_fro(p.term(N), ref) < 1e-10
 
 
+@pytest.mark.parametrize("route", ROUTES)
 @pytest.mark.parametrize("n,N", [(2, 2), (2, 3), (4, 4), (128, 2)])
-def test_smallest_and_largest_systems(npf, n, N):
+def test_smallest_and_largest_systems(npf, n, N, route):
     """n = 2 and 4 (one mostly padded sub-block) and n = 128, the largest system of the
     tensor-core path (K' = 256: every chunk full, |L0| may reach 2^22)."""
     sysm = _system(n, N, 5000 + n)
     ref = oracle.psiN(sysm.tensors[N], n, N, sysm.U, sysm.V, sysm.lam, p1_block=8)
     with npf.Plan(sysm.lam, sysm.U, sysm.V, N) as p:
+        set_route(npf, p, route)
         p.set_tensor(N, sysm.tensors[N])
         assert rel_fro(p.term(N), ref) < 1e-10
+        assert_route(p, route)
 
 
 def test_n128_order3_slabs(npf):

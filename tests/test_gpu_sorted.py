@@ -11,7 +11,7 @@ import pytest
 
 import npf_synth as S
 import oracle
-from tests._util import rel_fro
+from tests._util import ROUTES, assert_route, rel_fro, set_route
 
 pytestmark = pytest.mark.gpu
 
@@ -39,30 +39,36 @@ def _odd_system(n, N, seed):
     return lam, U, np.linalg.inv(U), S.random_packed_tensor_dense_fill(n, N, seed + N)
 
 
+@pytest.mark.parametrize("route", ROUTES)
 @pytest.mark.parametrize("n,N,precision", [
     (1, 3, "split_bf16"), (3, 2, "split_bf16"), (3, 4, "split_bf16"), (9, 3, "split_bf16"),
     (11, 4, "split_bf16"), (33, 3, "split_bf16"), (35, 3, "fp32"), (17, 4, "fp32"), (19, 4, "split_bf16"),
     (65, 3, "split_bf16"), (67, 2, "split_bf16"), (71, 3, "fp32")])
-def test_term_odd_sizes(npf, n, N, precision):
+def test_term_odd_sizes(npf, n, N, precision, route):
     lam, U, V, A = _odd_system(n, N, 40 * n + N)
     ref = oracle.psiN(A, n, N, U, V, lam, p1_block=8)
     with npf.Plan(lam, U, V, N, precision=precision) as p:
+        set_route(npf, p, route, precision)
         p.set_tensor(N, A)
         assert rel_fro(p.term(N), ref) < (1e-10 if precision == "split_bf16" else 1e-5)
+        assert_route(p, route, precision)
 
 
+@pytest.mark.parametrize("route", ROUTES)
 @pytest.mark.parametrize("n,N,m", [(9, 3, 1), (21, 3, 5), (13, 4, 7), (67, 3, 33)])
-def test_subset_odd_sizes(npf, n, N, m):
+def test_subset_odd_sizes(npf, n, N, m, route):
     lam, U, V, A = _odd_system(n, N, 50 * n + N)
     modes = np.random.default_rng(n).permutation(n)[:m]
     ref = oracle.psiN_subset(A, n, N, U, V, lam, modes)
     with npf.Plan(lam, U, V, N) as p:
+        set_route(npf, p, route)
         p.set_tensor(N, A)
         full = p.term(N)                       # the tables of every mode, then of the subset
         p.set_mode_subset(modes)
         assert rel_fro(p.term(N), ref) < 1e-10
         p.set_mode_subset(None)
         assert rel_fro(p.term(N), full) < 1e-12
+        assert_route(p, route)
 
 
 @pytest.mark.parametrize("n,N,tile", [(5, 3, 16), (70, 3, 16), (90, 2, 16), (100, 2, 16), (75, 2, 32)])
@@ -88,8 +94,9 @@ def test_regather_chunks(npf, n, N, m):
         assert rel_fro(p.term(N), ref) < 1e-10
 
 
+@pytest.mark.parametrize("route", ROUTES)
 @pytest.mark.parametrize("n,N", [(9, 3), (11, 4), (35, 3)])
-def test_few_upper_indices_and_new_modes(npf, n, N):
+def test_few_upper_indices_and_new_modes(npf, n, N, route):
     """Batches of a few upper indices, and modal data replaced in a plan whose tables exist."""
     lam, U, V, A = _odd_system(n, N, 60 * n + N)
     lam2, U2, V2, _ = _odd_system(n, N, 61 * n + N)
@@ -97,6 +104,7 @@ def test_few_upper_indices_and_new_modes(npf, n, N):
     dense = 2 * (rad ** (N - 1) * (rad * 4 * 6 + 4)) + 4096
     fixed = n * (-(-comb(n + N - 1, N) // 128) * 128) * 16 + n * comb(n + N - 1, N) * 32
     with npf.Plan(lam2, U2, V2, N) as p:
+        set_route(npf, p, route)
         p.set_tensor(N, A)
         p.term(N)
         p.set_option(npf.OPT_MEM_BUDGET, fixed + dense)
@@ -108,6 +116,7 @@ def test_few_upper_indices_and_new_modes(npf, n, N):
         with pytest.raises(npf.NpfError) as e:
             p.term(N)
         assert e.value.status == npf.NPF_ERR_OOM
+        assert_route(p, route)
 
 
 def test_scratch_stays_in_the_budget(npf):

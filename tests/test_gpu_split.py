@@ -11,7 +11,7 @@ import pytest
 
 import npf_synth as S
 import oracle
-from tests._util import make_plan, rel_fro
+from tests._util import ROUTES, assert_route, make_plan, rel_fro, set_route
 
 pytestmark = pytest.mark.gpu
 TOL = {"split_bf16": 1e-10, "fp32": 1e-5}
@@ -30,26 +30,32 @@ def npf():
     return m
 
 
+@pytest.mark.parametrize("route", ROUTES)
 @pytest.mark.parametrize("prec", ["split_bf16", "fp32"])
 @pytest.mark.parametrize("seed", [0, 1, 2])
-def test_small_system(npf, prec, seed):
+def test_small_system(npf, prec, seed, route):
     sysm = S.config_small(seed, orders=(2, 3))
     with make_plan(npf, sysm, 3, prec) as p:
+        set_route(npf, p, route, prec)
         for N in (2, 3):
             ref = oracle.psiN(sysm.tensors[N], 10, N, sysm.U, sysm.V, sysm.lam, p1_block=10)
             err = rel_fro(p.term(N), ref)
             assert err < TOL[prec], (N, err)
         ref = oracle.npf_orders(sysm, 3, p1_block=10)
         assert rel_fro(p.compute(3), ref) < TOL[prec]
+        assert_route(p, route, prec)
 
 
+@pytest.mark.parametrize("route", ROUTES)
 @pytest.mark.parametrize("n,N", [(6, 4), (10, 4)])
-def test_high_order_small_n(npf, n, N):
+def test_high_order_small_n(npf, n, N, route):
     sysm = S.modal_system(n, 3 * n + N)
     sysm.tensors[N] = S.random_packed_tensor(n, N, 17 + N)
     with make_plan(npf, sysm, N, "split_bf16") as p:
+        set_route(npf, p, route)
         ref = oracle.psiN(sysm.tensors[N], n, N, sysm.U, sysm.V, sysm.lam, p1_block=n)
         assert rel_fro(p.term(N), ref) < 1e-10
+        assert_route(p, route)
 
 
 def test_slabs_small(npf):
@@ -147,9 +153,10 @@ def test_n120_order4_slabs_against_stored_oracle(npf):
             assert rel_fro(p.modal_slab(4, [int(x) for x in pre]), ref) < 1e-10
 
 
+@pytest.mark.parametrize("route", ROUTES)
 @pytest.mark.parametrize("fp64q", [0, 1])
 @pytest.mark.parametrize("detune", [0.0, 5e-9, 2e-7])
-def test_resonance_clamp(npf, fp64q, detune):
+def test_resonance_clamp(npf, fp64q, detune, route):
     """Identity eigenvectors and lambda_2 = 2 lambda_0 + detune: the denominator of (i = 2,
     p = (0, 0)) is -detune; below eps = 1e-8 it is replaced by eps (Alg. 2 step 9), above it
     divides as is. Both quotient forms of the tensor-core divide against the oracle."""
@@ -161,8 +168,10 @@ def test_resonance_clamp(npf, fp64q, detune):
     ref = oracle.psiN(A2, n, N, U, V, lam, p1_block=n)
     with npf.Plan(lam, U, V, N, precision="split_bf16") as p:
         p.set_option(npf.OPT_FP64_QUOTIENT, fp64q)
+        set_route(npf, p, route)
         p.set_tensor(N, A2)
         got = p.term(N)
+        assert_route(p, route)
     assert rel_fro(got, ref) < 1e-10, rel_fro(got, ref)
     # the resonant entry dominates: |Psi_2[2, 0]| ~ |A| / (2 max(|D|, eps))
     assert abs(ref[2, 0]) > 1e5
@@ -186,9 +195,9 @@ def _gold(name):
 
 @pytest.mark.parametrize("n,seed", [(68, 0), (80, 1)])
 def test_order4_radix128_against_stored_oracle(npf, n, seed):
-    """Order 4 above 64 states takes the row radix 128: the kernel variant without sub-blocks,
-    the mirrored first contraction, the divide epilogue with the multiplicity weights and the
-    reduction epilogue, all compared in full with the oracle's Psi_4 (term) and NPF (compute).
+    """Order 4 above 64 states takes the row radix 128: the kernel variant without sub-blocks, two
+    regathers, the divide epilogue with the multiplicity weights and the reduction epilogue, all
+    compared in full with the oracle's Psi_4 (term) and NPF (compute).
     A forced budget of three upper indices per batch runs 23 batches at n = 68."""
     path = _gold(f"n{n}_seed{seed}_order4.npz")
     if not os.path.exists(path):

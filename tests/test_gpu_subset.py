@@ -4,7 +4,7 @@ import pytest
 
 import npf_synth as S
 import oracle
-from tests._util import make_plan, rel_fro
+from tests._util import ROUTES, assert_route, make_plan, rel_fro, set_route
 
 pytestmark = pytest.mark.gpu
 TOL = 1e-10
@@ -18,12 +18,14 @@ def npf():
     return m
 
 
+@pytest.mark.parametrize("route", ROUTES)
 @pytest.mark.parametrize("n,N,m", [(10, 3, 4), (60, 3, 20), (20, 4, 7)])
-def test_subset_term_and_npf(npf, n, N, m):
+def test_subset_term_and_npf(npf, n, N, m, route):
     sysm = S.config_blocks(n, seed=n + N, orders=(N,)) if n % 4 == 0 else S.config_small(1, orders=(N,))
     modes = np.random.default_rng(n * 10 + N).choice(n, m, replace=False)   # scrambled order
     ref = oracle.psiN_subset(sysm.tensors[N], n, N, sysm.U, sysm.V, sysm.lam, modes)
     with make_plan(npf, sysm, N, "split_bf16") as p:
+        set_route(npf, p, route)
         p.set_mode_subset(modes)
         got = p.term(N)
         assert rel_fro(got, ref) < TOL, rel_fro(got, ref)
@@ -35,6 +37,7 @@ def test_subset_term_and_npf(npf, n, N, m):
         p.set_mode_subset(None)
         full = oracle.psiN(sysm.tensors[N], n, N, sysm.U, sysm.V, sysm.lam, p1_block=n)
         assert rel_fro(p.term(N), full) < TOL
+        assert_route(p, route)
 
 
 def test_subset_of_all_modes_in_any_order(npf):

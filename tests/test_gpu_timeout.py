@@ -25,6 +25,7 @@ def test_bounded_wait_reports_timeout_and_recovers(npf):
     sysm = S.config_small(0, orders=(2,))
     ref = oracle.psiN(sysm.tensors[2], 10, 2, sysm.U, sysm.V, sysm.lam, p1_block=10)
     with make_plan(npf, sysm, 2, "split_bf16") as p:
+        p.set_option(npf.OPT_SLICES, 6)   # the tensor-core route at this size
         p.set_option(npf.OPT_DEBUG_STALL, 1)
         t0 = time.time()
         with pytest.raises(npf.NpfError) as e:
