@@ -40,10 +40,12 @@ def _fma(a, b, c):
     return (a.astype(x) * np.asarray(b, x) + c.astype(x)).astype(np.float32)
 
 
-@pytest.mark.parametrize("widths,rows", [([4, 48, 9], 1), ([5, 16, 32, 13], 64), ([4, 256, 64], 33)])
-def test_adam_steps_are_exact(widths, rows):
+@pytest.mark.parametrize("widths,rows,scale", [([4, 48, 9], 1, 1.0), ([5, 16, 32, 13], 64, 1.0), ([4, 256, 64], 33, 1.0),
+                                               ([4, 48, 9], 3, 1e-14), ([4, 48, 9], 3, 1e-22)])
+def test_adam_steps_are_exact(widths, rows, scale):
     """Adam's arithmetic bit for bit: FP32, every operation rounded to nearest, the moments' new terms
-    fused with their sums, two true divisions by the bias corrections. With equal rows the order of a
+    fused with their sums, true divisions (the inputs' scale brings the first layer's moments to the ends
+    of the range: squares below 2^-100 and below the normal numbers). With equal rows the order of a
     batch does not matter, so each step's gradient is npf_mlp_loss_grad's."""
     from paper_2509_08968_gb300 import build
     build.build()
@@ -51,13 +53,13 @@ def test_adam_steps_are_exact(widths, rows):
     from paper_2509_08968_gb300.surrogate import init_weights
     rng = np.random.default_rng(7 + rows)
     w = init_weights(widths, 2, 6)
-    X = np.repeat(rng.uniform(-1, 1, (1, widths[0])).astype(np.float32), rows, 0)
+    X = np.repeat((scale * rng.uniform(-1, 1, (1, widths[0]))).astype(np.float32), rows, 0)
     T = np.repeat(rng.standard_normal((1, widths[-1])).astype(np.float32), rows, 0)
     f = np.float32
     b1, b2, one = f(0.9), f(0.999), f(1.0)
     m, v = np.zeros_like(w), np.zeros_like(w)
     with Mlp(widths, w) as net:
-        for k in range(1, 5):
+        for k in range(1, 13):
             _, g = net.loss_grad(X, T)
             assert (g == 0).any() and (g != 0).any()
             net.train(X, T, 1, rows, 1e-2, seed=k)
