@@ -92,6 +92,13 @@ __device__ __forceinline__ long long shift_full(long long V, int sh)
 // 2^e for |e| < 1000 (double) / |e| < 127 (float)
 __device__ __forceinline__ double pow2d(int e) { return __longlong_as_double((long long)(1023 + e) << 52); }
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((127 + e) << 23); }
+// x 2^e for any e
+__device__ __forceinline__ double2 times_pow2(double2 x, int e)
+{
+    if (e <= -1000 || e >= 1000) return make_double2(scalbn(x.x, e), scalbn(x.y, e));
+    const double f = pow2d(e);
+    return make_double2(x.x * f, x.y * f);
+}
 
 // BF16 bits of d * 2^(-8 s) for an integer digit |d| <= 128 (exact).
 __device__ __forceinline__ uint32_t digit_bf16(int d, int s)
@@ -433,7 +440,11 @@ struct RowArgs {
     // EPI_REDUCE: rows are the sorted tuples (p_1 <= .. <= p_{N-1}) in colexicographic rank
     const uint32_t* tuples;  // 8 bits per index
     const float4* wpre;      // W[p_1][k] W[p_2][k] at k * ldw + the pair's colex rank (orders 3 and 4), as
-    int64_t ldw;             // double-float complex: the 32 rows of a warp read one run
+    int64_t ldw;             // double-float complex: the 32 rows of a warp read one run. Weights come
+                             // without their column's exponent eb[k], and G (of the order of
+                             // V^(2 - N)) with (N - 2) ev[k] added; the sums take both up in FP64, so
+                             // that eigenvectors of any normalisation keep to FP32's range
+    const int* ev;           // column exponents of the left eigenvectors (eb, unless W is another matrix)
     const int* tiles;        // the tiles that run (nullptr: every tile, skipped ones tested)
     const unsigned* ntiles_run;   // their count
     int kout;            // K entries written per row of the next operand (whole chunks of it)
@@ -449,7 +460,7 @@ struct RowArgs {
     double2* out_f64;    // EPI_SLAB: out[i * n + q]; EPI_REDUCE: Psi_N
     // EPI_DIVIDE / EPI_SLAB / EPI_REDUCE
     const double2* lam;
-    const float4* psi_df;    // the reduction weights W[p][k] (psi_{p k}) as double-float, at k*n + p
+    const float4* psi_df;    // the reduction weights W[p][k] (psi_{p k}) as double-float, at k*n + p (less eb[k])
     int i0;
     double invfact, eps;
     int divide;
@@ -860,7 +871,8 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
             float sg[2][6];
             bool row_in[2];
             int vcols = min(bnc, args.ncv - qbase);
-            const int ebv = st < 32 && st < bnc ? args.eb[qbase + st] : 0;
+            int ebv = st < 32 && st < bnc ? args.eb[qbase + st] : 0;
+            if (MODE == EPI_REDUCE && st < 32 && st < bnc) ebv += (N - 2) * args.ev[qbase + st];
             const int err = st == 0 && (t & 7) == 0 ? *(volatile int*)args.err : 0;
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
@@ -1024,6 +1036,8 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                         const float4 x = __ldg(args.psi_df + qc * n + red_w);
                         v = cmul(v, make_double2((double)x.x + (double)x.y, (double)x.z + (double)x.w));
                     }
+                    // the exponents of the N - 1 weights, and those taken from G
+                    v = times_pow2(v, (N - 1) * args.eb[qc] - (N - 2) * args.ev[qc]);
                     const int64_t at = (int64_t)(args.i0 + red_outer) * n + qc;
                     atomicAdd(&args.out_f64[at].x, -v.x);
                     atomicAdd(&args.out_f64[at].y, -v.y);
@@ -1417,8 +1431,8 @@ __global__ void k_zero_heads(int N, int nm, int kc, int lg, int Q, int nouter, c
 
 // Start of a term: the output (zeroed unless the term is added to it), the exponents of S, the error
 // flag (nullptr: a batch's, or one that holds earlier orders), and where they exist the pairs' weights
-// wpre[k][t] = W[p_1][k] W[p_2][k] (FP64 products as double-float complex) and the reduction rows'
-// heads (when their buffer is the reduction's own).
+// wpre[k][t] = W[p_1][k] W[p_2][k] 2^(-2 we[k]) (FP64 products as double-float complex) and the reduction
+// rows' heads (when their buffer is the reduction's own).
 struct TermInit {
     double2* out;
     int64_t cells;
@@ -1426,6 +1440,7 @@ struct TermInit {
     int n, nm;
     int* err;
     const double2* W;
+    const int* we;           // exponents of W's columns
     const uint32_t* pairs;
     int64_t npairs;
     float4* wpre;
@@ -1446,7 +1461,8 @@ __global__ void k_term_init(const __grid_constant__ TermInit a)
     for (int64_t t = t0; t < a.npairs * a.n; t += step) {
         const int k = (int)(t / a.npairs);
         const uint32_t p = a.pairs[t - k * a.npairs];
-        const double2 w = cmul(a.W[(int64_t)(p & 255u) * a.n + k], a.W[(int64_t)((p >> 8) & 255u) * a.n + k]);
+        const double2 w = times_pow2(cmul(a.W[(int64_t)(p & 255u) * a.n + k], a.W[(int64_t)((p >> 8) & 255u) * a.n + k]),
+                                     -2 * a.we[k]);
         const float rh = (float)w.x, ih = (float)w.y;
         a.wpre[t] = make_float4(rh, (float)(w.x - rh), ih, (float)(w.y - ih));
     }
@@ -1627,12 +1643,12 @@ static __global__ void k_slot_rows(int N, int count, const uint32_t* __restrict_
     sum[5 * count + idx] = b.c;
 }
 
-// W transposed, as double-float complex (Re hi, Re lo, Im hi, Im lo).
-static __global__ void k_to_df(int n, const double2* __restrict__ W, float4* __restrict__ out)
+// W transposed and less the exponent of its column, as double-float complex (Re hi, Re lo, Im hi, Im lo).
+static __global__ void k_to_df(int n, const double2* __restrict__ W, const int* __restrict__ we, float4* __restrict__ out)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n * n) return;
-    const double2 w = W[(t % n) * n + t / n];
+    const double2 w = times_pow2(W[(t % n) * n + t / n], -we[t / n]);
     const float rh = (float)w.x, ih = (float)w.y;
     out[t] = make_float4(rh, (float)(w.x - rh), ih, (float)(w.y - ih));
 }
@@ -1907,13 +1923,13 @@ static void fixed_matrix(Plan& p, int S, const double2* m, bool trans, bool comp
     NPF_CUDA(cudaGetLastError());
 }
 
-// The reduction's weights transposed, in double-float.
-static void to_df(Plan& p, const double2* m, float4*& out)
+// The reduction's weights transposed, in double-float (ex: their columns' exponents).
+static void to_df(Plan& p, const double2* m, const int* ex, float4*& out)
 {
     const int count = p.n * p.n;
     if (!out) NPF_CUDA(cudaMalloc(&out, (size_t)count * sizeof(float4)));
     LaunchScope ls(&p.prof, "split_to_df", p.stream);
-    k_to_df<<<(count + 255) / 256, 256, 0, p.stream>>>(p.n, m, out);
+    k_to_df<<<(count + 255) / 256, 256, 0, p.stream>>>(p.n, m, ex, out);
     NPF_CUDA(cudaGetLastError());
 }
 
@@ -1924,7 +1940,7 @@ static void fill_fixed(Plan& p, SplitOperand* so)
     fixed_matrix(p, S, p.d_U, false, true, so->phi, so->phi_e);      // K index a, column p: phi_{a p}
     fixed_matrix(p, S, p.d_V, true, false, so->psir, so->psir_e);    // real K index j, column i: psi_{i j}
     fixed_matrix(p, S, p.d_V, false, true, so->red, so->red_e);      // K index p, column k: psi_{p k}
-    to_df(p, p.d_V, so->psi_df);
+    to_df(p, p.d_V, so->red_e, so->psi_df);
 }
 
 static SplitOperand& prepare(Plan& p)
@@ -1947,7 +1963,7 @@ static SplitOperand& prepare(Plan& p)
 static void prepare_weights(Plan& p, SplitOperand& so, const double2* dW)
 {
     fixed_matrix(p, so.S, dW, false, true, so.wred, so.wred_e);
-    to_df(p, dW, so.w_df);
+    to_df(p, dW, so.wred_e, so.w_df);
 }
 
 // The slot tables of the order from the plan's eigenvalues.
@@ -2382,6 +2398,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
         a.nm = nm;
         a.err = p.err_override || (p.defer_err && p.err_live) ? nullptr : err;
         a.W = W ? W : p.d_V;
+        a.we = W ? so.wred_e : so.red_e;
         a.pairs = so.ptup[2];
         a.npairs = Q2;
         a.wpre = wpre;
@@ -2548,6 +2565,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
         a.kfrom = 1;                       // K = p_N >= the tile's smallest p_{N-1}
         a.ea = ER;
         a.eb = W ? so.wred_e : so.red_e;
+        a.ev = so.red_e;
         a.R = Qc;
         a.RB = (int)((Qc + NP - 1) / NP);
         a.num_tiles = (int64_t)cur * a.RB * a.ncol_tiles;

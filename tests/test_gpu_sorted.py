@@ -119,6 +119,32 @@ def test_few_upper_indices_and_new_modes(npf, n, N, route):
         assert_route(p, route)
 
 
+@pytest.mark.parametrize("n,N,e", [(40, 2, 100), (9, 3, 100), (40, 3, 100), (70, 3, 100), (11, 4, 100), (35, 4, 100)])
+def test_any_normalisation_of_the_eigenvectors(npf, n, N, e):
+    """U 2^x, V 2^-x is the same system (Psi_N scales as V): the products of weights, 2^(-(N - 1) x), leave
+    FP32's range, the sums over them must not."""
+    lam, U, V, A = _odd_system(n, N, 30 * n + N)
+    ref = oracle.psiN(A, n, N, U, V, lam, p1_block=8)
+    for x in (e, -e):
+        with npf.Plan(lam, U * 2.0 ** x, V * 2.0 ** -x, N) as p:
+            set_route(npf, p, "tensor")
+            p.set_tensor(N, A)
+            assert rel_fro(p.term(N) * 2.0 ** x, ref) < 1e-10
+            assert_route(p, "tensor")
+
+
+def test_interaction_of_a_tiny_excitation(npf):
+    """pN3 is of the order delta^3 (1e-36), far below FP32's range for its low parts."""
+    n, delta = 27, 1e-12
+    lam, U, V, A = _odd_system(n, 3, 8)
+    s = SimpleNamespace(n=n, lam=lam, U=U, V=V, tensors={3: A})
+    ref = oracle.interaction_npfs(s, 3, delta)
+    with npf.Plan(lam, U, V, 3) as p:
+        p.set_tensor(3, A)
+        got = p.interaction(3, delta)
+    assert rel_fro(got[2], ref[2]) < 1e-10 and rel_fro(got[0], ref[0]) < 1e-10
+
+
 def test_scratch_stays_in_the_budget(npf):
     """The upper indices of a batch are counted by the rows they take, which at 2 slices, order 3 and
     n = 32, 64, 128 are more than the dense rows that a budget is accepted by (17 MB here)."""
