@@ -225,6 +225,7 @@ int tuned_tile(Plan& p, int N)
             NPF_CUDA(cudaEventElapsedTime(&ms, e0, e1));
             if (ms < best) { best = ms; best_tile = t; }
         }
+        npf::split_check(p);   // (a pipeline that gave up has timed nothing)
     } catch (...) {
         p.tile_n = 0;
         cudaEventDestroy(e0);

@@ -59,3 +59,21 @@ def test_a_failed_call_leaves_its_outputs_alone(npf):
         p.set_option(npf.OPT_DEBUG_STALL, 0)
         assert rel_fro(p.interaction(3, 0.1), good) < 1e-10
         assert rel_fro(good, oracle.interaction_npfs(sysm, 3, 0.1)) < 1e-10
+
+
+def test_a_failed_tuning_is_not_kept(npf):
+    """The autotuner's terms that gave up leave no tile width behind for the process."""
+    n = 22
+    sysm = S.modal_system(n, 5)
+    sysm.tensors[2] = S.random_packed_tensor(n, 2, 6)
+    with make_plan(npf, sysm, 2, "split_bf16") as p:
+        p.set_option(npf.OPT_TILE_N, 0)
+        p.set_option(npf.OPT_DEBUG_STALL, 1)
+        with pytest.raises(npf.NpfError) as e:
+            p.term(2)
+        assert e.value.status == npf.NPF_ERR_TIMEOUT
+        assert npf.tuned_tile(n, 2, "split_bf16") == 0
+        p.set_option(npf.OPT_DEBUG_STALL, 0)
+        ref = oracle.psiN(sysm.tensors[2], n, 2, sysm.U, sysm.V, sysm.lam, p1_block=n)
+        assert rel_fro(p.term(2), ref) < 1e-10
+        assert npf.tuned_tile(n, 2, "split_bf16") in (16, 32)
