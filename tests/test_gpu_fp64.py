@@ -94,11 +94,14 @@ def test_error_codes(npf):
     assert e.value.status == npf.NPF_ERR_NOT_INVERSE
 
 
+@pytest.mark.parametrize("n", [10, 24, 28])
 @pytest.mark.parametrize("value", [np.nan, np.inf, 1j * np.nan])
-def test_modal_data_that_are_no_numbers_are_refused(npf, value):
+def test_modal_data_that_are_no_numbers_are_refused(npf, value, n):
     """A NaN or infinity in U or V makes entries of V U - I NaN: no inverse, and a refused set_modes
-    leaves the plan as it was."""
-    sysm = S.config_small(0, orders=(2,))
+    leaves the plan as it was. The check runs on the host up to n = 24; on both sides of it an error just
+    above the tolerance is refused and one below is not."""
+    sysm = S.modal_system(n, 7)
+    sysm.tensors[2] = S.random_packed_tensor(n, 2, 8)
     with npf.Plan(sysm.lam, sysm.U, sysm.V, 2, precision="fp64") as p:
         p.set_tensor(2, sysm.tensors[2])
         before = p.compute(2)
@@ -110,3 +113,13 @@ def test_modal_data_that_are_no_numbers_are_refused(npf, value):
                     call()
                 assert e.value.status == npf.NPF_ERR_NOT_INVERSE
         assert np.array_equal(p.compute(2), before)
+        row = np.linalg.norm(sysm.U[4], np.inf)   # V[3, 4] + d changes V U by up to d row
+        for d, status in ((2e-8 / row, npf.NPF_ERR_NOT_INVERSE), (0.5e-8 / row, npf.NPF_OK)):
+            V = sysm.V.copy()
+            V[3, 4] += d
+            try:
+                p.set_modes(sysm.lam, sysm.U, V)
+                got = npf.NPF_OK
+            except npf.NpfError as e:
+                got = e.status
+            assert got == status
