@@ -168,11 +168,12 @@ void launch_add(Plan& p, double2* acc, const double2* x, int64_t count)
     NPF_CUDA(cudaGetLastError());
 }
 
+// y = a x + b y (b = 0: y is only written)
 __global__ void k_axpy(double2* y, double a, const double2* x, double b, int64_t count)
 {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
          i += (int64_t)gridDim.x * blockDim.x) {
-        const double2 u = x[i], v = y[i];
+        const double2 u = x[i], v = b != 0.0 ? y[i] : make_double2(0.0, 0.0);
         y[i] = make_double2(fma(a, u.x, b * v.x), fma(a, u.y, b * v.y));
     }
 }

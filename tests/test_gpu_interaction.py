@@ -51,3 +51,20 @@ def test_missing_order_is_zero(npf, route):
         assert_route(p, route)
     assert np.all(got[1] == 0)
     assert rel_fro(got[2], ref[2]) < 1e-10 and rel_fro(got[0], ref[0]) < 1e-10
+
+
+@pytest.mark.parametrize("prec", ["split_bf16", "fp64"])
+def test_nothing_is_left_of_an_earlier_call(npf, prec):
+    """z(0) is formed anew: entries that an earlier call left as NaN (a tensor that held some) do not
+    reach a later interaction."""
+    sysm = S.config_small(1, orders=(2, 3))
+    ref = oracle.interaction_npfs(sysm, 3, 0.1)
+    bad = sysm.tensors[2].copy()
+    bad[0, 0] = np.nan
+    with make_plan(npf, sysm, 3, prec) as p:
+        p.set_tensor(2, bad)
+        assert np.isnan(p.compute(2)).any()
+        p.set_tensor(2, sysm.tensors[2])
+        got = p.interaction(3, 0.1)
+        for M in range(3):
+            assert rel_fro(got[M], ref[M]) < TOL[prec]
