@@ -96,9 +96,11 @@ enum npf_option {
 };
 
 /* Arithmetic of the dense contraction. In every form the resonance denominators are formed
- * exactly from the FP64 eigenvalues and the Psi_N sums and the NPF finish are FP64; the quotient
- * h = C / D is native FP64 in the FP64 form and double-float in the tensor-core forms (native FP64
- * with NPF_OPT_FP64_QUOTIENT). */
+ * exactly from the FP64 eigenvalues and the NPF finish is FP64; the quotient h = C / D is native FP64
+ * in the FP64 form and double-float in the tensor-core forms (native FP64 with
+ * NPF_OPT_FP64_QUOTIENT). The Psi_N sums are FP64 in the FP64 form; in the tensor-core forms a thread
+ * adds its weighted entries of up to 47 row blocks in double-float (about 47 bits) before they go into
+ * the FP64 sum, which leaves the forms' errors as FP64 sums of every block do. */
 enum npf_precision {
     NPF_PREC_FP64 = 0,        /* native FP64 (CUDA-core DFMA) contraction */
     NPF_PREC_SPLIT_BF16 = 1,  /* FP64-emulating BF16 slices on tcgen05 tensor cores, FP32
@@ -205,8 +207,8 @@ int npf_finish_terms(npf_handle* h, int count, const npf_c128* terms, npf_c128* 
 /* Rows i_lo <= i < i_hi of Psi_N (out[i*n + k], the other rows zero; host or device): the upper
  * index is independent across rows (Eq. 7 sums over the lower indices only), so disjoint row
  * ranges computed separately -- on several GPUs, or resumed after an interruption -- add up to
- * npf_get_term. The tensor-core forms only form those rows; the FP64 form runs its mode
- * products in full and reduces only those rows. Not available with a mode subset. */
+ * npf_get_term. The tensor-core forms, and the FP64 form where it runs in shared memory, only
+ * form those rows; else the FP64 form runs its mode products in full and reduces only those rows. Not available with a mode subset. */
 int npf_get_term_rows(npf_handle* h, int order, int i_lo, int i_hi, npf_c128* out);
 
 /* One modal slab h^i_{prefix, q}: out[i*n + q] for the fixed prefix p_1..p_{N-1} (N-1 ints in

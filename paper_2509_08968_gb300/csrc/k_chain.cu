@@ -15,11 +15,12 @@
 // Bound by the FP64 pipe (2 fused multiply-adds per clock and SM): a complex multiply-add takes 2
 // clocks an SM whatever feeds it, so the operands come straight from shared memory and L1 and the
 // index arithmetic of the sorted gathers hides behind them. Against the dense FP64 chain
-// (k_fp64.cu) it does a third of the operations at order 3: n = 60, orders 2 and 3, 28.4 -> 9.1 ms
-// (2.1 of them for tail blocks and latency); n = 8, order 3, 184 -> 59 us. Against the tensor-core
-// chain (eight launches and more an order) it is two launches, which is what small systems wait
-// for: n = 10, orders 2 and 3, 243 -> 62 us. One block per (i, p_N) keeps 24 n^2 bytes at order 3, so
-// that two blocks share an SM up to n = 66.
+// (k_fp64.cu) it does a third of the operations at order 3: n = 60, orders 2 and 3, 28.4 -> 9.0 ms
+// (8.4 at the rate of cuBLAS's DGEMM); n = 8, order 3, 184 -> 59 us. It is faster wherever it fits in shared
+// memory: order 2, n = 252 (of 255) 101 -> 62 ms; order 3, n = 66 and 92 (of 93) 58 -> 14 and 213 -> 69
+// ms; order 4, n = 36 (of 37) 154 -> 15 ms. Against the tensor-core chain (eight launches and more an order)
+// it is two launches, which is what small systems wait for: n = 10, orders 2 and 3, 243 -> 62 us. One
+// block per (i, p_N) keeps 26 n^2 bytes at order 3, so that two blocks share an SM up to n = 65.
 #include <algorithm>
 
 #include "k_device.cuh"
@@ -283,6 +284,9 @@ __global__ void __launch_bounds__(THREADS) k_chain(ChainArgs a)
     if (tid == 0) a.count[row] = 0u;
 }
 
+// Blocks per (i, p_4), which share its p_3: few blocks are too short a grid, many repeat the first two
+// stages. One / two / four take 91 / 58 / 55 us at n = 8, 156 / 141 / 129 at 12, 305 / 255 / 203 at 14, 610 /
+// 490 / 597 at 18, 921 / 826 / 942 at 20, 2102 / 2014 / 2283 at 24, 8725 / 9439 / 11850 at 32.
 int chunks_for(int N, int n) { return N < 4 ? 1 : n <= 12 ? 4 : n <= 20 ? 2 : 1; }
 
 size_t smem_bytes(int N, int n, int nm)

@@ -684,13 +684,11 @@ static __global__ void k_tile_list(RowArgs a, int lg, int* __restrict__ list, un
 //   warps 18, 19     : set-up: the next tile's tables (row exponents and indices, eigenvalue sums,
 //                      output rows) into the other of two buffers. Chains of dependent global loads,
 //                      they took 2 to 7 us a tile in front of the epilogue.
-// Bound per 32-column tile of a mode product at n = 120: 7.1 us, 5.4 of them its 315 MMAs (without any
-// TMA load the launches take 2.64 ms instead of 3.06); shared memory carries 1.08 MB of MMA operand
-// reads and 0.59 MB of TMA writes meanwhile (6.3 us at 128 bytes a clock). Below n = 64 and in the
-// divide and the reduction the epilogue bounds it. 32-column tiles in every mode: an epilogue and the next
-// tile's MMAs overlap, which one 64-column tile with all 512 TMEM columns (and a level-3 hold in
-// shared memory) allowed in part only: divide at n = 120, order 3, 1.83 -> 1.45 ms a call (1.39 now) (24 us a
-// 64-column tile before, 13 us a 32-column one now, of which the kept columns are fewer).
+// Bound per 32-column tile of a mode product at n = 120: 7.1 us, 5.4 of them its 315 MMAs; shared memory
+// carries 1.08 MB of MMA operand reads and 0.59 MB of TMA writes meanwhile (6.3 us at 128 bytes a
+// clock). Below n = 64 and in the divide and the reduction the epilogue bounds it. Tiles are 32 columns
+// wide in every mode, so that two accumulator sets fit TMEM and an epilogue overlaps the next tile's
+// MMAs: divide at n = 120, order 3, 1.39 ms a call against 1.83 with 64-column tiles in turn.
 template <int S, int MODE, bool SUBB>
 __global__ void __launch_bounds__(ROW_THREADS, 1)
     k_rows(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, RowArgs args)
@@ -1203,10 +1201,10 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
 #pragma unroll 1
                 for (int h = 0; h < 4; ++h) {
                     const int c2 = cbeg + 2 * h;
-                    // the weights of these columns, asked for before the accumulators (of a valid row and
-                    // column in any case): 1.44 -> 1.17 ms a call at n = 120, order 3 (n = 60, order 4: 1.72
-                    // -> 1.62); a round ahead of them spilled registers (1.73). Order 3: the whole weight W[p_1][k] W[p_2][k]; order 4: that,
-                    // and W[p_3][k] unless it is left to the sum
+                    // the weights of these columns, asked for before the accumulators (1.17 ms a call at n =
+                    // 120, order 3, against 1.44 behind them), of a valid row and column in any case.
+                    // Order 3: the whole weight W[p_1][k] W[p_2][k]; order 4: that, and W[p_3][k] unless it
+                    // is left to the sum
                     float4 w4[2];
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
@@ -1397,8 +1395,8 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
 // Zeros in the reduction rows' K entries that its tiles read but the divide does not write: from
 // the chunk of the tile's smallest p_{N-1} up to the row's own p_{N-1}, and from nm to the operand's
 // inner extent. It runs before the divide and clears whole 32-byte sectors (8 entries, also those that
-// the divide then writes): after it, entry by entry, each sector was a partial write that had to be
-// read from HBM first (0.52 -> 0.18 ms at n = 60, order 4; 5.8 -> 2.4 ms at n = 120, orders 3 and 4).
+// the divide then writes), since a partly written sector is read from HBM first: 0.18 ms at n = 60, order
+// 4, against 0.52 entry by entry behind the divide.
 // kc: complex K entries a chunk (a multiple of 8). t: one of 8 threads a row.
 template <int S>
 __device__ __forceinline__ void zero_head(int64_t t, int N, int nm, int kc, int lg, int Q, const uint32_t* __restrict__ tuples,
@@ -1483,10 +1481,9 @@ __global__ void k_term_init(const __grid_constant__ TermInit a)
 // share sectors. A block takes one outer index and a strided share of its rows, so that nothing
 // but the gather, the shifts and the digits is left per row: a rank is one of M + 1 row constants
 // plus a binomial of the lane's a, kept in registers, and a plane's address a 32-bit offset from the
-// block's. Computing whole ranks and 64-bit addresses per entry, a row a warp: 5.50 against 4.51 ms at
-// n = 60, order 4; 1.16 against 1.10 at n = 120, order 3 (6.65 GB: 6.0 TB/s). What bounds it is mixed:
-// HBM writes (4 S bytes an entry against 16 read per source entry) at n = 120, the scattered half of
-// the gathers and the integer instructions (IPC 0.65 a scheduler) below.
+// block's (4.51 ms at n = 60, order 4, against 5.50 with whole ranks and 64-bit addresses per entry).
+// Bound by HBM writes at n = 120 (4 S bytes an entry against 16 read per source entry: 1.10 ms for
+// 6.65 GB at order 3), below by the scattered half of the gathers and the integer instructions.
 template <int S, int M, int SRC, int CH, int RW>
 __global__ void __launch_bounds__(256)
     k_regather(const longlong2* __restrict__ V, int64_t Rsrc, int n, int nm, int nt, const uint32_t* __restrict__ ttup,
@@ -2262,8 +2259,8 @@ static void launch_rows(Plan& p, const char* name, const DataOp& A, const FixedO
 static double factorial(int N) { double f = 1; for (int t = 2; t <= N; ++t) f *= t; return f; }
 
 // The regather's variant: 32-entry chunks of a row (CH), and the rows that a warp takes at a time (RW),
-// so that three to six gathers are in flight. Twice as many rows were slower (n = 60, order 4: 4.51
-// against 4.88 ms; n = 120, order 3: 1.10 against 1.20), one row less slower at n = 60 and 75.
+// so that three to six gathers are in flight (twice the rows: n = 60, order 4, 4.88 ms against
+// 4.51, n = 120, order 3, 1.20 against 1.10; one row less was slower too).
 static constexpr int regather_rows(int ch) { return ch == 1 ? 4 : ch <= 3 ? 2 : 1; }
 template <int S, int M, int SRC>
 static decltype(&k_regather<S, M, SRC, 4, regather_rows(4)>) regather_kernel(int n)
@@ -2331,7 +2328,8 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     const int rlo = std::max(0, p.row_lo);                       // upper-index rows to form
     const int rhi = p.row_hi < 0 ? nm : std::min(p.row_hi, nm);
     // One batch of a small system: the reduction's rows get a buffer of their own, so that the first
-    // launch can clear their heads.
+    // launch can clear their heads (87 us a term against 90 at n = 60, order 2, 218 against 220 at n = 20,
+    // order 4; above 64 MB it is less than 1%: 568 against 575 at n = 60, order 3).
     const size_t red_bytes = (size_t)nm * Qc * row_bytes;
     const size_t fixed_bytes = s_bytes + wbytes + 10 * 256 + 1024;   // (and alignment, sE)
     const size_t all_bytes = fixed_bytes + (size_t)nm * per_i;
@@ -2356,7 +2354,9 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
         own_red &= ib == nm && all_bytes + red_bytes <= budget;
         keep &= ib == nm && all_bytes + red_bytes <= budget;
     }
-    // kept rows: up to 256 MB an order, in a buffer of the plan that a repeated interaction finds again
+    // kept rows, in a buffer of the plan that a repeated interaction finds again: an interaction of n = 60,
+    // orders 2 and 3, takes 802 us with them and 1309 without, and gains as much at every size (8.5 -> 4.9
+    // ms at n = 100, where they take 1.5 GB); 256 MB an order bounds the memory
     if (keep) {
         const size_t eb = (size_t)nm * Qc * sizeof(int);
         if (so.kept_bytes[N] != red_bytes + eb) {
