@@ -41,18 +41,21 @@ def _fma(a, b, c):
 
 
 @pytest.mark.parametrize("widths,rows,scale", [([4, 48, 9], 1, 1.0), ([5, 16, 32, 13], 64, 1.0), ([4, 256, 64], 33, 1.0),
-                                               ([4, 48, 9], 3, 1e-14), ([4, 48, 9], 3, 1e-22)])
+                                               ([4, 48, 9], 3, 1e-14), ([4, 48, 9], 3, 1e-22), ([4, 48, 9], 3, 1e9)])
 def test_adam_steps_are_exact(widths, rows, scale):
     """Adam's arithmetic bit for bit: FP32, every operation rounded to nearest, the moments' new terms
     fused with their sums, true divisions (the inputs' scale brings the first layer's moments to the ends
-    of the range: squares below 2^-100 and below the normal numbers). With equal rows the order of a
-    batch does not matter, so each step's gradient is npf_mlp_loss_grad's."""
+    of the range: squares below 2^-100, below the normal numbers and above 2^50; some weights start at
+    zero or next to it, where the smallest update counts). With equal rows the order of a batch does not
+    matter, so each step's gradient is npf_mlp_loss_grad's."""
     from paper_2509_08968_gb300 import build
     build.build()
     from paper_2509_08968_gb300.mlp import Mlp
     from paper_2509_08968_gb300.surrogate import init_weights
     rng = np.random.default_rng(7 + rows)
     w = init_weights(widths, 2, 6)
+    w[:, ::7] = 0
+    w[:, 3::7] *= np.float32(1e-20)
     X = np.repeat((scale * rng.uniform(-1, 1, (1, widths[0]))).astype(np.float32), rows, 0)
     T = np.repeat(rng.standard_normal((1, widths[-1])).astype(np.float32), rows, 0)
     f = np.float32
