@@ -441,10 +441,12 @@ struct RowArgs {
     const uint32_t* tuples;  // 8 bits per index
     const float4* wpre;      // W[p_1][k] W[p_2][k] at k * ldw + the pair's colex rank (orders 3 and 4), as
     int64_t ldw;             // double-float complex: the 32 rows of a warp read one run. Weights come
-                             // without their column's exponent eb[k], and G (of the order of
-                             // V^(2 - N)) with (N - 2) ev[k] added; the sums take both up in FP64, so
-                             // that eigenvectors of any normalisation keep to FP32's range
+                             // without their column's exponent eb[k], and G (of the order of A
+                             // V^(2 - N), S of A V) with (N - 1) ev[k] - es[i] added; the sums take both
+                             // up in FP64, so that eigenvectors of any normalisation and tensors of
+                             // any scale keep to FP32's range
     const int* ev;           // column exponents of the left eigenvectors (eb, unless W is another matrix)
+    const int* es;           // exponents of S by upper index
     const int* tiles;        // the tiles that run (nullptr: every tile, skipped ones tested)
     const unsigned* ntiles_run;   // their count
     int kout;            // K entries written per row of the next operand (whole chunks of it)
@@ -870,7 +872,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
             bool row_in[2];
             int vcols = min(bnc, args.ncv - qbase);
             int ebv = st < 32 && st < bnc ? args.eb[qbase + st] : 0;
-            if (MODE == EPI_REDUCE && st < 32 && st < bnc) ebv += (N - 2) * args.ev[qbase + st];
+            if (MODE == EPI_REDUCE && st < 32 && st < bnc) ebv += (N - 1) * args.ev[qbase + st] - args.es[args.i0 + tp.outer];
             const int err = st == 0 && (t & 7) == 0 ? *(volatile int*)args.err : 0;
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
@@ -1035,7 +1037,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1)
                         v = cmul(v, make_double2((double)x.x + (double)x.y, (double)x.z + (double)x.w));
                     }
                     // the exponents of the N - 1 weights, and those taken from G
-                    v = times_pow2(v, (N - 1) * args.eb[qc] - (N - 2) * args.ev[qc]);
+                    v = times_pow2(v, (N - 1) * (args.eb[qc] - args.ev[qc]) + args.es[args.i0 + red_outer]);
                     const int64_t at = (int64_t)(args.i0 + red_outer) * n + qc;
                     atomicAdd(&args.out_f64[at].x, -v.x);
                     atomicAdd(&args.out_f64[at].y, -v.y);
@@ -1434,7 +1436,7 @@ __global__ void k_zero_heads(int N, int nm, int kc, int lg, int Q, int nouter, c
 struct TermInit {
     double2* out;
     int64_t cells;
-    int* sE;
+    int* sE;                 // (nullptr: S stays)
     int n, nm;
     int* err;
     const double2* W;
@@ -1454,7 +1456,7 @@ __global__ void k_term_init(const __grid_constant__ TermInit a)
     pdl_wait();
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
     for (int64_t t = t0; t < a.cells; t += step) a.out[t] = make_double2(0.0, 0.0);
-    if (t0 < a.nm) a.sE[t0] = EXP_NONE;
+    if (t0 < a.nm && a.sE) a.sE[t0] = EXP_NONE;
     if (t0 == 0 && a.err) *a.err = 0;
     for (int64_t t = t0; t < a.npairs * a.n; t += step) {
         const int k = (int)(t / a.npairs);
@@ -2358,7 +2360,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     // orders 2 and 3, takes 802 us with them and 1309 without, and gains as much at every size (8.5 -> 4.9
     // ms at n = 100, where they take 1.5 GB); 256 MB an order bounds the memory
     if (keep) {
-        const size_t eb = (size_t)nm * Qc * sizeof(int);
+        const size_t eb = ((size_t)nm * Qc + nm) * sizeof(int);   // the rows' exponents and S's
         if (so.kept_bytes[N] != red_bytes + eb) {
             if (so.kept[N]) NPF_CUDA(cudaStreamSynchronize(p.stream));
             free_kept(so, N);
@@ -2377,7 +2379,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
     uint8_t* base = (uint8_t*)ar.base;
     auto take = [&](size_t bytes) { uint8_t* r = base; base += (bytes + 255) & ~(size_t)255; return r; };
     longlong2* Sv = (longlong2*)take(s_bytes);
-    int* sE = (int*)take(256 * sizeof(int));
+    int* sE = keep ? so.kept_e[N] + (size_t)nm * Qc : (int*)take(256 * sizeof(int));
     uint8_t* bufA = take((size_t)ib * a_per);
     uint8_t* bufB = take((size_t)ib * b_per);
     uint8_t* bufR = keep ? so.kept[N] : own_red ? take(red_bytes) : bufA;   // reduction rows
@@ -2393,7 +2395,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
         TermInit a{};
         a.out = d_out;
         a.cells = accumulate ? 0 : (int64_t)n * n;
-        a.sE = sE;
+        a.sE = again ? nullptr : sE;
         a.n = n;
         a.nm = nm;
         a.err = p.err_override || (p.defer_err && p.err_live) ? nullptr : err;
@@ -2566,6 +2568,7 @@ static void split_run(Plan& p, int N, double2* d_out, const int* prefix, const d
         a.ea = ER;
         a.eb = W ? so.wred_e : so.red_e;
         a.ev = so.red_e;
+        a.es = sE;
         a.R = Qc;
         a.RB = (int)((Qc + NP - 1) / NP);
         a.num_tiles = (int64_t)cur * a.RB * a.ncol_tiles;

@@ -133,6 +133,25 @@ def test_any_normalisation_of_the_eigenvectors(npf, n, N, e):
             assert_route(p, "tensor")
 
 
+@pytest.mark.parametrize("n,N", [(9, 2), (9, 3), (40, 3), (70, 3), (11, 4)])
+def test_any_scale_of_the_tensor(npf, n, N):
+    """Psi_N is linear in the tensor: scaled by 2^x beyond FP32's range, it is the same numbers times
+    2^x; an interaction's second reduction starts from kept rows."""
+    lam, U, V, A = _odd_system(n, N, 20 * n + N)
+    ref = oracle.psiN(A, n, N, U, V, lam, p1_block=8)
+    # far below the linear part: z(0) = 0.1 Psi, and pNN is linear in the tensor too
+    small = SimpleNamespace(n=n, lam=lam, U=U, V=V, tensors={N: A * 2.0 ** -60})
+    inter = oracle.interaction_npfs(small, N, 0.1)[N - 1] * 2.0 ** 60
+    for x in (110, -110, 300, -300):
+        with npf.Plan(lam, U, V, N) as p:
+            set_route(npf, p, "tensor")
+            p.set_tensor(N, A * 2.0 ** x)
+            assert rel_fro(p.term(N) * 2.0 ** -x, ref) < 1e-10
+            if x < 0:
+                assert rel_fro(p.interaction(N, 0.1)[N - 1] * 2.0 ** -x, inter) < 1e-10
+            assert_route(p, "tensor")
+
+
 def test_interaction_of_a_tiny_excitation(npf):
     """pN3 is of the order delta^3 (1e-36), far below FP32's range for its low parts."""
     n, delta = 27, 1e-12
